@@ -61,6 +61,7 @@ struct Sel {
     int64_t g;      // threshold gain (mode 1) / digit prefix (mode 2)
     int64_t rem;    // weight budget left for candidates with gain == g (mode 1) or with the
                     // current digit prefix (mode 2)
+    int64_t cut;    // mode 1: candidates with gain == g are approved up to this vertex id
 };
 
 enum { SEL_ALL = 0, SEL_THRESH = 1, SEL_REFINE = 2 };
@@ -96,7 +97,7 @@ struct Dev {
     int64_t *tot;           // [k] candidate weight per target block
     unsigned long long *hist;  // [k * kBins]
     Sel *sel;               // [k]
-    int64_t *tie;           // [k * n_tiles]
+    int64_t *tie;           // [k * n_tiles] weight of the candidates at the threshold gain
     int64_t *stats;         // [rounds * ST_N]
     int32_t *wq;            // [rounds * kWqPerRow] work counters of the single-instance persistent
                             // kernels (nullptr in batches: static assignment)

@@ -17,8 +17,8 @@
 //                  histogram of candidate weight by gain, scanned from the highest gain to
 //                  find the threshold gain G_t and the budget left for candidates with
 //                  gain == G_t (approval order (gain desc, id asc), inclusive prefix sums).
-//   k_tie_sum/k_tie_scan   per tile weight of the gain == G_t candidates, exclusive prefix over
-//                  tiles (tiles are in vertex-id order), so ties are approved in id order.
+//   k_tie_sum/k_tie_cut   per tile weight of the gain == G_t candidates, then the vertex id up to
+//                  which they fit the remaining budget (ties are approved in id order).
 //   k_apply        applies every approved move: Pi(u) = t, block weights, Phi(e,a)--,
 //                  Phi(e,t)++ with integer atomics, and Lambda(e), S1(e) and the objective
 //                  from the atomics' old values (each step of a pin count across 0/1/2 toggles
@@ -841,7 +841,7 @@ __global__ void __launch_bounds__(kThreads) k_select(const Dev *devs, const int2
             }
             if (tid == 0) {
                 Sel o;
-                o.mode = SEL_ALL; o.level = 0; o.g = 0; o.rem = 0;
+                o.mode = SEL_ALL; o.level = 0; o.g = 0; o.rem = 0; o.cut = 0;
                 d.sel[t] = o;
                 d.tot[t] = 0;
             }
@@ -878,6 +878,7 @@ __global__ void __launch_bounds__(kThreads) k_select(const Dev *devs, const int2
         const int fb = found_bin;
         const long long rem = cap - found_before;
         Sel o;
+        o.cut = 0;
         if (level == 0) {
             d.tot[t] = 0;
             if (fb < kBins - 1) {
@@ -940,45 +941,79 @@ __global__ void __launch_bounds__(kThreads) k_tie_sum(const Dev *devs, const int
     if (tid < d.k && thr[tid]) d.tie[(int64_t)tid * d.n_tiles + tile] = (int64_t)ts[tid];
 }
 
-// one CTA per block item: exclusive prefix of the tie weights over the tiles, in tile order
-__global__ void __launch_bounds__(1024) k_tie_scan(const Dev *devs, const int2 *items, int32_t n_items)
+// one CTA per block item with a threshold gain: the vertex id up to which the candidates at that
+// gain pass.  Their inclusive (KEY_A: exclusive) weight prefix in id order only grows, so the
+// passing ones are those up to one id: the tile where the prefix crosses the budget is found from
+// the tile sums (tiles are in id order), the id inside it from the tile's candidates.  The apply
+// step then only compares ids; rebuilding the prefix of every range that held a tie there (its
+// tile's earlier ranges read again, one candidate at a time) took 2.0 ms of the power-law
+// instance's 67.3 ms (50 M vertices, k = 64, 5 rounds) and 0.06 of the row-net one's 6.56 ms.
+template <int KEY = KEY_T>
+__global__ void __launch_bounds__(1024) k_tie_cut(const Dev *devs, const int2 *items, int32_t n_items)
 {
     __shared__ unsigned long long wt[32];
-    __shared__ unsigned long long carry;
+    __shared__ unsigned long long carry_s, cross_before;
+    __shared__ int32_t cross_tile;
+    __shared__ int32_t cut_s;
     if ((int32_t)blockIdx.x >= item_count(devs, items, n_items, 2)) return;
     int32_t t;
-    const Dev d = item_of(devs, items, blockIdx.x, t);
-    if (d.sel[t].mode != SEL_THRESH) return;
-    int64_t *row = d.tie + (int64_t)t * d.n_tiles;
-    if (threadIdx.x == 0) carry = 0;
+    const Dev &d = item_of(devs, items, blockIdx.x, t);
+    const Sel sl = d.sel[t];
+    if (sl.mode != SEL_THRESH) return;
+    const int tid = threadIdx.x;
+    const unsigned long long rem = (unsigned long long)sl.rem;
+    const int64_t *row = d.tie + (int64_t)t * d.n_tiles;
+    if (tid == 0) {
+        carry_s = 0;
+        cross_tile = -1;
+    }
     __syncthreads();
-    for (int64_t b = 0; b < d.n_tiles; b += blockDim.x) {
-        const int64_t i = b + threadIdx.x;
+    for (int32_t b = 0; b < d.n_tiles; b += (int32_t)blockDim.x) {
+        const int32_t i = b + tid;
         const unsigned long long v = i < d.n_tiles ? (unsigned long long)row[i] : 0;
-        const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-        unsigned long long x = v;
-        for (int o = 1; o < 32; o <<= 1) {
-            const unsigned long long y = __shfl_up_sync(kFull, x, o);
-            if (lane >= o) x += y;
-        }
-        if (lane == 31) wt[wid] = x;
-        __syncthreads();
-        if (wid == 0) {
-            const unsigned long long tt = wt[lane];
-            unsigned long long s = tt;
-            for (int o = 1; o < 32; o <<= 1) {
-                const unsigned long long y = __shfl_up_sync(kFull, s, o);
-                if (lane >= o) s += y;
-            }
-            wt[lane] = s - tt;
+        const unsigned long long ex = carry_s + block_scan_u64(v, wt);
+        // the tile of the candidate that first exceeds the budget: all of the earlier tiles'
+        // candidates pass, none of the later tiles' (under either rule)
+        if (ex <= rem && ex + v > rem) {
+            cross_tile = i;
+            cross_before = ex;
         }
         __syncthreads();
-        const unsigned long long ex = carry + wt[wid] + x - v;
-        if (i < d.n_tiles) row[i] = (int64_t)ex;
-        __syncthreads();
-        if (threadIdx.x == blockDim.x - 1) carry = ex + v;
+        if (cross_tile >= 0) break;
+        if (tid == (int)blockDim.x - 1) carry_s = ex + v;
         __syncthreads();
     }
+    const int32_t tile = cross_tile;
+    if (tile < 0) {   // everything fits
+        if (tid == 0) d.sel[t].cut = 0x7fffffff;
+        return;
+    }
+    // the crossing tile's candidates in id order, kTile slots
+    if (tid == 0) {
+        cut_s = tile * kTile - 1;
+        carry_s = cross_before;
+    }
+    __syncthreads();
+    for (int b = 0; b < kTile; b += (int)blockDim.x) {
+        const int slot = b + tid;
+        const int32_t range = tile * kWarps + slot / kRange;
+        unsigned long long v = 0;
+        int32_t u = -1;
+        if (range < d.n_ranges && slot % kRange < d.cand_cnt[range]) {
+            int key, tt, ul;
+            int32_t g;
+            if (decode_key<KEY>(d.cand[(int64_t)tile * kTile + slot], key, tt, g, ul) && key == t && g == (int32_t)sl.g) {
+                u = range * kRange + ul;
+                v = d.vw ? (unsigned long long)d.vw[u] : 1ull;
+            }
+        }
+        const unsigned long long ex = carry_s + block_scan_u64(v, wt);
+        if (u >= 0 && (KEY == KEY_A ? ex : ex + v) <= rem) atomicMax(&cut_s, u);
+        __syncthreads();
+        if (tid == (int)blockDim.x - 1) carry_s = ex + v;
+        __syncthreads();
+    }
+    if (tid == 0) d.sel[t].cut = cut_s;
 }
 
 // ------------------------------------------------------------------ apply
@@ -1065,112 +1100,47 @@ __device__ __forceinline__ long long apply_pins(const Dev &d, Rec *recs, const A
 
 // Per-warp approval state of one instance.
 struct ApplyInst {
-    int mode[64];
-    int32_t gthr[64];
-    long long rem[64];
+    int32_t gthr[64];    // a candidate of the block passes above this gain,
+    int32_t cut[64];     // or at it up to this vertex id
 };
 
-__device__ __forceinline__ bool apply_refresh(const Dev &d, ApplyInst &ai, int32_t &r)
+__device__ __forceinline__ void apply_refresh(const Dev &d, ApplyInst &ai, int32_t &r)
 {
     const int lane = threadIdx.x & 31;
-    int thr_any = 0;
     for (int t = lane; t < 64; t += 32) {
-        int md = SEL_ALL;
+        int32_t g = -1, cut = -1;   // every candidate passes (gains and priorities are >= 0)
         if (t < d.k) {
             const Sel sl = d.sel[t];
-            md = sl.mode;
-            ai.gthr[t] = (int32_t)sl.g;
-            ai.rem[t] = sl.rem;
+            if (sl.mode == SEL_THRESH) {
+                g = (int32_t)sl.g;
+                cut = (int32_t)sl.cut;
+            }
         }
-        ai.mode[t] = md;
-        thr_any |= md == SEL_THRESH;
+        ai.gthr[t] = g;
+        ai.cut[t] = cut;
     }
     r = d.rs[0];
     __syncwarp();
-    return __any_sync(kFull, thr_any) != 0;
 }
 
-// The id-ordered tie prefix of a range: per key block at its threshold gain, the weight of
-// the passing candidates at the threshold in the earlier ranges of the tile (the tile's
-// exclusive prefix plus the earlier ranges of the same tile).  Only needed, and only built,
-// when the range holds such a candidate; returns whether it does.
-template <int KEY>
-__device__ __forceinline__ bool range_tie_prefix(const Dev &d, int32_t range, bool any_thr, const ApplyInst &ai,
-                                                 unsigned long long *run, const uint64_t *cand, int32_t ncand)
-{
-    const int lane = threadIdx.x & 31;
-    const int *mode = ai.mode;
-    const int32_t *gthr = ai.gthr;
-    bool has_tie = false;
-    if (any_thr) {
-        bool tie = false;
-        for (int i = lane; i < ncand; i += 32) {
-            int t, ul, key;
-            int32_t g;
-            const bool in = decode_key<KEY>(cand[i], key, t, g, ul);
-            tie = tie || (in && mode[key] == SEL_THRESH && g == gthr[key]);
-        }
-        has_tie = __any_sync(kFull, tie) != 0;
-    }
-    if (has_tie) {
-        const int32_t tile = range / kWarps;
-        for (int t = lane; t < 64; t += 32)
-            run[t] = (t < d.k && mode[t] == SEL_THRESH)
-                         ? (unsigned long long)d.tie[(int64_t)t * d.n_tiles + tile] : 0ull;
-        __syncwarp();
-        for (int32_t pr = tile * kWarps; pr < range; ++pr) {
-            const int32_t n2 = d.cand_cnt[pr];
-            const uint64_t *c2 = d.cand + (int64_t)pr * kRange;
-            for (int i = lane; i < n2; i += 32) {
-                int t, ul, key;
-                int32_t g;
-                if (decode_key<KEY>(c2[i], key, t, g, ul) && mode[key] == SEL_THRESH && g == gthr[key])
-                    atomicAdd(&run[key], d.vw ? (unsigned long long)d.vw[pr * kRange + ul] : 1ull);
-            }
-        }
-        __syncwarp();
-    }
-    return has_tie;
-}
-
-// Approval of the candidate in this lane's slot of a 32-candidate chunk: above its key
-// block's threshold gain, or at it and within the block's remainder in id order (KEY_A:
-// the weight before it; otherwise: including its own weight).
+// Approval of the candidate in this lane's slot of a 32-candidate chunk: above its key block's
+// threshold gain, or at it up to the block's last id.
 template <int KEY>
 __device__ __forceinline__ bool approve_slot(const Dev &d, int32_t range, const uint64_t *cand, int32_t ncand,
-                                             int idx, const ApplyInst &ai, unsigned long long *run, int &t,
-                                             int &key, int32_t &g, int &ul, unsigned long long &cw)
+                                             int idx, const ApplyInst &ai, int &t, int &ul)
 {
-    const int lane = threadIdx.x & 31;
-    bool appr = false, tie = false;
-    t = 0; key = 0; g = 0; ul = 0; cw = 1;
-    if (idx < ncand) {
-        const bool in = decode_key<KEY>(cand[idx], key, t, g, ul);
-        if (d.vw) cw = (unsigned long long)d.vw[range * kRange + ul];
-        const int md = ai.mode[key];
-        if (in) {
-            if (md == SEL_ALL || g > ai.gthr[key]) appr = true;
-            else if (g == ai.gthr[key]) tie = true;
-        }
-    }
-    unsigned tm = __ballot_sync(kFull, tie);
-    while (tm) {
-        const int l = __ffs(tm) - 1;
-        tm &= tm - 1;
-        if (lane == l) {
-            appr = (long long)(run[key] + (KEY == KEY_A ? 0ull : cw)) <= ai.rem[key];
-            run[key] += cw;
-        }
-        __syncwarp();
-    }
-    return appr;
+    t = 0; ul = 0;
+    if (idx >= ncand) return false;
+    int key;
+    int32_t g;
+    if (!decode_key<KEY>(cand[idx], key, t, g, ul)) return false;
+    return g > ai.gthr[key] || (g == ai.gthr[key] && range * kRange + ul <= ai.cut[key]);
 }
 
 // One range item of the apply step (see k_apply).  KEY_T: LP (stamps the nets, records the
 // revert variant's source blocks); KEY_TS: rebalancing (no stamps).
 template <typename Rec, int KEY>
-__device__ __forceinline__ void apply_range(const Dev &d, int32_t range, int32_t r, bool any_thr,
-                                            const ApplyInst &ai, unsigned long long *run,
+__device__ __forceinline__ void apply_range(const Dev &d, int32_t range, int32_t r, const ApplyInst &ai,
                                             unsigned long long *bwd, ApplyWarp &w_, long long &idobj,
                                             int32_t &iappr, int32_t &ipins, int32_t &ishared)
 {
@@ -1179,16 +1149,14 @@ __device__ __forceinline__ void apply_range(const Dev &d, int32_t range, int32_t
     const int32_t ncand = d.cand_cnt[range];
     if (ncand == 0) return;
     const uint64_t *cand = d.cand + (int64_t)range * kRange;
-    range_tie_prefix<KEY>(d, range, any_thr, ai, run, cand, ncand);
     for (int32_t c0 = 0; c0 < ncand; c0 += 32) {
         const int idx = c0 + lane;
-        int t, key, ul;
-        int32_t g;
-        unsigned long long cw;
-        const bool appr = approve_slot<KEY>(d, range, cand, ncand, idx, ai, run, t, key, g, ul, cw);
+        int t, ul;
+        const bool appr = approve_slot<KEY>(d, range, cand, ncand, idx, ai, t, ul);
         int32_t deg = 0, jb = 0, a = 0;
         if (appr) {
             const int32_t u = range * kRange + ul;
+            const unsigned long long cw = d.vw ? (unsigned long long)d.vw[u] : 1ull;
             a = d.part[u];
             d.part[u] = (uint8_t)t;
             atomicAdd(&bwd[a], (unsigned long long)(-(long long)cw));
@@ -1219,17 +1187,15 @@ __device__ __forceinline__ void apply_range(const Dev &d, int32_t range, int32_t
 }
 
 // Persistent: each warp walks range items with a grid stride.  For each 32 candidates of a
-// range it decides approval (ties at a block's threshold gain in vertex-id order: the warp
-// starts from the tile's exclusive tie prefix and adds the ties of the earlier ranges of the
-// same tile itself, so warps never wait for each other), then applies the approved moves
-// over their incidences flattened across the lanes, so all atomics are in flight at once.
+// range it decides approval (threshold gain and last tied id of the target block, see
+// k_tie_cut), then applies the approved moves over their incidences flattened across the lanes,
+// so all atomics are in flight at once.
 // B as for k_gain.
 template <typename Rec, bool B, int KEY = KEY_T>
 __global__ void __launch_bounds__(kThreads, 4) k_apply(const Dev d0, const Dev *devs, const int2 *items,
                                                        int32_t n_items, int32_t rr, int32_t sub)
 {
     __shared__ ApplyInst ai_w[kWarps];
-    __shared__ unsigned long long run[kWarps][64];
     __shared__ unsigned long long bwd_w[kWarps][64];
     __shared__ ApplyWarp aw[kWarps];
     __shared__ Dev dsm[B ? kWarps : 1];
@@ -1243,10 +1209,8 @@ __global__ void __launch_bounds__(kThreads, 4) k_apply(const Dev d0, const Dev *
     long long dobj = 0;
     int32_t nappr = 0, npins = 0, r = 0, nshared = 0;
     int inst_prev = -1;
-    bool any_thr = false;
     const int32_t n_it = B ? n_items : d0.n_ranges;
-    // static assignment: the 8 warps of a CTA take the 8 ranges of one tile, whose candidates
-    // the tie prefixes read (measured faster here than the gain step's dynamic distribution)
+    // static assignment (measured faster here than the gain step's dynamic distribution)
     (void)sub;
     for (int32_t item = blockIdx.x * kWarps + wid; item < n_it; item += gridDim.x * kWarps) {
         long long idobj = 0;
@@ -1255,11 +1219,11 @@ __global__ void __launch_bounds__(kThreads, 4) k_apply(const Dev d0, const Dev *
             const int2 it = items[item];
             if (it.x != inst_prev) {
                 load_dev(dsm[wid], devs + it.x);
-                any_thr = apply_refresh(dsm[wid], ai_w[wid], r);
+                apply_refresh(dsm[wid], ai_w[wid], r);
                 inst_prev = it.x;
             }
             const Dev &d = dsm[wid];
-            apply_range<Rec, KEY>(d, it.y, r, any_thr, ai_w[wid], run[wid], bwd_w[wid], aw[wid], idobj, iappr, ipins,
+            apply_range<Rec, KEY>(d, it.y, r, ai_w[wid], bwd_w[wid], aw[wid], idobj, iappr, ipins,
                                   ishared);
             for (int o = 16; o; o >>= 1) {
                 idobj += __shfl_xor_sync(kFull, idobj, o);
@@ -1284,10 +1248,10 @@ __global__ void __launch_bounds__(kThreads, 4) k_apply(const Dev d0, const Dev *
             __syncwarp();
         } else {
             if (inst_prev < 0) {
-                any_thr = apply_refresh(d0, ai_w[wid], r);
+                apply_refresh(d0, ai_w[wid], r);
                 inst_prev = 0;
             }
-            apply_range<Rec, KEY>(d0, item, r, any_thr, ai_w[wid], run[wid], bwd_w[wid], aw[wid], idobj, iappr, ipins,
+            apply_range<Rec, KEY>(d0, item, r, ai_w[wid], bwd_w[wid], aw[wid], idobj, iappr, ipins,
                                   ishared);
             dobj += idobj;
             nappr += iappr;
@@ -1612,11 +1576,10 @@ __global__ void k_round_end(const Dev *devs, int32_t n_inst, int32_t rr, int32_t
 __global__ void __launch_bounds__(kThreads) k_rb_mark(const Dev d)
 {
     __shared__ ApplyInst ai_w[kWarps];
-    __shared__ unsigned long long run_w[kWarps][64];
     __shared__ unsigned long long tot_w[kWarps][64];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     int32_t r;
-    const bool any_thr = apply_refresh(d, ai_w[wid], r);
+    apply_refresh(d, ai_w[wid], r);
     tot_w[wid][lane] = 0;
     tot_w[wid][lane + 32] = 0;
     __syncwarp();
@@ -1624,16 +1587,12 @@ __global__ void __launch_bounds__(kThreads) k_rb_mark(const Dev d)
         const int32_t ncand = d.cand_cnt[range];
         if (ncand == 0) continue;
         uint64_t *cand = d.cand + (int64_t)range * kRange;
-        range_tie_prefix<KEY_A>(d, range, any_thr, ai_w[wid], run_w[wid], cand, ncand);
         for (int32_t c0 = 0; c0 < ncand; c0 += 32) {
             const int idx = c0 + lane;
-            int t, key, ul;
-            int32_t g;
-            unsigned long long cw;
-            const bool sel = approve_slot<KEY_A>(d, range, cand, ncand, idx, ai_w[wid], run_w[wid], t, key, g, ul, cw);
-            if (sel) {
+            int t, ul;
+            if (approve_slot<KEY_A>(d, range, cand, ncand, idx, ai_w[wid], t, ul)) {
                 cand[idx] |= kSelBit;
-                atomicAdd(&tot_w[wid][t], cw);
+                atomicAdd(&tot_w[wid][t], d.vw ? (unsigned long long)d.vw[range * kRange + ul] : 1ull);
             }
         }
         __syncwarp();
@@ -1803,7 +1762,7 @@ cudaError_t launch_round(const Plan &p, int32_t rr)
             }
         }
         k_tie_sum<<<p.n_tiles, kThreads, 0, p.st>>>(p.devs, p.tiles, p.n_tiles);
-        k_tie_scan<<<p.n_blocks, 1024, 0, p.st>>>(p.devs, p.blocks, p.n_blocks);
+        k_tie_cut<KEY_T><<<p.n_blocks, 1024, 0, p.st>>>(p.devs, p.blocks, p.n_blocks);
         n += 2;
         *p.launches += n;
         e = cudaGetLastError();
@@ -2147,7 +2106,7 @@ int64_t launch_stage(const Plan &p, bool levels)
         }
     }
     k_tie_sum<KEY><<<p.n_tiles, kThreads, 0, p.st>>>(p.devs, p.tiles, p.n_tiles);
-    k_tie_scan<<<p.n_blocks, 1024, 0, p.st>>>(p.devs, p.blocks, p.n_blocks);
+    k_tie_cut<KEY><<<p.n_blocks, 1024, 0, p.st>>>(p.devs, p.blocks, p.n_blocks);
     return n + 2;
 }
 
