@@ -80,6 +80,9 @@ struct Dev {
     const int32_t *inc;
     const int32_t *vw;      // nullptr: unit weights
     const int32_t *nw;      // net weights as given (nullptr: unit)
+    const int32_t *vnw;     // [n] W(u), the weight of u's nets (nullptr with unit nets: the degree)
+    int32_t bins;           // gains lie below this (a multiple of kThreads), or it is kBins
+    int32_t pad1;
     uint8_t *part;
     uint32_t *phi;
     int32_t *phi_wide;
@@ -94,7 +97,7 @@ struct Dev {
     uint16_t *sub_start;    // [n_ranges * (S + 1)]
     uint64_t *cand;         // [n_ranges * kRange] (gain << 32 | local << 8 | target)
     int32_t *cand_cnt;      // [n_ranges]
-    int64_t *tot;           // [k] candidate weight per target block
+    int64_t *tot;           // [k] candidate weight per key block (rebalancing)
     unsigned long long *hist;  // [k * kBins]
     Sel *sel;               // [k]
     int64_t *tie;           // [k * n_tiles] weight of the candidates at the threshold gain

@@ -138,13 +138,6 @@ template <typename Rec> struct RecIO;
 
 template <> struct RecIO<Rec16> {
     typedef uint32_t Lam;
-    // eligibility/b pass: s1, w, mv, and lam (same 16 bytes)
-    __device__ static void load_a(const Rec16 *r, Lam &s1, int32_t &w, int32_t &mv, Lam &lam, bool &has_lam)
-    {
-        const uint4 q = __ldg(reinterpret_cast<const uint4 *>(r));
-        s1 = q.x; w = (int32_t)q.y; mv = (int32_t)q.z; lam = q.w; has_lam = true;
-    }
-    __device__ static Lam load_lam(const Rec16 *r) { return __ldg(&r->lam); }
     __device__ static void load_full(const Rec16 *r, Lam &s1, int32_t &w, int32_t &mv, Lam &lam)
     {
         const uint4 q = __ldg(reinterpret_cast<const uint4 *>(r));
@@ -159,23 +152,13 @@ template <> struct RecIO<Rec16> {
 
 template <> struct RecIO<Rec32> {
     typedef uint64_t Lam;
-    __device__ static void load_a(const Rec32 *r, Lam &s1, int32_t &w, int32_t &mv, Lam &lam, bool &has_lam)
-    {
-        const uint4 q = __ldg(reinterpret_cast<const uint4 *>(r));
-        s1 = (uint64_t)q.x | ((uint64_t)q.y << 32); w = (int32_t)q.z; mv = (int32_t)q.w;
-        lam = 0; has_lam = false;
-    }
+    // the whole record is one 32-byte load (records are 32-byte aligned)
     __device__ static void load_full(const Rec32 *r, Lam &s1, int32_t &w, int32_t &mv, Lam &lam)
     {
-        const uint4 q = __ldg(reinterpret_cast<const uint4 *>(r));
-        const uint2 l = __ldg(reinterpret_cast<const uint2 *>(&r->lam));
-        s1 = (uint64_t)q.x | ((uint64_t)q.y << 32); w = (int32_t)q.z; mv = (int32_t)q.w;
-        lam = (uint64_t)l.x | ((uint64_t)l.y << 32);
-    }
-    __device__ static Lam load_lam(const Rec32 *r)
-    {
-        const uint2 q = __ldg(reinterpret_cast<const uint2 *>(&r->lam));
-        return (uint64_t)q.x | ((uint64_t)q.y << 32);
+        uint64_t wm;
+        [[maybe_unused]] uint64_t tail;
+        asm("ld.global.nc.v4.b64 {%0, %1, %2, %3}, [%4];" : "=l"(s1), "=l"(wm), "=l"(lam), "=l"(tail) : "l"(r));
+        w = (int32_t)(uint32_t)wm; mv = (int32_t)(uint32_t)(wm >> 32);
     }
     __device__ static void load_b(const Rec32 *r, Lam &lam, int32_t &w)
     {
@@ -190,20 +173,6 @@ template <typename Lam> __device__ __forceinline__ uint32_t hi32(Lam x)
     return sizeof(Lam) == 8 ? (uint32_t)((uint64_t)x >> 32) : 0u;
 }
 
-constexpr int kCache = 256;   // incidences per chunk whose (Lambda, omega) stay in shared memory
-
-template <typename Lam>
-struct alignas(16) GainWarp {
-    Lam lamc[kCache];            // Lambda(e) of the chunk's incidences, in flattened order
-    int32_t wc[kCache];          // omega(e)
-    unsigned long long T[32];
-    unsigned long long A2[32];   // AND of Lambda(e) over nets with Phi(e,a) >= 2 (balance moves)
-    int32_t W[32], b[32], jb[32], a[32], elig[32];
-    int32_t off[33];
-};
-static_assert(sizeof(GainWarp<uint32_t>) % 16 == 0 && sizeof(GainWarp<uint64_t>) % 16 == 0, "GainWarp alignment");
-static_assert(offsetof(GainWarp<uint32_t>, T) % 8 == 0 && offsetof(GainWarp<uint64_t>, T) % 8 == 0, "GainWarp alignment");
-
 __device__ __forceinline__ int slot_of(const int32_t *off, int32_t i)
 {
     int v = 0;
@@ -213,88 +182,23 @@ __device__ __forceinline__ int slot_of(const int32_t *off, int32_t i)
     return v;
 }
 
-// Connectivity of one vertex to every block of T, held as NP bit planes (bit t of plane p is
-// bit p of conn_t), accumulated with a ripple-carry adder on whole bitsets: adding omega(e) to
-// every block of Lambda(e) & T costs O(NP) word operations, whatever the number of blocks.
-// Returns the block of T with the largest conn_t (smallest id among equals) and its value.
-// Requires conn_t <= W(u) < 2^NP.
-template <typename Lam, typename Rec, int NP, bool UNIT>
-__device__ __forceinline__ void bitsliced_best(const GainWarp<Lam> &g, const Rec *recs, const int32_t *inc,
-                                               int32_t i_begin, int32_t i_end, int32_t jb, int32_t off,
-                                               Lam T, int &t_out, int32_t &conn_out, int32_t eq_value,
-                                               Lam &eq_out)
-{
-    Lam c[NP];
-#pragma unroll
-    for (int p = 0; p < NP; ++p) c[p] = 0;
-    for (int32_t i = i_begin; i < i_end; ++i) {
-        Lam lam;
-        int32_t w;
-        if (i < kCache) {
-            lam = g.lamc[i];
-            w = g.wc[i];
-        } else {
-            RecIO<Rec>::load_b(recs + (__ldg(&inc[jb + (i - off)]) & kNetMask), lam, w);
-            w &= 0x7fffffff;
-        }
-        const Lam x = lam & T;
-        if (UNIT) {
-            Lam carry = x;
-#pragma unroll
-            for (int p = 0; p < NP; ++p) {
-                const Lam t = c[p] & carry;
-                c[p] ^= carry;
-                carry = t;
-            }
-        } else {
-            Lam carry = 0;
-#pragma unroll
-            for (int p = 0; p < NP; ++p) {
-                const Lam ad = ((w >> p) & 1) ? x : (Lam)0;
-                const Lam cp = c[p];
-                c[p] = cp ^ ad ^ carry;
-                carry = (cp & ad) | (carry & (cp ^ ad));
-            }
-        }
-    }
-    Lam C = T;
-#pragma unroll
-    for (int p = NP - 1; p >= 0; --p) {
-        const Lam m = C & c[p];
-        C = m ? m : C;
-    }
-    const int t = lam_bits_ctz(C);
-    int32_t v = 0;
-#pragma unroll
-    for (int p = 0; p < NP; ++p) v |= (int32_t)((c[p] >> t) & 1) << p;
-    t_out = t;
-    conn_out = v;
-    // blocks of T whose conn equals eq_value (eq_value < 0: none)
-    Lam eq = eq_value >= 0 && (eq_value >> NP) == 0 ? T : (Lam)0;
-#pragma unroll
-    for (int p = 0; p < NP; ++p) eq &= ((eq_value >> p) & 1) ? c[p] : ~c[p];
-    eq_out = eq;
-}
-
-template <typename Lam, typename Rec, bool UNIT>
-__device__ __forceinline__ void best_by_planes(int np, const GainWarp<Lam> &g, const Rec *recs,
-                                               const int32_t *inc, int32_t ib, int32_t ie, int32_t jb,
-                                               int32_t off, Lam T, int &t, int32_t &conn, int32_t eqv, Lam &eq)
-{
-    if (np <= 4) bitsliced_best<Lam, Rec, 4, UNIT>(g, recs, inc, ib, ie, jb, off, T, t, conn, eqv, eq);
-    else if (np <= 6) bitsliced_best<Lam, Rec, 6, UNIT>(g, recs, inc, ib, ie, jb, off, T, t, conn, eqv, eq);
-    else if (np <= 8) bitsliced_best<Lam, Rec, 8, UNIT>(g, recs, inc, ib, ie, jb, off, T, t, conn, eqv, eq);
-    else bitsliced_best<Lam, Rec, 11, UNIT>(g, recs, inc, ib, ie, jb, off, T, t, conn, eqv, eq);
-}
-
 constexpr int32_t kPlaneMaxW = 2047;   // W(u) up to this uses bit planes (NP <= 11)
+// degrees above this are walked by the whole warp: its two passes cost about as many issue slots
+// as a lane's walk of this length with the other lanes idle
+constexpr int32_t kLaneDeg = 96;
+constexpr int kFeasW = 8;              // vertex weights up to this have a mask of blocks with room
 
 // Per-warp state of the gain step that depends on the instance.
 template <typename Lam>
 struct GainInst {
-    Lam feas1;           // blocks with room for a unit-weight vertex
     int32_t r;           // round number
     int32_t all_elig;    // first round: every vertex eligible
+};
+
+// per-warp tables of the instance: room left per block, and the blocks with room for weight c
+struct alignas(16) GainWarp {
+    long long slack[64];
+    unsigned long long feas[kFeasW + 1];
 };
 
 // Rebalancing pass settings (RB instances of the gain step).
@@ -304,260 +208,357 @@ struct RbArgs {
     int32_t off;     // added to the gain to make the approval priority non-negative
 };
 
+// What one pass over a vertex's nets gives.
+template <typename Lam>
+struct Nets {
+    Lam T;        // union of Lambda(e) over the nets with Phi(e,a) = 1
+    Lam A2;       // intersection over the others (balance moves)
+    int32_t b;    // omega of the nets with Phi(e,a) = 1
+    int32_t elig; // a net moved in round r - 1
+};
+
+template <typename Lam>
+__device__ __forceinline__ void take_net(Nets<Lam> &x, Lam s1, Lam lam, int32_t w, int32_t mv, int a, int32_t r)
+{
+    const bool alone = (s1 >> a) & 1;
+    if (alone) {
+        x.b += w;
+        x.T |= lam;
+    } else {
+        x.A2 &= lam;
+    }
+    if (moved_in_prev_round(mv, r)) x.elig = 1;
+}
+
+// blocks of T with room for weight cu
+template <typename Lam>
+__device__ __forceinline__ Lam with_room(Lam T, const GainWarp &g, int32_t cu)
+{
+    if (cu <= kFeasW) return T & (Lam)g.feas[cu];
+    for (Lam x = T; x; x &= x - 1) {
+        const int t = lam_bits_ctz(x);
+        if (g.slack[t] < cu) T &= ~((Lam)1 << t);
+    }
+    return T;
+}
+
+// One lane's vertex: a single walk over its nets that gathers each record once and accumulates
+// b(u), T, eligibility and, for all blocks at once, conn_t = omega({e in I(u) : t in Lambda(e)})
+// in NP bit planes held in registers (bit t of plane p is bit p of conn_t): adding omega(e) to
+// every block of Lambda(e) is a ripple-carry addition on whole bitsets, O(NP) word operations
+// whatever the number of blocks.  W(u) is known from creation, so NP is too (conn_t <= W(u) <
+// 2^NP).  kAhead records are in flight per lane.  Then the block of T with room with the largest
+// conn_t (smallest id among equals).  Against incidences spread over the lanes (a binary search
+// and three shared-memory atomics each, (Lambda, omega) kept for a second pass over the nets):
+// row-net 2M, k = 8, records in L2: 93 -> 56 us per launch of 5 M gathers; power-law 50M, k = 64,
+// bound by random sectors from DRAM: 1.77 -> 1.65 ms per launch of 86 M.
+template <typename Lam, typename Rec, int NP, bool UNIT, bool RB>
+__device__ __forceinline__ void lane_best(const Rec *recs, const int32_t *inc, int32_t jb, int32_t je, int a, int32_t r,
+                                          const GainWarp &g, int32_t cu, Lam kall, int32_t eq_value, Nets<Lam> &x,
+                                          Lam &T_all, Lam &T, int &t_out, int32_t &conn_out, Lam &eq_out)
+{
+    constexpr int kAhead = sizeof(Lam) == 8 ? 2 : 4;
+    Lam c[NP];
+#pragma unroll
+    for (int p = 0; p < NP; ++p) c[p] = 0;
+    for (int32_t j = jb; j < je; j += kAhead) {
+        int32_t e[kAhead];
+        Lam s1[kAhead], lam[kAhead];
+        int32_t w[kAhead], mv[kAhead];
+#pragma unroll
+        for (int q = 0; q < kAhead; ++q) e[q] = j + q < je ? (__ldg(&inc[j + q]) & kNetMask) : -1;
+#pragma unroll
+        for (int q = 0; q < kAhead; ++q) {
+            s1[q] = 0; lam[q] = 0; w[q] = 0; mv[q] = 0;
+            if (e[q] >= 0) RecIO<Rec>::load_full(recs + e[q], s1[q], w[q], mv[q], lam[q]);
+        }
+#pragma unroll
+        for (int q = 0; q < kAhead; ++q) {
+            if (e[q] < 0) continue;
+            const int32_t we = UNIT ? 1 : w[q] & 0x7fffffff;
+            take_net(x, s1[q], lam[q], we, mv[q], a, r);
+            if (UNIT) {
+                Lam carry = lam[q];
+#pragma unroll
+                for (int p = 0; p < NP; ++p) {
+                    const Lam t = c[p] & carry;
+                    c[p] ^= carry;
+                    carry = t;
+                }
+            } else {
+                Lam carry = 0;
+#pragma unroll
+                for (int p = 0; p < NP; ++p) {
+                    const Lam ad = ((we >> p) & 1) ? lam[q] : (Lam)0;
+                    const Lam cp = c[p];
+                    c[p] = cp ^ ad ^ carry;
+                    carry = (cp & ad) | (carry & (cp ^ ad));
+                }
+            }
+        }
+    }
+    T_all = x.elig ? (RB ? kall : x.T) & ~((Lam)1 << a) : (Lam)0;
+    T = with_room(T_all, g, cu);
+    Lam C = T;
+#pragma unroll
+    for (int p = NP - 1; p >= 0; --p) {
+        const Lam m = C & c[p];
+        C = m ? m : C;
+    }
+    t_out = -1;
+    conn_out = 0;
+    eq_out = 0;
+    if (T) {
+        const int t = lam_bits_ctz(C);
+#pragma unroll
+        for (int p = 0; p < NP; ++p) conn_out |= (int32_t)((c[p] >> t) & 1) << p;
+        t_out = t;
+    }
+    // balance moves: blocks of T with gain 0, conn_t = W - b (eq_value = W; < 0: not asked for)
+    if (eq_value >= 0) {
+        const int32_t v = eq_value - x.b;
+        Lam eq = T;
+#pragma unroll
+        for (int p = 0; p < NP; ++p) eq &= ((v >> p) & 1) ? c[p] : ~c[p];
+        eq_out = eq;
+    }
+}
+
 // One range item of the gain step (see k_gain); returns the number of candidates written.
 // RB: a rebalancing pass (Sec. 8): only vertices of overloaded blocks take part, their target
 // is the block with room of highest gain (any sign), and the candidate records its source
 // block (bits 16..23) and the priority gain + off; the per-block totals are by source block.
 template <typename Rec, bool RB>
-__device__ __forceinline__ int32_t gain_range(const Dev &d, int32_t range, int32_t s, GainWarp<typename RecIO<Rec>::Lam> &g,
-                                              const long long *slack, unsigned long long *tot,
-                                              const GainInst<typename RecIO<Rec>::Lam> &gi, int32_t &nel,
-                                              const RbArgs &rb)
+__device__ __forceinline__ int32_t gain_range(const Dev &d, int32_t range, int32_t s, const GainWarp &g,
+                                              uint8_t *picked, unsigned long long *tot, const GainInst<typename RecIO<Rec>::Lam> &gi,
+                                              int32_t &nel, const RbArgs &rb)
 {
     typedef typename RecIO<Rec>::Lam Lam;
     constexpr bool kWide = sizeof(Lam) == 8;
     const int lane = threadIdx.x & 31;
-    const Lam feas1 = gi.feas1;
-    const int32_t r = gi.r, all_elig = gi.all_elig;
+    const int32_t r = gi.r;
     const bool balance = !RB && (d.variant & 1) != 0;
-        const Rec *recs = reinterpret_cast<const Rec *>(d.rec);
-        const bool unit = d.nw == nullptr;
-        const int32_t rbase = range * kRange;
-        int32_t beg = 0, cnt = 0;
-        if (s < d.S) {
-            const uint16_t *ss = d.sub_start + (int64_t)range * (d.S + 1);
-            beg = ss[s];
-            cnt = (int32_t)ss[s + 1] - beg;
-        }
-        const uint8_t *list = d.sub_list + (int64_t)range * kRange + beg;
-        uint64_t *out = d.cand + (int64_t)range * kRange;
-        int32_t nout = 0;
-        nel = 0;
+    const Rec *recs = reinterpret_cast<const Rec *>(d.rec);
+    const bool unit = d.nw == nullptr;
+    const Lam kall = d.k >= (int)(8 * sizeof(Lam)) ? ~(Lam)0 : (((Lam)1 << d.k) - 1);
+    const int32_t rbase = range * kRange;
+    int32_t beg = 0, cnt = 0;
+    if (s < d.S) {
+        const uint16_t *ss = d.sub_start + (int64_t)range * (d.S + 1);
+        beg = ss[s];
+        cnt = (int32_t)ss[s + 1] - beg;
+    }
+    const uint8_t *list = d.sub_list + (int64_t)range * kRange + beg;
+    uint64_t *out = d.cand + (int64_t)range * kRange;
+    int32_t nout = 0;
+    nel = 0;
+    if (RB) {
+        // the vertices of overloaded blocks, few of a range, moved together first so that the
+        // lanes are full
+        int32_t kept = 0;
         for (int32_t c0 = 0; c0 < cnt; c0 += 32) {
-            const int32_t idx = c0 + lane;
-            const bool valid = idx < cnt;
-            int32_t ul = 0, cu = 1, deg = 0, jb = 0, a = 0;
-            if (valid) {
-                ul = list[idx];
-                const int32_t u = rbase + ul;
-                a = d.part[u];
-                cu = d.vw ? d.vw[u] : 1;
-                jb = d.vtx_off[u];
-                deg = d.vtx_off[u + 1] - jb;
-                if (RB && slack[a] >= 0) deg = 0;   // not in an overloaded block: no work
-            }
-            g.a[lane] = a;
-            g.jb[lane] = jb;
-            g.W[lane] = 0;
-            g.b[lane] = 0;
-            g.T[lane] = 0;
-            g.A2[lane] = ~0ull;
-            g.elig[lane] = RB ? (valid && slack[a] < 0) : all_elig;
-            int32_t incl = deg;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const int32_t y = __shfl_up_sync(kFull, incl, o);
-                if (lane >= o) incl += y;
-            }
-            const int32_t total = __shfl_sync(kFull, incl, 31);
-            const int32_t my_off = incl - deg;
-            g.off[lane] = my_off;
-            if (lane == 31) g.off[32] = total;
-            __syncwarp();
-            // ---- pass A over the flattened incidences
-            for (int32_t i0 = 0; i0 < total; i0 += 64) {
-                const int32_t i1 = i0 + lane, i2 = i0 + 32 + lane;
-                int v1 = 0, v2 = 0, e1 = 0, e2 = 0;
-                if (i1 < total) {
-                    v1 = slot_of(g.off, i1);
-                    e1 = __ldg(&d.inc[g.jb[v1] + (i1 - g.off[v1])]) & kNetMask;
-                }
-                if (i2 < total) {
-                    v2 = slot_of(g.off, i2);
-                    e2 = __ldg(&d.inc[g.jb[v2] + (i2 - g.off[v2])]) & kNetMask;
-                }
-                Lam s11 = 0, lam1 = 0, s12 = 0, lam2 = 0;
-                int32_t w1 = 0, mv1 = 0, w2 = 0, mv2 = 0;
-                if (i1 < total) RecIO<Rec>::load_full(recs + e1, s11, w1, mv1, lam1);
-                if (i2 < total) RecIO<Rec>::load_full(recs + e2, s12, w2, mv2, lam2);
-                if (i1 < total) {
-                    w1 &= 0x7fffffff;
-                    if (i1 < kCache) { g.lamc[i1] = lam1; g.wc[i1] = w1; }
-                    atomicAdd(&g.W[v1], w1);
-                    if ((s11 >> g.a[v1]) & 1) {
-                        atomicAdd(&g.b[v1], w1);
-                        atomicOr(&g.T[v1], (unsigned long long)lam1);
-                    } else if (balance) {
-                        atomicAnd(&g.A2[v1], (unsigned long long)lam1);
-                    }
-                    if (!RB && moved_in_prev_round(mv1, r)) g.elig[v1] = 1;
-                }
-                if (i2 < total) {
-                    w2 &= 0x7fffffff;
-                    if (i2 < kCache) { g.lamc[i2] = lam2; g.wc[i2] = w2; }
-                    atomicAdd(&g.W[v2], w2);
-                    if ((s12 >> g.a[v2]) & 1) {
-                        atomicAdd(&g.b[v2], w2);
-                        atomicOr(&g.T[v2], (unsigned long long)lam2);
-                    } else if (balance) {
-                        atomicAnd(&g.A2[v2], (unsigned long long)lam2);
-                    }
-                    if (!RB && moved_in_prev_round(mv2, r)) g.elig[v2] = 1;
-                }
-            }
-            __syncwarp();
-            // ---- per vertex: eligibility, candidate blocks, best block
-            const int32_t W = g.W[lane], b = g.b[lane];
-            const bool elig = valid && g.elig[lane] != 0;
-            const Lam kall = d.k >= (int)(8 * sizeof(Lam)) ? ~(Lam)0 : (((Lam)1 << d.k) - 1);
-            Lam T = elig ? (RB ? kall : (Lam)g.T[lane]) : (Lam)0;
-            T &= ~((Lam)1 << a);
-            const Lam T_all = T;   // before the room filter (balance moves need it)
-            if (d.vw) {
-                for (Lam x = T; x; x &= x - 1) {
-                    const int t = lam_bits_ctz(x);
-                    if (slack[t] < cu) T &= ~((Lam)1 << t);
-                }
-            } else {
-                T &= feas1;
-            }
-            const bool plane_path = T != 0 && W <= kPlaneMaxW;
-            const bool coop_path = T != 0 && W > kPlaneMaxW;
-            int32_t t_best = -1, g_best = 0;
-            const int32_t bw_ = b - W;
-            const unsigned wmax = __reduce_max_sync(kFull, plane_path ? (unsigned)W : 0u);
-            Lam zero_in = 0;   // blocks of T with gain exactly 0 (balance moves)
-            if (plane_path) {
-                const int np = 32 - __clz((int)wmax);   // 2^np > wmax >= conn_t
-                int t;
-                int32_t conn;
-                const int32_t eqv = balance ? W - b : -1;
-                if (unit) best_by_planes<Lam, Rec, true>(np, g, recs, d.inc, my_off, my_off + deg, jb, my_off, T, t, conn, eqv, zero_in);
-                else best_by_planes<Lam, Rec, false>(np, g, recs, d.inc, my_off, my_off + deg, jb, my_off, T, t, conn, eqv, zero_in);
-                const int32_t gg = bw_ + conn;
-                if (RB ? (rb.phase == 2 || gg >= 0) : gg > 0) {
-                    t_best = t;
-                    g_best = gg;
-                }
-            }
-            // ---- warp-cooperative pass for vertices with large incident net weight
-            unsigned hm = __ballot_sync(kFull, coop_path);
-            while (hm) {
-                const int src = __ffs(hm) - 1;
-                hm &= hm - 1;
-                const int32_t hjb = __shfl_sync(kFull, jb, src), hje = hjb + __shfl_sync(kFull, deg, src);
-                const int32_t hbw = __shfl_sync(kFull, bw_, src);
-                const uint32_t Tlo = __shfl_sync(kFull, lo32(T), src);
-                const uint32_t Thi = kWide ? __shfl_sync(kFull, hi32(T), src) : 0u;
-                int32_t acc0 = 0, acc1 = 0;
-                for (int32_t j0 = hjb; j0 < hje; j0 += 32) {
-                    const int32_t j = j0 + lane;
-                    Lam lam = 0;
-                    int32_t w = 0;
-                    if (j < hje) {
-                        RecIO<Rec>::load_b(recs + (__ldg(&d.inc[j]) & kNetMask), lam, w);
-                        w &= 0x7fffffff;
-                    }
-                    const int nn = min(32, hje - j0);
-                    const uint32_t llo = lo32(lam), lhi = hi32(lam);
-                    for (int q = 0; q < nn; ++q) {
-                        const uint32_t bl = __shfl_sync(kFull, llo, q);
-                        const int32_t wi = __shfl_sync(kFull, w, q);
-                        acc0 += ((bl >> lane) & 1) ? wi : 0;
-                        if (kWide) {
-                            const uint32_t bh = __shfl_sync(kFull, lhi, q);
-                            acc1 += ((bh >> lane) & 1) ? wi : 0;
-                        }
-                    }
-                }
-                // key = gain << 8 | (255 - block): the larger key is the higher gain, then the
-                // smaller block (RB: the gain's sign bit flipped, so negative gains order too)
-                unsigned long long key = 0;
-                if ((Tlo >> lane) & 1) {
-                    const int32_t gg = hbw + acc0;
-                    if (RB ? (rb.phase == 2 || gg >= 0) : gg > 0)
-                        key = ((unsigned long long)((uint32_t)gg ^ (RB ? 0x80000000u : 0u)) << 8) | (unsigned long long)(255 - lane);
-                }
-                if (kWide && ((Thi >> lane) & 1)) {
-                    const int32_t gg = hbw + acc1;
-                    if (RB ? (rb.phase == 2 || gg >= 0) : gg > 0) {
-                        const unsigned long long k2 = ((unsigned long long)((uint32_t)gg ^ (RB ? 0x80000000u : 0u)) << 8) | (unsigned long long)(255 - (lane + 32));
-                        key = k2 > key ? k2 : key;
-                    }
-                }
-#pragma unroll
-                for (int o = 16; o; o >>= 1) {
-                    const unsigned long long y = __shfl_xor_sync(kFull, key, o);
-                    key = y > key ? y : key;
-                }
-                if (lane == src && key) {
-                    t_best = 255 - (int)(key & 0xFF);
-                    g_best = (int32_t)((uint32_t)(key >> 8) ^ (RB ? 0x80000000u : 0u));
-                }
-                if (balance) {
-                    // zero-gain blocks of T among the ones this lane owns
-                    const unsigned zlo = __ballot_sync(kFull, ((Tlo >> lane) & 1) && hbw + acc0 == 0);
-                    const unsigned zhi = __ballot_sync(kFull, kWide && ((Thi >> lane) & 1) && hbw + acc1 == 0);
-                    if (lane == src) zero_in = kWide ? (Lam)((uint64_t)zlo | ((uint64_t)zhi << 32)) : (Lam)zlo;
-                }
-            }
-            if (balance && valid && elig && t_best < 0) {
-                // zero-gain moves that improve the balance (Sec. 6): blocks of T with gain 0, and
-                // blocks outside T that lie in every net where u is not alone (their gain is
-                // b - p_t = 0 exactly then); room and w(t) + c(u) < w(a); lightest block first
-                const Lam kmask = d.k >= (int)(8 * sizeof(Lam)) ? ~(Lam)0 : (((Lam)1 << d.k) - 1);
-                Lam z = (zero_in | ((Lam)g.A2[lane] & ~T_all & ~((Lam)1 << a))) & kmask;
-                const long long wa = d.lmax - slack[a];
-                long long best_w = 0;
-                for (Lam x = z; x; x &= x - 1) {
-                    const int t = lam_bits_ctz(x);
-                    const long long wt = d.lmax - slack[t];
-                    if (slack[t] < cu || wt + cu >= wa) continue;
-                    if (t_best < 0 || wt < best_w) {
-                        t_best = t;
-                        best_w = wt;
-                    }
-                }
-                g_best = 0;
-            }
-            nel += __popc(__ballot_sync(kFull, elig));
-            const unsigned cm = __ballot_sync(kFull, t_best >= 0);
-            if (t_best >= 0) {
-                const int pos = nout + __popc(cm & lanemask_lt());
-                if (RB) {
-                    out[pos] = ((uint64_t)(uint32_t)(g_best + rb.off) << 32) | ((uint32_t)a << 16) |
-                               ((uint32_t)ul << 8) | (uint32_t)t_best;
-                    atomicAdd(&tot[a], (unsigned long long)cu);
-                } else {
-                    out[pos] = ((uint64_t)(uint32_t)g_best << 32) | ((uint32_t)ul << 8) | (uint32_t)t_best;
-                    atomicAdd(&tot[t_best], (unsigned long long)cu);
-                }
-            }
-            if (!RB && t_best >= 0) {
-                // level-0 histogram of the approval step: candidate weight by target block and
-                // gain bin (no return value: a reduction in L2)
-                const int bin = g_best < kBins - 1 ? g_best : kBins - 1;
-                atomicAdd(&d.hist[(int64_t)t_best * kBins + bin], (unsigned long long)cu);
-            }
-            nout += __popc(cm);
-            __syncwarp();
+            const int32_t ul = c0 + lane < cnt ? list[c0 + lane] : 0;
+            const bool over = c0 + lane < cnt && g.slack[d.part[rbase + ul]] < 0;
+            const unsigned om = __ballot_sync(kFull, over);
+            if (over) picked[kept + __popc(om & lanemask_lt())] = (uint8_t)ul;
+            kept += __popc(om);
         }
-        return nout;
+        __syncwarp();
+        list = picked;
+        cnt = kept;
+    }
+    for (int32_t c0 = 0; c0 < cnt; c0 += 32) {
+        const int32_t idx = c0 + lane;
+        const bool valid = idx < cnt;
+        int32_t ul = 0, cu = 1, jb = 0, je = 0, a = 0, W = 0;
+        if (valid) {
+            ul = list[idx];
+            const int32_t u = rbase + ul;
+            a = d.part[u];
+            cu = d.vw ? d.vw[u] : 1;
+            jb = d.vtx_off[u];
+            je = d.vtx_off[u + 1];
+            W = unit ? je - jb : d.vnw[u];
+        }
+        Nets<Lam> x;
+        x.T = 0; x.A2 = ~(Lam)0; x.b = 0;
+        x.elig = valid && (RB || gi.all_elig);
+        Lam T_all = 0, T = 0, zero_in = 0;
+        int t_best = -1;
+        int32_t conn = 0;
+        const bool heavy = valid && (W > kPlaneMaxW || je - jb > kLaneDeg);
+        const bool light = valid && !heavy;
+        const unsigned wmax = __reduce_max_sync(kFull, light ? (unsigned)W : 0u);
+        if (light) {
+            const int np = 32 - __clz((int)wmax);   // 2^np > wmax >= conn_t
+            const int32_t eqv = balance ? W : -1;
+#define HGP_LANE(NP, U) lane_best<Lam, Rec, NP, U, RB>(recs, d.inc, jb, je, a, r, g, cu, kall, eqv, x, T_all, T, t_best, conn, zero_in)
+            if (unit) {
+                if (np <= 4) HGP_LANE(4, true);
+                else HGP_LANE(7, true);             // at most kLaneDeg nets
+            } else {
+                if (np <= 6) HGP_LANE(6, false);
+                else if (np <= 8) HGP_LANE(8, false);
+                else HGP_LANE(11, false);
+            }
+#undef HGP_LANE
+        }
+        __syncwarp();
+        const int32_t bw_ = x.b - W;
+        int32_t g_best = bw_ + conn;
+        if (!(light && t_best >= 0 && (RB ? (rb.phase == 2 || g_best >= 0) : g_best > 0))) {
+            t_best = -1;
+            g_best = 0;
+        }
+        // ---- vertices with many nets or large W: the whole warp on one vertex at a time
+        unsigned hm = __ballot_sync(kFull, heavy);
+        while (hm) {
+            const int src = __ffs(hm) - 1;
+            hm &= hm - 1;
+            const int32_t hjb = __shfl_sync(kFull, jb, src), hje = __shfl_sync(kFull, je, src);
+            const int32_t ha = __shfl_sync(kFull, a, src), hcu = __shfl_sync(kFull, cu, src);
+            const int32_t hW = __shfl_sync(kFull, W, src);
+            Nets<Lam> y;
+            y.T = 0; y.A2 = ~(Lam)0; y.b = 0; y.elig = RB || gi.all_elig;
+            for (int32_t j = hjb + lane; j < hje; j += 32) {
+                Lam s1, lam;
+                int32_t w, mv;
+                RecIO<Rec>::load_full(recs + (__ldg(&d.inc[j]) & kNetMask), s1, w, mv, lam);
+                take_net(y, s1, lam, w & 0x7fffffff, mv, ha, r);
+            }
+            y.b = __reduce_add_sync(kFull, y.b);
+            y.elig = __any_sync(kFull, y.elig);
+            uint32_t tl = __reduce_or_sync(kFull, lo32(y.T)), al = __reduce_and_sync(kFull, lo32(y.A2));
+            uint32_t th = kWide ? __reduce_or_sync(kFull, hi32(y.T)) : 0u;
+            uint32_t ah = kWide ? __reduce_and_sync(kFull, hi32(y.A2)) : 0u;
+            y.T = (Lam)((uint64_t)tl | ((uint64_t)th << 32));
+            y.A2 = (Lam)((uint64_t)al | ((uint64_t)ah << 32));
+            const Lam hTa = y.elig ? (RB ? kall : y.T) & ~((Lam)1 << ha) : (Lam)0;
+            const Lam hT = with_room(hTa, g, hcu);
+            if (lane == src) {
+                x = y;
+                T_all = hTa;
+                T = hT;
+            }
+            if (hT == 0) continue;
+            const uint32_t Tlo = lo32(hT), Thi = hi32(hT);
+            const int32_t hbw = y.b - hW;
+            int32_t acc0 = 0, acc1 = 0;
+            for (int32_t j0 = hjb; j0 < hje; j0 += 32) {
+                const int32_t j = j0 + lane;
+                Lam lam = 0;
+                int32_t w = 0;
+                if (j < hje) {
+                    RecIO<Rec>::load_b(recs + (__ldg(&d.inc[j]) & kNetMask), lam, w);
+                    w &= 0x7fffffff;
+                }
+                const int nn = min(32, hje - j0);
+                const uint32_t llo = lo32(lam), lhi = hi32(lam);
+                for (int q = 0; q < nn; ++q) {
+                    const uint32_t bl = __shfl_sync(kFull, llo, q);
+                    const int32_t wi = __shfl_sync(kFull, w, q);
+                    acc0 += ((bl >> lane) & 1) ? wi : 0;
+                    if (kWide) {
+                        const uint32_t bh = __shfl_sync(kFull, lhi, q);
+                        acc1 += ((bh >> lane) & 1) ? wi : 0;
+                    }
+                }
+            }
+            // key = gain << 8 | (255 - block): the larger key is the higher gain, then the
+            // smaller block (RB: the gain's sign bit flipped, so negative gains order too)
+            unsigned long long key = 0;
+            if ((Tlo >> lane) & 1) {
+                const int32_t gg = hbw + acc0;
+                if (RB ? (rb.phase == 2 || gg >= 0) : gg > 0)
+                    key = ((unsigned long long)((uint32_t)gg ^ (RB ? 0x80000000u : 0u)) << 8) | (unsigned long long)(255 - lane);
+            }
+            if (kWide && ((Thi >> lane) & 1)) {
+                const int32_t gg = hbw + acc1;
+                if (RB ? (rb.phase == 2 || gg >= 0) : gg > 0) {
+                    const unsigned long long k2 = ((unsigned long long)((uint32_t)gg ^ (RB ? 0x80000000u : 0u)) << 8) | (unsigned long long)(255 - (lane + 32));
+                    key = k2 > key ? k2 : key;
+                }
+            }
+#pragma unroll
+            for (int o = 16; o; o >>= 1) {
+                const unsigned long long y2 = __shfl_xor_sync(kFull, key, o);
+                key = y2 > key ? y2 : key;
+            }
+            if (lane == src && key) {
+                t_best = 255 - (int)(key & 0xFF);
+                g_best = (int32_t)((uint32_t)(key >> 8) ^ (RB ? 0x80000000u : 0u));
+            }
+            if (balance) {
+                // zero-gain blocks of T among the ones this lane owns
+                const unsigned zlo = __ballot_sync(kFull, ((Tlo >> lane) & 1) && hbw + acc0 == 0);
+                const unsigned zhi = __ballot_sync(kFull, kWide && ((Thi >> lane) & 1) && hbw + acc1 == 0);
+                if (lane == src) zero_in = kWide ? (Lam)((uint64_t)zlo | ((uint64_t)zhi << 32)) : (Lam)zlo;
+            }
+        }
+        if (balance && valid && x.elig && t_best < 0) {
+            // zero-gain moves that improve the balance (Sec. 6): blocks of T with gain 0, and
+            // blocks outside T that lie in every net where u is not alone (their gain is
+            // b - p_t = 0 exactly then); room and w(t) + c(u) < w(a); lightest block first
+            Lam z = (zero_in | (x.A2 & ~T_all & ~((Lam)1 << a))) & kall;
+            const long long wa = d.lmax - g.slack[a];
+            long long best_w = 0;
+            for (Lam y = z; y; y &= y - 1) {
+                const int t = lam_bits_ctz(y);
+                const long long wt = d.lmax - g.slack[t];
+                if (g.slack[t] < cu || wt + cu >= wa) continue;
+                if (t_best < 0 || wt < best_w) {
+                    t_best = t;
+                    best_w = wt;
+                }
+            }
+            g_best = 0;
+        }
+        nel += __popc(__ballot_sync(kFull, valid && x.elig));
+        const unsigned cm = __ballot_sync(kFull, t_best >= 0);
+        const bool small_c = __all_sync(kFull, cu < (1 << 26));   // 32 of them fit 32 bits
+        if (t_best >= 0) {
+            const int pos = nout + __popc(cm & lanemask_lt());
+            if (RB) {
+                out[pos] = ((uint64_t)(uint32_t)(g_best + rb.off) << 32) | ((uint32_t)a << 16) |
+                           ((uint32_t)ul << 8) | (uint32_t)t_best;
+                atomicAdd(&tot[a], (unsigned long long)cu);
+            } else {
+                out[pos] = ((uint64_t)(uint32_t)g_best << 32) | ((uint32_t)ul << 8) | (uint32_t)t_best;
+                // level-0 histogram of the approval step: candidate weight by target block and
+                // gain bin (a reduction in L2).  Gains are small numbers, so a warp's candidates
+                // share bins: one reduction per distinct (block, bin)
+                const int bin = g_best < kBins - 1 ? g_best : kBins - 1;
+                unsigned long long *slot = &d.hist[(int64_t)t_best * kBins + bin];
+                if (small_c) {
+                    const unsigned peers = __match_any_sync(cm, t_best * kBins + bin);
+                    const unsigned sum = __reduce_add_sync(peers, (unsigned)cu);
+                    if (lane == __ffs(peers) - 1) atomicAdd(slot, (unsigned long long)sum);
+                } else {
+                    atomicAdd(slot, (unsigned long long)cu);
+                }
+            }
+        }
+        nout += __popc(cm);
+        __syncwarp();
+    }
+    return nout;
 }
 
 template <typename Rec>
-__device__ __forceinline__ void gain_refresh(const Dev &d, long long *slack, GainInst<typename RecIO<Rec>::Lam> &gi)
+__device__ __forceinline__ void gain_refresh(const Dev &d, GainWarp &g, GainInst<typename RecIO<Rec>::Lam> &gi)
 {
-    typedef typename RecIO<Rec>::Lam Lam;
     const int lane = threadIdx.x & 31;
-    for (int t = lane; t < 64; t += 32) slack[t] = t < d.k ? d.lmax - d.bw[t] : -1;
     __syncwarp();
-    const unsigned lo = __ballot_sync(kFull, slack[lane] >= 1);
-    const unsigned hi = __ballot_sync(kFull, slack[lane + 32] >= 1);
-    if (sizeof(Lam) == 8) gi.feas1 = (Lam)((uint64_t)lo | ((uint64_t)hi << 32));
-    else gi.feas1 = (Lam)lo;
+    const long long s0 = lane < d.k ? d.lmax - d.bw[lane] : -1, s1 = lane + 32 < d.k ? d.lmax - d.bw[lane + 32] : -1;
+    g.slack[lane] = s0;
+    g.slack[lane + 32] = s1;
+    for (int c = 1; c <= kFeasW; ++c) {
+        const unsigned lo = __ballot_sync(kFull, s0 >= c), hi = __ballot_sync(kFull, s1 >= c);
+        if (lane == 0) g.feas[c] = (unsigned long long)lo | ((unsigned long long)hi << 32);
+    }
     gi.r = d.rs[0];
     gi.all_elig = d.rs[1] == 0;
+    __syncwarp();
 }
 
 // Dynamic work distribution of the single-instance persistent kernels: a warp takes its next
@@ -589,16 +590,10 @@ __device__ __forceinline__ void load_dev(Dev &dst, const Dev *src)
     __syncwarp();
 }
 
-// Persistent: each warp walks range items with a grid stride and takes the vertices of
-// sub-round s of a range 32 at a time (one slot per lane).
-//   pass A  flattened over the chunk's incidences (every record gather issued at once): W,
-//           b(u) (Sec. 5), eligibility (Sec. 6) and T = union of Lambda(e) over the nets with
-//           Phi(e,a) = 1, minus a and the blocks without room for c(u); (Lambda, omega) of each
-//           incidence is kept in shared memory.  Only blocks in T can have a positive gain,
-//           since g_t <= omega({e : Phi(e,a) = 1, t in Lambda(e)}).
-//   pass B  per vertex, conn_t = omega({e in I(u) : t in Lambda(e)}) for all t in T at once in
-//           bit planes, and the arg-max of g_t = b(u) - W + conn_t.
-// A vertex whose incident net weights exceed kPlaneMaxW uses a warp-cooperative pass instead.
+// Persistent: each warp walks range items and takes the vertices of sub-round s of a range 32 at a
+// time, one per lane (lane_best).  Only blocks in T can have a positive gain, since g_t <=
+// omega({e : Phi(e,a) = 1, t in Lambda(e)}); the best of them has the largest g_t = b(u) - W +
+// conn_t.  Vertices with more than kLaneDeg nets or W > kPlaneMaxW are walked by the whole warp.
 // B = false: one instance, d0 (parameter space), items are its ranges; B = true: a batch,
 // items name (instance, range) and each warp copies its item's instance into shared memory.
 template <typename Rec, bool B, bool RB = false>
@@ -606,17 +601,16 @@ __global__ void __launch_bounds__(kThreads, 4) k_gain(const Dev d0, const Dev *d
                                                       int32_t n_items, int32_t s, int32_t rr, RbArgs rb = RbArgs{0, 0, 0})
 {
     typedef typename RecIO<Rec>::Lam Lam;
-    __shared__ GainWarp<Lam> ws[kWarps];
-    __shared__ long long slack_w[kWarps][64];
-    __shared__ unsigned long long tot_w[kWarps][64];
+    __shared__ GainWarp ws[kWarps];
+    __shared__ unsigned long long tot_s[RB ? 64 : 1];
+    __shared__ uint8_t picked[RB ? kWarps : 1][kRange];
     __shared__ Dev dsm[B ? kWarps : 1];
     __shared__ unsigned long long cnt_s[2];
     __shared__ int warps_done;
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-    tot_w[wid][lane] = 0;
-    tot_w[wid][lane + 32] = 0;
+    if (RB && tid < 64) tot_s[tid] = 0;
     if (tid == 0) { cnt_s[0] = 0; cnt_s[1] = 0; warps_done = 0; }
-    __syncthreads();   // before any warp can add into another warp's slots (at its end)
+    __syncthreads();   // before any warp adds into them
     GainInst<Lam> gi;
     int32_t nelig = 0, ncand = 0;
     int inst_prev = -1;
@@ -629,48 +623,35 @@ __global__ void __launch_bounds__(kThreads, 4) k_gain(const Dev d0, const Dev *d
             const int2 it = items[item];
             if (it.x != inst_prev) {
                 load_dev(dsm[wid], devs + it.x);
-                gain_refresh<Rec>(dsm[wid], slack_w[wid], gi);
+                gain_refresh<Rec>(dsm[wid], ws[wid], gi);
                 inst_prev = it.x;
             }
             const Dev &d = dsm[wid];
             int32_t nel = 0;
-            const int32_t nout = gain_range<Rec, false>(d, it.y, s, ws[wid], slack_w[wid], tot_w[wid], gi, nel, rb);
-            if (lane == 0) d.cand_cnt[it.y] = nout;
-            // flush this item's totals into its own instance
-            unsigned long long *row = reinterpret_cast<unsigned long long *>(d.stats + (int64_t)rr * ST_N);
-            for (int t = lane; t < 64; t += 32) {
-                const unsigned long long v = tot_w[wid][t];
-                if (v) {
-                    atomicAdd(reinterpret_cast<unsigned long long *>(&d.tot[t]), v);
-                    tot_w[wid][t] = 0;
-                }
-            }
+            const int32_t nout = gain_range<Rec, false>(d, it.y, s, ws[wid], nullptr, tot_s, gi, nel, rb);
             if (lane == 0) {
+                d.cand_cnt[it.y] = nout;
+                unsigned long long *row = reinterpret_cast<unsigned long long *>(d.stats + (int64_t)rr * ST_N);
                 if (nel) atomicAdd(row + ST_ELIG, (unsigned long long)nel);
                 if (nout) atomicAdd(row + ST_CAND, (unsigned long long)nout);
             }
             __syncwarp();
         } else {
             if (inst_prev < 0) {
-                gain_refresh<Rec>(d0, slack_w[wid], gi);
+                gain_refresh<Rec>(d0, ws[wid], gi);
                 if (RB) gi.r = rb.r;
                 inst_prev = 0;
             }
             int32_t nel = 0;
-            const int32_t nout = gain_range<Rec, RB>(d0, item, s, ws[wid], slack_w[wid], tot_w[wid], gi, nel, rb);
+            const int32_t nout = gain_range<Rec, RB>(d0, item, s, ws[wid], picked[RB ? wid : 0], tot_s, gi, nel, rb);
             if (lane == 0) d0.cand_cnt[item] = nout;
             nelig += nel;
             ncand += nout;
         }
     }
     if (!B) {
-        // one instance: the warps add their partial sums into warp 0's slots as they finish and
-        // the last warp of the CTA flushes them with one atomic per block (no barrier, so warps
-        // that finish early do not wait for the slowest one)
-        if (wid != 0) {
-            for (int t = lane; t < 64; t += 32)
-                if (tot_w[wid][t]) atomicAdd(&tot_w[0][t], tot_w[wid][t]);
-        }
+        // one instance: the warps' partial sums meet in shared memory and the last warp of the CTA
+        // flushes them (no barrier, so warps that finish early do not wait for the slowest one)
         if (lane == 0) {
             if (nelig) atomicAdd(&cnt_s[0], (unsigned long long)nelig);
             if (ncand) atomicAdd(&cnt_s[1], (unsigned long long)ncand);
@@ -682,9 +663,11 @@ __global__ void __launch_bounds__(kThreads, 4) k_gain(const Dev d0, const Dev *d
         last = __shfl_sync(kFull, last, 0);
         if (last) {
             __threadfence_block();
-            for (int t = lane; t < 64 && t < d0.k; t += 32) {
-                const unsigned long long v = atomicAdd(&tot_w[0][t], 0ull);
-                if (v) atomicAdd(reinterpret_cast<unsigned long long *>(&d0.tot[t]), v);
+            if (RB) {
+                for (int t = lane; t < 64 && t < d0.k; t += 32) {
+                    const unsigned long long v = atomicAdd(&tot_s[t], 0ull);
+                    if (v) atomicAdd(reinterpret_cast<unsigned long long *>(&d0.tot[t]), v);
+                }
             }
             if (lane == 0) {
                 unsigned long long *row = reinterpret_cast<unsigned long long *>(d0.stats + (int64_t)rr * ST_N);
@@ -822,6 +805,7 @@ __global__ void __launch_bounds__(kThreads) k_select(const Dev *devs, const int2
     __shared__ unsigned long long wt[32];
     __shared__ int found_bin;
     __shared__ long long found_before;
+    __shared__ unsigned long long tot_s;
     const int tid = threadIdx.x;
     if ((int32_t)blockIdx.x >= item_count(devs, items, n_items, 2)) return;
     int32_t t;
@@ -829,31 +813,38 @@ __global__ void __launch_bounds__(kThreads) k_select(const Dev *devs, const int2
     Sel sl = d.sel[t];
     long long cap;
     int nbins;
+    unsigned long long *row = d.hist + (int64_t)t * kBins;
     if (level == 0) {
-        const long long tot = d.tot[t];
+        // LP: the gain step filled the level-0 row of every target block, the total is its sum
+        nbins = KEY == KEY_T ? d.bins : kBins;
+        long long tot = 0;
+        if (KEY == KEY_T) {
+            unsigned long long part = 0;
+            for (int b = tid; b < nbins; b += kThreads) part += row[b];
+            const unsigned long long before = block_scan_u64(part, wt);
+            if (tid == kThreads - 1) tot_s = before + part;
+            __syncthreads();
+            tot = (long long)tot_s;
+        } else {
+            tot = d.tot[t];
+        }
         cap = stage_cap<KEY>(d, t);
         if (tot == 0 || tot <= cap) {
-            if (KEY == KEY_T) {
-                // the gain step filled the level-0 row of every target block
-                unsigned long long *row0 = d.hist + (int64_t)t * kBins;
-                if (tot)
-                    for (int b = tid; b < kBins; b += kThreads) row0[b] = 0;
-            }
+            if (KEY == KEY_T && tot)
+                for (int b = tid; b < nbins; b += kThreads) row[b] = 0;
             if (tid == 0) {
                 Sel o;
                 o.mode = SEL_ALL; o.level = 0; o.g = 0; o.rem = 0; o.cut = 0;
                 d.sel[t] = o;
-                d.tot[t] = 0;
+                if (KEY != KEY_T) d.tot[t] = 0;
             }
             return;
         }
-        nbins = kBins;
     } else {
         if (sl.mode != SEL_REFINE || sl.level != level) return;
         cap = sl.rem;
         nbins = level == 1 ? 2048 : 1024;
     }
-    unsigned long long *row = d.hist + (int64_t)t * kBins;
     // thread i owns bins [nbins - per*(i+1), nbins - per*i), visited from high to low
     const int per = nbins / kThreads;
     const int hi = nbins - per * tid;
@@ -880,7 +871,7 @@ __global__ void __launch_bounds__(kThreads) k_select(const Dev *devs, const int2
         Sel o;
         o.cut = 0;
         if (level == 0) {
-            d.tot[t] = 0;
+            if (KEY != KEY_T) d.tot[t] = 0;
             if (fb < kBins - 1) {
                 o.mode = SEL_THRESH; o.level = 0; o.g = fb; o.rem = rem;
             } else {

@@ -336,9 +336,10 @@ __global__ void k_check_inputs(const int64_t *off64, int32_t *off32, int32_t m, 
 }
 
 // ------------------------------------------------------------------ per-vertex net weight
-// W(u) = sum of incident net weights must stay below 2^31 (int32 gain arithmetic)
+// W(u) = sum of incident net weights must stay below 2^31 (int32 gain arithmetic); kept in vnw
+// (weighted nets) for the gain step
 __global__ void k_vertex_netweight(const int32_t *vtx_off, const int32_t *inc, const int32_t *nw,
-                                   int32_t n, int32_t *err, unsigned long long *max_w)
+                                   int32_t n, int32_t *vnw, int32_t *err, unsigned long long *max_w)
 {
     if (input_invalid(err)) return;
     unsigned long long local = 0;
@@ -347,6 +348,7 @@ __global__ void k_vertex_netweight(const int32_t *vtx_off, const int32_t *inc, c
         int64_t s = 0;
         for (int32_t j = vtx_off[v]; j < vtx_off[v + 1]; ++j) s += nw ? nw[inc[j] & kNetMask] : 1;
         if (s >= (int64_t)1 << 31) atomicOr(err, ERR_UNSUPPORTED);
+        if (vnw) vnw[v] = (int32_t)s;
         local = max(local, (unsigned long long)s);
     }
     for (int o = 16; o; o >>= 1) local = max(local, __shfl_xor_sync(kFull, local, o));
@@ -1123,7 +1125,7 @@ size_t small_handle_bytes(int32_t n, int32_t m, int64_t P, int32_t k, const hgp_
     size_t b = 0;
     b += A(8 * (m + 1)) + A(4 * (m + 1)) + A(4 * P) + A(4 * (int64_t)n) + A(4 * 8);   // inputs, flags
     if (has_vw) b += A(4 * (int64_t)n);
-    if (has_nw) b += A(4 * (int64_t)m);
+    if (has_nw) b += A(4 * (int64_t)m) + A(4 * (int64_t)n);                           // and W(u)
     b += A(4 * (nb + 1)) + A(4 * (nm + 1));                                          // scan scratch
     b += A(4 * ((int64_t)n + 1)) + A(4 * P);                                         // vtx_off, inc
     b += A(n) + A(4 * (((int64_t)m * k * w + 3) / 4)) + A((int64_t)m * (k <= 32 ? 16 : 32)) + A(8 * (2 * 64 + 8));
@@ -1440,9 +1442,12 @@ int create_impl(int32_t n, int32_t m, const int64_t *net_offsets, const int32_t 
     d.inc = inc;
 
     unsigned long long *maxw_d = reinterpret_cast<unsigned long long *>(misc32 + 2);   // zeroed with misc32
+    int32_t *vnw = nullptr;
+    if (nw_d) CKF(dalloc(h, &vnw, n));
+    d.vnw = vnw;
     // the result of this check is read with the block weights at the end (nothing in between
     // depends on it)
-    k_vertex_netweight<<<grid_for(n, 256), 256, 0, st>>>(vtx_off, inc, nw_d, n, d.err, maxw_d); h->launches++;
+    k_vertex_netweight<<<grid_for(n, 256), 256, 0, st>>>(vtx_off, inc, nw_d, n, vnw, d.err, maxw_d); h->launches++;
     CKF(cudaGetLastError());
 
     // ---- state (Pi was stored by the input check)
@@ -1523,6 +1528,7 @@ int create_impl(int32_t n, int32_t m, const int64_t *net_offsets, const int32_t 
     if (host_err[0] & ERR_INVALID) return fail(HGP_ERR_INVALID);
     if (host_err[0] & ERR_UNSUPPORTED) return fail(HGP_ERR_UNSUPPORTED);
     h->max_vertex_netweight = (int64_t)maxw;
+    d.bins = (int32_t)std::min<int64_t>(kBins, ((int64_t)maxw + kThreads) / kThreads * kThreads);   // > maxw
     int64_t total = 0;
     for (int i = 0; i < k; ++i) total += bw[i];
     h->total_weight = total;

@@ -30,3 +30,23 @@ def test_ties_at_the_threshold_gain(n, weighted):
     hg = synth.random_small(n, n, n, 5, max_size=3, weighted=weighted, f=0.9)
     _check(hg, eps=0.004)
     _check(hg, eps=0.004, subrounds=1)
+
+
+@pytest.mark.parametrize("k", [2, 32, 33, 64])
+@pytest.mark.parametrize("m,scale", [(2_000, 0), (8_000, 0), (8_000, 1), (8_000, 6), (30_000, 0), (2_000, 1_000_000)])
+@pytest.mark.parametrize("balance", [False, True])
+def test_degrees_and_net_weights(k, m, scale, balance):
+    """300 vertices of about 23, 93 and 350 nets: below, around and above the degree (96) from which a
+    warp walks a vertex's nets together; net weights (scale > 0) put W(u) around and above 2047, the
+    last value the bit planes hold."""
+    hg = synth.random_small(k, 300, m, k, max_size=6, weighted=True, f=0.6)
+    hg.net_w = (hg.net_w * scale).astype(np.int32) if scale else None
+    hg.vertex_w = (hg.vertex_w * 3 - 2).astype(np.int32)      # 1..13: beside the weights with a mask of their own
+    hg.eps = 0.2
+    from paper_2010_10272_gb300 import HGP
+    h = HGP.from_hypergraph(hg, seed=9, balance_moves=balance)
+    o = oracle.Oracle.from_hypergraph(hg, subrounds=4, seed=9, balance_moves=balance)
+    want, _ = o.refine(4)
+    assert np.array_equal(h.refine(4)[:, :5], want[:, :5])
+    assert np.array_equal(h.partition(), o.partition())
+    h.close()
