@@ -15,18 +15,24 @@
 #pragma once
 
 #include <cuda_runtime.h>
+#include <math.h>
 #include <stdint.h>
 
 #include "hgp.h"
 
 namespace hgp {
 
-constexpr int kRange = 256;              // consecutive vertices handled by one warp
+constexpr int kSeg = 32;                 // list entries of a segment: one per lane
 constexpr int kWarps = 8;                // warps per tile CTA
 constexpr int kRvSlotBytes = 32;         // one slot of the revert variant's hash table
 constexpr int kWqPerRow = 128;           // work counters per stats row: 64 sub-rounds x 2 kernels
-constexpr int kTile = kRange * kWarps;   // vertices per tile (one CTA)
 constexpr int kThreads = 32 * kWarps;
+// consecutive vertices whose sub-round lists are built together.  A warp takes a list 32 entries
+// (a segment) at a time: the longer the list, the fewer of its segments are partly empty (with
+// S = 4, 512 +- 20 entries of 2048 vertices; of 256 vertices it was 64 +- 7, so that every second
+// list had a third segment of a few entries)
+constexpr int kTile = 2048;
+constexpr int kMaxSeg = kTile / kSeg;
 constexpr int kBins = 4096;              // approval histogram bins (gains 1..4094 exact)
 constexpr int kNever = -2;               // move-stamp round meaning "never moved"
 constexpr uint32_t kWideFlag = 0x80000000u;
@@ -68,11 +74,21 @@ enum { SEL_ALL = 0, SEL_THRESH = 1, SEL_REFINE = 2 };
 enum { ST_OBJ = 0, ST_CAND = 1, ST_APPR = 2, ST_ELIG = 3, ST_MAXW = 4, ST_MOVED = 5, ST_REV = 6, ST_N = 7 };
 enum { ERR_INVALID = 1, ERR_UNSUPPORTED = 2, ERR_TABLE = 4 };
 
+// segments per tile: two standard deviations above the mean length of a sub-round's list
+inline int32_t segments_of(int32_t S)
+{
+    const double mean = (double)kTile / S;
+    const double len = mean + 2.0 * sqrt(mean * (1.0 - 1.0 / S));
+    const int32_t s = (int32_t)((len + kSeg - 1) / kSeg);
+    return s < 1 ? 1 : (s > kMaxSeg ? kMaxSeg : s);
+}
+
 struct Dev {
     int32_t n, m, k, P;
     int32_t S;
     int32_t phi_w;          // 1, 2 or 4
-    int32_t n_ranges, n_tiles;
+    int32_t n_tiles;
+    int32_t nseg;           // segments per tile and sub-round; the last one takes the list's rest
     int64_t lmax;
     const int32_t *net_off;
     const int32_t *pins;
@@ -93,10 +109,11 @@ struct Dev {
     int64_t *bw;
     int64_t *obj;
     // scratch
-    uint8_t *sub_list;      // [n_ranges * kRange] local vertex offsets grouped by sub-round
-    uint16_t *sub_start;    // [n_ranges * (S + 1)]
-    uint64_t *cand;         // [n_ranges * kRange] (gain << 32 | local << 8 | target)
-    int32_t *cand_cnt;      // [n_ranges]
+    uint16_t *sub_list;     // [n_tiles * kTile] vertex offsets in the tile grouped by sub-round
+    uint16_t *sub_start;    // [n_tiles * (S + 1)]
+    uint64_t *cand;         // [n_tiles * kTile] (gain << 32 | offset << 8 | target); a segment's
+                            // candidates start at slot kSeg * segment of its tile
+    int32_t *cand_cnt;      // [n_tiles * nseg]
     int64_t *tot;           // [k] candidate weight per key block (rebalancing)
     unsigned long long *hist;  // [k * kBins]
     Sel *sel;               // [k]
@@ -111,7 +128,7 @@ struct Dev {
     int32_t *rs;            // round state on the device: rs[0] = next round r, rs[1] = 0 while
                             // every vertex is eligible (first round), 1 afterwards
     // revert variant only (nullptr otherwise)
-    uint8_t *rv_src;        // [n_ranges * kRange] per candidate slot: block an approved move left,
+    uint8_t *rv_src;        // [n_tiles * kTile] per candidate slot: block an approved move left,
                             // | 0x80 when it is to be undone; 0xFF when not approved
     void *rv_tab;           // hash table of (net, block) order statistics of the sub-round's moves
     int64_t rv_cap;         // its capacity in slots (a power of two >= 2 P)

@@ -3,8 +3,9 @@
 // One round r = round_prep, then for each sub-round s: gain -> approval -> apply, then
 // round_end.  Kernels and what they compute:
 //
-//   k_round_prep   splitmix64(seed ^ (r << 32 | u)) mod S for every vertex, and per warp range
-//                  of 256 vertices a list of its vertices grouped by sub-round (id order kept).
+//   k_round_prep   splitmix64(seed ^ (r << 32 | u)) mod S for every vertex, and per tile of 2048
+//                  vertices a list of its vertices grouped by sub-round (id order kept); the
+//                  sub-round kernels take such a list in segments of 32.
 //   k_gain         for each active vertex u (a = Pi(u)), against the frozen state:
 //                  W = omega(I(u)), b(u) = omega({e : Phi(e,a) = 1}) (Sec. 5), eligibility
 //                  (a net of u moved in round r-1, Sec. 6), and the best target
@@ -27,7 +28,7 @@
 //
 // Every kernel takes the instance state as `const Dev *devs` in device memory and a list of
 // work items.  A single-handle launch passes items == nullptr: item i is the handle's own
-// range / tile / block i.  A batch launch passes (instance, local index) pairs covering many
+// tile / block i.  A batch launch passes (instance, local index) pairs covering many
 // handles at once, so one launch per phase refines a whole batch.
 #include <cuda_runtime.h>
 #include <stddef.h>
@@ -66,69 +67,115 @@ __device__ __forceinline__ const Dev &item_of(const Dev *devs, const int2 *items
     return devs[0];
 }
 
+enum { ITEM_TILE = 1, ITEM_BLOCK = 2 };
 __device__ __forceinline__ int32_t item_count(const Dev *devs, const int2 *items, int32_t n_items, int kind)
 {
     if (items) return n_items;
-    return kind == 0 ? devs[0].n_ranges : (kind == 1 ? devs[0].n_tiles : devs[0].k);
+    return kind == ITEM_TILE ? devs[0].n_tiles : devs[0].k;
 }
 
+// A run of segments of one tile's candidates, spread over the lanes of a warp: candidate i of the
+// run is in slot at(i).  At most 32 segments.
+struct SegRun {
+    int32_t off[33];    // exclusive prefix of the segments' counts
+    int32_t slot0;      // first slot of the run (in Dev::cand / rv_src)
+    __device__ __forceinline__ int32_t load(const Dev &d, int32_t tile, int32_t s0, int32_t s1)
+    {
+        const int lane = threadIdx.x & 31;
+        const int32_t c = s0 + lane < s1 ? d.cand_cnt[(int64_t)tile * d.nseg + s0 + lane] : 0;
+        int32_t incl = c;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int32_t y = __shfl_up_sync(kFull, incl, o);
+            if (lane >= o) incl += y;
+        }
+        __syncwarp();
+        off[lane] = incl - c;
+        if (lane == 31) off[32] = incl;
+        if (lane == 0) slot0 = tile * kTile + s0 * kSeg;
+        __syncwarp();
+        return off[32];
+    }
+    __device__ __forceinline__ int32_t at(int32_t i) const
+    {
+        int v = 0;
+#pragma unroll
+        for (int st = 16; st; st >>= 1)
+            if (off[v + st] <= i) v += st;
+        return slot0 + v * kSeg + (i - off[v]);
+    }
+};
+
+// the segments of a tile that warp wid of a CTA of kWarps takes: [s0, s1)
+__device__ __forceinline__ void warp_segments(const Dev &d, int wid, int32_t &s0, int32_t &s1)
+{
+    const int32_t per = (d.nseg + kWarps - 1) / kWarps;
+    s0 = min(d.nseg, wid * per);
+    s1 = min(d.nseg, s0 + per);
+}
+
+// vertex of a candidate: its slot's tile and the offset in it
+__device__ __forceinline__ int32_t cand_vertex(int32_t slot, int ul) { return slot / kTile * kTile + ul; }
+
 // ------------------------------------------------------------------ round preparation
-// warp per range item
+// CTA per tile item; warp w hashes the tile's vertices [256 w, 256 w + 256), 8 per lane
 // r_ovr >= 0: hash with that round number instead of the device round state (rebalancing)
 __global__ void __launch_bounds__(kThreads) k_round_prep(const Dev *devs, const int2 *items, int32_t n_items,
                                                          int32_t r_ovr = -1)
 {
-    __shared__ uint8_t subs[kWarps][kRange];
-    __shared__ int32_t cnt[kWarps][65];
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const int32_t item = blockIdx.x * kWarps + wid;
-    if (item >= item_count(devs, items, n_items, 0)) return;
-    int32_t range;
-    const Dev d = item_of(devs, items, item, range);
+    __shared__ int32_t cnt[64][kWarps];   // then the first list position of (sub-round, warp)
+    __shared__ int32_t tot[64];
+    constexpr int kPer = kTile / kThreads;
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    if ((int32_t)blockIdx.x >= item_count(devs, items, n_items, ITEM_TILE)) return;
+    int32_t tile;
+    const Dev &d = item_of(devs, items, blockIdx.x, tile);
     const int32_t r = r_ovr >= 0 ? r_ovr : d.rs[0];
     const uint64_t seed = d.seed;
-    const int32_t base = range * kRange;
-    const int32_t nv = min(kRange, d.n - base);
     const int32_t S = d.S;
+    const int32_t nv = min(kTile, d.n - tile * kTile);
     const bool pow2 = (S & (S - 1)) == 0;
-    for (int i = lane; i <= S; i += 32) cnt[wid][i] = 0;
-    __syncwarp();
-    for (int c = 0; c < kRange / 32; ++c) {
-        const int idx = c * 32 + lane;
-        if (idx < nv) {
-            const uint32_t u = (uint32_t)(base + idx);
-            const uint64_t z = splitmix64_output(seed ^ (((uint64_t)(uint32_t)r << 32) | u));
-            const int sv = pow2 ? (int)(z & (uint64_t)(S - 1)) : (int)(z % (uint64_t)S);
-            subs[wid][idx] = (uint8_t)sv;
-            atomicAdd(&cnt[wid][sv], 1);
-        }
+    for (int i = tid; i < S * kWarps; i += kThreads) (&cnt[0][0])[i] = 0;
+    __syncthreads();
+    int sv[kPer];
+    const int first = wid * (kTile / kWarps) + lane;
+#pragma unroll
+    for (int c = 0; c < kPer; ++c) {
+        const int idx = first + c * 32;
+        const uint32_t u = (uint32_t)(tile * kTile + idx);
+        const uint64_t z = splitmix64_output(seed ^ (((uint64_t)(uint32_t)r << 32) | u));
+        sv[c] = idx < nv ? (pow2 ? (int)(z & (uint64_t)(S - 1)) : (int)(z % (uint64_t)S)) : -1;
+        const unsigned peers = __match_any_sync(kFull, sv[c]);
+        if (sv[c] >= 0 && lane == __ffs(peers) - 1) cnt[sv[c]][wid] += __popc(peers);
+        __syncwarp();
     }
-    __syncwarp();
-    uint16_t *ss = d.sub_start + (int64_t)range * (S + 1);
-    if (lane == 0) {
+    __syncthreads();
+    if (tid < S) {
+        int32_t t = 0;
+        for (int w = 0; w < kWarps; ++w) t += cnt[tid][w];
+        tot[tid] = t;
+    }
+    __syncthreads();
+    uint16_t *ss = d.sub_start + (int64_t)tile * (S + 1);
+    if (tid <= S) {
         int32_t run = 0;
-        for (int i = 0; i < S; ++i) {
-            const int32_t c = cnt[wid][i];
-            cnt[wid][i] = run;
-            ss[i] = (uint16_t)run;
-            run += c;
-        }
-        ss[S] = (uint16_t)run;
+        for (int i = 0; i < tid; ++i) run += tot[i];
+        ss[tid] = (uint16_t)run;
+        if (tid < S)
+            for (int w = 0; w < kWarps; ++w) {
+                const int32_t c = cnt[tid][w];
+                cnt[tid][w] = run;
+                run += c;
+            }
     }
-    __syncwarp();
-    uint8_t *list = d.sub_list + (int64_t)range * kRange;
-    for (int c = 0; c < kRange / 32; ++c) {
-        const int idx = c * 32 + lane;
-        const bool act = idx < nv;
-        const unsigned mask = __ballot_sync(kFull, act);
-        if (act) {
-            const int sv = subs[wid][idx];
-            const unsigned peers = __match_any_sync(mask, sv);
-            const int pos = cnt[wid][sv] + __popc(peers & lanemask_lt());
-            list[pos] = (uint8_t)idx;
-            __syncwarp(mask);
-            if (lane == __ffs(peers) - 1) cnt[wid][sv] += __popc(peers);
-        }
+    __syncthreads();
+    uint16_t *list = d.sub_list + (int64_t)tile * kTile;
+#pragma unroll
+    for (int c = 0; c < kPer; ++c) {
+        const unsigned peers = __match_any_sync(kFull, sv[c]);
+        if (sv[c] >= 0) list[cnt[sv[c]][wid] + __popc(peers & lanemask_lt())] = (uint16_t)(first + c * 32);
+        __syncwarp();
+        if (sv[c] >= 0 && lane == __ffs(peers) - 1) cnt[sv[c]][wid] += __popc(peers);
         __syncwarp();
     }
 }
@@ -186,6 +233,7 @@ constexpr int32_t kPlaneMaxW = 2047;   // W(u) up to this uses bit planes (NP <=
 // degrees above this are walked by the whole warp: its two passes cost about as many issue slots
 // as a lane's walk of this length with the other lanes idle
 constexpr int32_t kLaneDeg = 96;
+constexpr int kRbSegs = 6;             // segments of a rebalancing item
 constexpr int kFeasW = 8;              // vertex weights up to this have a mask of blocks with room
 
 // Per-warp state of the gain step that depends on the instance.
@@ -324,14 +372,15 @@ __device__ __forceinline__ void lane_best(const Rec *recs, const int32_t *inc, i
     }
 }
 
-// One range item of the gain step (see k_gain); returns the number of candidates written.
+// Segments [seg, seg_end) of one tile's list of sub-round s (see k_gain); returns the number of
+// candidates written, to the slots of segment seg.
 // RB: a rebalancing pass (Sec. 8): only vertices of overloaded blocks take part, their target
 // is the block with room of highest gain (any sign), and the candidate records its source
-// block (bits 16..23) and the priority gain + off; the per-block totals are by source block.
+// block (bits 19..24) and the priority gain + off; the per-block totals are by source block.
 template <typename Rec, bool RB>
-__device__ __forceinline__ int32_t gain_range(const Dev &d, int32_t range, int32_t s, const GainWarp &g,
-                                              uint8_t *picked, unsigned long long *tot, const GainInst<typename RecIO<Rec>::Lam> &gi,
-                                              int32_t &nel, const RbArgs &rb)
+__device__ __forceinline__ int32_t gain_seg(const Dev &d, int32_t tile, int32_t seg, int32_t seg_end, int32_t s,
+                                            const GainWarp &g, uint16_t *picked, unsigned long long *tot,
+                                            const GainInst<typename RecIO<Rec>::Lam> &gi, int32_t &nel, const RbArgs &rb)
 {
     typedef typename RecIO<Rec>::Lam Lam;
     constexpr bool kWide = sizeof(Lam) == 8;
@@ -341,26 +390,25 @@ __device__ __forceinline__ int32_t gain_range(const Dev &d, int32_t range, int32
     const Rec *recs = reinterpret_cast<const Rec *>(d.rec);
     const bool unit = d.nw == nullptr;
     const Lam kall = d.k >= (int)(8 * sizeof(Lam)) ? ~(Lam)0 : (((Lam)1 << d.k) - 1);
-    const int32_t rbase = range * kRange;
-    int32_t beg = 0, cnt = 0;
-    if (s < d.S) {
-        const uint16_t *ss = d.sub_start + (int64_t)range * (d.S + 1);
-        beg = ss[s];
-        cnt = (int32_t)ss[s + 1] - beg;
-    }
-    const uint8_t *list = d.sub_list + (int64_t)range * kRange + beg;
-    uint64_t *out = d.cand + (int64_t)range * kRange;
-    int32_t nout = 0;
+    const int32_t rbase = tile * kTile;
     nel = 0;
+    if (s >= d.S) return 0;
+    const uint16_t *ss = d.sub_start + (int64_t)tile * (d.S + 1);
+    const int32_t beg = ss[s] + seg * kSeg, end = ss[s + 1];
+    int32_t cnt = (seg_end == d.nseg ? end : min(end, (int32_t)ss[s] + seg_end * kSeg)) - beg;
+    if (cnt <= 0) return 0;
+    const uint16_t *list = d.sub_list + (int64_t)tile * kTile + beg;
+    uint64_t *out = d.cand + (int64_t)tile * kTile + seg * kSeg;
+    int32_t nout = 0;
     if (RB) {
-        // the vertices of overloaded blocks, few of a range, moved together first so that the
+        // the vertices of overloaded blocks, few of a list, moved together first so that the
         // lanes are full
         int32_t kept = 0;
         for (int32_t c0 = 0; c0 < cnt; c0 += 32) {
             const int32_t ul = c0 + lane < cnt ? list[c0 + lane] : 0;
             const bool over = c0 + lane < cnt && g.slack[d.part[rbase + ul]] < 0;
             const unsigned om = __ballot_sync(kFull, over);
-            if (over) picked[kept + __popc(om & lanemask_lt())] = (uint8_t)ul;
+            if (over) picked[kept + __popc(om & lanemask_lt())] = (uint16_t)ul;
             kept += __popc(om);
         }
         __syncwarp();
@@ -519,7 +567,7 @@ __device__ __forceinline__ int32_t gain_range(const Dev &d, int32_t range, int32
         if (t_best >= 0) {
             const int pos = nout + __popc(cm & lanemask_lt());
             if (RB) {
-                out[pos] = ((uint64_t)(uint32_t)(g_best + rb.off) << 32) | ((uint32_t)a << 16) |
+                out[pos] = ((uint64_t)(uint32_t)(g_best + rb.off) << 32) | ((uint32_t)a << 19) |
                            ((uint32_t)ul << 8) | (uint32_t)t_best;
                 atomicAdd(&tot[a], (unsigned long long)cu);
             } else {
@@ -561,25 +609,6 @@ __device__ __forceinline__ void gain_refresh(const Dev &d, GainWarp &g, GainInst
     __syncwarp();
 }
 
-// Dynamic work distribution of the single-instance persistent kernels: a warp takes its next
-// range item from a per-launch device counter (zeroed before the launch), so the last items go
-// to whichever warps are free instead of a fixed stride.
-__device__ __forceinline__ int32_t take_item(int32_t *counter)
-{
-    int32_t it = 0;
-    if ((threadIdx.x & 31) == 0) it = atomicAdd(counter, 1);
-    return __shfl_sync(kFull, it, 0);
-}
-
-// the counter increment is issued by lane 0 before the current item is processed; its result
-// is only read (broadcast) when the item is done, so the round trip overlaps the work
-__device__ __forceinline__ int32_t take_item_early(int32_t *counter)
-{
-    int32_t it = 0;
-    if ((threadIdx.x & 31) == 0) it = atomicAdd(counter, 1);
-    return it;
-}
-
 // copies devs[inst] into a warp's shared slot
 __device__ __forceinline__ void load_dev(Dev &dst, const Dev *src)
 {
@@ -590,20 +619,25 @@ __device__ __forceinline__ void load_dev(Dev &dst, const Dev *src)
     __syncwarp();
 }
 
-// Persistent: each warp walks range items and takes the vertices of sub-round s of a range 32 at a
-// time, one per lane (lane_best).  Only blocks in T can have a positive gain, since g_t <=
-// omega({e : Phi(e,a) = 1, t in Lambda(e)}); the best of them has the largest g_t = b(u) - W +
-// conn_t.  Vertices with more than kLaneDeg nets or W > kPlaneMaxW are walked by the whole warp.
-// B = false: one instance, d0 (parameter space), items are its ranges; B = true: a batch,
-// items name (instance, range) and each warp copies its item's instance into shared memory.
+// Persistent: each warp walks work items, a segment of one tile's sub-round list each (a
+// rebalancing item is kRbSegs segments, few of whose vertices take part), one vertex per lane
+// (lane_best).  Only blocks in T can have a positive gain, since g_t <= omega({e : Phi(e,a) = 1,
+// t in Lambda(e)}); the best of them has the largest g_t = b(u) - W + conn_t.  Vertices with more
+// than kLaneDeg nets or W > kPlaneMaxW are walked by the whole warp.
+// B = false: one instance, d0 (parameter space); B = true: a batch, items name (instance, tile)
+// and each warp copies its item's instance into shared memory.  per_tile: items per tile (batches:
+// the members' largest number of segments).  Work is handed out dynamically: a warp's first item is its index, the next
+// ones come from a per-launch device counter, `take` of them at a time (so that a large
+// instance's 10^5 items do not queue at one address), fetched while the items before are worked on.
 template <typename Rec, bool B, bool RB = false>
 __global__ void __launch_bounds__(kThreads, 4) k_gain(const Dev d0, const Dev *devs, const int2 *items,
-                                                      int32_t n_items, int32_t s, int32_t rr, RbArgs rb = RbArgs{0, 0, 0})
+                                                      int32_t n_items, int32_t per_tile, int32_t take, int32_t s,
+                                                      int32_t rr, RbArgs rb = RbArgs{0, 0, 0})
 {
     typedef typename RecIO<Rec>::Lam Lam;
     __shared__ GainWarp ws[kWarps];
     __shared__ unsigned long long tot_s[RB ? 64 : 1];
-    __shared__ uint8_t picked[RB ? kWarps : 1][kRange];
+    __shared__ uint16_t picked[RB ? kWarps : 1][RB ? kTile : 1];
     __shared__ Dev dsm[B ? kWarps : 1];
     __shared__ unsigned long long cnt_s[2];
     __shared__ int warps_done;
@@ -614,40 +648,61 @@ __global__ void __launch_bounds__(kThreads, 4) k_gain(const Dev d0, const Dev *d
     GainInst<Lam> gi;
     int32_t nelig = 0, ncand = 0;
     int inst_prev = -1;
-    const int32_t n_it = B ? n_items : d0.n_ranges;
+    const int32_t n_it = (B ? n_items : d0.n_tiles) * per_tile;
+    const int32_t warps = gridDim.x * kWarps;
     int32_t *wq = d0.wq + ((int64_t)rr * 64 + s) * 2;
-    int32_t next_raw = 0;
-    for (int32_t item = take_item(wq); item < n_it; item = __shfl_sync(kFull, next_raw, 0)) {
-        next_raw = take_item_early(wq);
-        if (B) {
-            const int2 it = items[item];
-            if (it.x != inst_prev) {
-                load_dev(dsm[wid], devs + it.x);
-                gain_refresh<Rec>(dsm[wid], ws[wid], gi);
-                inst_prev = it.x;
-            }
-            const Dev &d = dsm[wid];
+    int32_t group = blockIdx.x * kWarps + wid;
+    while ((int64_t)group * take < n_it) {
+        // issued by lane 0 now, read (broadcast) when the items are done
+        int32_t next = 0;
+        if (lane == 0 && (int64_t)warps * take < n_it) next = atomicAdd(wq, 1);
+        const int32_t it1 = min(n_it, (group + 1) * take);
+        for (int32_t it = group * take; it < it1; ++it) {
+            int32_t tile = it / per_tile;
+            const int32_t seg = (it - tile * per_tile) * (RB ? kRbSegs : 1);
             int32_t nel = 0;
-            const int32_t nout = gain_range<Rec, false>(d, it.y, s, ws[wid], nullptr, tot_s, gi, nel, rb);
-            if (lane == 0) {
-                d.cand_cnt[it.y] = nout;
-                unsigned long long *row = reinterpret_cast<unsigned long long *>(d.stats + (int64_t)rr * ST_N);
-                if (nel) atomicAdd(row + ST_ELIG, (unsigned long long)nel);
-                if (nout) atomicAdd(row + ST_CAND, (unsigned long long)nout);
+            if (B) {
+                const int2 im = items[tile];
+                tile = im.y;
+                if (im.x != inst_prev) {
+                    __syncwarp();
+                    load_dev(dsm[wid], devs + im.x);
+                    gain_refresh<Rec>(dsm[wid], ws[wid], gi);
+                    inst_prev = im.x;
+                }
+                const Dev &d = dsm[wid];
+                if (seg >= d.nseg) continue;
+                const int32_t nout = gain_seg<Rec, false>(d, tile, seg, seg + 1, s, ws[wid], nullptr, tot_s, gi, nel, rb);
+                if (lane == 0) {
+                    d.cand_cnt[(int64_t)tile * d.nseg + seg] = nout;
+                    unsigned long long *row = reinterpret_cast<unsigned long long *>(d.stats + (int64_t)rr * ST_N);
+                    if (nel) atomicAdd(row + ST_ELIG, (unsigned long long)nel);
+                    if (nout) atomicAdd(row + ST_CAND, (unsigned long long)nout);
+                }
+                __syncwarp();
+            } else {
+                if (inst_prev < 0) {
+                    gain_refresh<Rec>(d0, ws[wid], gi);
+                    if (RB) gi.r = rb.r;
+                    inst_prev = 0;
+                }
+                const int32_t seg_end = RB ? min(d0.nseg, seg + kRbSegs) : seg + 1;
+                const int32_t nout = gain_seg<Rec, RB>(d0, tile, seg, seg_end, s, ws[wid], picked[RB ? wid : 0], tot_s,
+                                                       gi, nel, rb);
+                int32_t *cnt = d0.cand_cnt + (int64_t)tile * d0.nseg + seg;
+                if (RB) {
+                    // the item's candidates lie together, filled segments first
+                    const int32_t q = lane, left = max(0, nout - q * kSeg);
+                    if (q < seg_end - seg) cnt[q] = seg + q == d0.nseg - 1 ? left : min(kSeg, left);
+                } else if (lane == 0) {
+                    *cnt = nout;
+                }
+                nelig += nel;
+                ncand += nout;
             }
-            __syncwarp();
-        } else {
-            if (inst_prev < 0) {
-                gain_refresh<Rec>(d0, ws[wid], gi);
-                if (RB) gi.r = rb.r;
-                inst_prev = 0;
-            }
-            int32_t nel = 0;
-            const int32_t nout = gain_range<Rec, RB>(d0, item, s, ws[wid], picked[RB ? wid : 0], tot_s, gi, nel, rb);
-            if (lane == 0) d0.cand_cnt[item] = nout;
-            nelig += nel;
-            ncand += nout;
         }
+        group = warps + __shfl_sync(kFull, next, 0);
+        if ((int64_t)warps * take >= n_it) break;
     }
     if (!B) {
         // one instance: the warps' partial sums meet in shared memory and the last warp of the CTA
@@ -683,24 +738,24 @@ __global__ void __launch_bounds__(kThreads, 4) k_gain(const Dev d0, const Dev *d
 __device__ __forceinline__ void decode(uint64_t c, int &t, int32_t &g, int &ul)
 {
     t = (int)(c & 0xFF);
-    ul = (int)((c >> 8) & 0xFF);
+    ul = (int)((c >> 8) & (kTile - 1));
     g = (int32_t)(c >> 32);
 }
 
 // Which block an approval stage groups a candidate by, and which candidates take part:
 //   KEY_T   LP: by target block, all candidates, inclusive prefix <= L_max - w(t);
-//   KEY_A   rebalancing, source side: by source block (bits 16..23), all candidates, a
+//   KEY_A   rebalancing, source side: by source block (bits 19..24), all candidates, a
 //           candidate passes while the weight before it is <= w(a) - L_max - 1 (exclusive);
 //   KEY_TS  rebalancing, target side: by target block, only candidates marked by KEY_A
-//           (bit 24), inclusive prefix <= L_max - w(t).
+//           (bit 25), inclusive prefix <= L_max - w(t).
 enum { KEY_T = 0, KEY_A = 1, KEY_TS = 2 };
-constexpr uint64_t kSelBit = 1ull << 24;
+constexpr uint64_t kSelBit = 1ull << 25;
 
 template <int KEY>
 __device__ __forceinline__ bool decode_key(uint64_t c, int &key, int &t, int32_t &g, int &ul)
 {
     decode(c, t, g, ul);
-    key = KEY == KEY_A ? (int)((c >> 16) & 0xFF) : t;
+    key = KEY == KEY_A ? (int)((c >> 19) & 0x3F) : t;
     return KEY != KEY_TS || (c & kSelBit) != 0;
 }
 
@@ -721,49 +776,48 @@ __device__ __forceinline__ int refine_digit(int32_t v, int level, int64_t prefix
     return v & 1023;
 }
 
-// warp per range item: histogram of candidate weight by gain for saturated key blocks
+// CTA per tile item: histogram of candidate weight by gain for saturated key blocks
 template <int KEY = KEY_T>
 __global__ void __launch_bounds__(kThreads) k_hist(const Dev *devs, const int2 *items, int32_t n_items, int level)
 {
-    __shared__ int active[kWarps][64];
-    __shared__ long long prefix[kWarps][64];
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const int32_t item = blockIdx.x * kWarps + wid;
-    if (item >= item_count(devs, items, n_items, 0)) return;
-    int32_t range;
-    const Dev d = item_of(devs, items, item, range);
-    int a_any = 0;
-    for (int t = lane; t < 64; t += 32) {
-        int a = 0;
-        if (t < d.k) {
-            if (level == 0) {
-                a = d.tot[t] > 0 && d.tot[t] > stage_cap<KEY>(d, t);
-            } else {
-                const Sel sl = d.sel[t];
-                a = sl.mode == SEL_REFINE && sl.level == level;
-                prefix[wid][t] = sl.g;
-            }
+    __shared__ int active[64];
+    __shared__ long long prefix[64];
+    __shared__ SegRun run_w[kWarps];
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    if ((int32_t)blockIdx.x >= item_count(devs, items, n_items, ITEM_TILE)) return;
+    int32_t tile;
+    const Dev &d = item_of(devs, items, blockIdx.x, tile);
+    int a = 0;
+    if (tid < d.k) {
+        if (level == 0) {
+            a = d.tot[tid] > 0 && d.tot[tid] > stage_cap<KEY>(d, tid);
+        } else {
+            const Sel sl = d.sel[tid];
+            a = sl.mode == SEL_REFINE && sl.level == level;
+            prefix[tid] = sl.g;
         }
-        active[wid][t] = a;
-        a_any |= a;
     }
-    if (!__any_sync(kFull, a_any)) return;
-    __syncwarp();
-    const int32_t n = d.cand_cnt[range];
-    const uint64_t *cand = d.cand + (int64_t)range * kRange;
-    for (int i = lane; i < n; i += 32) {
+    if (tid < 64) active[tid] = a;
+    if (!__syncthreads_or(a)) return;
+    int32_t s0, s1;
+    warp_segments(d, wid, s0, s1);
+    if (s0 >= s1) return;
+    SegRun &run = run_w[wid];
+    const int32_t n = run.load(d, tile, s0, s1);
+    for (int32_t i = lane; i < n; i += 32) {
+        const int32_t slot = run.at(i);
         int t, ul, key;
         int32_t g;
-        if (!decode_key<KEY>(cand[i], key, t, g, ul) || !active[wid][key]) continue;
+        if (!decode_key<KEY>(d.cand[slot], key, t, g, ul) || !active[key]) continue;
         t = key;
-        const unsigned long long c = d.vw ? (unsigned long long)d.vw[range * kRange + ul] : 1ull;
+        const unsigned long long c = d.vw ? (unsigned long long)d.vw[cand_vertex(slot, ul)] : 1ull;
         int bin;
         if (level == 0) {
             bin = g < kBins - 1 ? g : kBins - 1;
         } else {
             if (g < kBins - 1) continue;
             bool match;
-            bin = refine_digit(g - (kBins - 1), level, prefix[wid][t], match);
+            bin = refine_digit(g - (kBins - 1), level, prefix[t], match);
             if (!match) continue;
         }
         atomicAdd(&d.hist[(int64_t)t * kBins + bin], c);
@@ -807,7 +861,7 @@ __global__ void __launch_bounds__(kThreads) k_select(const Dev *devs, const int2
     __shared__ long long found_before;
     __shared__ unsigned long long tot_s;
     const int tid = threadIdx.x;
-    if ((int32_t)blockIdx.x >= item_count(devs, items, n_items, 2)) return;
+    if ((int32_t)blockIdx.x >= item_count(devs, items, n_items, ITEM_BLOCK)) return;
     int32_t t;
     const Dev d = item_of(devs, items, blockIdx.x, t);
     Sel sl = d.sel[t];
@@ -889,7 +943,7 @@ __global__ void __launch_bounds__(kThreads) k_select(const Dev *devs, const int2
     }
 }
 
-// one CTA per tile item (instance, tile of 8 ranges): weight of the candidates at their
+// one CTA per tile item (instance, tile): weight of the candidates at their
 // block's threshold gain, per block
 template <int KEY = KEY_T>
 __global__ void __launch_bounds__(kThreads) k_tie_sum(const Dev *devs, const int2 *items, int32_t n_items)
@@ -897,9 +951,10 @@ __global__ void __launch_bounds__(kThreads) k_tie_sum(const Dev *devs, const int
     __shared__ int thr[64];
     __shared__ int32_t gthr[64];
     __shared__ unsigned long long ts[64];
+    __shared__ SegRun run_w[kWarps];
     __shared__ int any;
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-    if ((int32_t)blockIdx.x >= item_count(devs, items, n_items, 1)) return;
+    if ((int32_t)blockIdx.x >= item_count(devs, items, n_items, ITEM_TILE)) return;
     int32_t tile;
     const Dev d = item_of(devs, items, blockIdx.x, tile);
     if (tid == 0) any = 0;
@@ -917,15 +972,16 @@ __global__ void __launch_bounds__(kThreads) k_tie_sum(const Dev *devs, const int
     }
     __syncthreads();
     if (!any) return;
-    const int32_t range = tile * kWarps + wid;
-    if (range < d.n_ranges) {
-        const int32_t n = d.cand_cnt[range];
-        const uint64_t *cand = d.cand + (int64_t)range * kRange;
-        for (int i = lane; i < n; i += 32) {
+    int32_t s0, s1;
+    warp_segments(d, wid, s0, s1);
+    if (s0 < s1) {
+        const int32_t n = run_w[wid].load(d, tile, s0, s1);
+        for (int32_t i = lane; i < n; i += 32) {
+            const int32_t slot = run_w[wid].at(i);
             int t, ul, key;
             int32_t g;
-            if (decode_key<KEY>(cand[i], key, t, g, ul) && thr[key] && g == gthr[key])
-                atomicAdd(&ts[key], d.vw ? (unsigned long long)d.vw[range * kRange + ul] : 1ull);
+            if (decode_key<KEY>(d.cand[slot], key, t, g, ul) && thr[key] && g == gthr[key])
+                atomicAdd(&ts[key], d.vw ? (unsigned long long)d.vw[cand_vertex(slot, ul)] : 1ull);
         }
     }
     __syncthreads();
@@ -936,8 +992,8 @@ __global__ void __launch_bounds__(kThreads) k_tie_sum(const Dev *devs, const int
 // gain pass.  Their inclusive (KEY_A: exclusive) weight prefix in id order only grows, so the
 // passing ones are those up to one id: the tile where the prefix crosses the budget is found from
 // the tile sums (tiles are in id order), the id inside it from the tile's candidates.  The apply
-// step then only compares ids; rebuilding the prefix of every range that held a tie there (its
-// tile's earlier ranges read again, one candidate at a time) took 2.0 ms of the power-law
+// step then only compares ids; rebuilding the prefix of every 256 vertices that held a tie there
+// (the earlier ones of the tile read again, one candidate at a time) took 2.0 ms of the power-law
 // instance's 67.3 ms (50 M vertices, k = 64, 5 rounds) and 0.06 of the row-net one's 6.56 ms.
 template <int KEY = KEY_T>
 __global__ void __launch_bounds__(1024) k_tie_cut(const Dev *devs, const int2 *items, int32_t n_items)
@@ -946,7 +1002,7 @@ __global__ void __launch_bounds__(1024) k_tie_cut(const Dev *devs, const int2 *i
     __shared__ unsigned long long carry_s, cross_before;
     __shared__ int32_t cross_tile;
     __shared__ int32_t cut_s;
-    if ((int32_t)blockIdx.x >= item_count(devs, items, n_items, 2)) return;
+    if ((int32_t)blockIdx.x >= item_count(devs, items, n_items, ITEM_BLOCK)) return;
     int32_t t;
     const Dev &d = item_of(devs, items, blockIdx.x, t);
     const Sel sl = d.sel[t];
@@ -987,14 +1043,14 @@ __global__ void __launch_bounds__(1024) k_tie_cut(const Dev *devs, const int2 *i
     __syncthreads();
     for (int b = 0; b < kTile; b += (int)blockDim.x) {
         const int slot = b + tid;
-        const int32_t range = tile * kWarps + slot / kRange;
+        const int32_t seg = min(slot / kSeg, d.nseg - 1);
         unsigned long long v = 0;
         int32_t u = -1;
-        if (range < d.n_ranges && slot % kRange < d.cand_cnt[range]) {
+        if (slot - seg * kSeg < d.cand_cnt[(int64_t)tile * d.nseg + seg]) {
             int key, tt, ul;
             int32_t g;
             if (decode_key<KEY>(d.cand[(int64_t)tile * kTile + slot], key, tt, g, ul) && key == t && g == (int32_t)sl.g) {
-                u = range * kRange + ul;
+                u = tile * kTile + ul;
                 v = d.vw ? (unsigned long long)d.vw[u] : 1ull;
             }
         }
@@ -1015,6 +1071,14 @@ struct alignas(16) ApplyWarp {
     int32_t jb[32];
     int32_t a[32];
     int32_t t[32];
+};
+
+// Approved moves of a warp that wait until 32 of them fill its lanes.
+constexpr int kDecide = 4;            // candidates a lane decides at a time
+constexpr int kQueue = 32 * (kDecide + 1);
+struct alignas(16) MoveQueue {
+    int32_t u[kQueue];
+    uint16_t at[kQueue];    // source block | target block << 8
 };
 
 // Applies up to kPins moved pins per lane (vertex moved a -> t, incident net e): Phi(e,a)--,
@@ -1114,79 +1178,142 @@ __device__ __forceinline__ void apply_refresh(const Dev &d, ApplyInst &ai, int32
     __syncwarp();
 }
 
-// Approval of the candidate in this lane's slot of a 32-candidate chunk: above its key block's
-// threshold gain, or at it up to the block's last id.
+// Approval of candidate i of a run: above its key block's threshold gain, or at it up to the
+// block's last id.
 template <int KEY>
-__device__ __forceinline__ bool approve_slot(const Dev &d, int32_t range, const uint64_t *cand, int32_t ncand,
-                                             int idx, const ApplyInst &ai, int &t, int &ul)
+__device__ __forceinline__ bool approve(uint64_t c, int32_t slot, const ApplyInst &ai, int &t, int32_t &u)
 {
-    t = 0; ul = 0;
-    if (idx >= ncand) return false;
-    int key;
+    int key, ul;
     int32_t g;
-    if (!decode_key<KEY>(cand[idx], key, t, g, ul)) return false;
-    return g > ai.gthr[key] || (g == ai.gthr[key] && range * kRange + ul <= ai.cut[key]);
+    if (!decode_key<KEY>(c, key, t, g, ul)) return false;
+    u = cand_vertex(slot, ul);
+    return g > ai.gthr[key] || (g == ai.gthr[key] && u <= ai.cut[key]);
 }
 
-// One range item of the apply step (see k_apply).  KEY_T: LP (stamps the nets, records the
-// revert variant's source blocks); KEY_TS: rebalancing (no stamps).
+// Applies the queued moves [first, first + 32) (at most `queued` in all) over their incidences,
+// flattened across the lanes.
 template <typename Rec, int KEY>
-__device__ __forceinline__ void apply_range(const Dev &d, int32_t range, int32_t r, const ApplyInst &ai,
-                                            unsigned long long *bwd, ApplyWarp &w_, long long &idobj,
-                                            int32_t &iappr, int32_t &ipins, int32_t &ishared)
+__device__ __forceinline__ void apply_queue(const Dev &d, const MoveQueue &mq, int32_t first, int32_t queued,
+                                            int32_t r, ApplyWarp &w_,
+                                            long long &dobj, int32_t &npins, int32_t &nshared)
 {
     const int lane = threadIdx.x & 31;
     Rec *recs = reinterpret_cast<Rec *>(d.rec);
-    const int32_t ncand = d.cand_cnt[range];
-    if (ncand == 0) return;
-    const uint64_t *cand = d.cand + (int64_t)range * kRange;
-    for (int32_t c0 = 0; c0 < ncand; c0 += 32) {
-        const int idx = c0 + lane;
-        int t, ul;
-        const bool appr = approve_slot<KEY>(d, range, cand, ncand, idx, ai, t, ul);
-        int32_t deg = 0, jb = 0, a = 0;
-        if (appr) {
-            const int32_t u = range * kRange + ul;
-            const unsigned long long cw = d.vw ? (unsigned long long)d.vw[u] : 1ull;
-            a = d.part[u];
-            d.part[u] = (uint8_t)t;
-            atomicAdd(&bwd[a], (unsigned long long)(-(long long)cw));
-            atomicAdd(&bwd[t], cw);
-            jb = d.vtx_off[u];
-            deg = d.vtx_off[u + 1] - jb;
-            ++iappr;
-            ipins += deg;
-        }
-        if (KEY == KEY_T && d.rv_src && idx < ncand) d.rv_src[(int64_t)range * kRange + idx] = appr ? (uint8_t)a : kRvNone;
-        int32_t incl = deg;
+    int32_t deg = 0, jb = 0, a = 0, t = 0;
+    if (first + lane < queued) {
+        const int32_t u = mq.u[first + lane], at = mq.at[first + lane];
+        a = at & 0xFF;
+        t = at >> 8;
+        jb = d.vtx_off[u];
+        deg = d.vtx_off[u + 1] - jb;
+        npins += deg;
+    }
+    int32_t incl = deg;
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int32_t y = __shfl_up_sync(kFull, incl, o);
-            if (lane >= o) incl += y;
+    for (int o = 1; o < 32; o <<= 1) {
+        const int32_t y = __shfl_up_sync(kFull, incl, o);
+        if (lane >= o) incl += y;
+    }
+    const int32_t total = __shfl_sync(kFull, incl, 31);
+    w_.off[lane] = incl - deg;
+    w_.jb[lane] = jb;
+    w_.a[lane] = a;
+    w_.t[lane] = t;
+    if (lane == 31) w_.off[32] = total;
+    __syncwarp();
+    for (int32_t i0 = 0; i0 < total; i0 += 32 * kPins)
+        dobj += apply_pins<Rec, KEY == KEY_T, KEY == KEY_T>(d, recs, w_, i0 + lane, total, r, &nshared);
+    __syncwarp();
+}
+
+// Segments [s0, s1) of one tile in the apply step (see k_apply).  KEY_T: LP (stamps the nets,
+// records the revert variant's source blocks); KEY_TS: rebalancing (no stamps).
+template <typename Rec, int KEY>
+__device__ __forceinline__ void apply_segs(const Dev &d, int32_t tile, int32_t s0, int32_t s1, int32_t r,
+                                           const ApplyInst &ai, unsigned long long *bwd, SegRun &run, ApplyWarp &w_,
+                                           MoveQueue &mq, int32_t &queued, long long &dobj, int32_t &nappr,
+                                           int32_t &npins, int32_t &nshared)
+{
+    const int lane = threadIdx.x & 31;
+    const int32_t ncand = run.load(d, tile, s0, s1);
+    for (int32_t c0 = 0; c0 < ncand; c0 += 32 * kDecide) {
+        // kDecide candidates per lane, their loads in flight together
+        int32_t slot[kDecide], u[kDecide];
+        int t[kDecide], a[kDecide];
+        uint64_t c[kDecide];
+        bool appr[kDecide];
+#pragma unroll
+        for (int q = 0; q < kDecide; ++q) {
+            const int32_t i = c0 + q * 32 + lane;
+            slot[q] = i < ncand ? run.at(i) : -1;
+            c[q] = slot[q] >= 0 ? d.cand[slot[q]] : 0;
         }
-        const int32_t total = __shfl_sync(kFull, incl, 31);
-        w_.off[lane] = incl - deg;
-        w_.jb[lane] = jb;
-        w_.a[lane] = a;
-        w_.t[lane] = t;
-        if (lane == 31) w_.off[32] = total;
+#pragma unroll
+        for (int q = 0; q < kDecide; ++q) {
+            t[q] = 0; a[q] = 0; u[q] = 0;
+            appr[q] = slot[q] >= 0 && approve<KEY>(c[q], slot[q], ai, t[q], u[q]);
+            if (appr[q]) a[q] = d.part[u[q]];
+        }
+#pragma unroll
+        for (int q = 0; q < kDecide; ++q) {
+            if (KEY == KEY_T && d.rv_src && slot[q] >= 0) d.rv_src[slot[q]] = appr[q] ? (uint8_t)a[q] : kRvNone;
+            const unsigned am = __ballot_sync(kFull, appr[q]);
+            if (am == 0) continue;
+            if (appr[q]) {
+                const unsigned long long cw = d.vw ? (unsigned long long)d.vw[u[q]] : 1ull;
+                d.part[u[q]] = (uint8_t)t[q];
+                if (!d.vw) {
+                    // unit weights: one update per distinct block
+                    const unsigned pa = __match_any_sync(am, a[q]), pt = __match_any_sync(am, t[q]);
+                    if (lane == __ffs(pa) - 1) atomicAdd(&bwd[a[q]], (unsigned long long)(-(long long)__popc(pa)));
+                    if (lane == __ffs(pt) - 1) atomicAdd(&bwd[t[q]], (unsigned long long)__popc(pt));
+                } else {
+                    atomicAdd(&bwd[a[q]], (unsigned long long)(-(long long)cw));
+                    atomicAdd(&bwd[t[q]], cw);
+                }
+                ++nappr;
+                const int pos = queued + __popc(am & lanemask_lt());
+                mq.u[pos] = u[q];
+                mq.at[pos] = (uint16_t)(a[q] | (t[q] << 8));
+            }
+            queued += __popc(am);
+        }
         __syncwarp();
-        for (int32_t i0 = 0; i0 < total; i0 += 32 * kPins)
-            idobj += apply_pins<Rec, KEY == KEY_T, KEY == KEY_T>(d, recs, w_, i0 + lane, total, r, &ishared);
+        int32_t first = 0;
+        for (; queued - first >= 32; first += 32)
+            apply_queue<Rec, KEY>(d, mq, first, queued, r, w_, dobj, npins, nshared);
+        if (first && queued - first > 0) {   // the rest moves to the front
+            int32_t u2 = 0;
+            uint16_t at2 = 0;
+            if (first + lane < queued) {
+                u2 = mq.u[first + lane];
+                at2 = mq.at[first + lane];
+            }
+            __syncwarp();
+            mq.u[lane] = u2;
+            mq.at[lane] = at2;
+        }
+        queued -= first;
         __syncwarp();
     }
 }
 
-// Persistent: each warp walks range items with a grid stride.  For each 32 candidates of a
-// range it decides approval (threshold gain and last tied id of the target block, see
-// k_tie_cut), then applies the approved moves over their incidences flattened across the lanes,
-// so all atomics are in flight at once.
+// Persistent: each warp walks work items with a grid stride, `per` consecutive segments of a tile
+// each.  For each 32 candidates it decides approval (threshold gain and last tied id of the target
+// block, see k_tie_cut) and queues the approved ones; whenever 32 are queued, from whichever items,
+// it applies them over their incidences flattened across the lanes, so all atomics are in flight
+// at once.  (In a saturated sub-round a fifth of the candidates is approved: without the queue a
+// chunk had 6 moves and 40 of the 128 pins it can have in flight.  Row-net 2M 35 -> 32 us per
+// launch, power-law 50M 1.05 -> 0.98 ms; the queue with one candidate decided per lane at a time,
+// a chain of loads for every 32, was slower than no queue, 42 us and 1.19 ms.)
 // B as for k_gain.
 template <typename Rec, bool B, int KEY = KEY_T>
 __global__ void __launch_bounds__(kThreads, 4) k_apply(const Dev d0, const Dev *devs, const int2 *items,
-                                                       int32_t n_items, int32_t rr, int32_t sub)
+                                                       int32_t n_items, int32_t nseg, int32_t per, int32_t rr)
 {
     __shared__ ApplyInst ai_w[kWarps];
+    __shared__ SegRun run_w[kWarps];
+    __shared__ MoveQueue mq_w[kWarps];
     __shared__ unsigned long long bwd_w[kWarps][64];
     __shared__ ApplyWarp aw[kWarps];
     __shared__ Dev dsm[B ? kWarps : 1];
@@ -1198,58 +1325,69 @@ __global__ void __launch_bounds__(kThreads, 4) k_apply(const Dev d0, const Dev *
     if (tid == 0) { objd = 0; napp = 0; mpins = 0; warps_done = 0; }
     __syncthreads();   // before any warp can add into another warp's slots (at its end)
     long long dobj = 0;
-    int32_t nappr = 0, npins = 0, r = 0, nshared = 0;
+    int32_t nappr = 0, npins = 0, r = 0, nshared = 0, queued = 0;
     int inst_prev = -1;
-    const int32_t n_it = B ? n_items : d0.n_ranges;
+    const int32_t groups = (nseg + per - 1) / per;
+    const int32_t n_it = (B ? n_items : d0.n_tiles) * groups;
+    // a batch instance's queue, block weights and counters, before the warp turns to another one
+    auto leave = [&](const Dev &d) {
+        if (queued) apply_queue<Rec, KEY>(d, mq_w[wid], 0, queued, r, aw[wid], dobj, npins, nshared);
+        queued = 0;
+        for (int o = 16; o; o >>= 1) {
+            dobj += __shfl_xor_sync(kFull, dobj, o);
+            nappr += __shfl_xor_sync(kFull, nappr, o);
+            npins += __shfl_xor_sync(kFull, npins, o);
+        }
+        __syncwarp();
+        for (int t = lane; t < 64; t += 32) {
+            const unsigned long long v = bwd_w[wid][t];
+            if (v) {
+                atomicAdd(reinterpret_cast<unsigned long long *>(&d.bw[t]), v);
+                bwd_w[wid][t] = 0;
+            }
+        }
+        if (lane == 0) {
+            unsigned long long *row = reinterpret_cast<unsigned long long *>(d.stats + (int64_t)rr * ST_N);
+            if (dobj) atomicAdd(reinterpret_cast<unsigned long long *>(d.obj), (unsigned long long)dobj);
+            if (nappr) atomicAdd(row + ST_APPR, (unsigned long long)nappr);
+            if (npins) atomicAdd(row + ST_MOVED, (unsigned long long)npins);
+        }
+        dobj = 0;
+        nappr = 0;
+        npins = 0;
+        __syncwarp();
+    };
     // static assignment (measured faster here than the gain step's dynamic distribution)
-    (void)sub;
     for (int32_t item = blockIdx.x * kWarps + wid; item < n_it; item += gridDim.x * kWarps) {
-        long long idobj = 0;
-        int32_t iappr = 0, ipins = 0, ishared = 0;
+        int32_t tile = item / groups;
+        const int32_t s0 = (item - tile * groups) * per;
         if (B) {
-            const int2 it = items[item];
+            const int2 it = items[tile];
+            tile = it.y;
             if (it.x != inst_prev) {
+                if (inst_prev >= 0) leave(dsm[wid]);
                 load_dev(dsm[wid], devs + it.x);
                 apply_refresh(dsm[wid], ai_w[wid], r);
                 inst_prev = it.x;
             }
             const Dev &d = dsm[wid];
-            apply_range<Rec, KEY>(d, it.y, r, ai_w[wid], bwd_w[wid], aw[wid], idobj, iappr, ipins,
-                                  ishared);
-            for (int o = 16; o; o >>= 1) {
-                idobj += __shfl_xor_sync(kFull, idobj, o);
-                iappr += __shfl_xor_sync(kFull, iappr, o);
-                ipins += __shfl_xor_sync(kFull, ipins, o);
-            }
-            __syncwarp();
-            for (int t = lane; t < 64; t += 32) {
-                const unsigned long long v = bwd_w[wid][t];
-                if (v) {
-                    atomicAdd(reinterpret_cast<unsigned long long *>(&d.bw[t]), v);
-                    bwd_w[wid][t] = 0;
-                }
-            }
-            if (lane == 0) {
-                unsigned long long *row = reinterpret_cast<unsigned long long *>(d.stats + (int64_t)rr * ST_N);
-                if (idobj) atomicAdd(reinterpret_cast<unsigned long long *>(d.obj), (unsigned long long)idobj);
-                if (iappr) atomicAdd(row + ST_APPR, (unsigned long long)iappr);
-                if (ipins) atomicAdd(row + ST_MOVED, (unsigned long long)ipins);
-                if (KEY == KEY_T && ipins && d.rv_cnt) atomicAdd(d.rv_cnt, (unsigned long long)ipins);
-            }
-            __syncwarp();
+            if (s0 >= d.nseg) continue;
+            apply_segs<Rec, KEY>(d, tile, s0, min(d.nseg, s0 + per), r, ai_w[wid], bwd_w[wid], run_w[wid], aw[wid],
+                                 mq_w[wid], queued, dobj, nappr, npins, nshared);
         } else {
             if (inst_prev < 0) {
                 apply_refresh(d0, ai_w[wid], r);
                 inst_prev = 0;
             }
-            apply_range<Rec, KEY>(d0, item, r, ai_w[wid], bwd_w[wid], aw[wid], idobj, iappr, ipins,
-                                  ishared);
-            dobj += idobj;
-            nappr += iappr;
-            npins += ipins;
-            nshared += ishared;
+            apply_segs<Rec, KEY>(d0, tile, s0, min(d0.nseg, s0 + per), r, ai_w[wid], bwd_w[wid], run_w[wid], aw[wid],
+                                 mq_w[wid], queued, dobj, nappr, npins, nshared);
         }
     }
+    if (B) {
+        if (inst_prev >= 0) leave(dsm[wid]);
+        return;
+    }
+    if (queued) apply_queue<Rec, KEY>(d0, mq_w[wid], 0, queued, r, aw[wid], dobj, npins, nshared);
     if (!B && KEY == KEY_T && d0.rv_cnt) {
         // revert variant: moved incidences on nets with several movers (sizes the order-statistics table)
         nshared = __reduce_add_sync(kFull, nshared);
@@ -1372,34 +1510,36 @@ struct alignas(16) RvWarp {
 
 enum { RV_INSERT = 0, RV_EVAL = 1 };
 
-// Warp per range: the approved movers of each 32 candidates, their incidences flattened over
+// CTA per tile, a run of its segments per warp: the approved movers of each 32 candidates, their incidences flattened over
 // the lanes, one of the passes above per launch.
 template <typename Rec, int PASS>
 __global__ void __launch_bounds__(kThreads) k_rv_pass(const Dev d)
 {
     __shared__ RvWarp rw_[kWarps];
+    __shared__ SegRun run_w[kWarps];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const int32_t range = blockIdx.x * kWarps + wid;
-    if (range >= d.n_ranges) return;
-    const int32_t ncand = d.cand_cnt[range];
+    int32_t s0, s1;
+    warp_segments(d, wid, s0, s1);
+    if (s0 >= s1) return;
+    SegRun &run = run_w[wid];
+    const int32_t ncand = run.load(d, blockIdx.x, s0, s1);
     if (ncand == 0) return;
     RvWarp &rw = rw_[wid];
     const uint64_t mask = (PASS == RV_INSERT || PASS == RV_EVAL) ? rv_slots(d) - 1 : 0;
     RvSlot *tab = reinterpret_cast<RvSlot *>(d.rv_tab);
     const Rec *recs = reinterpret_cast<const Rec *>(d.rec);
-    const uint64_t *cand = d.cand + (int64_t)range * kRange;
-    uint8_t *src = d.rv_src + (int64_t)range * kRange;
+    uint8_t *src = d.rv_src;
     bool lost = false;
     for (int32_t c0 = 0; c0 < ncand; c0 += 32) {
-        const int idx = c0 + lane;
+        const int32_t idx = c0 + lane < ncand ? run.at(c0 + lane) : 0;
         int32_t deg = 0, jb = 0, u = 0;
         int t = 0, a = 0;
-        const uint8_t sa = idx < ncand ? src[idx] : kRvNone;
+        const uint8_t sa = c0 + lane < ncand ? src[idx] : kRvNone;
         if (sa != kRvNone) {
             int ul;
             int32_t g;
-            decode(cand[idx], t, g, ul);
-            u = range * kRange + ul;
+            decode(d.cand[idx], t, g, ul);
+            u = cand_vertex(idx, ul);
             a = sa;
             jb = d.vtx_off[u];
             deg = d.vtx_off[u + 1] - jb;
@@ -1466,31 +1606,32 @@ __global__ void __launch_bounds__(kThreads) k_rv_pass(const Dev d)
     if (lost) atomicOr(d.err, ERR_TABLE);
 }
 
-// Warp per range: the marked moves go back to their source blocks (Phi, Lambda, S1, block
+// CTA per tile, a run of its segments per warp: the marked moves go back to their source blocks (Phi, Lambda, S1, block
 // weights, objective as in the apply step; the nets keep their round-r stamps).  Resets the
 // sub-round's moved-incidence count for the next sub-round.
 template <typename Rec>
 __global__ void __launch_bounds__(kThreads) k_rv_revert(const Dev d, int32_t rr)
 {
     __shared__ ApplyWarp aw[kWarps];
+    __shared__ SegRun run_w[kWarps];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const int32_t range = blockIdx.x * kWarps + wid;
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         d.rv_cnt[0] = 0;
         d.rv_cnt[1] = 0;
     }
-    if (range >= d.n_ranges) return;
-    const int32_t ncand = d.cand_cnt[range];
+    int32_t s0, s1;
+    warp_segments(d, wid, s0, s1);
+    if (s0 >= s1) return;
+    SegRun &run = run_w[wid];
+    const int32_t ncand = run.load(d, blockIdx.x, s0, s1);
     if (ncand == 0) return;
-    const uint8_t *src = d.rv_src + (int64_t)range * kRange;
-    const uint64_t *cand = d.cand + (int64_t)range * kRange;
     Rec *recs = reinterpret_cast<Rec *>(d.rec);
     const int32_t r = d.rs[0];
     long long dobj = 0;
     int32_t nrev = 0;
     for (int32_t c0 = 0; c0 < ncand; c0 += 32) {
-        const int idx = c0 + lane;
-        const uint8_t sa = idx < ncand ? src[idx] : kRvNone;
+        const int32_t idx = c0 + lane < ncand ? run.at(c0 + lane) : 0;
+        const uint8_t sa = c0 + lane < ncand ? d.rv_src[idx] : kRvNone;
         const bool back = sa != kRvNone && (sa & kRvBack);
         if (!__any_sync(kFull, back)) continue;
         int32_t deg = 0, jb = 0;
@@ -1498,8 +1639,8 @@ __global__ void __launch_bounds__(kThreads) k_rv_revert(const Dev d, int32_t rr)
         if (back) {
             int ul;
             int32_t g;
-            decode(cand[idx], t, g, ul);
-            const int32_t u = range * kRange + ul;
+            decode(d.cand[idx], t, g, ul);
+            const int32_t u = cand_vertex(idx, ul);
             a = sa & 0x3F;
             d.part[u] = (uint8_t)a;
             const long long cw = d.vw ? d.vw[u] : 1;
@@ -1561,12 +1702,13 @@ __global__ void k_round_end(const Dev *devs, int32_t n_inst, int32_t rr, int32_t
     }
 }
 
-// Rebalancing, source side (KEY_A): persistent, a warp per range item with a grid stride (the
+// Rebalancing, source side (KEY_A): persistent, a CTA per tile with a grid stride (the
 // per-block thresholds are read once per warp); marks the candidates that may leave their block
-// (bit 24) and adds their weights to the per-target totals of the target-side stage.
+// (bit 25) and adds their weights to the per-target totals of the target-side stage.
 __global__ void __launch_bounds__(kThreads) k_rb_mark(const Dev d)
 {
     __shared__ ApplyInst ai_w[kWarps];
+    __shared__ SegRun run_w[kWarps];
     __shared__ unsigned long long tot_w[kWarps][64];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     int32_t r;
@@ -1574,50 +1716,57 @@ __global__ void __launch_bounds__(kThreads) k_rb_mark(const Dev d)
     tot_w[wid][lane] = 0;
     tot_w[wid][lane + 32] = 0;
     __syncwarp();
-    for (int32_t range = blockIdx.x * kWarps + wid; range < d.n_ranges; range += gridDim.x * kWarps) {
-        const int32_t ncand = d.cand_cnt[range];
-        if (ncand == 0) continue;
-        uint64_t *cand = d.cand + (int64_t)range * kRange;
-        for (int32_t c0 = 0; c0 < ncand; c0 += 32) {
-            const int idx = c0 + lane;
-            int t, ul;
-            if (approve_slot<KEY_A>(d, range, cand, ncand, idx, ai_w[wid], t, ul)) {
-                cand[idx] |= kSelBit;
-                atomicAdd(&tot_w[wid][t], d.vw ? (unsigned long long)d.vw[range * kRange + ul] : 1ull);
+    int32_t s0, s1;
+    warp_segments(d, wid, s0, s1);
+    for (int32_t tile = blockIdx.x; tile < d.n_tiles && s0 < s1; tile += gridDim.x) {
+        const int32_t ncand = run_w[wid].load(d, tile, s0, s1);
+        for (int32_t i = lane; i < ncand; i += 32) {
+            const int32_t slot = run_w[wid].at(i);
+            int t;
+            int32_t u;
+            const uint64_t c = d.cand[slot];
+            if (approve<KEY_A>(c, slot, ai_w[wid], t, u)) {
+                d.cand[slot] = c | kSelBit;
+                atomicAdd(&tot_w[wid][t], d.vw ? (unsigned long long)d.vw[u] : 1ull);
             }
         }
-        __syncwarp();
     }
     __syncwarp();
     for (int t = lane; t < 64 && t < d.k; t += 32)
         if (tot_w[wid][t]) atomicAdd(reinterpret_cast<unsigned long long *>(&d.tot[t]), tot_w[wid][t]);
 }
 
-__global__ void k_expand_candidates(const Dev *devs, int32_t *target, int64_t *gain)
+__global__ void __launch_bounds__(kThreads) k_expand_candidates(const Dev *devs, int32_t *target, int64_t *gain)
 {
-    const Dev d = devs[0];
-    const int lane = threadIdx.x & 31;
-    const int32_t range = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (range >= d.n_ranges) return;
-    const int32_t n = d.cand_cnt[range];
-    for (int i = lane; i < n; i += 32) {
+    __shared__ SegRun run_w[kWarps];
+    const Dev &d = devs[0];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    int32_t s0, s1;
+    warp_segments(d, wid, s0, s1);
+    if (s0 >= s1) return;
+    const int32_t n = run_w[wid].load(d, blockIdx.x, s0, s1);
+    for (int32_t i = lane; i < n; i += 32) {
+        const int32_t slot = run_w[wid].at(i);
         int t, ul;
         int32_t g;
-        decode(d.cand[(int64_t)range * kRange + i], t, g, ul);
-        target[range * kRange + ul] = t;
-        gain[range * kRange + ul] = g;
+        decode(d.cand[slot], t, g, ul);
+        target[cand_vertex(slot, ul)] = t;
+        gain[cand_vertex(slot, ul)] = g;
     }
 }
 
 // ------------------------------------------------------------------ launch plans (host)
 // A set of instances with one record type, launched together: one instance with its own
-// ranges (items == nullptr), or a batch group with explicit (instance, local index) items.
+// tiles (items == nullptr), or a batch group with explicit (instance, local index) items.
 struct Plan {
     Dev d0{};                     // single instance: its state by value (kernel parameter)
     const Dev *devs = nullptr;
-    const int2 *ranges = nullptr, *tiles = nullptr, *blocks = nullptr;
-    int32_t n_ranges = 0, n_tiles = 0, n_blocks = 0, n_inst = 0;
+    const int2 *tiles = nullptr, *blocks = nullptr;
+    int32_t n_tiles = 0, n_blocks = 0, n_inst = 0;
     int32_t S_max = 0;
+    int32_t nseg = 1;      // segments per tile (batches: the members' largest)
+    int32_t take = 1;      // gain items a warp takes at a time
+    int32_t per = 1;       // segments per apply item
     bool levels = false;   // some instance can have gains >= kBins - 1
     bool rec32 = false;
     bool revert = false;   // revert variant (single instance only)
@@ -1627,29 +1776,40 @@ struct Plan {
     hgp_handle *prof = nullptr;   // per-phase event timing (single-instance launches only)
 };
 
+// persistent grid of ctas_per_sm CTAs per SM (0: as many as fit), at most one warp per work item
 template <typename K>
-int persistent_grid(int device, K kernel, int32_t n_ranges)
+int persistent_grid(int device, K kernel, int ctas_per_sm, int64_t n_items)
 {
-    int sms = 0, per_sm = 0;
+    int sms = 0, per_sm = ctas_per_sm;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kThreads, 0);
+    if (per_sm <= 0) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kThreads, 0);
     (void)cudaGetLastError();
     int64_t g = (int64_t)(sms > 0 ? sms : 1) * (per_sm > 0 ? per_sm : 1);
-    const int64_t need = (n_ranges + kWarps - 1) / kWarps;
+    const int64_t need = (n_items + kWarps - 1) / kWarps;
     if (g > need) g = need;
     return (int)(g < 1 ? 1 : g);
 }
 
-void set_grids(Plan &p, int device)
+// Grids and work granularity of the gain and apply kernels.  A gain item is one segment; a warp
+// takes several at a time once it has 32 or more of them (the counter is one address).  An apply
+// item is as many segments as leave a warp one item (its candidates are decided together), at
+// most half a tile.
+void set_grids(Plan &p, int device, int gain_ctas, int apply_ctas)
 {
-    const bool b = p.ranges != nullptr;
+    const bool b = p.tiles != nullptr;
+    const int64_t segs = (int64_t)p.n_tiles * p.nseg;
     if (p.rec32) {
-        p.grid_gain = persistent_grid(device, b ? k_gain<Rec32, true> : k_gain<Rec32, false>, p.n_ranges);
-        p.grid_apply = persistent_grid(device, b ? k_apply<Rec32, true> : k_apply<Rec32, false>, p.n_ranges);
+        p.grid_gain = persistent_grid(device, b ? k_gain<Rec32, true> : k_gain<Rec32, false>, gain_ctas, segs);
+        p.grid_apply = persistent_grid(device, b ? k_apply<Rec32, true> : k_apply<Rec32, false>, apply_ctas, segs);
     } else {
-        p.grid_gain = persistent_grid(device, b ? k_gain<Rec16, true> : k_gain<Rec16, false>, p.n_ranges);
-        p.grid_apply = persistent_grid(device, b ? k_apply<Rec16, true> : k_apply<Rec16, false>, p.n_ranges);
+        p.grid_gain = persistent_grid(device, b ? k_gain<Rec16, true> : k_gain<Rec16, false>, gain_ctas, segs);
+        p.grid_apply = persistent_grid(device, b ? k_apply<Rec16, true> : k_apply<Rec16, false>, apply_ctas, segs);
     }
+    p.take = (int32_t)std::min<int64_t>(4, std::max<int64_t>(1, segs / ((int64_t)p.grid_gain * kWarps * 8)));
+    int64_t per = (segs + (int64_t)p.grid_apply * kWarps - 1) / ((int64_t)p.grid_apply * kWarps);
+    per = std::min<int64_t>(std::max<int64_t>(per, 1), std::min<int64_t>(32, (p.nseg + 1) / 2));
+    const int64_t groups = (p.nseg + per - 1) / per;
+    p.per = (int32_t)((p.nseg + groups - 1) / groups);
 }
 
 // Per-phase event timing (profiling mode): a pair of events around each phase instance.
@@ -1709,22 +1869,20 @@ cudaError_t collect_profile(hgp_handle *h)
     return e;
 }
 
-unsigned warp_grid(int32_t n_items) { return (unsigned)((n_items + kWarps - 1) / kWarps); }
-
 cudaError_t launch_gain(const Plan &p, int32_t s, int32_t rr)
 {
-    const bool b = p.ranges != nullptr;
-    if (p.rec32 && b) k_gain<Rec32, true><<<p.grid_gain, kThreads, 0, p.st>>>(p.d0, p.devs, p.ranges, p.n_ranges, s, rr);
-    else if (p.rec32) k_gain<Rec32, false><<<p.grid_gain, kThreads, 0, p.st>>>(p.d0, p.devs, p.ranges, p.n_ranges, s, rr);
-    else if (b) k_gain<Rec16, true><<<p.grid_gain, kThreads, 0, p.st>>>(p.d0, p.devs, p.ranges, p.n_ranges, s, rr);
-    else k_gain<Rec16, false><<<p.grid_gain, kThreads, 0, p.st>>>(p.d0, p.devs, p.ranges, p.n_ranges, s, rr);
+    const bool b = p.tiles != nullptr;
+    if (p.rec32 && b) k_gain<Rec32, true><<<p.grid_gain, kThreads, 0, p.st>>>(p.d0, p.devs, p.tiles, p.n_tiles, p.nseg, p.take, s, rr);
+    else if (p.rec32) k_gain<Rec32, false><<<p.grid_gain, kThreads, 0, p.st>>>(p.d0, p.devs, p.tiles, p.n_tiles, p.nseg, p.take, s, rr);
+    else if (b) k_gain<Rec16, true><<<p.grid_gain, kThreads, 0, p.st>>>(p.d0, p.devs, p.tiles, p.n_tiles, p.nseg, p.take, s, rr);
+    else k_gain<Rec16, false><<<p.grid_gain, kThreads, 0, p.st>>>(p.d0, p.devs, p.tiles, p.n_tiles, p.nseg, p.take, s, rr);
     *p.launches += 1;
     return cudaGetLastError();
 }
 
 cudaError_t launch_prep(const Plan &p)
 {
-    k_round_prep<<<warp_grid(p.n_ranges), kThreads, 0, p.st>>>(p.devs, p.ranges, p.n_ranges);
+    k_round_prep<<<p.n_tiles, kThreads, 0, p.st>>>(p.devs, p.tiles, p.n_tiles);
     *p.launches += 1;
     return cudaGetLastError();
 }
@@ -1747,7 +1905,7 @@ cudaError_t launch_round(const Plan &p, int32_t rr)
         n += 1;
         if (p.levels) {
             for (int level = 1; level <= 3; ++level) {
-                k_hist<<<warp_grid(p.n_ranges), kThreads, 0, p.st>>>(p.devs, p.ranges, p.n_ranges, level);
+                k_hist<<<p.n_tiles, kThreads, 0, p.st>>>(p.devs, p.tiles, p.n_tiles, level);
                 k_select<<<p.n_blocks, kThreads, 0, p.st>>>(p.devs, p.blocks, p.n_blocks, level);
                 n += 2;
             }
@@ -1760,19 +1918,19 @@ cudaError_t launch_round(const Plan &p, int32_t rr)
         if (e == cudaSuccess) e = phase_end(p.prof, PH_APPROVE, n);
         if (e == cudaSuccess) e = phase_begin(p.prof);
         if (e != cudaSuccess) break;
-        const bool b = p.ranges != nullptr;
+        const bool b = p.tiles != nullptr;
         if (p.revert) e = cudaMemsetAsync(p.d0.rv_net, 0, sizeof(int32_t) * (size_t)p.d0.m, p.st);
         if (e != cudaSuccess) break;
-        if (p.rec32 && b) k_apply<Rec32, true><<<p.grid_apply, kThreads, 0, p.st>>>(p.d0, p.devs, p.ranges, p.n_ranges, rr, s);
-        else if (p.rec32) k_apply<Rec32, false><<<p.grid_apply, kThreads, 0, p.st>>>(p.d0, p.devs, p.ranges, p.n_ranges, rr, s);
-        else if (b) k_apply<Rec16, true><<<p.grid_apply, kThreads, 0, p.st>>>(p.d0, p.devs, p.ranges, p.n_ranges, rr, s);
-        else k_apply<Rec16, false><<<p.grid_apply, kThreads, 0, p.st>>>(p.d0, p.devs, p.ranges, p.n_ranges, rr, s);
+        if (p.rec32 && b) k_apply<Rec32, true><<<p.grid_apply, kThreads, 0, p.st>>>(p.d0, p.devs, p.tiles, p.n_tiles, p.nseg, p.per, rr);
+        else if (p.rec32) k_apply<Rec32, false><<<p.grid_apply, kThreads, 0, p.st>>>(p.d0, p.devs, p.tiles, p.n_tiles, p.nseg, p.per, rr);
+        else if (b) k_apply<Rec16, true><<<p.grid_apply, kThreads, 0, p.st>>>(p.d0, p.devs, p.tiles, p.n_tiles, p.nseg, p.per, rr);
+        else k_apply<Rec16, false><<<p.grid_apply, kThreads, 0, p.st>>>(p.d0, p.devs, p.tiles, p.n_tiles, p.nseg, p.per, rr);
         *p.launches += 1;
         e = cudaGetLastError();
         if (e == cudaSuccess) e = phase_end(p.prof, PH_APPLY, 1);
         if (p.revert && e == cudaSuccess) e = phase_begin(p.prof);
         if (e == cudaSuccess && p.revert) {
-            const unsigned g = warp_grid(p.n_ranges);
+            const unsigned g = p.n_tiles;
             // the apply step counted the movers of every net and the shared incidences
             k_rv_clear<<<p.grid_apply * 4, kThreads, 0, p.st>>>(p.d0);
             if (p.rec32) {
@@ -1817,25 +1975,13 @@ cudaError_t sync_dev(hgp_handle *h)
     return e;
 }
 
-// persistent grid of ctas_per_sm CTAs per SM (at most one warp per range item), or `fallback`
-int grid_override(int device, int ctas_per_sm, int fallback, int32_t n_ranges)
-{
-    if (ctas_per_sm <= 0) return fallback;
-    int sms = 0;
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
-    int64_t g = (int64_t)sms * ctas_per_sm;
-    const int64_t need = (n_ranges + kWarps - 1) / kWarps;
-    if (g > need) g = need;
-    return (int)(g < 1 ? 1 : g);
-}
-
 Plan single_plan(hgp_handle *h)
 {
     Plan p;
     p.d0 = h->d;
     p.devs = h->d_dev;
-    p.n_ranges = h->d.n_ranges;
     p.n_tiles = h->d.n_tiles;
+    p.nseg = h->d.nseg;
     p.n_blocks = h->d.k;
     p.n_inst = 1;
     p.S_max = h->d.S;
@@ -1843,13 +1989,16 @@ Plan single_plan(hgp_handle *h)
     p.rec32 = h->d.k > 32;
     p.revert = h->d.rv_src != nullptr;
     if (!h->grid_gain) {
-        Plan q = p;
-        set_grids(q, h->device);
-        h->grid_gain = grid_override(h->device, h->gain_ctas, q.grid_gain, p.n_ranges);
-        h->grid_apply = grid_override(h->device, h->apply_ctas, q.grid_apply, p.n_ranges);
+        set_grids(p, h->device, h->gain_ctas, h->apply_ctas);
+        h->grid_gain = p.grid_gain;
+        h->grid_apply = p.grid_apply;
+        h->gain_take = p.take;
+        h->apply_per = p.per;
     }
     p.grid_gain = h->grid_gain;
     p.grid_apply = h->grid_apply;
+    p.take = h->gain_take;
+    p.per = h->apply_per;
     p.st = h->stream;
     p.launches = &h->launches;
     p.prof = h->profiling ? h : nullptr;
@@ -2038,7 +2187,7 @@ int debug_candidates(hgp_handle *h, int32_t s, int32_t *target, int64_t *gain)
     if (e == cudaSuccess) e = cudaMemsetAsync(d.tot, 0, sizeof(int64_t) * 64, st);
     if (e == cudaSuccess) e = cudaMemsetAsync(d.hist, 0, sizeof(unsigned long long) * (size_t)d.k * kBins, st);
     if (e == cudaSuccess) {
-        k_expand_candidates<<<(d.n_ranges * 32 + 255) / 256, 256, 0, st>>>(h->d_dev, t_d, g_d);
+        k_expand_candidates<<<d.n_tiles, kThreads, 0, st>>>(h->d_dev, t_d, g_d);
         h->launches++;
         e = cudaGetLastError();
     }
@@ -2086,12 +2235,12 @@ template <int KEY>
 int64_t launch_stage(const Plan &p, bool levels)
 {
     int64_t n = 0;
-    k_hist<KEY><<<warp_grid(p.n_ranges), kThreads, 0, p.st>>>(p.devs, p.ranges, p.n_ranges, 0);
+    k_hist<KEY><<<p.n_tiles, kThreads, 0, p.st>>>(p.devs, p.tiles, p.n_tiles, 0);
     k_select<KEY><<<p.n_blocks, kThreads, 0, p.st>>>(p.devs, p.blocks, p.n_blocks, 0);
     n += 2;
     if (levels) {
         for (int level = 1; level <= 3; ++level) {
-            k_hist<KEY><<<warp_grid(p.n_ranges), kThreads, 0, p.st>>>(p.devs, p.ranges, p.n_ranges, level);
+            k_hist<KEY><<<p.n_tiles, kThreads, 0, p.st>>>(p.devs, p.tiles, p.n_tiles, level);
             k_select<KEY><<<p.n_blocks, kThreads, 0, p.st>>>(p.devs, p.blocks, p.n_blocks, level);
             n += 2;
         }
@@ -2106,16 +2255,17 @@ int64_t launch_stage(const Plan &p, bool levels)
 template <typename Rec>
 cudaError_t launch_rebalance_pass(const Plan &p, int32_t pass, RbArgs rb, bool levels)
 {
-    k_round_prep<<<warp_grid(p.n_ranges), kThreads, 0, p.st>>>(p.devs, p.ranges, p.n_ranges, rb.r);
+    k_round_prep<<<p.n_tiles, kThreads, 0, p.st>>>(p.devs, p.tiles, p.n_tiles, rb.r);
     *p.launches += 1;
     for (int32_t s = 0; s < p.S_max; ++s) {
-        k_gain<Rec, false, true><<<p.grid_gain, kThreads, 0, p.st>>>(p.d0, p.devs, p.ranges, p.n_ranges, s, pass, rb);
+        k_gain<Rec, false, true><<<p.grid_gain, kThreads, 0, p.st>>>(p.d0, p.devs, p.tiles, p.n_tiles, (p.nseg + kRbSegs - 1) / kRbSegs, 1, s,
+                                                                    pass, rb);
         *p.launches += 1;
         *p.launches += launch_stage<KEY_A>(p, levels);
         k_rb_mark<<<p.grid_apply, kThreads, 0, p.st>>>(p.d0);
         *p.launches += 1;
         *p.launches += launch_stage<KEY_TS>(p, levels);
-        k_apply<Rec, false, KEY_TS><<<p.grid_apply, kThreads, 0, p.st>>>(p.d0, p.devs, p.ranges, p.n_ranges, pass, s);
+        k_apply<Rec, false, KEY_TS><<<p.grid_apply, kThreads, 0, p.st>>>(p.d0, p.devs, p.tiles, p.n_tiles, p.nseg, p.per, pass);
         *p.launches += 1;
     }
     k_round_end<<<1, 128, 0, p.st>>>(p.devs, 1, pass, 0);
@@ -2208,7 +2358,7 @@ struct hgp_batch {
         Plan plan;
         std::vector<int32_t> members;           // indices into hs
         Dev *d_devs = nullptr;
-        int2 *d_items = nullptr;                // ranges, then tiles, then blocks
+        int2 *d_items = nullptr;                // tiles, then blocks
         int32_t *d_wq = nullptr;                // gain-step work counters [stats_cap * kWqPerRow]
     } g[2];
     int64_t *d_stats = nullptr;
@@ -2265,28 +2415,27 @@ int build_groups(hgp_batch *b, int32_t cap)
         gr.plan = Plan();
         if (gr.members.empty()) continue;
         std::vector<Dev> devs;
-        std::vector<int2> ranges, tiles, blocks;
-        int32_t S_max = 0;
+        std::vector<int2> tiles, blocks;
+        int32_t S_max = 0, nseg = 1;
         bool levels = false;
         for (size_t j = 0; j < gr.members.size(); ++j) {
             const hgp_handle *h = b->hs[gr.members[j]];
             Dev d = h->d;
             d.stats = b->d_stats + (int64_t)gr.members[j] * cap * ST_N;
             devs.push_back(d);
-            for (int32_t r = 0; r < d.n_ranges; ++r) ranges.push_back(make_int2((int)j, r));
             for (int32_t t = 0; t < d.n_tiles; ++t) tiles.push_back(make_int2((int)j, t));
             for (int32_t t = 0; t < d.k; ++t) blocks.push_back(make_int2((int)j, t));
             S_max = d.S > S_max ? d.S : S_max;
+            nseg = d.nseg > nseg ? d.nseg : nseg;
             levels = levels || h->max_vertex_netweight >= kBins - 1;
         }
-        const size_t n_items = ranges.size() + tiles.size() + blocks.size();
+        const size_t n_items = tiles.size() + blocks.size();
         e = dev_alloc(reinterpret_cast<void **>(&gr.d_devs), sizeof(Dev) * devs.size(), b->stream);
         if (e == cudaSuccess) e = dev_alloc(reinterpret_cast<void **>(&gr.d_items), sizeof(int2) * n_items, b->stream);
         if (e == cudaSuccess)
             e = dev_alloc(reinterpret_cast<void **>(&gr.d_wq), sizeof(int32_t) * kWqPerRow * (size_t)cap, b->stream);
         std::vector<int2> all;
         all.reserve(n_items);
-        all.insert(all.end(), ranges.begin(), ranges.end());
         all.insert(all.end(), tiles.begin(), tiles.end());
         all.insert(all.end(), blocks.begin(), blocks.end());
         // pageable sources: each call returns once its source has been staged
@@ -2301,19 +2450,16 @@ int build_groups(hgp_batch *b, int32_t cap)
         Plan &p = gr.plan;
         p.d0.wq = gr.d_wq;   // the batch kernels read only the work counters from d0
         p.devs = gr.d_devs;
-        p.ranges = gr.d_items;
-        p.tiles = gr.d_items + ranges.size();
-        p.blocks = gr.d_items + ranges.size() + tiles.size();
-        p.n_ranges = (int32_t)ranges.size();
+        p.tiles = gr.d_items;
+        p.blocks = gr.d_items + tiles.size();
+        p.nseg = nseg;
         p.n_tiles = (int32_t)tiles.size();
         p.n_blocks = (int32_t)blocks.size();
         p.n_inst = (int32_t)devs.size();
         p.S_max = S_max;
         p.levels = levels;
         p.rec32 = gi == 1;
-        set_grids(p, b->device);
-        p.grid_gain = grid_override(b->device, b->gain_ctas, p.grid_gain, p.n_ranges);
-        p.grid_apply = grid_override(b->device, b->apply_ctas, p.grid_apply, p.n_ranges);
+        set_grids(p, b->device, b->gain_ctas, b->apply_ctas);
         p.st = b->stream;
         p.launches = &b->launches;
     }

@@ -1116,7 +1116,7 @@ size_t small_handle_bytes(int32_t n, int32_t m, int64_t P, int32_t k, const hgp_
                           bool has_vw, bool has_nw)
 {
     auto A = [](int64_t bytes) -> size_t { return (size_t)((bytes < 1 ? 1 : bytes) + 255) / 256 * 256; };
-    const int64_t n_ranges = (n + kRange - 1) / kRange, n_tiles = (n_ranges + kWarps - 1) / kWarps;
+    const int64_t n_tiles = ((int64_t)n + kTile - 1) / kTile, nseg = segments_of(o.subrounds);
     const int64_t S = o.subrounds, nm = n > m ? n : m;
     const int w = o.phi_width ? o.phi_width : (max_size <= 255 ? 1 : 2);
     const int64_t nr_ctas = m > 0 ? std::min<int64_t>((m + 2047) / 2048, 1216) : 0;
@@ -1129,12 +1129,12 @@ size_t small_handle_bytes(int32_t n, int32_t m, int64_t P, int32_t k, const hgp_
     b += A(4 * (nb + 1)) + A(4 * (nm + 1));                                          // scan scratch
     b += A(4 * ((int64_t)n + 1)) + A(4 * P);                                         // vtx_off, inc
     b += A(n) + A(4 * (((int64_t)m * k * w + 3) / 4)) + A((int64_t)m * (k <= 32 ? 16 : 32)) + A(8 * (2 * 64 + 8));
-    b += A(n_ranges * kRange) + A(2 * n_ranges * (S + 1)) + A(8 * n_ranges * kRange) + A(4 * n_ranges);
+    b += A(2 * n_tiles * kTile) + A(2 * n_tiles * (S + 1)) + A(8 * n_tiles * kTile) + A(4 * n_tiles * nseg);
     b += A(8 * 64) + A(8 * (int64_t)k * kBins) + A((int64_t)sizeof(Sel) * 64) + A(8 * (int64_t)k * n_tiles);
     if (o.revert_negative) {
         int64_t cap = 1024;
         while (cap < 2 * P) cap <<= 1;
-        b += A(n_ranges * kRange) + A(16) + A(4 * (int64_t)m) + A(cap * kRvSlotBytes);
+        b += A(n_tiles * kTile) + A(16) + A(4 * (int64_t)m) + A(cap * kRvSlotBytes);
     }
     b += A(16);                                                                     // round state
     b += A(8 * ST_N * 16 + 4 * kWqPerRow * 16);                                      // statistics
@@ -1210,8 +1210,8 @@ int create_impl(int32_t n, int32_t m, const int64_t *net_offsets, const int32_t 
     d.k = k;
     d.P = (int32_t)P;
     d.S = o.subrounds;
-    d.n_ranges = (n + kRange - 1) / kRange;
-    d.n_tiles = (d.n_ranges + kWarps - 1) / kWarps;
+    d.n_tiles = (int32_t)(((int64_t)n + kTile - 1) / kTile);
+    d.nseg = segments_of(d.S);
 
 #define CKF(call)                                  \
     do {                                           \
@@ -1467,17 +1467,16 @@ int create_impl(int32_t n, int32_t m, const int64_t *net_offsets, const int32_t 
     d.obj = small + 64;
 
     // ---- per-sub-round scratch
-    uint8_t *sub_list = nullptr;
-    uint16_t *sub_start = nullptr;
+    uint16_t *sub_list = nullptr, *sub_start = nullptr;
     uint64_t *cand = nullptr;
     int32_t *cand_cnt = nullptr;
     int64_t *tot = nullptr, *tie = nullptr;
     unsigned long long *hist = nullptr;
     Sel *sel = nullptr;
-    CKF(dalloc(h, &sub_list, (int64_t)d.n_ranges * kRange));
-    CKF(dalloc(h, &sub_start, (int64_t)d.n_ranges * (d.S + 1)));
-    CKF(dalloc(h, &cand, (int64_t)d.n_ranges * kRange));
-    CKF(dalloc(h, &cand_cnt, d.n_ranges));
+    CKF(dalloc(h, &sub_list, (int64_t)d.n_tiles * kTile));
+    CKF(dalloc(h, &sub_start, (int64_t)d.n_tiles * (d.S + 1)));
+    CKF(dalloc(h, &cand, (int64_t)d.n_tiles * kTile));
+    CKF(dalloc(h, &cand_cnt, (int64_t)d.n_tiles * d.nseg));
     CKF(dalloc(h, &tot, 64));
     CKF(dalloc(h, &hist, (int64_t)k * kBins));
     CKF(dalloc(h, &sel, 64));
@@ -1500,7 +1499,7 @@ int create_impl(int32_t n, int32_t m, const int64_t *net_offsets, const int32_t 
         int64_t cap = 1024;
         while (cap < 2 * (int64_t)P) cap <<= 1;
         int32_t *rv_net = nullptr;
-        CKF(dalloc(h, &rv_src, (int64_t)d.n_ranges * kRange));
+        CKF(dalloc(h, &rv_src, (int64_t)d.n_tiles * kTile));
         CKF(dalloc(h, &rv_cnt, 2));
         CKF(dalloc(h, &rv_net, m));
         CKF(dalloc(h, reinterpret_cast<uint4 **>(&d.rv_tab), cap * kRvSlotBytes / 16));

@@ -50,3 +50,35 @@ def test_degrees_and_net_weights(k, m, scale, balance):
     assert np.array_equal(h.refine(4)[:, :5], want[:, :5])
     assert np.array_equal(h.partition(), o.partition())
     h.close()
+
+
+@pytest.mark.parametrize("S", [1, 2, 3, 7, 64])
+def test_tiles_and_segments(S):
+    """Sub-round lists of whole, partial and single-vertex tiles (2048 vertices) cut into segments of
+    32, alone and as members of one batch, and rebalancing from an overloaded start."""
+    from paper_2010_10272_gb300 import HGP, Batch
+    hgs = [synth.random_small(7 * n + S, n, n + 3, k, max_size=5, weighted=n % 2 == 0, f=0.7)
+           for n, k in ((4, 2), (31, 3), (2048, 40), (2049, 5), (5000, 16), (5000, 64))]
+    for hg in hgs:
+        _check(hg, rounds=3, subrounds=S)
+    subs = [S, S, S, 2, S, S]                                  # one member with its own count
+    hs = [HGP.from_hypergraph(hg, subrounds=s, seed=9) for hg, s in zip(hgs, subs)]
+    b = Batch(hs)
+    got = b.refine(3)
+    for i, hg in enumerate(hgs):
+        o = oracle.Oracle.from_hypergraph(hg, subrounds=subs[i], seed=9)
+        want, _ = o.refine(3)
+        assert np.array_equal(got[i][:, :5], want[:, :5])
+        assert np.array_equal(hs[i].partition(), o.partition())
+    b.close()
+    for h, hg, s in zip(hs, hgs, subs):
+        over = hg.part.copy()
+        over[: max(1, hg.n * 2 // 3)] = 0
+        h.set_partition(over)
+        o = oracle.Oracle.from_hypergraph(hg, part=over, subrounds=s, seed=9)
+        st, ph = h.rebalance(8)
+        want, wph = o.rebalance(8)[:2]
+        assert np.array_equal(st[:, :5], want[:, :5]) and np.array_equal(ph, wph)
+        assert np.array_equal(h.partition(), o.partition())
+        h.close()
+
