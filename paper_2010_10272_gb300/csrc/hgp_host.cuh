@@ -36,7 +36,7 @@ struct hgp_handle {
     // CUDA-graph cache: one refine() of `graph_rounds` rounds
     cudaGraphExec_t graph_exec = nullptr;
     int32_t graph_rounds = 0;
-    int32_t *d_round = nullptr;   // device round state (Dev::rs)
+    uint8_t *part_next = nullptr; // [n] a new partition between its check and its initialisation
     hgp::Dev *d_dev = nullptr;    // device copy of d, read by the kernels
     bool dev_dirty = true;        // d changed since the last upload
     int64_t graph_launches = 0;   // kernels in one replay of graph_exec

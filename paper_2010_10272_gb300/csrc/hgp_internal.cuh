@@ -72,6 +72,8 @@ struct Sel {
 
 enum { SEL_ALL = 0, SEL_THRESH = 1, SEL_REFINE = 2 };
 enum { ST_OBJ = 0, ST_CAND = 1, ST_APPR = 2, ST_ELIG = 3, ST_MAXW = 4, ST_MOVED = 5, ST_REV = 6, ST_N = 7 };
+// Dev::acc: block weights, objective, CTAs done
+enum { ACC_BW = 0, ACC_OBJ = 64, ACC_DONE = 65, kAccN = 66 };
 enum { ERR_INVALID = 1, ERR_UNSUPPORTED = 2, ERR_TABLE = 4 };
 
 // segments per tile: two standard deviations above the mean length of a sub-round's list
@@ -122,6 +124,7 @@ struct Dev {
     int32_t *wq;            // [rounds * kWqPerRow] work counters of the single-instance persistent
                             // kernels (nullptr in batches: static assignment)
     int32_t *err;
+    unsigned long long *acc;  // [kAccN] sums of a state initialisation, zero between them
     uint64_t seed;          // sub-round hash seed
     int32_t variant;        // bit 0: zero-gain balance moves; bit 1: revert negative moves
     int32_t pad0;

@@ -10,9 +10,11 @@
 #include <stdint.h>
 #include <string.h>
 
+#include <algorithm>
 #include <atomic>
 #include <mutex>
 #include <new>
+#include <type_traits>
 
 #include "hgp_host.cuh"
 
@@ -21,6 +23,7 @@ using namespace hgp;
 namespace {
 
 constexpr unsigned kFull = 0xffffffffu;
+constexpr int kDefaultSmem = 32 << 10;   // dynamic shared memory beside the static arrays (48 KB in all)
 
 // ------------------------------------------------------------------ prefix sums (int32)
 constexpr int kScanThreads = 1024;
@@ -284,21 +287,6 @@ __global__ void __launch_bounds__(256) k_nr_pins(const int32_t *off, const int32
     }
 }
 
-__global__ void k_check_vertices(const int32_t *vw, const int32_t *part_in, int32_t n, int32_t k,
-                                 int32_t *err)
-{
-    bool bad = false;
-    for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < n;
-         v += (int64_t)gridDim.x * blockDim.x) {
-        if (vw && vw[v] < 1) bad = true;
-        if (part_in) {
-            const int32_t p = part_in[v];
-            if (p < 0 || p >= k) bad = true;
-        }
-    }
-    if (__any_sync(kFull, bad) && (threadIdx.x & 31) == 0) atomicOr(err, ERR_INVALID);
-}
-
 // Creation queues its kernels behind the input checks without waiting for their verdict (for
 // instances whose net sizes the host reads itself, see create_impl): every kernel that indexes
 // by a pin, a vertex id or a block then returns at once when the checks flagged the input, and
@@ -309,13 +297,68 @@ __device__ __forceinline__ bool input_invalid(const int32_t *guard)
     return guard && (*reinterpret_cast<const volatile int32_t *>(guard) & ERR_INVALID) != 0;
 }
 
-// The creation's checks of the offsets (converted to int32 on the way), the net and vertex
-// weights and the partition in one launch; the valid partition entries are stored as the 1-byte
-// Pi at the same time.
-__global__ void k_check_inputs(const int64_t *off64, int32_t *off32, int32_t m, int64_t P, const int32_t *nw,
-                               const int32_t *vw, const int32_t *part_in, int32_t n, int32_t k, uint8_t *part,
-                               int32_t *err)
+// Adds the weights c (>= 1) of the lanes with ok to the shared block weights w, one update per
+// distinct block of the warp (same-address updates would queue up).
+__device__ __forceinline__ void add_block_weights(unsigned long long *w, bool ok, int blk, const int32_t *vw, int64_t v)
 {
+    const unsigned mask = __ballot_sync(kFull, ok);
+    if (!ok) return;
+    const unsigned peers = __match_any_sync(mask, blk);
+    unsigned long long sum = __popc(peers);
+    if (vw) {   // two halves: 32 sums of either fit 32 bits
+        const uint32_t c = (uint32_t)vw[v];
+        sum = (unsigned long long)__reduce_add_sync(peers, c & 0xFFFFu) +
+              ((unsigned long long)__reduce_add_sync(peers, c >> 16) << 16);
+    }
+    if ((int)(threadIdx.x & 31) == __ffs(peers) - 1) atomicAdd(&w[blk], sum);
+}
+
+// Stores the valid entries of a partition as 1-byte Pi and adds their vertices' weights to w (shared,
+// 64 zeros); returns whether an entry was out of range.
+__device__ __forceinline__ bool stage_partition(const int32_t *part_in, int32_t n, int32_t k, const int32_t *vw,
+                                                uint8_t *part, unsigned long long *w)
+{
+    bool bad = false;
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t v0 = blockIdx.x * (int64_t)blockDim.x + (threadIdx.x & ~31); v0 < n; v0 += stride) {
+        const int64_t v = v0 + (threadIdx.x & 31);
+        const int32_t p = v < n ? part_in[v] : -1;
+        const bool ok = p >= 0 && p < k;
+        if (v < n && !ok) bad = true;
+        if (ok) part[v] = (uint8_t)p;
+        add_block_weights(w, ok, p, vw, v);
+    }
+    return bad;
+}
+
+__device__ __forceinline__ void flush_block_weights(const unsigned long long *w, int32_t k, unsigned long long *acc)
+{
+    __syncthreads();
+    if (threadIdx.x < k && w[threadIdx.x]) atomicAdd(&acc[ACC_BW + threadIdx.x], w[threadIdx.x]);
+}
+
+// A new partition: range check, 1-byte Pi and block weights in one pass over it.
+__global__ void __launch_bounds__(256) k_stage_partition(const int32_t *part_in, int32_t n, int32_t k, const int32_t *vw,
+                                                         uint8_t *part, unsigned long long *acc, int32_t *err)
+{
+    __shared__ unsigned long long w[64];
+    if (threadIdx.x < 64) w[threadIdx.x] = 0;
+    __syncthreads();
+    const bool bad = stage_partition(part_in, n, k, vw, part, w);
+    if (__any_sync(kFull, bad) && (threadIdx.x & 31) == 0) atomicOr(err, ERR_INVALID);
+    flush_block_weights(w, k, acc);
+}
+
+// The creation's checks of the offsets (converted to int32 on the way), the net and vertex
+// weights and the partition in one launch; the partition is stored and weighed at the same time.
+__global__ void __launch_bounds__(256) k_check_inputs(const int64_t *off64, int32_t *off32, int32_t m, int64_t P,
+                                                      const int32_t *nw, const int32_t *vw, const int32_t *part_in,
+                                                      int32_t n, int32_t k, uint8_t *part, unsigned long long *acc,
+                                                      int32_t *err)
+{
+    __shared__ unsigned long long w[64];
+    if (threadIdx.x < 64) w[threadIdx.x] = 0;
+    __syncthreads();
     bool bad = false;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     const int64_t t0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
@@ -326,13 +369,12 @@ __global__ void k_check_inputs(const int64_t *off64, int32_t *off32, int32_t m, 
         if (e < m && nw && nw[e] < 1) bad = true;
         off32[e] = (int32_t)(a < 0 ? 0 : (a > P ? P : a));
     }
-    for (int64_t v = t0; v < n; v += stride) {
-        if (vw && vw[v] < 1) bad = true;
-        const int32_t p = part_in[v];
-        if (p < 0 || p >= k) bad = true;
-        else part[v] = (uint8_t)p;
-    }
+    if (vw)
+        for (int64_t v = t0; v < n; v += stride)
+            if (vw[v] < 1) bad = true;
+    if (stage_partition(part_in, n, k, vw, part, w)) bad = true;
     if (__any_sync(kFull, bad) && (threadIdx.x & 31) == 0) atomicOr(err, ERR_INVALID);
+    flush_block_weights(w, k, acc);
 }
 
 // ------------------------------------------------------------------ per-vertex net weight
@@ -610,247 +652,314 @@ __global__ void k_wide_flags(const int32_t *off, int32_t m, int32_t narrow_max, 
 }
 
 // ------------------------------------------------------------------ state initialisation
-__global__ void k_copy_part(const int32_t *in, uint8_t *part, int32_t n)
-{
-    for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < n;
-         v += (int64_t)gridDim.x * blockDim.x)
-        part[v] = (uint8_t)in[v];
-}
-
-__global__ void k_block_weights(Dev d, const int32_t *guard)
-{
-    if (input_invalid(guard)) return;
-    __shared__ unsigned long long w[64];
-    if (threadIdx.x < 64) w[threadIdx.x] = 0;
-    __syncthreads();
-    for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < d.n;
-         v += (int64_t)gridDim.x * blockDim.x)
-        atomicAdd(&w[d.part[v]], (unsigned long long)(d.vw ? d.vw[v] : 1));
-    __syncthreads();
-    if (threadIdx.x < d.k && w[threadIdx.x])
-        atomicAdd(reinterpret_cast<unsigned long long *>(&d.bw[threadIdx.x]), w[threadIdx.x]);
-}
-
-// Counts Phi(e, .) from the partition, writes the Phi rows, the records (Lambda, S1, omega,
-// stamp) and adds (lambda(e) - 1) * omega(e) to the objective.  A warp takes 32 consecutive nets,
-// one per lane: a net of at most kSmallNet pins is counted by its lane in registers; larger nets
-// are then counted by the whole warp, one at a time, with shared-memory counters.  The 32 Phi
-// rows are assembled in shared memory and written as one contiguous block (coalesced, and no
-// separate zeroing of the table); the rows of nets in the wide table stay zero there.
-constexpr int kSmallNet = 8;
+// Phi(e, .) counted from the partition, the Phi rows, the records (Lambda, S1, omega, stamp) and the
+// objective sum (lambda(e) - 1) * omega(e).
 constexpr int kInitWarps = 8;
+constexpr int32_t kInitBig = 2048;   // larger nets (or beyond a narrow entry) take a whole CTA
 
+// streaming stores: the table and the records exceed L2, where the partition has to stay
 template <typename Rec>
 __device__ __forceinline__ void write_record(const Dev &d, int64_t e, uint64_t lam, uint64_t s1, int32_t wf)
 {
-    Rec *rec = reinterpret_cast<Rec *>(d.rec) + e;
+    uint4 *rec = reinterpret_cast<uint4 *>(reinterpret_cast<Rec *>(d.rec) + e);
     if constexpr (sizeof(Rec) == 16) {
-        Rec r;
-        r.s1 = (uint32_t)s1;
-        r.w = wf;
-        r.mv = kNever * 2;
-        r.lam = (uint32_t)lam;
-        *rec = r;
+        __stcs(rec, make_uint4((uint32_t)s1, (uint32_t)wf, (uint32_t)(kNever * 2), (uint32_t)lam));
     } else {
-        Rec r;
-        r.s1 = s1;
-        r.w = wf;
-        r.mv = kNever * 2;
-        r.lam = lam;
-        r.w2 = wf;
-        r.pad = 0;
-        *rec = r;
+        __stcs(rec, make_uint4((uint32_t)s1, (uint32_t)(s1 >> 32), (uint32_t)wf, (uint32_t)(kNever * 2)));
+        __stcs(rec + 1, make_uint4((uint32_t)lam, (uint32_t)(lam >> 32), (uint32_t)wf, 0u));
     }
 }
 
-// entry i of the staged row block (rows of `wb` bytes per net, entries of `w` bytes)
-__device__ __forceinline__ void stage_set(uint8_t *blk, int row, int i, int w, int wb, int32_t v)
+__device__ __forceinline__ int32_t narrow_max_of(const Dev &d)
 {
-    uint8_t *p = blk + row * wb + i * w;
+    return d.phi_w == 1 ? 255 : (d.phi_w == 2 ? 65535 : 0x7fffffff);
+}
+
+// One net, by the whole CTA (256 threads); cnt: 64 shared counters.  Returns the net's objective
+// term in thread 0.
+template <typename Rec>
+__device__ __forceinline__ long long init_net_cta(const Dev &d, const uint8_t *part, int64_t e, int32_t *cnt)
+{
+    const int lane = threadIdx.x & 31;
+    const int w = d.phi_w;
+    long long obj = 0;
+    if (threadIdx.x < 64) cnt[threadIdx.x] = 0;
+    __syncthreads();
+    const int32_t b = d.net_off[e], sz = d.net_off[e + 1] - b;
+    for (int32_t j0 = 0; j0 < sz; j0 += 4 * (int32_t)blockDim.x) {
+        int blk[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {   // four pins per thread in flight
+            const int32_t j = j0 + q * (int32_t)blockDim.x + (int32_t)threadIdx.x;
+            blk[q] = j < sz ? d.pins[b + j] : -1;
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) blk[q] = blk[q] >= 0 ? part[blk[q]] : -1;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const unsigned peers = __match_any_sync(kFull, blk[q]);
+            if (blk[q] >= 0 && lane == __ffs(peers) - 1) atomicAdd(&cnt[blk[q]], (int)__popc(peers));
+        }
+    }
+    __syncthreads();
+    const bool wide = d.widx != nullptr && sz > narrow_max_of(d);
+    uint8_t *row = reinterpret_cast<uint8_t *>(d.phi) + e * (int64_t)(d.k * w);
+    for (int i = threadIdx.x; i < d.k; i += blockDim.x) {
+        const int32_t v = wide ? 0 : cnt[i];
+        if (w == 1) row[i] = (uint8_t)v;
+        else if (w == 2) reinterpret_cast<uint16_t *>(row)[i] = (uint16_t)v;
+        else reinterpret_cast<int32_t *>(row)[i] = v;
+        if (wide) d.phi_wide[(int64_t)d.widx[e] * d.k + i] = cnt[i];
+    }
+    if (threadIdx.x < 32) {
+        const unsigned lo_lam = __ballot_sync(kFull, lane < d.k && cnt[lane] > 0);
+        const unsigned lo_s1 = __ballot_sync(kFull, lane < d.k && cnt[lane] == 1);
+        const unsigned hi_lam = __ballot_sync(kFull, lane + 32 < d.k && cnt[lane + 32] > 0);
+        const unsigned hi_s1 = __ballot_sync(kFull, lane + 32 < d.k && cnt[lane + 32] == 1);
+        if (lane == 0) {
+            const int32_t wv = d.nw ? d.nw[e] : 1;
+            write_record<Rec>(d, e, (uint64_t)lo_lam | ((uint64_t)hi_lam << 32),
+                              (uint64_t)lo_s1 | ((uint64_t)hi_s1 << 32), wv | (wide ? (int32_t)kWideFlag : 0));
+            const int lambda = __popc(lo_lam) + __popc(hi_lam);
+            if (lambda > 0) obj = (long long)(lambda - 1) * wv;
+        }
+    }
+    __syncthreads();
+    return obj;
+}
+
+// The nets of the large-net prefix of the internal order, one CTA per net: k_init_nets would give all
+// of them to its first CTAs.
+template <typename Rec>
+__global__ void __launch_bounds__(256) k_init_big(Dev d, const uint8_t *part, int32_t m_big, const int32_t *guard)
+{
+    if (input_invalid(guard)) return;
+    __shared__ int32_t cnt[64];
+    long long obj = 0;
+    for (int64_t e = blockIdx.x; e < m_big; e += gridDim.x) obj += init_net_cta<Rec>(d, part, e, cnt);
+    if (threadIdx.x == 0 && obj) atomicAdd(&d.acc[ACC_OBJ], (unsigned long long)obj);
+}
+
+// entry i of the staged row block (rows of `wb` bytes per net, entries of `w` bytes)
+__device__ __forceinline__ void stage_set(uint32_t *blk, int row, int i, int w, int wb, int32_t v)
+{
+    uint8_t *p = reinterpret_cast<uint8_t *>(blk) + row * wb + i * w;
     if (w == 1) *p = (uint8_t)v;
     else if (w == 2) *reinterpret_cast<uint16_t *>(p) = (uint16_t)v;
     else *reinterpret_cast<int32_t *>(p) = v;
 }
 
+// One lane's net of at most N pins, counted in registers: pin i stands for its block if no earlier
+// pin is in it, with the number of pins that are.
+template <int N>
+struct LaneNet {
+    int blk[N], c[N];   // c: 0 unless pin i stands for its block
+    __device__ __forceinline__ void count(const int32_t *pins, const uint8_t *part, int32_t b, int32_t size)
+    {
+#pragma unroll
+        for (int i = 0; i < N; ++i) blk[i] = i < size ? __ldcs(&pins[b + i]) : -1;
+#pragma unroll
+        for (int i = 0; i < N; ++i) {
+            blk[i] = i < size ? (int)part[blk[i]] : -1 - i;   // no two absent pins alike
+            c[i] = i < size;
+        }
+#pragma unroll
+        for (int i = 1; i < N; ++i) {
+            bool merged = false;
+#pragma unroll
+            for (int j = 0; j < i; ++j) {
+                const bool same = !merged && c[j] > 0 && blk[j] == blk[i];
+                c[j] += same;
+                merged = merged || same;
+            }
+            if (merged) c[i] = 0;
+        }
+    }
+    __device__ __forceinline__ void sets(uint64_t &lam, uint64_t &s1) const
+    {
+#pragma unroll
+        for (int i = 0; i < N; ++i) {
+            if (c[i] > 0) lam |= 1ull << blk[i];
+            if (c[i] == 1) s1 |= 1ull << blk[i];
+        }
+    }
+    template <bool CLEAR>
+    __device__ __forceinline__ void stage(uint32_t *rows, int row, int w, int wb) const
+    {
+#pragma unroll
+        for (int i = 0; i < N; ++i)
+            if (c[i] > 0) stage_set(rows, row, blk[i], w, wb, CLEAR ? 0 : c[i]);
+    }
+};
+
+// The nets from e_begin on, 32 consecutive ones per warp.  Where none of the 32 has more than 4
+// pins, each lane counts its own in registers.  Else the lanes walk the 32 nets' pins, one run
+// in memory, flattened, four each in flight: counts by shared-memory atomics, whose old values give
+// the Lambda and S1 flips (a warp per net of more than 8 pins took the 32 nets one after another).
+// The 32 Phi rows are written as one contiguous block (no separate zeroing of the table).  Nets
+// beyond kInitBig pins or a narrow entry are left to the whole CTA.  Row-net 2M (20 M pins, k = 8):
+// 325 -> 137 us; power-law 50M (345 M pins, k = 64, 2-byte entries): 4.2 -> 3.2 ms, of which the
+// gathers of Pi take about 2.  4 CTAs per SM: with 5 (48 registers, spills) the power-law table took
+// 6.7 ms, with 3 the row-net one 160 us.
+// The last CTA to finish stores the block weights and the objective and resets the round state
+// (and the sums), so no other launch does; part, when another buffer than d.part, is copied there.
 template <typename Rec>
-__global__ void __launch_bounds__(kInitWarps * 32) k_init_nets(Dev d, int32_t e_begin, const int32_t *guard)
+__global__ void __launch_bounds__(kInitWarps * 32, 4) k_init_nets(Dev d, const uint8_t *part, int32_t e_begin,
+                                                               const int32_t *guard)
 {
     if (input_invalid(guard)) return;
-    __shared__ int32_t cnt[kInitWarps][64];
-    __shared__ long long part_obj[kInitWarps];
+    typedef typename std::conditional<sizeof(Rec) == 16, uint32_t, uint64_t>::type Lam;
+    constexpr int kHalves = sizeof(Lam) / 4;
+    __shared__ int32_t off33_w[kInitWarps][33];
+    __shared__ int32_t src_w[kInitWarps][32];
+    __shared__ uint32_t lam_w[kInitWarps][32 * kHalves], s1_w[kInitWarps][32 * kHalves];
+    __shared__ int32_t cnt[64];
+    __shared__ int32_t big_list[kInitWarps * 32];
+    __shared__ int32_t n_big;
+    __shared__ unsigned long long obj_s;
+    __shared__ bool last;
     extern __shared__ __align__(16) uint32_t stage_dyn[];   // kInitWarps blocks of 32 rows
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const int64_t warps = (int64_t)gridDim.x * kInitWarps;
-    const int32_t narrow_max = d.phi_w == 1 ? 255 : (d.phi_w == 2 ? 65535 : 0x7fffffff);
     const int w = d.phi_w, wb = d.k * d.phi_w;       // bytes per entry / per row
     const int blk_words = (32 * wb + 15) / 16 * 4;   // one warp's block, 16-byte multiple
-    uint32_t *stage_w = stage_dyn + wid * blk_words;
-    uint8_t *stage = reinterpret_cast<uint8_t *>(stage_w);
+    const int32_t big_from = min(kInitBig, narrow_max_of(d));
+    const uint32_t fmask = w == 1 ? 0xFFu : (w == 2 ? 0xFFFFu : 0xFFFFFFFFu);
+    uint32_t *stage = stage_dyn + wid * blk_words;
+    int32_t *off33 = off33_w[wid];
+    if (threadIdx.x == 0) {
+        n_big = 0;
+        obj_s = 0;
+    }
+    __syncthreads();
     long long obj = 0;
-    for (int64_t e0 = e_begin + ((int64_t)blockIdx.x * kInitWarps + wid) * 32; e0 < d.m; e0 += warps * 32) {
-        const int32_t rows = (int32_t)min((int64_t)32, (int64_t)d.m - e0);
-        for (int i = lane; i < blk_words; i += 32) stage_w[i] = 0;
-        __syncwarp();
-        const int64_t e = e0 + lane;
+    constexpr int kPerCta = kInitWarps * 32;
+    uint4 *s4 = reinterpret_cast<uint4 *>(stage);
+    for (int i = lane; i < blk_words / 4; i += 32) s4[i] = make_uint4(0, 0, 0, 0);   // and zero after every group
+    __syncwarp();
+    auto store_rows = [&](int64_t e0, int32_t rows) {
+        // the block of rows e0 .. e0 + rows - 1 starts at byte e0 * wb of the table
+        const int64_t byte0 = e0 * (int64_t)wb;
+        uint8_t *dst = reinterpret_cast<uint8_t *>(d.phi) + byte0;
+        if ((byte0 & 15) == 0 && (rows * wb) % 16 == 0) {
+            uint4 *d4 = reinterpret_cast<uint4 *>(dst);
+            for (int i = lane; i < rows * wb / 16; i += 32) __stcs(&d4[i], s4[i]);
+        } else {
+            // byte-exact tail (the table's rows need not be 16-byte multiples for small k)
+            const uint8_t *s8 = reinterpret_cast<const uint8_t *>(stage);
+            for (int i = lane; i < rows * wb; i += 32) dst[i] = s8[i];
+        }
+    };
+    for (int64_t c0 = e_begin + (int64_t)blockIdx.x * kPerCta; c0 < d.m; c0 += (int64_t)gridDim.x * kPerCta) {
+        const int64_t e0 = c0 + wid * 32, e = e0 + lane;
+        const int32_t rows = (int32_t)max((int64_t)0, min((int64_t)32, (int64_t)d.m - e0));
         int32_t b = 0, size = 0;
         if (e < d.m) {
             b = d.net_off[e];
             size = d.net_off[e + 1] - b;
         }
-        const bool small = e < d.m && size <= kSmallNet;
-        if (small) {
-            int32_t blk[kSmallNet], c[kSmallNet];
-            int nd = 0;
-#pragma unroll
-            for (int i = 0; i < kSmallNet; ++i) {
-                blk[i] = -1;
-                c[i] = 0;
-            }
-#pragma unroll
-            for (int i = 0; i < kSmallNet; ++i) {
-                if (i < size) {
-                    const int bk = d.part[d.pins[b + i]];
-                    bool found = false;
-#pragma unroll
-                    for (int j = 0; j < kSmallNet; ++j) {
-                        if (blk[j] == bk) { ++c[j]; found = true; }
-                    }
-                    if (!found) {
-#pragma unroll
-                        for (int j = 0; j < kSmallNet; ++j)
-                            if (j == nd) { blk[j] = bk; c[j] = 1; }
-                        ++nd;
-                    }
-                }
-            }
-            uint64_t lam = 0, s1 = 0;
-#pragma unroll
-            for (int j = 0; j < kSmallNet; ++j) {
-                if (j < nd) {
-                    lam |= 1ull << blk[j];
-                    if (c[j] == 1) s1 |= 1ull << blk[j];
-                    stage_set(stage, lane, blk[j], w, wb, c[j]);
-                }
-            }
-            const int32_t wv = d.nw ? d.nw[e] : 1;
-            write_record<Rec>(d, e, lam, s1, wv);
-            if (nd > 0) obj += (long long)(nd - 1) * wv;
-        }
-        // larger nets: the whole warp on one net at a time
-        unsigned big = __ballot_sync(kFull, e < d.m && !small);
-        while (big) {
-            const int src = __ffs(big) - 1;
-            big &= big - 1;
-            const int64_t ee = e0 + src;
-            const int32_t bb = __shfl_sync(kFull, b, src), sz = __shfl_sync(kFull, size, src);
-            cnt[wid][lane] = 0;
-            cnt[wid][lane + 32] = 0;
+        const bool big = size > big_from;
+        const int32_t wv = e < d.m && d.nw ? d.nw[e] : 1;
+        const int32_t most = (int32_t)__reduce_max_sync(kFull, (unsigned)size);
+        uint64_t lam = 0, s1 = 0;
+        auto in_registers = [&](auto net) {
+            net.count(d.pins, part, b, size);
+            net.sets(lam, s1);
+            net.template stage<false>(stage, lane, w, wb);
             __syncwarp();
-            for (int32_t base = bb; base < bb + sz; base += 32) {
-                const int32_t j = base + lane;
-                const bool act = j < bb + sz;
-                const unsigned mask = __ballot_sync(kFull, act);
-                if (act) {
-                    const int blk = d.part[d.pins[j]];
-                    const unsigned peers = __match_any_sync(mask, blk);
-                    if (lane == __ffs(peers) - 1) cnt[wid][blk] += __popc(peers);
-                }
-                __syncwarp();
-            }
-            const int32_t wv = d.nw ? d.nw[ee] : 1;
-            const bool wide = d.widx != nullptr && sz > narrow_max;
-            const int32_t wrow = wide ? d.widx[ee] : 0;
-            for (int i = lane; i < d.k; i += 32) {
-                if (wide) d.phi_wide[(int64_t)wrow * d.k + i] = cnt[wid][i];
-                else stage_set(stage, src, i, w, wb, cnt[wid][i]);
-            }
-            const unsigned lo_lam = __ballot_sync(kFull, lane < d.k && cnt[wid][lane] > 0);
-            const unsigned lo_s1 = __ballot_sync(kFull, lane < d.k && cnt[wid][lane] == 1);
-            const unsigned hi_lam = __ballot_sync(kFull, lane + 32 < d.k && cnt[wid][lane + 32] > 0);
-            const unsigned hi_s1 = __ballot_sync(kFull, lane + 32 < d.k && cnt[wid][lane + 32] == 1);
-            if (lane == 0) {
-                const int32_t wf = wv | (wide ? (int32_t)kWideFlag : 0);
-                write_record<Rec>(d, ee, (uint64_t)lo_lam | ((uint64_t)hi_lam << 32),
-                                  (uint64_t)lo_s1 | ((uint64_t)hi_s1 << 32), wf);
-                const int lambda = __popc(lo_lam) + __popc(hi_lam);
-                if (lambda > 0) obj += (long long)(lambda - 1) * wv;
-            }
+            store_rows(e0, rows);
             __syncwarp();
-        }
-        __syncwarp();
-        // the block of rows e0 .. e0 + rows - 1 starts at byte e0 * wb of the table
-        const int64_t byte0 = e0 * (int64_t)wb;
-        uint8_t *dst = reinterpret_cast<uint8_t *>(d.phi) + byte0;
-        if ((byte0 & 15) == 0 && (rows * wb) % 16 == 0) {
-            const uint4 *s4 = reinterpret_cast<const uint4 *>(stage_w);
-            uint4 *d4 = reinterpret_cast<uint4 *>(dst);
-            for (int i = lane; i < rows * wb / 16; i += 32) d4[i] = s4[i];
+            net.template stage<true>(stage, lane, w, wb);
+        };
+        if (most <= 4) {
+            in_registers(LaneNet<4>());
         } else {
-            // byte-exact tail (the table's rows need not be 16-byte multiples for small k)
-            for (int i = lane; i < rows * wb; i += 32) dst[i] = stage[i];
+#pragma unroll
+            for (int h = 0; h < kHalves; ++h) {
+                lam_w[wid][h * 32 + lane] = 0;
+                s1_w[wid][h * 32 + lane] = 0;
+            }
+            const int32_t sz = big ? 0 : size;
+            int32_t incl = sz;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int32_t y = __shfl_up_sync(kFull, incl, o);
+                if (lane >= o) incl += y;
+            }
+            off33[lane] = incl - sz;
+            src_w[wid][lane] = b - (incl - sz);
+            if (lane == 31) off33[32] = incl;
+            if (big) big_list[atomicAdd(&n_big, 1)] = (int32_t)e;
+            __syncwarp();
+            const int32_t total = off33[32];
+            for (int32_t i0 = 0; i0 < total; i0 += 128) {
+                int v[4], blk[4];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const int32_t i = i0 + q * 32 + lane;
+                    v[q] = i < total ? pin_net(off33, i) : 0;
+                    blk[q] = i < total ? __ldcs(&d.pins[src_w[wid][v[q]] + i]) : -1;
+                }
+#pragma unroll
+                for (int q = 0; q < 4; ++q) blk[q] = blk[q] >= 0 ? part[blk[q]] : -1;
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    if (blk[q] < 0) continue;
+                    const int at = v[q] * wb + blk[q] * w;
+                    const int sh = (at & 3) * 8;
+                    const uint32_t old = (atomicAdd(&stage[at >> 2], 1u << sh) >> sh) & fmask;
+                    const uint32_t bit = 1u << (blk[q] & 31);
+                    const int word = (blk[q] >> 5) * 32 + v[q];
+                    if (old == 0) atomicOr(&lam_w[wid][word], bit);
+                    if (old <= 1) atomicXor(&s1_w[wid][word], bit);
+                }
+            }
+            __syncwarp();
+            lam = lam_w[wid][lane];
+            s1 = s1_w[wid][lane];
+            if (kHalves == 2) {
+                lam |= (uint64_t)lam_w[wid][32 * (kHalves - 1) + lane] << 32;
+                s1 |= (uint64_t)s1_w[wid][32 * (kHalves - 1) + lane] << 32;
+            }
+            store_rows(e0, rows);
+            __syncwarp();
+            for (int i = lane; i < blk_words / 4; i += 32) s4[i] = make_uint4(0, 0, 0, 0);
+        }
+        if (e < d.m && !big) {
+            write_record<Rec>(d, e, lam, s1, wv);
+            if (lam) obj += (long long)(__popcll(lam) - 1) * wv;
         }
         __syncwarp();
+        // large nets of the CTA's 256; their rows were written as zeros above, before the barrier
+        if (__syncthreads_or(big)) {
+            const int32_t nb = n_big;
+            for (int32_t i = 0; i < nb; ++i) obj += init_net_cta<Rec>(d, part, big_list[i], cnt);
+            if (threadIdx.x == 0) n_big = 0;
+            __syncthreads();
+        }
+    }
+    if (part != d.part) {
+        const int64_t t0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, stride = (int64_t)gridDim.x * blockDim.x;
+        const int64_t n16 = d.n / 16;
+        for (int64_t i = t0; i < n16; i += stride)
+            reinterpret_cast<uint4 *>(d.part)[i] = reinterpret_cast<const uint4 *>(part)[i];
+        for (int64_t i = n16 * 16 + t0; i < d.n; i += stride) d.part[i] = part[i];
     }
     for (int o = 16; o; o >>= 1) obj += __shfl_xor_sync(kFull, obj, o);
-    if (lane == 0) part_obj[wid] = obj;
+    if (lane == 0 && obj) atomicAdd(&obj_s, (unsigned long long)obj);
     __syncthreads();
     if (threadIdx.x == 0) {
-        long long s = 0;
-        for (int i = 0; i < kInitWarps; ++i) s += part_obj[i];
-        if (s) atomicAdd(reinterpret_cast<unsigned long long *>(d.obj), (unsigned long long)s);
+        if (obj_s) atomicAdd(&d.acc[ACC_OBJ], obj_s);
+        __threadfence();
+        last = atomicAdd(&d.acc[ACC_DONE], 1ull) == gridDim.x - 1;
     }
-}
-
-// The nets of at least kBigNet pins, stored first in internal order (the prefix [0, m_big),
-// rounded up to whole 32-net groups), one CTA per net: k_init_nets would give all of them to
-// the first few warps.  Same results as k_init_nets for these nets (the narrow row of a net in
-// the wide table is written as zeros).
-template <typename Rec>
-__global__ void __launch_bounds__(256) k_init_big(Dev d, int32_t m_big, const int32_t *guard)
-{
-    if (input_invalid(guard)) return;
-    __shared__ int32_t cnt[64];
-    const int lane = threadIdx.x & 31;
-    const int32_t narrow_max = d.phi_w == 1 ? 255 : (d.phi_w == 2 ? 65535 : 0x7fffffff);
-    const int w = d.phi_w, wb = d.k * d.phi_w;
-    long long obj = 0;
-    for (int64_t e = blockIdx.x; e < m_big; e += gridDim.x) {
-        if (threadIdx.x < 64) cnt[threadIdx.x] = 0;
-        __syncthreads();
-        const int32_t b = d.net_off[e], sz = d.net_off[e + 1] - b;
-        for (int32_t j0 = 0; j0 < sz; j0 += blockDim.x) {
-            const int32_t j = j0 + threadIdx.x;
-            const bool act = j < sz;
-            const unsigned mask = __ballot_sync(kFull, act);
-            if (act) {
-                const int blk = d.part[d.pins[b + j]];
-                const unsigned peers = __match_any_sync(mask, blk);
-                if (lane == __ffs(peers) - 1) atomicAdd(&cnt[blk], (int)__popc(peers));
-            }
-        }
-        __syncthreads();
-        const bool wide = d.widx != nullptr && sz > narrow_max;
-        uint8_t *row = reinterpret_cast<uint8_t *>(d.phi) + e * (int64_t)wb;
-        for (int i = threadIdx.x; i < d.k; i += blockDim.x) {
-            stage_set(row, 0, i, w, wb, wide ? 0 : cnt[i]);
-            if (wide) d.phi_wide[(int64_t)d.widx[e] * d.k + i] = cnt[i];
-        }
-        if (threadIdx.x < 32) {
-            const unsigned lo_lam = __ballot_sync(kFull, lane < d.k && cnt[lane] > 0);
-            const unsigned lo_s1 = __ballot_sync(kFull, lane < d.k && cnt[lane] == 1);
-            const unsigned hi_lam = __ballot_sync(kFull, lane + 32 < d.k && cnt[lane + 32] > 0);
-            const unsigned hi_s1 = __ballot_sync(kFull, lane + 32 < d.k && cnt[lane + 32] == 1);
-            if (lane == 0) {
-                const int32_t wv = d.nw ? d.nw[e] : 1;
-                write_record<Rec>(d, e, (uint64_t)lo_lam | ((uint64_t)hi_lam << 32),
-                                  (uint64_t)lo_s1 | ((uint64_t)hi_s1 << 32), wv | (wide ? (int32_t)kWideFlag : 0));
-                const int lambda = __popc(lo_lam) + __popc(hi_lam);
-                if (lambda > 0) obj += (long long)(lambda - 1) * wv;
-            }
-        }
-        __syncthreads();
-    }
-    if (threadIdx.x == 0 && obj) atomicAdd(reinterpret_cast<unsigned long long *>(d.obj), (unsigned long long)obj);
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    if (threadIdx.x < d.k) d.bw[threadIdx.x] = (int64_t)__ldcg(&d.acc[ACC_BW + threadIdx.x]);
+    if (threadIdx.x == 64) *d.obj = (int64_t)__ldcg(&d.acc[ACC_OBJ]);
+    if (threadIdx.x < 2) d.rs[threadIdx.x] = 0;   // round 0, every vertex eligible
+    __syncthreads();
+    if (threadIdx.x < kAccN) d.acc[threadIdx.x] = 0;
 }
 
 // ------------------------------------------------------------------ getters
@@ -1065,48 +1174,42 @@ cudaError_t dalloc(hgp_handle *h, T **p, int64_t count)
         }                                          \
     } while (0)
 
-// guard: the creation's error flag while creating (kernels skip flagged input), else nullptr
-int init_state(hgp_handle *h, const int32_t *guard)
+// State of the partition in `part` (d.part, or a buffer that is copied there); its block weights are
+// in d.acc.  guard: the creation's error flag while creating (kernels skip flagged input), else nullptr
+int init_state(hgp_handle *h, const uint8_t *part, const int32_t *guard)
 {
     Dev &d = h->d;
     cudaStream_t st = h->stream;
-    CK(cudaMemsetAsync(d.bw, 0, sizeof(int64_t) * d.k, st));
-    CK(cudaMemsetAsync(d.obj, 0, sizeof(int64_t), st));
-    // round 0, every vertex eligible
-    CK(cudaMemsetAsync(d.rs, 0, 2 * sizeof(int32_t), st));
-    // the net kernel writes every narrow Phi row (zeros included); the wide table's rows are
-    // written by their nets, but a row of a net with zero pins in range stays as zeroed here
-    if (d.phi_wide && h->n_wide > 0) CK(cudaMemsetAsync(d.phi_wide, 0, sizeof(int32_t) * (size_t)h->n_wide * d.k, st));
-    k_block_weights<<<grid_for(d.n, 256), 256, 0, st>>>(d, guard); h->launches++;
-    CK(cudaGetLastError());
     const int32_t e_begin = h->m_big32;
     if (e_begin > 0) {
         const int gb = e_begin < 152 * 16 ? e_begin : 152 * 16;
-        if (d.k <= 32) k_init_big<Rec16><<<gb, 256, 0, st>>>(d, e_begin, guard);
-        else k_init_big<Rec32><<<gb, 256, 0, st>>>(d, e_begin, guard);
+        if (d.k <= 32) k_init_big<Rec16><<<gb, 256, 0, st>>>(d, part, e_begin, guard);
+        else k_init_big<Rec32><<<gb, 256, 0, st>>>(d, part, e_begin, guard);
         h->launches++;
     }
-    if (d.m > e_begin) {
-        const int g = grid_for(((int64_t)d.m - e_begin + 31) / 32 * 32, kInitWarps * 32, 152 * 16);
-        auto init_smem = [](int k, int w) { return kInitWarps * (32 * k * w + 15) / 16 * 16; };
-        const int smem = init_smem(d.k, d.phi_w);
-        // the attribute is the kernel's largest need over every k and entry width (the same
-        // value from every caller), so concurrent creations cannot lower it under each other
-        if (d.k <= 32) {
-            cudaFuncSetAttribute(k_init_nets<Rec16>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 init_smem(32, 4));
-            k_init_nets<Rec16><<<g, kInitWarps * 32, smem, st>>>(d, e_begin, guard); h->launches++;
-        } else {
-            cudaFuncSetAttribute(k_init_nets<Rec32>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 init_smem(64, 4));
-            k_init_nets<Rec32><<<g, kInitWarps * 32, smem, st>>>(d, e_begin, guard); h->launches++;
-        }
+    const int g = grid_for(std::max<int64_t>((int64_t)d.m - e_begin, 1), kInitWarps * 32, 152 * 16);
+    auto init_smem = [](int k, int w) { return kInitWarps * (32 * k * w + 15) / 16 * 16; };
+    const int smem = init_smem(d.k, d.phi_w);
+    // beyond the default limit the attribute is the kernel's largest need over every k and entry
+    // width (the same value from every caller), so concurrent creations cannot lower it under
+    // each other
+    if (d.k <= 32) {
+        if (smem > kDefaultSmem)
+            CK(cudaFuncSetAttribute(k_init_nets<Rec16>, cudaFuncAttributeMaxDynamicSharedMemorySize, init_smem(32, 4)));
+        k_init_nets<Rec16><<<g, kInitWarps * 32, smem, st>>>(d, part, e_begin, guard);
+    } else {
+        if (smem > kDefaultSmem)
+            CK(cudaFuncSetAttribute(k_init_nets<Rec32>, cudaFuncAttributeMaxDynamicSharedMemorySize, init_smem(64, 4)));
+        k_init_nets<Rec32><<<g, kInitWarps * 32, smem, st>>>(d, part, e_begin, guard);
     }
+    h->launches++;
     CK(cudaGetLastError());
     h->next_round = 0;
     h->all_eligible = true;
     return HGP_OK;
 }
+
+constexpr int kSmallN = 72 + kAccN;   // int64 entries of a handle's small state (see create_impl)
 
 // Device bytes of every buffer create_impl (and the first refine) allocates for a handle made
 // from host inputs of fewer than kHostSizesMaxNets nets, each rounded up to 256 bytes: the arena
@@ -1123,12 +1226,12 @@ size_t small_handle_bytes(int32_t n, int32_t m, int64_t P, int32_t k, const hgp_
     const int64_t scan_count = std::max<int64_t>(nm + 1, kNrRanks * nr_ctas + 1);
     const int64_t nb = (scan_count + kScanChunk - 1) / kScanChunk;
     size_t b = 0;
-    b += A(8 * (m + 1)) + A(4 * (m + 1)) + A(4 * P) + A(4 * (int64_t)n) + A(4 * 8);   // inputs, flags
+    b += A(8 * (m + 1)) + A(4 * (m + 1)) + A(4 * P) + A(4 * (int64_t)n);   // inputs
     if (has_vw) b += A(4 * (int64_t)n);
     if (has_nw) b += A(4 * (int64_t)m) + A(4 * (int64_t)n);                           // and W(u)
     b += A(4 * (nb + 1)) + A(4 * (nm + 1));                                          // scan scratch
     b += A(4 * ((int64_t)n + 1)) + A(4 * P);                                         // vtx_off, inc
-    b += A(n) + A(4 * (((int64_t)m * k * w + 3) / 4)) + A((int64_t)m * (k <= 32 ? 16 : 32)) + A(8 * (2 * 64 + 8));
+    b += 2 * A(n) + A(4 * (((int64_t)m * k * w + 3) / 4)) + A((int64_t)m * (k <= 32 ? 16 : 32)) + A(8 * kSmallN);
     b += A(2 * n_tiles * kTile) + A(2 * n_tiles * (S + 1)) + A(8 * n_tiles * kTile) + A(4 * n_tiles * nseg);
     b += A(8 * 64) + A(8 * (int64_t)k * kBins) + A((int64_t)sizeof(Sel) * 64) + A(8 * (int64_t)k * n_tiles);
     if (o.revert_negative) {
@@ -1136,7 +1239,6 @@ size_t small_handle_bytes(int32_t n, int32_t m, int64_t P, int32_t k, const hgp_
         while (cap < 2 * P) cap <<= 1;
         b += A(n_tiles * kTile) + A(16) + A(4 * (int64_t)m) + A(cap * kRvSlotBytes);
     }
-    b += A(16);                                                                     // round state
     b += A(8 * ST_N * 16 + 4 * kWqPerRow * 16);                                      // statistics
     b += A(sizeof(Dev));                                                            // device Dev
     return b;
@@ -1251,16 +1353,24 @@ int create_impl(int32_t n, int32_t m, const int64_t *net_offsets, const int32_t 
 
     // ---- inputs
     int64_t *off64 = nullptr;
-    int32_t *part_in = nullptr, *tmp = nullptr, *misc32 = nullptr;
+    int32_t *part_in = nullptr, *tmp = nullptr;
     int32_t *net_off = nullptr, *pins_d = nullptr, *vw_d = nullptr, *nw_d = nullptr;
     CKF(dalloc(h, &off64, (int64_t)m + 1));
     CKF(dalloc(h, &net_off, (int64_t)m + 1));
     CKF(dalloc(h, &pins_d, P));
     CKF(dalloc(h, &part_in, n));
-    CKF(dalloc(h, &misc32, 8));   // err, max net size
-    CKF(cudaMemsetAsync(misc32, 0, 8 * sizeof(int32_t), st));
-    d.err = misc32;
-    int32_t *max_size_d = misc32 + 1;
+    // small state: block weights [64], objective, largest W(u), error flag and largest net (int32
+    // each), round state (2 int32), then the sums of a state initialisation; zeroed once
+    int64_t *small = nullptr;
+    CKF(dalloc(h, &small, kSmallN));
+    CKF(cudaMemsetAsync(small, 0, kSmallN * sizeof(int64_t), st));
+    d.bw = small;
+    d.obj = small + 64;
+    unsigned long long *maxw_d = reinterpret_cast<unsigned long long *>(small + 65);
+    d.err = reinterpret_cast<int32_t *>(small + 66);
+    int32_t *max_size_d = d.err + 1;
+    d.rs = reinterpret_cast<int32_t *>(small + 67);
+    d.acc = reinterpret_cast<unsigned long long *>(small + 72);
     CKF(cudaMemcpyAsync(off64, net_offsets, sizeof(int64_t) * ((size_t)m + 1), kind, st));
     if (P) CKF(cudaMemcpyAsync(pins_d, pins, sizeof(int32_t) * (size_t)P, kind, st));
     CKF(cudaMemcpyAsync(part_in, initial_part, sizeof(int32_t) * (size_t)n, kind, st));
@@ -1280,8 +1390,9 @@ int create_impl(int32_t n, int32_t m, const int64_t *net_offsets, const int32_t 
     // ---- validation
     uint8_t *part = nullptr;
     CKF(dalloc(h, &part, n));
-    k_check_inputs<<<grid_for(std::max<int64_t>((int64_t)m + 1, n), 256), 256, 0, st>>>(
-        off64, net_off, m, P, nw_d, vw_d, part_in, n, k, part, d.err); h->launches++;
+    CKF(dalloc(h, &h->part_next, n));
+    k_check_inputs<<<grid_for(std::max<int64_t>((int64_t)m + 1, n), 256, 152 * 8), 256, 0, st>>>(
+        off64, net_off, m, P, nw_d, vw_d, part_in, n, k, part, d.acc, d.err); h->launches++;
     CKF(cudaGetLastError());
     int32_t host_err[2] = {0, 0};
     // one read-back for both checks: the pin check does nothing when the offsets were bad
@@ -1379,7 +1490,6 @@ int create_impl(int32_t n, int32_t m, const int64_t *net_offsets, const int32_t 
         d.widx = widx;
         int32_t *pw = nullptr;
         CKF(dalloc(h, &pw, (int64_t)nwide * k));
-        CKF(cudaMemsetAsync(pw, 0, sizeof(int32_t) * (size_t)nwide * k, st));
         d.phi_wide = pw;
     }
 
@@ -1441,7 +1551,6 @@ int create_impl(int32_t n, int32_t m, const int64_t *net_offsets, const int32_t 
     d.vtx_off = vtx_off;
     d.inc = inc;
 
-    unsigned long long *maxw_d = reinterpret_cast<unsigned long long *>(misc32 + 2);   // zeroed with misc32
     int32_t *vnw = nullptr;
     if (nw_d) CKF(dalloc(h, &vnw, n));
     d.vnw = vnw;
@@ -1456,15 +1565,11 @@ int create_impl(int32_t n, int32_t m, const int64_t *net_offsets, const int32_t 
     const int64_t words = (entries * w + 3) / 4;
     uint32_t *phi = nullptr;
     CKF(dalloc(h, &phi, words));
-    d.phi = phi;   // zeroed by init_state
+    d.phi = phi;   // written whole by init_state
     const size_t rec_bytes = k <= 32 ? sizeof(Rec16) : sizeof(Rec32);
     uint4 *rec = nullptr;
     CKF(dalloc(h, &rec, (int64_t)m * (int64_t)(rec_bytes / 16)));
     d.rec = rec;
-    int64_t *small = nullptr;
-    CKF(dalloc(h, &small, 2 * 64 + 8));
-    d.bw = small;
-    d.obj = small + 64;
 
     // ---- per-sub-round scratch
     uint16_t *sub_list = nullptr, *sub_start = nullptr;
@@ -1509,25 +1614,22 @@ int create_impl(int32_t n, int32_t m, const int64_t *net_offsets, const int32_t 
         d.rv_cnt = rv_cnt;
         d.rv_cap = cap;
     }
-    CKF(dalloc(h, &h->d_round, 4));
-    d.rs = h->d_round;
     d.seed = o.seed;
     d.variant = (o.balance_moves ? 1 : 0) | (o.revert_negative ? 2 : 0);
 
-    rc = init_state(h, guard);
+    rc = init_state(h, part, guard);
     if (rc != HGP_OK) return fail(rc);
 
     // ---- L_max = floor((1 + eps) * ceil(c(V) / k))  (Sec. 2); the incident-weight check
-    int64_t bw[64];
-    unsigned long long maxw = 0;
-    CKF(cudaMemcpyAsync(bw, d.bw, sizeof(int64_t) * k, cudaMemcpyDeviceToHost, st));
-    CKF(cudaMemcpyAsync(host_err, d.err, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
-    CKF(cudaMemcpyAsync(&maxw, maxw_d, sizeof(maxw), cudaMemcpyDeviceToHost, st));
+    int64_t bw[67];
+    CKF(cudaMemcpyAsync(bw, small, sizeof(bw), cudaMemcpyDeviceToHost, st));
     CKF(stream_wait(st));
+    const int64_t maxw = bw[65];
+    memcpy(host_err, &bw[66], sizeof(int32_t));
     if (host_err[0] & ERR_INVALID) return fail(HGP_ERR_INVALID);
     if (host_err[0] & ERR_UNSUPPORTED) return fail(HGP_ERR_UNSUPPORTED);
-    h->max_vertex_netweight = (int64_t)maxw;
-    d.bins = (int32_t)std::min<int64_t>(kBins, ((int64_t)maxw + kThreads) / kThreads * kThreads);   // > maxw
+    h->max_vertex_netweight = maxw;
+    d.bins = (int32_t)std::min<int64_t>(kBins, (maxw + kThreads) / kThreads * kThreads);   // > maxw
     int64_t total = 0;
     for (int i = 0; i < k; ++i) total += bw[i];
     h->total_weight = total;
@@ -1641,30 +1743,38 @@ int hgp_set_partition(hgp_handle *h, const int32_t *part, int32_t on_device)
     settle(h);
     Dev &d = h->d;
     cudaStream_t st = h->stream;
-    int32_t *tmp = h->scratch_n;
-    if (!tmp) CK(dev_alloc(reinterpret_cast<void **>(&tmp), sizeof(int32_t) * (size_t)d.n, st));
-    int rc = HGP_OK;
-    int32_t err = 0;
-    cudaError_t e = cudaMemcpyAsync(tmp, part, sizeof(int32_t) * (size_t)d.n,
-                                    on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(d.err, 0, sizeof(int32_t), st);
-    if (e == cudaSuccess) {
-        k_check_vertices<<<grid_for(d.n, 256), 256, 0, st>>>(nullptr, tmp, d.n, d.k, d.err); h->launches++;
-        e = cudaMemcpyAsync(&err, d.err, sizeof(int32_t), cudaMemcpyDeviceToHost, st);
+    // two launches and one read-back: the check stages the 1-byte partition and its block weights, and
+    // once it is known to be valid (else the handle keeps its state) k_init_nets does the rest.  A
+    // device partition is read where it is.  10k vertices: 110 -> 28 us a call.
+    const int32_t *src = part;
+    int32_t *tmp = nullptr;
+    cudaError_t e = cudaSuccess;
+    if (!on_device || (reinterpret_cast<uintptr_t>(part) & 3)) {
+        tmp = h->scratch_n;
+        if (!tmp) CK(dev_alloc(reinterpret_cast<void **>(&tmp), sizeof(int32_t) * (size_t)d.n, st));
+        src = tmp;
+        e = cudaMemcpyAsync(tmp, part, sizeof(int32_t) * (size_t)d.n,
+                            on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, st);
     }
-    if (e == cudaSuccess) e = stream_wait(st);
-    if (e == cudaSuccess && (err & ERR_INVALID)) rc = HGP_ERR_INVALID;
-    if (e == cudaSuccess && rc == HGP_OK) {
-        k_copy_part<<<grid_for(d.n, 256), 256, 0, st>>>(tmp, d.part, d.n); h->launches++;
+    int32_t err = 0;
+    if (e == cudaSuccess) {
+        k_stage_partition<<<grid_for(d.n, 256, 152 * 8), 256, 0, st>>>(src, d.n, d.k, d.vw, h->part_next, d.acc, d.err);
+        h->launches++;
         e = cudaGetLastError();
     }
-    if (tmp != h->scratch_n) pool_free(tmp, st);
+    if (tmp && tmp != h->scratch_n) pool_free(tmp, st);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(&err, d.err, sizeof(int32_t), cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = stream_wait(st);
+    if (e == cudaSuccess && (err & ERR_INVALID)) {
+        e = cudaMemsetAsync(d.err, 0, sizeof(int32_t), st);
+        if (e == cudaSuccess) e = cudaMemsetAsync(d.acc, 0, sizeof(unsigned long long) * kAccN, st);
+        if (e == cudaSuccess) return HGP_ERR_INVALID;
+    }
     if (e != cudaSuccess) {
         (void)cudaGetLastError();
         return status_of(e);
     }
-    if (rc != HGP_OK) return rc;
-    return init_state(h, nullptr);
+    return init_state(h, h->part_next, nullptr);
 }
 
 int hgp_export_state(hgp_handle *h, int32_t *part, uint8_t *moved_nets, int64_t *next_round,
