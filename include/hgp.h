@@ -76,7 +76,9 @@ typedef struct {
                             checkpoints always use input net ids; bit 4 (fault injection,
                             for tests of the error path): after each hgp_refine the maintained
                             objective is lowered by one from the host, so that check mode
-                            reports HGP_ERR_INTERNAL [0] */
+                            reports HGP_ERR_INTERNAL; bit 5: hgp_refine uses the launches of
+                            large instances whatever the size (small ones otherwise run a whole
+                            call as one thread-block cluster; the results are the same) [0] */
     int32_t graph;       /* 1: hgp_refine captures its launches as a CUDA graph on the first call
                             with a given round count and replays it afterwards [0]; ignored
                             while profiling is on */

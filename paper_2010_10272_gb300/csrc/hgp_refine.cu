@@ -183,16 +183,22 @@ __global__ void __launch_bounds__(kThreads) k_round_prep(const Dev *devs, const 
 // ------------------------------------------------------------------ gain + best target
 template <typename Rec> struct RecIO;
 
+// COH: the record may have been changed by another SM earlier in the same launch (hgp_small.cuh), so
+// it is read from L2; else through the read-only path.
 template <> struct RecIO<Rec16> {
     typedef uint32_t Lam;
+    template <bool COH>
     __device__ static void load_full(const Rec16 *r, Lam &s1, int32_t &w, int32_t &mv, Lam &lam)
     {
-        const uint4 q = __ldg(reinterpret_cast<const uint4 *>(r));
+        const uint4 *p = reinterpret_cast<const uint4 *>(r);
+        const uint4 q = COH ? __ldcg(p) : __ldg(p);
         s1 = q.x; w = (int32_t)q.y; mv = (int32_t)q.z; lam = q.w;
     }
+    template <bool COH>
     __device__ static void load_b(const Rec16 *r, Lam &lam, int32_t &w)
     {
-        const uint4 q = __ldg(reinterpret_cast<const uint4 *>(r));
+        const uint4 *p = reinterpret_cast<const uint4 *>(r);
+        const uint4 q = COH ? __ldcg(p) : __ldg(p);
         lam = q.w; w = (int32_t)q.y;
     }
 };
@@ -200,16 +206,25 @@ template <> struct RecIO<Rec16> {
 template <> struct RecIO<Rec32> {
     typedef uint64_t Lam;
     // the whole record is one 32-byte load (records are 32-byte aligned)
+    template <bool COH>
     __device__ static void load_full(const Rec32 *r, Lam &s1, int32_t &w, int32_t &mv, Lam &lam)
     {
+        if (COH) {
+            const uint4 q = __ldcg(reinterpret_cast<const uint4 *>(r)), l = __ldcg(reinterpret_cast<const uint4 *>(r) + 1);
+            s1 = (uint64_t)q.x | ((uint64_t)q.y << 32); w = (int32_t)q.z; mv = (int32_t)q.w;
+            lam = (uint64_t)l.x | ((uint64_t)l.y << 32);
+            return;
+        }
         uint64_t wm;
         [[maybe_unused]] uint64_t tail;
         asm("ld.global.nc.v4.b64 {%0, %1, %2, %3}, [%4];" : "=l"(s1), "=l"(wm), "=l"(lam), "=l"(tail) : "l"(r));
         w = (int32_t)(uint32_t)wm; mv = (int32_t)(uint32_t)(wm >> 32);
     }
+    template <bool COH>
     __device__ static void load_b(const Rec32 *r, Lam &lam, int32_t &w)
     {
-        const uint4 q = __ldg(reinterpret_cast<const uint4 *>(&r->lam));
+        const uint4 *p = reinterpret_cast<const uint4 *>(&r->lam);
+        const uint4 q = COH ? __ldcg(p) : __ldg(p);
         lam = (uint64_t)q.x | ((uint64_t)q.y << 32); w = (int32_t)q.z;
     }
 };
@@ -300,7 +315,7 @@ __device__ __forceinline__ Lam with_room(Lam T, const GainWarp &g, int32_t cu)
 // and three shared-memory atomics each, (Lambda, omega) kept for a second pass over the nets):
 // row-net 2M, k = 8, records in L2: 93 -> 56 us per launch of 5 M gathers; power-law 50M, k = 64,
 // bound by random sectors from DRAM: 1.77 -> 1.65 ms per launch of 86 M.
-template <typename Lam, typename Rec, int NP, bool UNIT, bool RB>
+template <typename Lam, typename Rec, int NP, bool UNIT, bool RB, bool COH>
 __device__ __forceinline__ void lane_best(const Rec *recs, const int32_t *inc, int32_t jb, int32_t je, int a, int32_t r,
                                           const GainWarp &g, int32_t cu, Lam kall, int32_t eq_value, Nets<Lam> &x,
                                           Lam &T_all, Lam &T, int &t_out, int32_t &conn_out, Lam &eq_out)
@@ -318,7 +333,7 @@ __device__ __forceinline__ void lane_best(const Rec *recs, const int32_t *inc, i
 #pragma unroll
         for (int q = 0; q < kAhead; ++q) {
             s1[q] = 0; lam[q] = 0; w[q] = 0; mv[q] = 0;
-            if (e[q] >= 0) RecIO<Rec>::load_full(recs + e[q], s1[q], w[q], mv[q], lam[q]);
+            if (e[q] >= 0) RecIO<Rec>::template load_full<COH>(recs + e[q], s1[q], w[q], mv[q], lam[q]);
         }
 #pragma unroll
         for (int q = 0; q < kAhead; ++q) {
@@ -372,6 +387,157 @@ __device__ __forceinline__ void lane_best(const Rec *recs, const int32_t *inc, i
     }
 }
 
+// The best target of the vertex in this lane (a = its block, cu its weight, [jb, je) its nets, W their
+// weight): block t_best (-1: none) and its gain; returns eligibility.  The warp calls it together.
+template <typename Rec, bool RB, bool COH>
+__device__ __forceinline__ bool gain_vertex(const Dev &d, const GainWarp &g, const GainInst<typename RecIO<Rec>::Lam> &gi,
+                                            const RbArgs &rb, bool valid, int32_t a, int32_t cu, int32_t jb, int32_t je,
+                                            int32_t W, int &t_best, int32_t &g_best)
+{
+    typedef typename RecIO<Rec>::Lam Lam;
+    constexpr bool kWide = sizeof(Lam) == 8;
+    const int lane = threadIdx.x & 31;
+    const int32_t r = gi.r;
+    const bool balance = !RB && (d.variant & 1) != 0;
+    const Rec *recs = reinterpret_cast<const Rec *>(d.rec);
+    const bool unit = d.nw == nullptr;
+    const Lam kall = d.k >= (int)(8 * sizeof(Lam)) ? ~(Lam)0 : (((Lam)1 << d.k) - 1);
+    Nets<Lam> x;
+    x.T = 0; x.A2 = ~(Lam)0; x.b = 0;
+    x.elig = valid && (RB || gi.all_elig);
+    Lam T_all = 0, T = 0, zero_in = 0;
+    t_best = -1;
+    int32_t conn = 0;
+    const bool heavy = valid && (W > kPlaneMaxW || je - jb > kLaneDeg);
+    const bool light = valid && !heavy;
+    const unsigned wmax = __reduce_max_sync(kFull, light ? (unsigned)W : 0u);
+    if (light) {
+        const int np = 32 - __clz((int)wmax);   // 2^np > wmax >= conn_t
+        const int32_t eqv = balance ? W : -1;
+#define HGP_LANE(NP, U) lane_best<Lam, Rec, NP, U, RB, COH>(recs, d.inc, jb, je, a, r, g, cu, kall, eqv, x, T_all, T, t_best, conn, zero_in)
+        if (unit) {
+            if (np <= 4) HGP_LANE(4, true);
+            else HGP_LANE(7, true);             // at most kLaneDeg nets
+        } else {
+            if (np <= 6) HGP_LANE(6, false);
+            else if (np <= 8) HGP_LANE(8, false);
+            else HGP_LANE(11, false);
+        }
+#undef HGP_LANE
+    }
+    __syncwarp();
+    const int32_t bw_ = x.b - W;
+    g_best = bw_ + conn;
+    if (!(light && t_best >= 0 && (RB ? (rb.phase == 2 || g_best >= 0) : g_best > 0))) {
+        t_best = -1;
+        g_best = 0;
+    }
+    // ---- vertices with many nets or large W: the whole warp on one vertex at a time
+    unsigned hm = __ballot_sync(kFull, heavy);
+    while (hm) {
+        const int src = __ffs(hm) - 1;
+        hm &= hm - 1;
+        const int32_t hjb = __shfl_sync(kFull, jb, src), hje = __shfl_sync(kFull, je, src);
+        const int32_t ha = __shfl_sync(kFull, a, src), hcu = __shfl_sync(kFull, cu, src);
+        const int32_t hW = __shfl_sync(kFull, W, src);
+        Nets<Lam> y;
+        y.T = 0; y.A2 = ~(Lam)0; y.b = 0; y.elig = RB || gi.all_elig;
+        for (int32_t j = hjb + lane; j < hje; j += 32) {
+            Lam s1, lam;
+            int32_t w, mv;
+            RecIO<Rec>::template load_full<COH>(recs + (__ldg(&d.inc[j]) & kNetMask), s1, w, mv, lam);
+            take_net(y, s1, lam, w & 0x7fffffff, mv, ha, r);
+        }
+        y.b = __reduce_add_sync(kFull, y.b);
+        y.elig = __any_sync(kFull, y.elig);
+        uint32_t tl = __reduce_or_sync(kFull, lo32(y.T)), al = __reduce_and_sync(kFull, lo32(y.A2));
+        uint32_t th = kWide ? __reduce_or_sync(kFull, hi32(y.T)) : 0u;
+        uint32_t ah = kWide ? __reduce_and_sync(kFull, hi32(y.A2)) : 0u;
+        y.T = (Lam)((uint64_t)tl | ((uint64_t)th << 32));
+        y.A2 = (Lam)((uint64_t)al | ((uint64_t)ah << 32));
+        const Lam hTa = y.elig ? (RB ? kall : y.T) & ~((Lam)1 << ha) : (Lam)0;
+        const Lam hT = with_room(hTa, g, hcu);
+        if (lane == src) {
+            x = y;
+            T_all = hTa;
+            T = hT;
+        }
+        if (hT == 0) continue;
+        const uint32_t Tlo = lo32(hT), Thi = hi32(hT);
+        const int32_t hbw = y.b - hW;
+        int32_t acc0 = 0, acc1 = 0;
+        for (int32_t j0 = hjb; j0 < hje; j0 += 32) {
+            const int32_t j = j0 + lane;
+            Lam lam = 0;
+            int32_t w = 0;
+            if (j < hje) {
+                RecIO<Rec>::template load_b<COH>(recs + (__ldg(&d.inc[j]) & kNetMask), lam, w);
+                w &= 0x7fffffff;
+            }
+            const int nn = min(32, hje - j0);
+            const uint32_t llo = lo32(lam), lhi = hi32(lam);
+            for (int q = 0; q < nn; ++q) {
+                const uint32_t bl = __shfl_sync(kFull, llo, q);
+                const int32_t wi = __shfl_sync(kFull, w, q);
+                acc0 += ((bl >> lane) & 1) ? wi : 0;
+                if (kWide) {
+                    const uint32_t bh = __shfl_sync(kFull, lhi, q);
+                    acc1 += ((bh >> lane) & 1) ? wi : 0;
+                }
+            }
+        }
+        // key = gain << 8 | (255 - block): the larger key is the higher gain, then the
+        // smaller block (RB: the gain's sign bit flipped, so negative gains order too)
+        unsigned long long key = 0;
+        if ((Tlo >> lane) & 1) {
+            const int32_t gg = hbw + acc0;
+            if (RB ? (rb.phase == 2 || gg >= 0) : gg > 0)
+                key = ((unsigned long long)((uint32_t)gg ^ (RB ? 0x80000000u : 0u)) << 8) | (unsigned long long)(255 - lane);
+        }
+        if (kWide && ((Thi >> lane) & 1)) {
+            const int32_t gg = hbw + acc1;
+            if (RB ? (rb.phase == 2 || gg >= 0) : gg > 0) {
+                const unsigned long long k2 = ((unsigned long long)((uint32_t)gg ^ (RB ? 0x80000000u : 0u)) << 8) | (unsigned long long)(255 - (lane + 32));
+                key = k2 > key ? k2 : key;
+            }
+        }
+#pragma unroll
+        for (int o = 16; o; o >>= 1) {
+            const unsigned long long y2 = __shfl_xor_sync(kFull, key, o);
+            key = y2 > key ? y2 : key;
+        }
+        if (lane == src && key) {
+            t_best = 255 - (int)(key & 0xFF);
+            g_best = (int32_t)((uint32_t)(key >> 8) ^ (RB ? 0x80000000u : 0u));
+        }
+        if (balance) {
+            // zero-gain blocks of T among the ones this lane owns
+            const unsigned zlo = __ballot_sync(kFull, ((Tlo >> lane) & 1) && hbw + acc0 == 0);
+            const unsigned zhi = __ballot_sync(kFull, kWide && ((Thi >> lane) & 1) && hbw + acc1 == 0);
+            if (lane == src) zero_in = kWide ? (Lam)((uint64_t)zlo | ((uint64_t)zhi << 32)) : (Lam)zlo;
+        }
+    }
+    if (balance && valid && x.elig && t_best < 0) {
+        // zero-gain moves that improve the balance (Sec. 6): blocks of T with gain 0, and
+        // blocks outside T that lie in every net where u is not alone (their gain is
+        // b - p_t = 0 exactly then); room and w(t) + c(u) < w(a); lightest block first
+        Lam z = (zero_in | (x.A2 & ~T_all & ~((Lam)1 << a))) & kall;
+        const long long wa = d.lmax - g.slack[a];
+        long long best_w = 0;
+        for (Lam y = z; y; y &= y - 1) {
+            const int t = lam_bits_ctz(y);
+            const long long wt = d.lmax - g.slack[t];
+            if (g.slack[t] < cu || wt + cu >= wa) continue;
+            if (t_best < 0 || wt < best_w) {
+                t_best = t;
+                best_w = wt;
+            }
+        }
+        g_best = 0;
+    }
+    return valid && x.elig;
+}
+
 // Segments [seg, seg_end) of one tile's list of sub-round s (see k_gain); returns the number of
 // candidates written, to the slots of segment seg.
 // RB: a rebalancing pass (Sec. 8): only vertices of overloaded blocks take part, their target
@@ -382,14 +548,8 @@ __device__ __forceinline__ int32_t gain_seg(const Dev &d, int32_t tile, int32_t 
                                             const GainWarp &g, uint16_t *picked, unsigned long long *tot,
                                             const GainInst<typename RecIO<Rec>::Lam> &gi, int32_t &nel, const RbArgs &rb)
 {
-    typedef typename RecIO<Rec>::Lam Lam;
-    constexpr bool kWide = sizeof(Lam) == 8;
     const int lane = threadIdx.x & 31;
-    const int32_t r = gi.r;
-    const bool balance = !RB && (d.variant & 1) != 0;
-    const Rec *recs = reinterpret_cast<const Rec *>(d.rec);
     const bool unit = d.nw == nullptr;
-    const Lam kall = d.k >= (int)(8 * sizeof(Lam)) ? ~(Lam)0 : (((Lam)1 << d.k) - 1);
     const int32_t rbase = tile * kTile;
     nel = 0;
     if (s >= d.S) return 0;
@@ -428,140 +588,10 @@ __device__ __forceinline__ int32_t gain_seg(const Dev &d, int32_t tile, int32_t 
             je = d.vtx_off[u + 1];
             W = unit ? je - jb : d.vnw[u];
         }
-        Nets<Lam> x;
-        x.T = 0; x.A2 = ~(Lam)0; x.b = 0;
-        x.elig = valid && (RB || gi.all_elig);
-        Lam T_all = 0, T = 0, zero_in = 0;
-        int t_best = -1;
-        int32_t conn = 0;
-        const bool heavy = valid && (W > kPlaneMaxW || je - jb > kLaneDeg);
-        const bool light = valid && !heavy;
-        const unsigned wmax = __reduce_max_sync(kFull, light ? (unsigned)W : 0u);
-        if (light) {
-            const int np = 32 - __clz((int)wmax);   // 2^np > wmax >= conn_t
-            const int32_t eqv = balance ? W : -1;
-#define HGP_LANE(NP, U) lane_best<Lam, Rec, NP, U, RB>(recs, d.inc, jb, je, a, r, g, cu, kall, eqv, x, T_all, T, t_best, conn, zero_in)
-            if (unit) {
-                if (np <= 4) HGP_LANE(4, true);
-                else HGP_LANE(7, true);             // at most kLaneDeg nets
-            } else {
-                if (np <= 6) HGP_LANE(6, false);
-                else if (np <= 8) HGP_LANE(8, false);
-                else HGP_LANE(11, false);
-            }
-#undef HGP_LANE
-        }
-        __syncwarp();
-        const int32_t bw_ = x.b - W;
-        int32_t g_best = bw_ + conn;
-        if (!(light && t_best >= 0 && (RB ? (rb.phase == 2 || g_best >= 0) : g_best > 0))) {
-            t_best = -1;
-            g_best = 0;
-        }
-        // ---- vertices with many nets or large W: the whole warp on one vertex at a time
-        unsigned hm = __ballot_sync(kFull, heavy);
-        while (hm) {
-            const int src = __ffs(hm) - 1;
-            hm &= hm - 1;
-            const int32_t hjb = __shfl_sync(kFull, jb, src), hje = __shfl_sync(kFull, je, src);
-            const int32_t ha = __shfl_sync(kFull, a, src), hcu = __shfl_sync(kFull, cu, src);
-            const int32_t hW = __shfl_sync(kFull, W, src);
-            Nets<Lam> y;
-            y.T = 0; y.A2 = ~(Lam)0; y.b = 0; y.elig = RB || gi.all_elig;
-            for (int32_t j = hjb + lane; j < hje; j += 32) {
-                Lam s1, lam;
-                int32_t w, mv;
-                RecIO<Rec>::load_full(recs + (__ldg(&d.inc[j]) & kNetMask), s1, w, mv, lam);
-                take_net(y, s1, lam, w & 0x7fffffff, mv, ha, r);
-            }
-            y.b = __reduce_add_sync(kFull, y.b);
-            y.elig = __any_sync(kFull, y.elig);
-            uint32_t tl = __reduce_or_sync(kFull, lo32(y.T)), al = __reduce_and_sync(kFull, lo32(y.A2));
-            uint32_t th = kWide ? __reduce_or_sync(kFull, hi32(y.T)) : 0u;
-            uint32_t ah = kWide ? __reduce_and_sync(kFull, hi32(y.A2)) : 0u;
-            y.T = (Lam)((uint64_t)tl | ((uint64_t)th << 32));
-            y.A2 = (Lam)((uint64_t)al | ((uint64_t)ah << 32));
-            const Lam hTa = y.elig ? (RB ? kall : y.T) & ~((Lam)1 << ha) : (Lam)0;
-            const Lam hT = with_room(hTa, g, hcu);
-            if (lane == src) {
-                x = y;
-                T_all = hTa;
-                T = hT;
-            }
-            if (hT == 0) continue;
-            const uint32_t Tlo = lo32(hT), Thi = hi32(hT);
-            const int32_t hbw = y.b - hW;
-            int32_t acc0 = 0, acc1 = 0;
-            for (int32_t j0 = hjb; j0 < hje; j0 += 32) {
-                const int32_t j = j0 + lane;
-                Lam lam = 0;
-                int32_t w = 0;
-                if (j < hje) {
-                    RecIO<Rec>::load_b(recs + (__ldg(&d.inc[j]) & kNetMask), lam, w);
-                    w &= 0x7fffffff;
-                }
-                const int nn = min(32, hje - j0);
-                const uint32_t llo = lo32(lam), lhi = hi32(lam);
-                for (int q = 0; q < nn; ++q) {
-                    const uint32_t bl = __shfl_sync(kFull, llo, q);
-                    const int32_t wi = __shfl_sync(kFull, w, q);
-                    acc0 += ((bl >> lane) & 1) ? wi : 0;
-                    if (kWide) {
-                        const uint32_t bh = __shfl_sync(kFull, lhi, q);
-                        acc1 += ((bh >> lane) & 1) ? wi : 0;
-                    }
-                }
-            }
-            // key = gain << 8 | (255 - block): the larger key is the higher gain, then the
-            // smaller block (RB: the gain's sign bit flipped, so negative gains order too)
-            unsigned long long key = 0;
-            if ((Tlo >> lane) & 1) {
-                const int32_t gg = hbw + acc0;
-                if (RB ? (rb.phase == 2 || gg >= 0) : gg > 0)
-                    key = ((unsigned long long)((uint32_t)gg ^ (RB ? 0x80000000u : 0u)) << 8) | (unsigned long long)(255 - lane);
-            }
-            if (kWide && ((Thi >> lane) & 1)) {
-                const int32_t gg = hbw + acc1;
-                if (RB ? (rb.phase == 2 || gg >= 0) : gg > 0) {
-                    const unsigned long long k2 = ((unsigned long long)((uint32_t)gg ^ (RB ? 0x80000000u : 0u)) << 8) | (unsigned long long)(255 - (lane + 32));
-                    key = k2 > key ? k2 : key;
-                }
-            }
-#pragma unroll
-            for (int o = 16; o; o >>= 1) {
-                const unsigned long long y2 = __shfl_xor_sync(kFull, key, o);
-                key = y2 > key ? y2 : key;
-            }
-            if (lane == src && key) {
-                t_best = 255 - (int)(key & 0xFF);
-                g_best = (int32_t)((uint32_t)(key >> 8) ^ (RB ? 0x80000000u : 0u));
-            }
-            if (balance) {
-                // zero-gain blocks of T among the ones this lane owns
-                const unsigned zlo = __ballot_sync(kFull, ((Tlo >> lane) & 1) && hbw + acc0 == 0);
-                const unsigned zhi = __ballot_sync(kFull, kWide && ((Thi >> lane) & 1) && hbw + acc1 == 0);
-                if (lane == src) zero_in = kWide ? (Lam)((uint64_t)zlo | ((uint64_t)zhi << 32)) : (Lam)zlo;
-            }
-        }
-        if (balance && valid && x.elig && t_best < 0) {
-            // zero-gain moves that improve the balance (Sec. 6): blocks of T with gain 0, and
-            // blocks outside T that lie in every net where u is not alone (their gain is
-            // b - p_t = 0 exactly then); room and w(t) + c(u) < w(a); lightest block first
-            Lam z = (zero_in | (x.A2 & ~T_all & ~((Lam)1 << a))) & kall;
-            const long long wa = d.lmax - g.slack[a];
-            long long best_w = 0;
-            for (Lam y = z; y; y &= y - 1) {
-                const int t = lam_bits_ctz(y);
-                const long long wt = d.lmax - g.slack[t];
-                if (g.slack[t] < cu || wt + cu >= wa) continue;
-                if (t_best < 0 || wt < best_w) {
-                    t_best = t;
-                    best_w = wt;
-                }
-            }
-            g_best = 0;
-        }
-        nel += __popc(__ballot_sync(kFull, valid && x.elig));
+        int t_best;
+        int32_t g_best;
+        const bool elig = gain_vertex<Rec, RB, false>(d, g, gi, rb, valid, a, cu, jb, je, W, t_best, g_best);
+        nel += __popc(__ballot_sync(kFull, elig));
         const unsigned cm = __ballot_sync(kFull, t_best >= 0);
         const bool small_c = __all_sync(kFull, cu < (1 << 26));   // 32 of them fit 32 bits
         if (t_best >= 0) {
@@ -592,21 +622,26 @@ __device__ __forceinline__ int32_t gain_seg(const Dev &d, int32_t tile, int32_t 
     return nout;
 }
 
-template <typename Rec>
-__device__ __forceinline__ void gain_refresh(const Dev &d, GainWarp &g, GainInst<typename RecIO<Rec>::Lam> &gi)
+__device__ __forceinline__ void room_tables(const Dev &d, const int64_t *bw, GainWarp &g)
 {
     const int lane = threadIdx.x & 31;
     __syncwarp();
-    const long long s0 = lane < d.k ? d.lmax - d.bw[lane] : -1, s1 = lane + 32 < d.k ? d.lmax - d.bw[lane + 32] : -1;
+    const long long s0 = lane < d.k ? d.lmax - bw[lane] : -1, s1 = lane + 32 < d.k ? d.lmax - bw[lane + 32] : -1;
     g.slack[lane] = s0;
     g.slack[lane + 32] = s1;
     for (int c = 1; c <= kFeasW; ++c) {
         const unsigned lo = __ballot_sync(kFull, s0 >= c), hi = __ballot_sync(kFull, s1 >= c);
         if (lane == 0) g.feas[c] = (unsigned long long)lo | ((unsigned long long)hi << 32);
     }
+    __syncwarp();
+}
+
+template <typename Rec>
+__device__ __forceinline__ void gain_refresh(const Dev &d, GainWarp &g, GainInst<typename RecIO<Rec>::Lam> &gi)
+{
+    room_tables(d, d.bw, g);
     gi.r = d.rs[0];
     gi.all_elig = d.rs[1] == 0;
-    __syncwarp();
 }
 
 // copies devs[inst] into a warp's shared slot
@@ -1193,15 +1228,15 @@ __device__ __forceinline__ bool approve(uint64_t c, int32_t slot, const ApplyIns
 // Applies the queued moves [first, first + 32) (at most `queued` in all) over their incidences,
 // flattened across the lanes.
 template <typename Rec, int KEY>
-__device__ __forceinline__ void apply_queue(const Dev &d, const MoveQueue &mq, int32_t first, int32_t queued,
-                                            int32_t r, ApplyWarp &w_,
+__device__ __forceinline__ void apply_queue(const Dev &d, const int32_t *qu, const uint16_t *qat, int32_t first,
+                                            int32_t queued, int32_t r, ApplyWarp &w_,
                                             long long &dobj, int32_t &npins, int32_t &nshared)
 {
     const int lane = threadIdx.x & 31;
     Rec *recs = reinterpret_cast<Rec *>(d.rec);
     int32_t deg = 0, jb = 0, a = 0, t = 0;
     if (first + lane < queued) {
-        const int32_t u = mq.u[first + lane], at = mq.at[first + lane];
+        const int32_t u = qu[first + lane], at = qat[first + lane];
         a = at & 0xFF;
         t = at >> 8;
         jb = d.vtx_off[u];
@@ -1281,7 +1316,7 @@ __device__ __forceinline__ void apply_segs(const Dev &d, int32_t tile, int32_t s
         __syncwarp();
         int32_t first = 0;
         for (; queued - first >= 32; first += 32)
-            apply_queue<Rec, KEY>(d, mq, first, queued, r, w_, dobj, npins, nshared);
+            apply_queue<Rec, KEY>(d, mq.u, mq.at, first, queued, r, w_, dobj, npins, nshared);
         if (first && queued - first > 0) {   // the rest moves to the front
             int32_t u2 = 0;
             uint16_t at2 = 0;
@@ -1331,7 +1366,7 @@ __global__ void __launch_bounds__(kThreads, 4) k_apply(const Dev d0, const Dev *
     const int32_t n_it = (B ? n_items : d0.n_tiles) * groups;
     // a batch instance's queue, block weights and counters, before the warp turns to another one
     auto leave = [&](const Dev &d) {
-        if (queued) apply_queue<Rec, KEY>(d, mq_w[wid], 0, queued, r, aw[wid], dobj, npins, nshared);
+        if (queued) apply_queue<Rec, KEY>(d, mq_w[wid].u, mq_w[wid].at, 0, queued, r, aw[wid], dobj, npins, nshared);
         queued = 0;
         for (int o = 16; o; o >>= 1) {
             dobj += __shfl_xor_sync(kFull, dobj, o);
@@ -1387,7 +1422,7 @@ __global__ void __launch_bounds__(kThreads, 4) k_apply(const Dev d0, const Dev *
         if (inst_prev >= 0) leave(dsm[wid]);
         return;
     }
-    if (queued) apply_queue<Rec, KEY>(d0, mq_w[wid], 0, queued, r, aw[wid], dobj, npins, nshared);
+    if (queued) apply_queue<Rec, KEY>(d0, mq_w[wid].u, mq_w[wid].at, 0, queued, r, aw[wid], dobj, npins, nshared);
     if (!B && KEY == KEY_T && d0.rv_cnt) {
         // revert variant: moved incidences on nets with several movers (sizes the order-statistics table)
         nshared = __reduce_add_sync(kFull, nshared);
@@ -1432,6 +1467,8 @@ __global__ void __launch_bounds__(kThreads, 4) k_apply(const Dev d0, const Dev *
         }
     }
 }
+
+#include "hgp_small.cuh"
 
 // ------------------------------------------------------------------ revert variant
 // Attributed gains (Sec. 5.2) of a sub-round's approved moves, with every net seeing its moves
@@ -2005,8 +2042,47 @@ Plan single_plan(hgp_handle *h)
     return p;
 }
 
-cudaError_t enqueue_rounds(const Plan &p, int64_t *stats, int32_t rounds)
+// Whether a handle's rounds run as one cluster (hgp_small.cuh): instances of up to kSmallVertices
+// vertices and kSmallPins pins on a device that can hold the cluster.  Per-phase profiling and the revert variant take
+// the launches of the general path.
+bool small_plan(const Plan &p, int device, int32_t debug)
 {
+    if (p.prof || p.revert || p.tiles || p.d0.n > kSmallVertices || (debug & 32)) return false;
+    if (p.d0.P > (p.rec32 ? kSmallPinsWide : kSmallPins)) return false;
+    static std::mutex mu;
+    static int8_t ready[64][2];   // per device and record type: 0 not asked yet, 1 yes, 2 no
+    if (device < 0 || device >= 64) return false;
+    std::lock_guard<std::mutex> lk(mu);
+    int8_t &r = ready[device][p.rec32];
+    if (r == 0) {
+        auto kernel = p.rec32 ? k_small<Rec32> : k_small<Rec16>;
+        cudaLaunchAttribute at;
+        cudaLaunchConfig_t cfg = small_config(kSmallVertices, nullptr, &at);
+        int clusters = 0;
+        cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cfg.dynamicSmemBytes);
+        if (e == cudaSuccess) e = cudaOccupancyMaxActiveClusters(&clusters, kernel, &cfg);
+        if (e != cudaSuccess) (void)cudaGetLastError();
+        r = e == cudaSuccess && clusters > 0 ? 1 : 2;
+    }
+    return r == 1;
+}
+
+cudaError_t launch_small(const Plan &p, int32_t rounds, int64_t max_netweight)
+{
+    int nd = 1;
+    while (nd < 4 && (max_netweight >> (kSmDigit * nd)) > 0) ++nd;
+    cudaLaunchAttribute at;
+    const cudaLaunchConfig_t cfg = small_config(p.d0.n, p.st, &at);
+    *p.launches += 1;
+    return p.rec32 ? cudaLaunchKernelEx(&cfg, k_small<Rec32>, p.d0, rounds, (int32_t)nd)
+                   : cudaLaunchKernelEx(&cfg, k_small<Rec16>, p.d0, rounds, (int32_t)nd);
+}
+
+cudaError_t enqueue_rounds(const Plan &p, int64_t *stats, int32_t rounds, bool small, int64_t max_netweight)
+{
+    if (small) return launch_small(p, rounds, max_netweight);
     cudaError_t e = cudaMemsetAsync(stats, 0, sizeof(int64_t) * ST_N * (size_t)rounds, p.st);
     if (e == cudaSuccess && p.d0.wq) e = cudaMemsetAsync(p.d0.wq, 0, sizeof(int32_t) * kWqPerRow * (size_t)rounds, p.st);
     for (int32_t rr = 0; rr < rounds && e == cudaSuccess; ++rr) e = launch_round(p, rr);
@@ -2090,6 +2166,7 @@ int refine_rounds(hgp_handle *h, int32_t rounds, hgp_round_stats *stats)
     }
     Plan p = single_plan(h);
     const bool use_graph = h->graph && !h->profiling;
+    const bool small = small_plan(p, h->device, h->debug);
     if (use_graph) {
         if (!h->graph_exec || h->graph_rounds != rounds) {
             if (h->graph_exec) {
@@ -2103,7 +2180,7 @@ int refine_rounds(hgp_handle *h, int32_t rounds, hgp_round_stats *stats)
             cudaGraph_t graph = nullptr;
             e = cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeThreadLocal);
             if (e == cudaSuccess) {
-                const cudaError_t e2 = enqueue_rounds(q, h->d.stats, rounds);
+                const cudaError_t e2 = enqueue_rounds(q, h->d.stats, rounds, small, h->max_vertex_netweight);
                 e = cudaStreamEndCapture(h->stream, &graph);
                 if (e2 != cudaSuccess) e = e2;
             }
@@ -2117,7 +2194,7 @@ int refine_rounds(hgp_handle *h, int32_t rounds, hgp_round_stats *stats)
         if (e == cudaSuccess) e = cudaGraphLaunch(h->graph_exec, h->stream);
         if (e == cudaSuccess) h->launches += h->graph_launches;
     } else {
-        e = enqueue_rounds(p, h->d.stats, rounds);
+        e = enqueue_rounds(p, h->d.stats, rounds, small, h->max_vertex_netweight);
         if (e == cudaSuccess) e = collect_profile(h);
     }
     if (e != cudaSuccess) {

@@ -4,22 +4,27 @@ import pytest
 
 import oracle
 import synth
+from parity_util import compare_state
 
 pytestmark = pytest.mark.gpu
 
 
+LAUNCHES = 32   # debug bit: the launches of large instances whatever the size
+
+
 def _check(hg, rounds=4, subrounds=4, eps=None, **kw):
+    """Both ways a small instance can run: as one cluster, and by the launches of large ones."""
     from paper_2010_10272_gb300 import HGP
     if eps is not None:
         hg.eps = eps
-    h = HGP.from_hypergraph(hg, subrounds=subrounds, seed=9, **kw)
-    o = oracle.Oracle.from_hypergraph(hg, subrounds=subrounds, seed=9)
+    o = oracle.Oracle.from_hypergraph(hg, subrounds=subrounds, seed=9, **kw)
     want, _ = o.refine(rounds)
-    got = h.refine(rounds)
-    assert np.array_equal(got[:, :5], want[:, :5])
-    assert np.array_equal(h.partition(), o.partition())
-    assert h.objective() == o.objective() == h.objective_from_phi()
-    h.close()
+    for debug in (0, LAUNCHES):
+        h = HGP.from_hypergraph(hg, subrounds=subrounds, seed=9, debug=debug, **kw)
+        got = np.concatenate([h.refine(1), h.refine(rounds - 1)])
+        assert np.array_equal(got[:, :5], want[:, :5])
+        compare_state(h, o)
+        h.close()
 
 
 @pytest.mark.parametrize("n", [2047, 2048, 2049, 4096, 6145, 33_000])
@@ -42,14 +47,7 @@ def test_degrees_and_net_weights(k, m, scale, balance):
     hg = synth.random_small(k, 300, m, k, max_size=6, weighted=True, f=0.6)
     hg.net_w = (hg.net_w * scale).astype(np.int32) if scale else None
     hg.vertex_w = (hg.vertex_w * 3 - 2).astype(np.int32)      # 1..13: beside the weights with a mask of their own
-    hg.eps = 0.2
-    from paper_2010_10272_gb300 import HGP
-    h = HGP.from_hypergraph(hg, seed=9, balance_moves=balance)
-    o = oracle.Oracle.from_hypergraph(hg, subrounds=4, seed=9, balance_moves=balance)
-    want, _ = o.refine(4)
-    assert np.array_equal(h.refine(4)[:, :5], want[:, :5])
-    assert np.array_equal(h.partition(), o.partition())
-    h.close()
+    _check(hg, eps=0.2, balance_moves=balance)
 
 
 @pytest.mark.parametrize("S", [1, 2, 3, 7, 64])
@@ -82,3 +80,19 @@ def test_tiles_and_segments(S):
         assert np.array_equal(h.partition(), o.partition())
         h.close()
 
+
+
+@pytest.mark.parametrize("n,k,weighted", [(131_072, 64, False), (131_073, 7, True), (120_001, 17, True), (257, 64, True)])
+@pytest.mark.parametrize("graph", [0, 1])
+def test_largest_and_smallest_cluster_instances(n, k, weighted, graph):
+    """At the line between one cluster and separate launches, saturated blocks among them; replayed
+    as a graph too."""
+    from paper_2010_10272_gb300 import HGP
+    hg = synth.random_small(n + k, n, n, k, max_size=4, weighted=weighted, f=0.8, eps=0.01)   # 2.5 n pins
+    o = oracle.Oracle.from_hypergraph(hg, subrounds=4, seed=9)
+    want, _ = o.refine(6)
+    h = HGP.from_hypergraph(hg, seed=9, graph=graph)
+    got = np.concatenate([h.refine(3), h.refine(3)])
+    assert np.array_equal(got[:, :5], want[:, :5])
+    compare_state(h, o, check_phi=n < 1000)
+    h.close()
