@@ -418,10 +418,11 @@ void hgp_destroy(hgp_handle *h);
  * Memory pool (no counterpart in the paper).  Handles and batches take their device memory
  * from a stream-ordered pool the library keeps per device (allocations and releases are
  * queued on the owner's stream and never synchronise the device, so handles can be created
- * and destroyed while other handles' kernels run).  By default freed memory goes back to the
- * system at the next synchronisation; this call lets the pool of the current device keep up
- * to `bytes` of freed memory for reuse, which a caller that creates and destroys many
- * handles (a serving loop) may want.  HGP_ERR_INVALID for bytes < 0.
+ * and destroyed while other handles' kernels run).  By default the pool keeps up to 1/64 of the
+ * device's memory of what was freed, for the next handles; more than that goes back to the system
+ * at the next synchronisation, and an allocation that fails gives back everything the pool keeps
+ * before it is tried again.  This call sets how many bytes the pool of the current device may
+ * keep (0: give everything back at the next synchronisation).  HGP_ERR_INVALID for bytes < 0.
  */
 int hgp_set_pool_retention(int64_t bytes);
 

@@ -75,8 +75,8 @@ inline int status_of(cudaError_t e)
 // Device memory of handles and batches comes from a library-owned stream-ordered memory pool
 // of the current device (cudaMallocFromPoolAsync / cudaFreeAsync on the owner's stream), so
 // creating or destroying a handle never implies a device-wide synchronisation and can overlap
-// with kernels of other handles (the serving loop relies on this).  Freed memory goes back to
-// the system at the next synchronisation unless hgp_set_pool_retention keeps some of it.
+// with kernels of other handles (the serving loop relies on this).  The pool keeps a bounded
+// amount of freed memory (hgp_set_pool_retention).
 cudaError_t library_pool(cudaMemPool_t *out);
 // Waits on the host for the work queued on st: spinning in cudaStreamSynchronize, or, after
 // hgp_set_blocking_waits(1), sleeping on a blocking-sync event recorded on st.

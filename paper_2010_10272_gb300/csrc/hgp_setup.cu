@@ -1053,6 +1053,7 @@ int grid_for(int64_t work, int threads, int cap = 152 * 32)
 namespace hgp {
 
 static constexpr int kMaxPoolDevices = 64;
+static constexpr uint64_t kPoolKeepShare = 64;   // default retention: this fraction of the device's memory
 static std::mutex g_pool_mu;
 static cudaMemPool_t g_pool[kMaxPoolDevices];
 
@@ -1082,6 +1083,18 @@ cudaError_t library_pool(cudaMemPool_t *out)
             g_pool[dev] = nullptr;
             return e;
         }
+        // keep up to 1/64 of the device's memory (4.4 GB of 284) between handles: mapping it
+        // afresh and unmapping it at the next synchronisation took as long as the work itself
+        // (creating and closing a 5M-vertex level 6.4 -> 3.6 ms, a 500k-pin request 457 -> 261
+        // us, contraction of 10M vertices 10.4 -> 6.8 ms).  Memory freed on another stream is only
+        // reused once it is free there, never by making a stream wait for the other.
+        size_t free_b = 0, total_b = 0;
+        uint64_t keep = 0;
+        if (cudaMemGetInfo(&free_b, &total_b) == cudaSuccess) keep = total_b / kPoolKeepShare;
+        int no = 0;
+        if (cudaMemPoolSetAttribute(g_pool[dev], cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess ||
+            cudaMemPoolSetAttribute(g_pool[dev], cudaMemPoolReuseAllowInternalDependencies, &no) != cudaSuccess)
+            (void)cudaGetLastError();
         g_pool_ready[dev].store(g_pool[dev], std::memory_order_release);
     }
     *out = g_pool[dev];
@@ -1128,6 +1141,11 @@ cudaError_t dev_alloc(void **p, size_t bytes, cudaStream_t st)
     cudaMemPool_t pool = nullptr;
     cudaError_t e = library_pool(&pool);
     if (e == cudaSuccess) e = cudaMallocFromPoolAsync(p, bytes, pool, st);
+    if (e == cudaErrorMemoryAllocation) {
+        // what the pool keeps may be what is missing: give it back and try once more
+        (void)cudaGetLastError();
+        if (cudaMemPoolTrimTo(pool, 0) == cudaSuccess) e = cudaMallocFromPoolAsync(p, bytes, pool, st);
+    }
     if (e != cudaSuccess) {
         (void)cudaGetLastError();
         *p = nullptr;

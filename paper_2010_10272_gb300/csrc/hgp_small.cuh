@@ -26,11 +26,11 @@ constexpr int kSmRow = kSmBins + kSmBins / 16;       // padded: a lane sums 16 c
 constexpr int kSmIdBits = 2 * kSmDigit;
 constexpr int32_t kSmMaxN = 1 << kSmIdBits;
 // Instances that run this way.  Its time grows with the pins (16 SMs), that of the launches hardly
-// does at this size: 5 rounds, planted, k = 4: 284 / 361 / 487 / 605 / 765 us at 90 / 180 / 360 / 540
-// / 786 thousand pins against 783-818 us; row-net, k = 64: 469 / 657 / 951 / 1231 us at 150 / 300 /
-// 600 / 900 thousand against 1041-1106 us.
+// does at this size.  5 rounds, planted, k = 4: 286 / 362 / 487 / 605 us at 90 / 180 / 360 / 540
+// thousand pins against 526-553 us; row-net, k = 64: 470 / 653 / 951 us at 150 / 300 / 600 thousand
+// against 797-855 us.
 constexpr int32_t kSmallVertices = 1 << 17;
-constexpr int32_t kSmallPins = 1 << 19, kSmallPinsWide = 3 << 17;   // k <= 32, k > 32
+constexpr int32_t kSmallPins = 7 << 16, kSmallPinsWide = 11 << 15;   // 459k for k <= 32, 360k for k > 32
 constexpr int kSmPerHome = (64 + kSmCtas - 1) / kSmCtas;
 static_assert(kSmallVertices <= kSmMaxN, "ids of two digits");
 
