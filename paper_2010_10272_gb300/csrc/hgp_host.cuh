@@ -18,6 +18,7 @@ struct hgp_handle {
     bool all_eligible = true;     // first round after creation / set_partition
     int32_t n_wide = 0;
     int32_t m_big = 0;            // internal order: nets [0, m_big) have at least kBigNet pins
+    int32_t m_huge = 0;           // and nets [0, m_huge) at least kHugeNet
     int32_t m_big32 = 0;          // m_big rounded up to whole 32-net groups (at most m)
     int64_t max_vertex_netweight = 0;   // max_u sum_{e in I(u)} omega(e)
     int64_t total_weight = 0;

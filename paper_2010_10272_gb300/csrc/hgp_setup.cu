@@ -141,46 +141,68 @@ __device__ __forceinline__ int pin_net(const int32_t *off33, int32_t i)
 }
 
 // pins in [0, n) and strictly increasing inside every net; the largest net size.  Runs after
-// k_check_inputs and does nothing if that found an error.  A warp walks 32 nets' pins at once,
-// coalesced.
+// k_check_inputs and does nothing if that found an error.  Whatever the nets' sizes, every thread
+// walks pins and nets with one stride: the steps of the whole pin array that do not increase are
+// counted, and so are those at the first pin of a net, which are allowed; the nets are increasing
+// exactly if the two counts are equal.  (A warp per 32 nets spent the time of the longest net:
+// power-law 5M, nets of up to 100,000 pins, 676 -> 50 us.)  The last CTA compares the counts.
 __global__ void __launch_bounds__(256) k_check_pins(const int32_t *off, const int32_t *pins, int32_t m, int32_t n,
-                                                    int32_t *err, int32_t *max_size)
+                                                    int64_t P, int32_t *err, int32_t *max_size,
+                                                    unsigned long long *acc)
 {
-    __shared__ int32_t off33_w[8][33];
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    int32_t *off33 = off33_w[wid];
+    __shared__ long long diff_s;
+    __shared__ int32_t max_s;
     // the offsets may only be trusted when the checks before found nothing (they ran to
     // completion earlier on the same stream, so their flag is final)
     if (*reinterpret_cast<volatile int32_t *>(err) & ERR_INVALID) return;
-    const int64_t warps = (int64_t)gridDim.x * 8;
-    int32_t local_max = 0;
-    bool bad = false;
-    for (int64_t e0 = ((int64_t)blockIdx.x * 8 + wid) * 32; e0 < m; e0 += warps * 32) {
-        int32_t sz;
-        const int32_t base = net_group(off, e0, m, off33, sz);
-        local_max = max(local_max, sz);
-        const int32_t total = off33[32];
-        for (int32_t i0 = lane; i0 < total; i0 += 128) {   // four pins (and predecessors) per lane
-            int32_t vq[4], pq[4];
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const int32_t i = i0 + 32 * q;
-                vq[q] = i < total ? pins[base + i] : 0;
-                pq[q] = i < total && i > 0 ? pins[base + i - 1] : -1;
-            }
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const int32_t i = i0 + 32 * q;
-                if (i >= total) continue;
-                if (vq[q] < 0 || vq[q] >= n) bad = true;
-                if (i > off33[pin_net(off33, i)] && pq[q] >= vq[q]) bad = true;
-            }
-        }
-        __syncwarp();
+    if (threadIdx.x == 0) {
+        diff_s = 0;
+        max_s = 0;
     }
-    if (__any_sync(kFull, bad) && lane == 0) atomicOr(err, ERR_INVALID);
-    for (int o = 16; o; o >>= 1) local_max = max(local_max, __shfl_xor_sync(kFull, local_max, o));
-    if (lane == 0) atomicMax(max_size, local_max);
+    __syncthreads();
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    const int64_t t0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    bool bad = false;
+    int32_t diff = 0, local_max = 0;
+    for (int64_t j0 = t0; j0 < P; j0 += 4 * stride) {   // four pins (and predecessors) per thread in flight
+        int32_t v[4], q[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int64_t j = j0 + i * stride;
+            v[i] = j < P ? pins[j] : 0;
+            q[i] = j < P && j > 0 ? pins[j - 1] : -1;
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            if (j0 + i * stride >= P) continue;
+            if (v[i] < 0 || v[i] >= n) bad = true;
+            if (j0 + i * stride > 0) diff += q[i] >= v[i];
+        }
+    }
+    for (int64_t e = t0; e < m; e += stride) {
+        const int32_t b = off[e], sz = off[e + 1] - b;
+        local_max = max(local_max, sz);
+        if (sz > 0 && b > 0) diff -= pins[b - 1] >= pins[b];
+    }
+    if (__any_sync(kFull, bad) && (threadIdx.x & 31) == 0) atomicOr(err, ERR_INVALID);
+    diff = __reduce_add_sync(kFull, diff);
+    local_max = (int32_t)__reduce_max_sync(kFull, (unsigned)local_max);
+    if ((threadIdx.x & 31) == 0) {
+        if (diff) atomicAdd(reinterpret_cast<unsigned long long *>(&diff_s), (unsigned long long)(long long)diff);
+        atomicMax(&max_s, local_max);
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        if (diff_s) atomicAdd(&acc[ACC_OBJ], (unsigned long long)diff_s);
+        atomicMax(max_size, max_s);
+        __threadfence();
+        if (atomicAdd(&acc[ACC_DONE], 1ull) == gridDim.x - 1) {
+            __threadfence();
+            if (__ldcg(&acc[ACC_OBJ]) != 0) atomicOr(err, ERR_INVALID);
+            acc[ACC_OBJ] = 0;
+            acc[ACC_DONE] = 0;
+        }
+    }
 }
 
 // ------------------------------------------------------------------ internal net order
@@ -211,9 +233,11 @@ __global__ void __launch_bounds__(kNrThreads) k_nr_count(const int32_t *off, int
     if (threadIdx.x < kNrRanks) cnt[(int64_t)threadIdx.x * gridDim.x + blockIdx.x] = c[threadIdx.x];
 }
 
-// same chunks: internal id of every net (stable inside a rank) and the sizes in internal order
+// same chunks: internal id of every net (stable inside a rank), the sizes in internal order, and where
+// the pins of the large-net prefix [0, m_big) come from
 __global__ void __launch_bounds__(kNrThreads) k_nr_place(const int32_t *off, int32_t m, int32_t per_cta,
-                                                         const int32_t *base, int32_t *perm, int32_t *size_int)
+                                                         const int32_t *base, int32_t *perm, int32_t *size_int,
+                                                         int32_t m_big, int32_t *src_big)
 {
     constexpr int W = kNrThreads / 32;
     __shared__ int32_t run[kNrRanks];
@@ -238,6 +262,7 @@ __global__ void __launch_bounds__(kNrThreads) k_nr_place(const int32_t *off, int
             for (int w = 0; w < wid; ++w) pos += wc[w][rk];
             perm[e] = pos;
             size_int[pos] = size;
+            if (pos < m_big) src_big[pos] = off[e];
         }
         __syncthreads();
         if (threadIdx.x < kNrRanks) {
@@ -250,40 +275,101 @@ __global__ void __launch_bounds__(kNrThreads) k_nr_place(const int32_t *off, int
 }
 
 // pins (and net weights) into internal order; a warp copies the pins of 32 consecutive input
-// nets, reading them as one coalesced run
+// nets, reading them as one coalesced run but for the nets of the large-net prefix, whose pins
+// k_nr_pins_big copies (power-law 5M: 640 us with them -> 74 + 37 us)
 __global__ void __launch_bounds__(256) k_nr_pins(const int32_t *off, const int32_t *pins, const int32_t *nw,
-                                                 int32_t m, const int32_t *perm, const int32_t *off_int,
-                                                 int32_t *pins_int, int32_t *nw_int)
+                                                 int32_t m, int32_t m_big, const int32_t *perm,
+                                                 const int32_t *off_int, int32_t *pins_int, int32_t *nw_int)
 {
     __shared__ int32_t off33_w[8][33];
-    __shared__ int32_t dst_w[8][32];
+    __shared__ int32_t dst_w[8][32], src_w[8][32];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     int32_t *off33 = off33_w[wid];
     const int64_t warps = (int64_t)gridDim.x * 8;
     for (int64_t e0 = ((int64_t)blockIdx.x * 8 + wid) * 32; e0 < m; e0 += warps * 32) {
-        int32_t sz;
-        const int32_t src = net_group(off, e0, m, off33, sz);
         const int64_t e = e0 + lane;
+        int32_t src = 0, sz = 0;
         if (e < m) {
+            src = off[e];
+            sz = off[e + 1] - src;
             const int32_t q = perm[e];
             dst_w[wid][lane] = off_int[q];
             if (nw) nw_int[q] = nw[e];
+            if (q < m_big) sz = 0;
         }
+        int32_t incl = sz;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int32_t y = __shfl_up_sync(kFull, incl, o);
+            if (lane >= o) incl += y;
+        }
+        off33[lane] = incl - sz;
+        src_w[wid][lane] = src;
+        if (lane == 31) off33[32] = incl;
         __syncwarp();
         const int32_t total = off33[32];
         for (int32_t i0 = lane; i0 < total; i0 += 128) {   // four loads in flight per lane
-            int32_t vq[4];
-#pragma unroll
-            for (int q = 0; q < 4; ++q) vq[q] = i0 + 32 * q < total ? pins[src + i0 + 32 * q] : 0;
+            int32_t vq[4], at[4];
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
                 const int32_t i = i0 + 32 * q;
-                if (i >= total) continue;
-                const int sl = pin_net(off33, i);
-                pins_int[dst_w[wid][sl] + (i - off33[sl])] = vq[q];
+                const int sl = i < total ? pin_net(off33, i) : 0;
+                vq[q] = i < total ? __ldcs(&pins[src_w[wid][sl] + (i - off33[sl])]) : 0;
+                at[q] = dst_w[wid][sl] + (i - off33[sl]);
             }
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                if (i0 + 32 * q < total) pins_int[at[q]] = vq[q];
         }
         __syncwarp();
+    }
+}
+
+// the pins of the large-net prefix into internal order: a CTA per kBigChunk of them, whose nets'
+// offsets and sources sit in shared memory
+constexpr int kBigChunk = 8192;
+constexpr int32_t kBigNet = 256;                   // nets of the prefix have at least this many pins
+constexpr int kBigWin = kBigChunk / kBigNet + 3;   // offsets of the nets a chunk overlaps, + 1
+
+// the net of the prefix that holds pin p0: the largest e < m_big with off[e] <= p0
+__device__ __forceinline__ int32_t net_of_pin(const int32_t *off, int32_t m_big, int32_t p0)
+{
+    int32_t lo = 0, hi = m_big - 1;
+    while (lo < hi) {
+        const int32_t mid = (lo + hi + 1) >> 1;
+        if (off[mid] <= p0) lo = mid;
+        else hi = mid - 1;
+    }
+    return lo;
+}
+
+__device__ __forceinline__ int win_slot(const int32_t *win, int32_t j)
+{
+    int sl = 0;   // the largest slot with win[sl] <= j
+#pragma unroll
+    for (int step = 32; step; step >>= 1)
+        if (sl + step < kBigWin && win[sl + step] <= j) sl += step;
+    return sl;
+}
+
+__global__ void __launch_bounds__(1024) k_nr_pins_big(const int32_t *off_int, const int32_t *src_big, const int32_t *pins,
+                                                      int32_t m_big, int32_t *pins_int)
+{
+    __shared__ int32_t win[kBigWin], src[kBigWin];
+    __shared__ int32_t first;
+    const int32_t p0 = blockIdx.x * kBigChunk;
+    const int32_t p1 = min(off_int[m_big], p0 + kBigChunk);
+    if (threadIdx.x == 0) first = net_of_pin(off_int, m_big, p0);
+    __syncthreads();
+    if (threadIdx.x < kBigWin) {
+        win[threadIdx.x] = off_int[min(m_big, first + (int32_t)threadIdx.x)];
+        src[threadIdx.x] = src_big[min(m_big - 1, first + (int32_t)threadIdx.x)];
+    }
+    __syncthreads();
+#pragma unroll 4
+    for (int32_t j = p0 + threadIdx.x; j < p1; j += blockDim.x) {
+        const int sl = win_slot(win, j);
+        pins_int[j] = pins[src[sl] + (j - win[sl])];
     }
 }
 
@@ -297,53 +383,84 @@ __device__ __forceinline__ bool input_invalid(const int32_t *guard)
     return guard && (*reinterpret_cast<const volatile int32_t *>(guard) & ERR_INVALID) != 0;
 }
 
-// Adds the weights c (>= 1) of the lanes with ok to the shared block weights w, one update per
-// distinct block of the warp (same-address updates would queue up).
-__device__ __forceinline__ void add_block_weights(unsigned long long *w, bool ok, int blk, const int32_t *vw, int64_t v)
+// Per-CTA block weights: counts of unit weights (32-bit, native shared atomics), or sums.
+struct BlockSums {
+    unsigned long long w[64];
+    uint32_t c[64];
+};
+constexpr int kFewBlocks = 8;   // up to this k a warp's lanes share blocks: one update per distinct block
+
+__device__ __forceinline__ void add_block_weights(BlockSums &b, bool ok, int blk, int32_t k, const int32_t *vw, int64_t v)
 {
+    if (!vw && k > kFewBlocks) {
+        if (ok) atomicAdd(&b.c[blk], 1u);
+        return;
+    }
     const unsigned mask = __ballot_sync(kFull, ok);
     if (!ok) return;
     const unsigned peers = __match_any_sync(mask, blk);
-    unsigned long long sum = __popc(peers);
-    if (vw) {   // two halves: 32 sums of either fit 32 bits
-        const uint32_t c = (uint32_t)vw[v];
-        sum = (unsigned long long)__reduce_add_sync(peers, c & 0xFFFFu) +
-              ((unsigned long long)__reduce_add_sync(peers, c >> 16) << 16);
+    const bool lead = (int)(threadIdx.x & 31) == __ffs(peers) - 1;
+    if (!vw) {
+        if (lead) atomicAdd(&b.c[blk], (uint32_t)__popc(peers));
+        return;
     }
-    if ((int)(threadIdx.x & 31) == __ffs(peers) - 1) atomicAdd(&w[blk], sum);
+    // two halves: 32 sums of either fit 32 bits
+    const uint32_t x = (uint32_t)vw[v];
+    const unsigned long long sum = (unsigned long long)__reduce_add_sync(peers, x & 0xFFFFu) +
+                                   ((unsigned long long)__reduce_add_sync(peers, x >> 16) << 16);
+    if (lead) atomicAdd(&b.w[blk], sum);
+}
+
+__device__ __forceinline__ void clear_block_weights(BlockSums &b)
+{
+    if (threadIdx.x < 64) {
+        b.w[threadIdx.x] = 0;
+        b.c[threadIdx.x] = 0;
+    }
+    __syncthreads();
+}
+
+__device__ __forceinline__ void flush_block_weights(const BlockSums &b, int32_t k, unsigned long long *acc)
+{
+    __syncthreads();
+    if (threadIdx.x < k) {
+        const unsigned long long v = b.w[threadIdx.x] + b.c[threadIdx.x];
+        if (v) atomicAdd(&acc[ACC_BW + threadIdx.x], v);
+    }
 }
 
 // Stores the valid entries of a partition as 1-byte Pi and adds their vertices' weights to w (shared,
-// 64 zeros); returns whether an entry was out of range.
+// cleared); returns whether an entry was out of range.
 __device__ __forceinline__ bool stage_partition(const int32_t *part_in, int32_t n, int32_t k, const int32_t *vw,
-                                                uint8_t *part, unsigned long long *w)
+                                                uint8_t *part, BlockSums &w)
 {
     bool bad = false;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t v0 = blockIdx.x * (int64_t)blockDim.x + (threadIdx.x & ~31); v0 < n; v0 += stride) {
-        const int64_t v = v0 + (threadIdx.x & 31);
-        const int32_t p = v < n ? part_in[v] : -1;
-        const bool ok = p >= 0 && p < k;
-        if (v < n && !ok) bad = true;
-        if (ok) part[v] = (uint8_t)p;
-        add_block_weights(w, ok, p, vw, v);
+    for (int64_t v0 = blockIdx.x * (int64_t)blockDim.x + (threadIdx.x & ~31); v0 < n; v0 += 4 * stride) {
+        int32_t p[4];   // four entries per lane in flight
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int64_t v = v0 + q * stride + (threadIdx.x & 31);
+            p[q] = v < n ? __ldcs(&part_in[v]) : 0;
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int64_t v = v0 + q * stride + (threadIdx.x & 31);
+            const bool in = p[q] >= 0 && p[q] < k, ok = v < n && in;
+            if (!in) bad = true;
+            if (ok) part[v] = (uint8_t)p[q];
+            add_block_weights(w, ok, p[q], k, vw, v);
+        }
     }
     return bad;
-}
-
-__device__ __forceinline__ void flush_block_weights(const unsigned long long *w, int32_t k, unsigned long long *acc)
-{
-    __syncthreads();
-    if (threadIdx.x < k && w[threadIdx.x]) atomicAdd(&acc[ACC_BW + threadIdx.x], w[threadIdx.x]);
 }
 
 // A new partition: range check, 1-byte Pi and block weights in one pass over it.
 __global__ void __launch_bounds__(256) k_stage_partition(const int32_t *part_in, int32_t n, int32_t k, const int32_t *vw,
                                                          uint8_t *part, unsigned long long *acc, int32_t *err)
 {
-    __shared__ unsigned long long w[64];
-    if (threadIdx.x < 64) w[threadIdx.x] = 0;
-    __syncthreads();
+    __shared__ BlockSums w;
+    clear_block_weights(w);
     const bool bad = stage_partition(part_in, n, k, vw, part, w);
     if (__any_sync(kFull, bad) && (threadIdx.x & 31) == 0) atomicOr(err, ERR_INVALID);
     flush_block_weights(w, k, acc);
@@ -356,9 +473,8 @@ __global__ void __launch_bounds__(256) k_check_inputs(const int64_t *off64, int3
                                                       int32_t n, int32_t k, uint8_t *part, unsigned long long *acc,
                                                       int32_t *err)
 {
-    __shared__ unsigned long long w[64];
-    if (threadIdx.x < 64) w[threadIdx.x] = 0;
-    __syncthreads();
+    __shared__ BlockSums w;
+    clear_block_weights(w);
     bool bad = false;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     const int64_t t0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
@@ -410,9 +526,8 @@ constexpr int32_t kReorderMinNets = 1 << 20;
 constexpr int64_t kReorderSkew = 8;
 // host inputs with fewer nets than this: the host reads the net sizes (see create_impl)
 constexpr int32_t kHostSizesMaxNets = 1 << 20;
-// in internal order, nets of at least this many pins (a prefix) get their own CTAs at creation
-// and initialisation (a power of two: size classes are powers of two)
-constexpr int32_t kBigNet = 256;
+// in internal order, nets of at least kBigNet pins (a prefix) get their own CTAs at creation and
+// initialisation (a power of two: size classes are powers of two)
 
 __global__ void k_degrees(const int32_t *pins, int64_t P, int32_t *deg, const int32_t *guard)
 {
@@ -449,12 +564,12 @@ constexpr int kTpMaxBuckets = 4096;
 constexpr int kTpShift = 14;             // 16384 vertices per bucket, unless that gives too few
 constexpr int kTpMinShift = 8;           // buckets for the GPU (small instances) or too many
 constexpr int kTpSmemShift = 14;         // buckets up to this size count in shared memory
-// nets per scatter CTA, at most (fewer when the instance has few nets): each CTA's walk over its
-// nets is a chain of dependent loads, so many short walks beat few long ones even though every
-// CTA reserves a range in every bucket (power-law creation: 16384 -> 30.1 ms, 4096 -> 25.1 ms,
-// 2048 -> 23.3 ms, 512 -> 23.1 ms)
-constexpr int kTpNetsPerCta = 2048;
-constexpr int kTpMinCtas = 608;          // target CTAs per launch (4 per SM)
+constexpr int kTpMinCtas = 608;          // target buckets and CTAs per launch (4 per SM)
+constexpr int kTpThreads = 512;
+// pins per scatter CTA, at most: every CTA reserves a range in every bucket.  Cut by pins, not by
+// nets: in internal order 2048 nets are 6,000 pins or 400,000, and the launch took as long as
+// the latter (power-law 5M 779 -> 351 us, 50M 5.85 -> 5.0 ms)
+constexpr int kTpMaxPins = 32768, kTpMinPins = 4096;
 
 __global__ void __launch_bounds__(256) k_tp_hist(const int32_t *pins, int64_t P, int bshift, int32_t nb,
                                                  int32_t *bucket_cnt, const int32_t *guard)
@@ -470,24 +585,41 @@ __global__ void __launch_bounds__(256) k_tp_hist(const int32_t *pins, int64_t P,
         if (h[i]) atomicAdd(&bucket_cnt[i], h[i]);
 }
 
-// CTA per per_cta nets; pass 0 counts its pins per bucket, then one range per bucket is
-// reserved, pass 1 writes the pairs.  A warp walks the pins of 32 nets at once (coalesced).
-__global__ void __launch_bounds__(256) k_tp_scatter(const int32_t *off, const int32_t *pins, int32_t m,
+// the first net e in [lo, hi] with off[e] >= p (hi if there is none before it)
+__device__ __forceinline__ int32_t first_net_at(const int32_t *off, int32_t lo, int32_t hi, int32_t p)
+{
+    while (lo < hi) {
+        const int32_t mid = lo + ((hi - lo) >> 1);
+        if (off[mid] >= p) hi = mid;
+        else lo = mid + 1;
+    }
+    return lo;
+}
+
+// CTA per per_cta pins: the nets from e_begin on that start there.  Pass 0 counts their pins per
+// bucket, then one range per bucket is reserved, pass 1 writes the pairs.  A warp walks the pins of
+// 32 nets at once (coalesced).
+__global__ void __launch_bounds__(kTpThreads) k_tp_scatter(const int32_t *off, const int32_t *pins, int32_t m,
                                                     int32_t e_begin, int bshift, int32_t nb, int32_t narrow_max,
                                                     int32_t per_cta, int32_t *bucket_cur, unsigned long long *pairs,
                                                     const int32_t *guard)
 {
     if (input_invalid(guard)) return;
+    constexpr int kW = kTpThreads / 32;
     __shared__ int32_t cur[kTpMaxBuckets];
-    __shared__ int32_t off33_w[8][33];
+    __shared__ int32_t off33_w[kW][33];
+    __shared__ int32_t bound[2];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     int32_t *off33 = off33_w[wid];
-    const int64_t e_lo = e_begin + (int64_t)blockIdx.x * per_cta;
-    const int64_t e_hi = min((int64_t)m, e_lo + per_cta);
+    if (threadIdx.x < 2) {
+        const int64_t p = off[e_begin] + ((int64_t)blockIdx.x + threadIdx.x) * per_cta;
+        bound[threadIdx.x] = p > off[m] ? m : first_net_at(off, e_begin, m, (int32_t)p);
+    }
     for (int i = threadIdx.x; i < nb; i += blockDim.x) cur[i] = 0;
     __syncthreads();
-    for (int pass = 0; pass < 2; ++pass) {
-        for (int64_t e0 = e_lo + 32 * wid; e0 < e_hi; e0 += 32 * 8) {
+    const int64_t e_lo = bound[0], e_hi = bound[1];
+    auto walk = [&](auto each) {   // each(pin, net, whether wide)
+        for (int64_t e0 = e_lo + 32 * wid; e0 < e_hi; e0 += 32 * kW) {
             int32_t sz;
             const int32_t base = net_group(off, e0, e_hi, off33, sz);
             const int32_t total = off33[32];
@@ -497,72 +629,54 @@ __global__ void __launch_bounds__(256) k_tp_scatter(const int32_t *off, const in
 #pragma unroll
                 for (int q = 0; q < 4; ++q) vq[q] = i0 + 32 * q < total ? pins[base + i0 + 32 * q] : -1;
 #pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    if (vq[q] < 0) continue;
-                    const int32_t i = i0 + 32 * q, v = vq[q];
-                    const int32_t pos = atomicAdd(&cur[v >> bshift], 1);
-                    if (pass == 1) {
-                        const int sl = pin_net(off33, i);
-                        const uint32_t ef = (uint32_t)(e0 + sl) | (off33[sl + 1] - off33[sl] > narrow_max ? kWideFlag : 0u);
-                        pairs[pos] = ((unsigned long long)(uint32_t)v << 32) | ef;
-                    }
-                }
+                for (int q = 0; q < 4; ++q)
+                    if (vq[q] >= 0) each(vq[q], e0, i0 + 32 * q);
             }
             __syncwarp();
         }
-        __syncthreads();
-        if (pass == 0) {
-            for (int i = threadIdx.x; i < nb; i += blockDim.x) {
-                const int32_t c = cur[i];
-                cur[i] = c ? atomicAdd(&bucket_cur[i], c) : 0;
-            }
-            __syncthreads();
-        }
+    };
+    walk([&](int32_t v, int64_t, int32_t) { atomicAdd(&cur[v >> bshift], 1); });   // no old value: a reduction
+    __syncthreads();
+    for (int i = threadIdx.x; i < nb; i += blockDim.x) {
+        const int32_t c = cur[i];
+        cur[i] = c ? atomicAdd(&bucket_cur[i], c) : 0;
     }
+    __syncthreads();
+    walk([&](int32_t v, int64_t e0, int32_t i) {
+        const int32_t pos = atomicAdd(&cur[v >> bshift], 1);
+        const int sl = pin_net(off33, i);
+        const uint32_t ef = (uint32_t)(e0 + sl) | (off33[sl + 1] - off33[sl] > narrow_max ? kWideFlag : 0u);
+        pairs[pos] = ((unsigned long long)(uint32_t)v << 32) | ef;
+    });
 }
 
 // The pins of the large-net prefix [0, m_big) of the internal order (nets of at least kBigNet
-// pins), split into chunks of kTpBigChunk pins, one CTA each, so that no CTA takes many large
-// nets.  A chunk overlaps at most kTpBigChunk / kBigNet + 2 nets, whose offsets are staged in
-// shared memory.  Same two passes as k_tp_scatter.
-constexpr int kTpBigChunk = 8192;
-constexpr int kTpBigWin = kTpBigChunk / kBigNet + 3;   // offsets of the nets a chunk overlaps, + 1
-
-__global__ void __launch_bounds__(256) k_tp_scatter_big(const int32_t *off, const int32_t *pins, int32_t m_big,
-                                                        int bshift, int32_t nb, int32_t narrow_max,
-                                                        int32_t *bucket_cur, unsigned long long *pairs,
-                                                        const int32_t *guard)
+// pins), split into chunks of kBigChunk pins, one CTA each, so that no CTA takes many large
+// nets.  Same two passes as k_tp_scatter.
+__global__ void __launch_bounds__(kTpThreads) k_tp_scatter_big(const int32_t *off, const int32_t *pins, int32_t m_big,
+                                                               int bshift, int32_t nb, int32_t narrow_max,
+                                                               int32_t *bucket_cur, unsigned long long *pairs,
+                                                               const int32_t *guard)
 {
     if (input_invalid(guard)) return;
     __shared__ int32_t cur[kTpMaxBuckets];
-    __shared__ int32_t win[kTpBigWin];
+    __shared__ int32_t win[kBigWin];
     __shared__ int32_t first;
     const int32_t p_end = off[m_big];
-    const int32_t p0 = blockIdx.x * kTpBigChunk;
-    const int32_t p1 = min(p_end, p0 + kTpBigChunk);
-    if (threadIdx.x == 0) {   // the net holding pin p0: the largest e < m_big with off[e] <= p0
-        int32_t lo = 0, hi = m_big - 1;
-        while (lo < hi) {
-            const int32_t mid = (lo + hi + 1) >> 1;
-            if (off[mid] <= p0) lo = mid;
-            else hi = mid - 1;
-        }
-        first = lo;
-    }
+    const int32_t p0 = blockIdx.x * kBigChunk;
+    const int32_t p1 = min(p_end, p0 + kBigChunk);
+    if (threadIdx.x == 0) first = net_of_pin(off, m_big, p0);
     for (int i = threadIdx.x; i < nb; i += blockDim.x) cur[i] = 0;
     __syncthreads();
     const int32_t e_f = first;
-    for (int i = threadIdx.x; i < kTpBigWin; i += blockDim.x) win[i] = off[min(m_big, e_f + i)];
+    if (threadIdx.x < kBigWin) win[threadIdx.x] = off[min(m_big, e_f + (int32_t)threadIdx.x)];
     __syncthreads();
     for (int pass = 0; pass < 2; ++pass) {
         for (int32_t j = p0 + threadIdx.x; j < p1; j += blockDim.x) {
             const int32_t v = pins[j];
             const int32_t pos = atomicAdd(&cur[v >> bshift], 1);
             if (pass == 1) {
-                int sl = 0;   // the largest slot with win[sl] <= j
-#pragma unroll
-                for (int step = 32; step; step >>= 1)
-                    if (sl + step < kTpBigWin && win[sl + step] <= j) sl += step;
+                const int sl = win_slot(win, j);
                 const uint32_t ef = (uint32_t)(e_f + sl) | (win[sl + 1] - win[sl] > narrow_max ? kWideFlag : 0u);
                 pairs[pos] = ((unsigned long long)(uint32_t)v << 32) | ef;
             }
@@ -675,7 +789,11 @@ __device__ __forceinline__ int32_t narrow_max_of(const Dev &d)
     return d.phi_w == 1 ? 255 : (d.phi_w == 2 ? 65535 : 0x7fffffff);
 }
 
-// One net, by the whole CTA (256 threads); cnt: 64 shared counters.  Returns the net's objective
+// k_init_big: nets of at least kHugeNet pins take CTAs of 1024 threads (the largest net's walk is as
+// long as the launch), the others of 256 (power-law 5M: 250 us with 256 for all -> 74 + 32)
+constexpr int32_t kHugeNet = 4096;
+
+// One net, by the whole CTA (at least 64 threads); cnt: 64 shared counters.  Returns the net's objective
 // term in thread 0.
 template <typename Rec>
 __device__ __forceinline__ long long init_net_cta(const Dev &d, const uint8_t *part, int64_t e, int32_t *cnt)
@@ -731,12 +849,12 @@ __device__ __forceinline__ long long init_net_cta(const Dev &d, const uint8_t *p
 // The nets of the large-net prefix of the internal order, one CTA per net: k_init_nets would give all
 // of them to its first CTAs.
 template <typename Rec>
-__global__ void __launch_bounds__(256) k_init_big(Dev d, const uint8_t *part, int32_t m_big, const int32_t *guard)
+__global__ void __launch_bounds__(1024) k_init_big(Dev d, const uint8_t *part, int32_t e0, int32_t e1, const int32_t *guard)
 {
     if (input_invalid(guard)) return;
     __shared__ int32_t cnt[64];
     long long obj = 0;
-    for (int64_t e = blockIdx.x; e < m_big; e += gridDim.x) obj += init_net_cta<Rec>(d, part, e, cnt);
+    for (int64_t e = e0 + (int64_t)blockIdx.x; e < e1; e += gridDim.x) obj += init_net_cta<Rec>(d, part, e, cnt);
     if (threadIdx.x == 0 && obj) atomicAdd(&d.acc[ACC_OBJ], (unsigned long long)obj);
 }
 
@@ -1199,10 +1317,12 @@ int init_state(hgp_handle *h, const uint8_t *part, const int32_t *guard)
     Dev &d = h->d;
     cudaStream_t st = h->stream;
     const int32_t e_begin = h->m_big32;
-    if (e_begin > 0) {
-        const int gb = e_begin < 152 * 16 ? e_begin : 152 * 16;
-        if (d.k <= 32) k_init_big<Rec16><<<gb, 256, 0, st>>>(d, part, e_begin, guard);
-        else k_init_big<Rec32><<<gb, 256, 0, st>>>(d, part, e_begin, guard);
+    for (int huge = 1; huge >= 0; --huge) {
+        const int32_t e0 = huge ? 0 : h->m_huge, e1 = huge ? h->m_huge : e_begin;
+        if (e0 >= e1) continue;
+        const int threads = huge ? 1024 : 256, gb = std::min(e1 - e0, 152 * (huge ? 2 : 16));
+        if (d.k <= 32) k_init_big<Rec16><<<gb, threads, 0, st>>>(d, part, e0, e1, guard);
+        else k_init_big<Rec32><<<gb, threads, 0, st>>>(d, part, e0, e1, guard);
         h->launches++;
     }
     const int g = grid_for(std::max<int64_t>((int64_t)d.m - e_begin, 1), kInitWarps * 32, 152 * 16);
@@ -1415,7 +1535,8 @@ int create_impl(int32_t n, int32_t m, const int64_t *net_offsets, const int32_t 
     int32_t host_err[2] = {0, 0};
     // one read-back for both checks: the pin check does nothing when the offsets were bad
     if (m > 0) {
-        k_check_pins<<<grid_for(m, 256), 256, 0, st>>>(net_off, pins_d, m, n, d.err, max_size_d); h->launches++;
+        k_check_pins<<<grid_for(std::max<int64_t>(P / 4, m), 256, 152 * 8), 256, 0, st>>>(net_off, pins_d, m, n, P, d.err,
+                                                                                    max_size_d, d.acc); h->launches++;
         CKF(cudaGetLastError());
     }
     const int32_t *guard = nullptr;
@@ -1463,17 +1584,30 @@ int create_impl(int32_t n, int32_t m, const int64_t *net_offsets, const int32_t 
         CKF(scan(cnt, base, nslots));
         int big_rank = 0;   // first rank of the nets below kBigNet pins
         while (((int64_t)1 << (31 - big_rank)) >= kBigNet) ++big_rank;
+        int huge_rank = 0;
+        while (((int64_t)1 << (31 - huge_rank)) >= kHugeNet) ++huge_rank;
         int32_t mb = 0;
+        CKF(cudaMemcpyAsync(&h->m_huge, base + (int64_t)huge_rank * nr_ctas, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
         CKF(cudaMemcpyAsync(&mb, base + (int64_t)big_rank * nr_ctas, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
         CKF(stream_wait(st));
-        k_nr_place<<<(unsigned)nr_ctas, kNrThreads, 0, st>>>(net_off, m, per_cta, base, perm, tmp); h->launches++;
+        int32_t *src_big = nullptr;   // where the pins of the large-net prefix come from
+        if (mb > 0) CKF(dev_alloc(reinterpret_cast<void **>(&src_big), sizeof(int32_t) * (size_t)mb, st));
+        k_nr_place<<<(unsigned)nr_ctas, kNrThreads, 0, st>>>(net_off, m, per_cta, base, perm, tmp, mb, src_big);
+        h->launches++;
         CKF(scan(tmp, off_int, m));   // sizes in internal order -> offsets (off_int[m] = P)
-        k_nr_pins<<<grid_for((int64_t)m * 32, 256), 256, 0, st>>>(net_off, pins_d, nw_d, m, perm, off_int,
-                                                                  pins_int, nw_int); h->launches++;
-        CKF(cudaGetLastError());
-        CKF(pool_free(cnt, st));
         CKF(cudaMemcpyAsync(&p_big, off_int + mb, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
+        k_nr_pins<<<grid_for((int64_t)m, 256), 256, 0, st>>>(net_off, pins_d, nw_d, m, mb, perm, off_int, pins_int,
+                                                             nw_int); h->launches++;
+        CKF(cudaGetLastError());
         CKF(stream_wait(st));
+        if (p_big > 0) {
+            k_nr_pins_big<<<(unsigned)((p_big + kBigChunk - 1) / kBigChunk), 1024, 0, st>>>(off_int, src_big, pins_d, mb,
+                                                                                            pins_int);
+            h->launches++;
+            CKF(cudaGetLastError());
+        }
+        CKF(pool_free(cnt, st));
+        if (src_big) CKF(pool_free(src_big, st));
         h->m_big = mb;
         h->m_big32 = (int32_t)std::min((int64_t)m, ((int64_t)mb + 31) / 32 * 32);
         release(net_off);
@@ -1530,9 +1664,8 @@ int create_impl(int32_t n, int32_t m, const int64_t *net_offsets, const int32_t 
         while (buckets(bshift) > kTpMaxBuckets) ++bshift;
         const int32_t nbk = (int32_t)buckets(bshift);
         const int32_t e_begin = h->m_big;   // the large-net prefix goes to k_tp_scatter_big
-        const int64_t m_rest = (int64_t)m - e_begin;
-        int64_t per_cta = (m_rest + kTpMinCtas - 1) / kTpMinCtas;
-        per_cta = per_cta < 512 ? 512 : (per_cta > kTpNetsPerCta ? kTpNetsPerCta : per_cta);
+        const int64_t p_rest = P - p_big;
+        const int64_t per_cta = std::min<int64_t>(kTpMaxPins, std::max<int64_t>(kTpMinPins, p_rest / kTpMinCtas));
         int32_t *bk = nullptr;           // counts [nbk + 1], offsets [nbk + 1], cursors [nbk]
         unsigned long long *pairs = nullptr;
         CKF(dev_alloc(reinterpret_cast<void **>(&bk), sizeof(int32_t) * (3 * (size_t)nbk + 2), st));
@@ -1542,13 +1675,13 @@ int create_impl(int32_t n, int32_t m, const int64_t *net_offsets, const int32_t 
         k_tp_hist<<<grid_for(P, 256, 152 * 8), 256, 0, st>>>(pins_d, P, bshift, nbk, bk_cnt, guard); h->launches++;
         CKF(scan(bk_cnt, bk_off, nbk));
         CKF(cudaMemcpyAsync(bk_cur, bk_off, sizeof(int32_t) * (size_t)nbk, cudaMemcpyDeviceToDevice, st));
-        const int64_t sc = (m_rest + per_cta - 1) / per_cta;
+        const int64_t sc = (p_rest + per_cta - 1) / per_cta;
         if (e_begin > 0 && p_big > 0) {
-            k_tp_scatter_big<<<(unsigned)((p_big + kTpBigChunk - 1) / kTpBigChunk), 256, 0, st>>>(
+            k_tp_scatter_big<<<(unsigned)((p_big + kBigChunk - 1) / kBigChunk), kTpThreads, 0, st>>>(
                 net_off, pins_d, e_begin, bshift, nbk, narrow_max, bk_cur, pairs, guard); h->launches++;
         }
         if (sc > 0) {
-            k_tp_scatter<<<(unsigned)sc, 256, 0, st>>>(net_off, pins_d, m, e_begin, bshift, nbk, narrow_max,
+            k_tp_scatter<<<(unsigned)sc, kTpThreads, 0, st>>>(net_off, pins_d, m, e_begin, bshift, nbk, narrow_max,
                                                        (int32_t)per_cta, bk_cur, pairs, guard); h->launches++;
         }
         if (bshift <= kTpSmemShift) {

@@ -43,3 +43,32 @@ def test_state_of_a_new_partition(phi_width, k, sizes):
         compare_state(h, o)
         assert np.array_equal(h.refine(2)[:, :5], o.refine(2)[0])
     h.close()
+
+
+@pytest.mark.parametrize("debug", [0, 2, 4, 6])
+@pytest.mark.parametrize("where", ["first", "middle", "last"])
+def test_pin_order_is_checked_wherever_it_breaks(debug, where):
+    """A repeated or falling pin inside a net is refused, a falling step between two nets is not; with
+    empty nets, nets of one pin and a net of 100,000 among them, on every creation path."""
+    from paper_2010_10272_gb300 import HGP, HGPError
+    rng = np.random.default_rng(3)
+    n = 120_000
+    size = rng.integers(0, 4, 30_000)
+    size[17_000] = 100_000
+    size[20_000] = 9_000
+    pins = np.concatenate([np.sort(rng.choice(n, s, replace=False)) for s in size]).astype(np.int32)
+    off = np.concatenate([[0], np.cumsum(size)]).astype(np.int64)
+    part = rng.integers(0, 9, n).astype(np.int32)
+    h = HGP(n, size.size, off, pins, 9, 0.03, part, debug=debug)
+    compare_state(h, oracle.Oracle(n, size.size, off, pins, 9, 0.03, part))
+    h.close()
+    at = {"first": off[np.flatnonzero(size >= 2)[0]], "middle": off[17_000] + 50_000,
+          "last": off[np.flatnonzero(size >= 2)[-1]]}[where]
+    for delta in (0, 1):
+        bad = pins.copy()
+        bad[at + 1] = bad[at] - delta
+        for device in (False, True):
+            a = [torch.from_numpy(x).cuda() if device else x for x in (off, bad, part)]
+            with pytest.raises(HGPError) as ei:
+                HGP(n, size.size, a[0], a[1], 9, 0.03, a[2], debug=debug, device=device)
+            assert ei.value.code == 1
