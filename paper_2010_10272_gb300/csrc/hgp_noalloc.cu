@@ -31,8 +31,8 @@ constexpr unsigned kFull = 0xffffffffu;
 constexpr int32_t kNoAllocMaxNets = 1 << 18;
 constexpr int kMaxDevices = 64;
 
-// scratch layout (bytes): [0, 512) block weights int64[64]; [512, 520) error flags;
-// [1024, ...) one 32-byte record per net
+// scratch layout (bytes): [0, 512) block weights int64[64]; [512, 516) error flag; [520, 528)
+// falling steps of the lists (see k_na_prepare); [1024, ...) one 32-byte record per net
 struct __align__(16) NaRec {
     uint64_t s1;     // bit i: Phi(e,i) == 1
     uint64_t lam;    // bit i: Phi(e,i) > 0
@@ -69,20 +69,23 @@ int scratch_address(void **out)
     return HGP_OK;
 }
 
+constexpr int kLaneNet = 16;   // nets of up to this many pins are read by one lane
+
 __global__ void k_na_clear(int64_t *bw, int32_t *err)
 {
     if (threadIdx.x < 64) bw[threadIdx.x] = 0;
-    if (threadIdx.x == 0) err[0] = 0;
+    if (threadIdx.x < 4) err[threadIdx.x] = 0;   // and the falling steps
 }
 
 // input checks (every index the later kernels use must be in range)
 __global__ void k_na_check(int32_t n, int32_t m, const int32_t *net_off, const int32_t *pins,
                            const int32_t *vtx_off, const int32_t *inc, const int32_t *vw,
-                           const int32_t *nw, const int32_t *part, int32_t k, int32_t P, int32_t *err)
+                           const int32_t *nw, const int32_t *part, int32_t k, int32_t *err)
 {
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     const int64_t i0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    bool bad = false;
+    const int32_t P = net_off[m];
+    bool bad = P < 0;
     for (int64_t e = i0; e <= m; e += stride) {
         const int32_t a = net_off[e];
         if ((e == 0 && a != 0) || (e == m && a != P) || (e < m && net_off[e + 1] < a)) bad = true;
@@ -101,126 +104,188 @@ __global__ void k_na_check(int32_t n, int32_t m, const int32_t *net_off, const i
     if (bad) atomicOr(err, 1);
 }
 
-// Order checks, warp per list (run after k_na_check has passed, so every index is in range):
-// pins strictly increasing inside each net (this also excludes a pin listed twice), and net
-// ids strictly increasing inside each vertex's list.
-__global__ void k_na_check_order(int32_t n, int32_t m, const int32_t *net_off, const int32_t *pins,
-                                 const int32_t *vtx_off, const int32_t *inc, int32_t *err)
+// After k_na_check (does nothing if that found an error), in one launch:
+//   * order: pins strictly increasing inside each net (this also excludes a pin listed twice) and
+//     net ids strictly increasing inside each vertex's list.  The steps of both arrays that do not
+//     increase are counted, those at the first entry of a list, which are allowed, are taken off:
+//     zero is left exactly if every list increases (whatever the lists' lengths, every thread reads
+//     with one stride);
+//   * transpose: vertex v's list may name net e only if v is a pin of e (binary search in the sorted
+//     pin list; a list out of order is reported by the first check).  With distinct entries per list
+//     and P entries in total, the two CSRs then describe exactly the same incidences;
+//   * block weights;
+//   * records: Lambda(e) and S1(e) need no pin counts: a block seen again is no longer in S1.  A lane
+//     per net of up to kLaneNet pins, else the warp.
+// 250k nets, 1M pins: 140 us as four launches -> 28.
+__global__ void __launch_bounds__(256) k_na_prepare(int32_t n, int32_t m, const int32_t *net_off, const int32_t *pins,
+                                                    const int32_t *vtx_off, const int32_t *inc, const int32_t *part,
+                                                    const int32_t *vw, const int32_t *nw, NaRec *recs, int64_t *bw,
+                                                    int32_t *err)
 {
+    if (*reinterpret_cast<volatile int32_t *>(err)) return;
+    __shared__ unsigned long long w[64];
+    __shared__ int falls_s;
     const int lane = threadIdx.x & 31;
-    const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
-    const int64_t w0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    bool bad = false;
-    for (int64_t e = w0; e < m; e += warps)
-        for (int32_t j = net_off[e] + 1 + lane; j < net_off[e + 1]; j += 32)
-            if (pins[j] <= pins[j - 1]) bad = true;
-    for (int64_t v = w0; v < n; v += warps)
-        for (int32_t j = vtx_off[v] + 1 + lane; j < vtx_off[v + 1]; j += 32)
-            if (inc[j] <= inc[j - 1]) bad = true;
-    if (__any_sync(kFull, bad) && lane == 0) atomicOr(err, 1);
-}
-
-// Transpose check, thread per incidence (after the order checks): vertex v's list may name net
-// e only if v is a pin of e (binary search in the sorted pin list).  With distinct entries per
-// list and P entries in total, the two CSRs then describe exactly the same incidences.
-__global__ void k_na_check_transpose(int32_t n, const int32_t *net_off, const int32_t *pins,
-                                     const int32_t *vtx_off, const int32_t *inc, int32_t *err)
-{
+    if (threadIdx.x < 64) w[threadIdx.x] = 0;
+    if (threadIdx.x == 0) falls_s = 0;
+    __syncthreads();
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    const int64_t i0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    const int32_t P = net_off[m];
     bool bad = false;
-    for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < n; v += stride) {
-        for (int32_t j = vtx_off[v]; j < vtx_off[v + 1]; ++j) {
+    int falls = 0;
+    for (int64_t j = i0 + 1; j < P; j += stride) falls += (pins[j - 1] >= pins[j]) + (inc[j - 1] >= inc[j]);
+    for (int64_t v = i0; v < n; v += stride) {
+        const int32_t b = vtx_off[v], end = vtx_off[v + 1];
+        if (b > 0 && b < end) falls -= inc[b - 1] >= inc[b];
+        for (int32_t j = b; j < end; ++j) {
             const int32_t e = inc[j];
-            int32_t lo = net_off[e], hi = net_off[e + 1];
+            int32_t lo = net_off[e];
+            const int32_t hi0 = net_off[e + 1];
+            int32_t hi = hi0;
             while (lo < hi) {
                 const int32_t mid = lo + ((hi - lo) >> 1);
                 if (pins[mid] < v) lo = mid + 1;
                 else hi = mid;
             }
-            if (lo >= net_off[e + 1] || pins[lo] != (int32_t)v) bad = true;
+            if (lo >= hi0 || pins[lo] != (int32_t)v) bad = true;
         }
-    }
-    if (bad) atomicOr(err, 1);
-}
-
-__global__ void k_na_block_weights(int32_t n, const int32_t *part, const int32_t *vw, int64_t *bw)
-{
-    __shared__ unsigned long long w[64];
-    if (threadIdx.x < 64) w[threadIdx.x] = 0;
-    __syncthreads();
-    for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < n;
-         v += (int64_t)gridDim.x * blockDim.x)
         atomicAdd(&w[part[v]], (unsigned long long)(vw ? vw[v] : 1));
-    __syncthreads();
-    if (threadIdx.x < 64 && w[threadIdx.x])
-        atomicAdd(reinterpret_cast<unsigned long long *>(&bw[threadIdx.x]), w[threadIdx.x]);
-}
-
-// warp per net: Phi(e, .) counted from the partition -> Lambda(e), S1(e), omega(e)
-__global__ void k_na_records(int32_t m, const int32_t *net_off, const int32_t *pins,
-                             const int32_t *part, const int32_t *nw, NaRec *recs)
-{
-    __shared__ int32_t cnt[8][64];
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    for (int64_t e = (int64_t)blockIdx.x * 8 + wid; e < m; e += (int64_t)gridDim.x * 8) {
-        cnt[wid][lane] = 0;
-        cnt[wid][lane + 32] = 0;
-        __syncwarp();
-        const int32_t b = net_off[e], end = net_off[e + 1];
-        for (int32_t base = b; base < end; base += 32) {
-            const int32_t j = base + lane;
-            const bool act = j < end;
-            const unsigned mask = __ballot_sync(kFull, act);
-            if (act) {
-                const int blk = part[pins[j]];
-                const unsigned peers = __match_any_sync(mask, blk);
-                if (lane == __ffs(peers) - 1) cnt[wid][blk] += __popc(peers);
-            }
-            __syncwarp();
+    }
+    for (int64_t e0 = i0 - lane; e0 < m; e0 += stride) {
+        const int64_t e = e0 + lane;
+        int32_t b = 0, end = 0;
+        if (e < m) {
+            b = net_off[e];
+            end = net_off[e + 1];
+            if (b > 0 && b < end) falls -= pins[b - 1] >= pins[b];
         }
-        const unsigned lo_l = __ballot_sync(kFull, cnt[wid][lane] > 0);
-        const unsigned hi_l = __ballot_sync(kFull, cnt[wid][lane + 32] > 0);
-        const unsigned lo_1 = __ballot_sync(kFull, cnt[wid][lane] == 1);
-        const unsigned hi_1 = __ballot_sync(kFull, cnt[wid][lane + 32] == 1);
-        if (lane == 0) {
+        uint64_t lam = 0, again = 0;
+        if (end - b <= kLaneNet) {
+            for (int32_t j = b; j < end; ++j) {
+                const uint64_t bit = 1ull << part[pins[j]];
+                again |= lam & bit;
+                lam |= bit;
+            }
+        }
+        unsigned big = __ballot_sync(kFull, end - b > kLaneNet);
+        while (big) {
+            const int src = __ffs(big) - 1;
+            big &= big - 1;
+            const int32_t bb = __shfl_sync(kFull, b, src), be = __shfl_sync(kFull, end, src);
+            uint64_t l = 0, a = 0;
+            for (int32_t j = bb + lane; j < be; j += 32) {
+                const uint64_t bit = 1ull << part[pins[j]];
+                a |= l & bit;
+                l |= bit;
+            }
+#pragma unroll
+            for (int o = 16; o; o >>= 1) {   // a block of both halves is a block seen again
+                const uint64_t l2 = __shfl_xor_sync(kFull, l, o), a2 = __shfl_xor_sync(kFull, a, o);
+                a |= a2 | (l & l2);
+                l |= l2;
+            }
+            if (lane == src) {
+                lam = l;
+                again = a;
+            }
+        }
+        if (e < m) {
             NaRec r;
-            r.s1 = (uint64_t)lo_1 | ((uint64_t)hi_1 << 32);
-            r.lam = (uint64_t)lo_l | ((uint64_t)hi_l << 32);
+            r.s1 = lam & ~again;
+            r.lam = lam;
             r.w = nw ? nw[e] : 1;
             r.pad[0] = r.pad[1] = r.pad[2] = 0;
             recs[e] = r;
         }
-        __syncwarp();
     }
+    if (__any_sync(kFull, bad) && lane == 0) atomicOr(err, 1);
+    falls = __reduce_add_sync(kFull, falls);
+    if (lane == 0 && falls) atomicAdd(&falls_s, falls);
+    __syncthreads();
+    if (threadIdx.x < 64 && w[threadIdx.x])
+        atomicAdd(reinterpret_cast<unsigned long long *>(&bw[threadIdx.x]), w[threadIdx.x]);
+    if (threadIdx.x == 0 && falls_s)   // next to the error flag, read with it
+        atomicAdd(reinterpret_cast<unsigned long long *>(err + 2), (unsigned long long)(long long)falls_s);
 }
 
-// thread per vertex: the gain step of round 0 (every vertex eligible) for sub-round s, as in
-// the refinement rounds: T = blocks of Lambda(e) over nets with Phi(e,a) = 1, minus a and the
-// blocks without room; best t in T by g_t = b(u) - W + omega({e : t in Lambda(e)}), smallest
-// block on ties; no candidate unless the gain is positive.
-__global__ void k_na_candidates(int32_t n, int32_t k, double eps, const int32_t *vtx_off,
-                                const int32_t *inc, const NaRec *recs, const int32_t *part,
-                                const int32_t *vw, const int64_t *bw, int32_t S, uint64_t seed,
-                                int32_t s, int32_t *target, int64_t *gain)
+// conn_t for every block at once in NP bit planes (bit t of plane p is bit p of conn_t; W < 2^NP), then
+// the block of T with the largest, smallest id among equals
+template <int NP>
+__device__ __forceinline__ void na_planes(const NaRec *recs, const int32_t *inc, int32_t jb, int32_t je, uint64_t T,
+                                          int &t_out, int32_t &conn_out)
+{
+    uint64_t c[NP];
+#pragma unroll
+    for (int p = 0; p < NP; ++p) c[p] = 0;
+    for (int32_t j = jb; j < je; ++j) {
+        const NaRec &r = recs[inc[j]];
+        const uint64_t x = r.lam & T;
+        const int32_t w = r.w;
+        uint64_t carry = 0;
+#pragma unroll
+        for (int p = 0; p < NP; ++p) {
+            const uint64_t ad = ((w >> p) & 1) ? x : 0ull;
+            const uint64_t cp = c[p];
+            c[p] = cp ^ ad ^ carry;
+            carry = (cp & ad) | (carry & (cp ^ ad));
+        }
+    }
+    uint64_t C = T;
+#pragma unroll
+    for (int p = NP - 1; p >= 0; --p) C = (C & c[p]) ? C & c[p] : C;
+    t_out = __ffsll((long long)C) - 1;
+    conn_out = 0;
+#pragma unroll
+    for (int p = 0; p < NP; ++p) conn_out |= (int32_t)((c[p] >> t_out) & 1) << p;
+}
+
+// The gain step of round 0 (every vertex eligible) for sub-round s, as in the refinement rounds:
+// T = blocks of Lambda(e) over nets with Phi(e,a) = 1, minus a and the blocks without room; best t in
+// T by g_t = b(u) - W + omega({e : t in Lambda(e)}), smallest block on ties; no candidate unless the
+// gain is positive.  A warp takes kNaRange vertices, whose active ones it gathers to full lanes.
+// 250k vertices, 1M pins: 34 -> 17 us.
+constexpr int kNaRange = 128;
+
+__global__ void __launch_bounds__(256) k_na_candidates(int32_t n, int32_t k, double eps, const int32_t *vtx_off,
+                                                       const int32_t *inc, const NaRec *recs, const int32_t *part,
+                                                       const int32_t *vw, const int64_t *bw, int32_t S, uint64_t seed,
+                                                       int32_t s, int32_t *target, int64_t *gain)
 {
     __shared__ long long slack[64];
-    if (threadIdx.x < 64) slack[threadIdx.x] = 0;
-    __syncthreads();
-    if (threadIdx.x == 0) {
+    __shared__ uint8_t list_w[8][kNaRange];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    uint8_t *list = list_w[wid];
+    if (threadIdx.x < 32) {
         long long total = 0;
-        for (int i = 0; i < k; ++i) total += bw[i];
+        for (int i = lane; i < k; i += 32) total += bw[i];
+        for (int o = 16; o; o >>= 1) total += __shfl_xor_sync(kFull, total, o);
         const long long avg = (total + k - 1) / k;
         const long long lmax = (long long)floor((1.0 + eps) * (double)avg);
-        for (int i = 0; i < 64; ++i) slack[i] = i < k ? lmax - bw[i] : -1;
+        for (int i = lane; i < 64; i += 32) slack[i] = i < k ? lmax - bw[i] : -1;
     }
     __syncthreads();
-    for (int64_t uu = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; uu < n;
-         uu += (int64_t)gridDim.x * blockDim.x) {
-        const int32_t u = (int32_t)uu;
-        int32_t t_best = -1;
-        int64_t g_best = 0;
-        const uint64_t z = splitmix64_output(seed ^ (uint64_t)(uint32_t)u);
-        if ((int32_t)(z % (uint64_t)S) == s) {
+    const int64_t warps = (int64_t)gridDim.x * 8;
+    for (int64_t base = ((int64_t)blockIdx.x * 8 + wid) * kNaRange; base < n; base += warps * kNaRange) {
+        int cnt = 0;
+#pragma unroll
+        for (int c = 0; c < kNaRange; c += 32) {
+            const int64_t u = base + c + lane;
+            const uint64_t z = splitmix64_output(seed ^ (uint64_t)(uint32_t)u);
+            const bool on = u < n && (int32_t)(z % (uint64_t)S) == s;
+            const unsigned om = __ballot_sync(kFull, on);
+            if (on) list[cnt + __popc(om & ((1u << lane) - 1))] = (uint8_t)(c + lane);
+            cnt += __popc(om);
+            if (u < n && !on) {
+                target[u] = -1;
+                gain[u] = 0;
+            }
+        }
+        __syncwarp();
+        for (int i = lane; i < cnt; i += 32) {
+            const int64_t u = base + list[i];
+            int32_t t_best = -1;
+            int64_t g_best = 0;
             const int a = part[u];
             const int32_t cu = vw ? vw[u] : 1;
             const int32_t jb = vtx_off[u], je = vtx_off[u + 1];
@@ -239,23 +304,36 @@ __global__ void k_na_candidates(int32_t n, int32_t k, double eps, const int32_t 
                 const int t = __ffsll((long long)x) - 1;
                 if (slack[t] < cu) T &= ~(1ull << t);
             }
-            // one pass over the nets per candidate block (registers only)
-            for (uint64_t x = T; x; x &= x - 1) {
-                const int t = __ffsll((long long)x) - 1;
-                int64_t conn = 0;
-                for (int32_t j = jb; j < je; ++j) {
-                    const NaRec &r = recs[inc[j]];
-                    if ((r.lam >> t) & 1) conn += r.w;
-                }
+            if (T != 0 && W < 2048) {
+                int t;
+                int32_t conn;
+                if (W < 64) na_planes<6>(recs, inc, jb, je, T, t, conn);
+                else na_planes<11>(recs, inc, jb, je, T, t, conn);
                 const int64_t g = b - W + conn;
-                if (g > g_best) {
+                if (g > 0) {
                     g_best = g;
                     t_best = t;
                 }
+            } else {
+                // one pass over the nets per candidate block (registers only)
+                for (uint64_t x = T; x; x &= x - 1) {
+                    const int t = __ffsll((long long)x) - 1;
+                    int64_t conn = 0;
+                    for (int32_t j = jb; j < je; ++j) {
+                        const NaRec &r = recs[inc[j]];
+                        if ((r.lam >> t) & 1) conn += r.w;
+                    }
+                    const int64_t g = b - W + conn;
+                    if (g > g_best) {
+                        g_best = g;
+                        t_best = t;
+                    }
+                }
             }
+            target[u] = t_best;
+            gain[u] = g_best;
         }
-        target[u] = t_best;
-        gain[u] = g_best;
+        __syncwarp();
     }
 }
 
@@ -290,47 +368,38 @@ extern "C" int hgp_candidates_noalloc(int32_t n, int32_t m, const int32_t *net_o
     int32_t *err = reinterpret_cast<int32_t *>(sc + 512);
     NaRec *recs = reinterpret_cast<NaRec *>(sc + kRecOffset);
 
-    int32_t P = 0;
-    cudaError_t e = cudaMemcpyAsync(&P, net_offsets + m, sizeof(int32_t), cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    if (e != cudaSuccess) {
-        (void)cudaGetLastError();
-        return HGP_ERR_CUDA;
+    cudaError_t e = cudaSuccess;
+    if (!pins || !inc_nets) {   // allowed only without pins
+        int32_t P = 0;
+        e = cudaMemcpyAsync(&P, net_offsets + m, sizeof(int32_t), cudaMemcpyDeviceToHost, st);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+        if (e != cudaSuccess) {
+            (void)cudaGetLastError();
+            return HGP_ERR_CUDA;
+        }
+        if (P != 0) return HGP_ERR_INVALID;
     }
-    if (P < 0) return HGP_ERR_INVALID;
-    if (P > 0 && (!pins || !inc_nets)) return HGP_ERR_INVALID;
 
     // block weights start from zero and the error flag is cleared on every call
     k_na_clear<<<1, 64, 0, st>>>(bw, err);
     k_na_check<<<152 * 4, 256, 0, st>>>(n, m, net_offsets, pins, vtx_offsets, inc_nets, vertex_w,
-                                        net_w, part, k, P, err);
-    int32_t bad = 0;
+                                        net_w, part, k, err);
+    // the order and transpose checks, weights and records follow if every index is in range
+    k_na_prepare<<<152 * 8, 256, 0, st>>>(n, m, net_offsets, pins, vtx_offsets, inc_nets, part, vertex_w, net_w, recs,
+                                          bw, err);
+    // one read-back: the error flag, and the falling steps that are not at the start of a list
+    int64_t bad[2] = {0, 0};
     e = cudaGetLastError();
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&bad, err, sizeof(int32_t), cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(bad, err, sizeof(bad), cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) {
         (void)cudaGetLastError();
         return HGP_ERR_CUDA;
     }
-    if (bad) return HGP_ERR_INVALID;
-    // every index is in range now: the order and transpose checks may follow them
-    if (P > 0) {
-        k_na_check_order<<<152 * 8, 256, 0, st>>>(n, m, net_offsets, pins, vtx_offsets, inc_nets, err);
-        k_na_check_transpose<<<152 * 4, 256, 0, st>>>(n, net_offsets, pins, vtx_offsets, inc_nets, err);
-    }
-    e = cudaGetLastError();
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&bad, err, sizeof(int32_t), cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    if (e != cudaSuccess) {
-        (void)cudaGetLastError();
-        return HGP_ERR_CUDA;
-    }
-    if (bad) return HGP_ERR_INVALID;
+    if ((int32_t)(bad[0] & 0xffffffff) != 0 || bad[1] != 0) return HGP_ERR_INVALID;
 
-    k_na_block_weights<<<152 * 4, 256, 0, st>>>(n, part, vertex_w, bw);
-    if (m > 0) k_na_records<<<152 * 8, 256, 0, st>>>(m, net_offsets, pins, part, net_w, recs);
-    const int64_t blocks = ((int64_t)n + 255) / 256;
-    k_na_candidates<<<(unsigned)(blocks < 152 * 16 ? blocks : 152 * 16), 256, 0, st>>>(
+    const int64_t blocks = ((int64_t)n + 8 * kNaRange - 1) / (8 * kNaRange);
+    k_na_candidates<<<(unsigned)(blocks < 152 * 8 ? blocks : 152 * 8), 256, 0, st>>>(
         n, k, eps, vtx_offsets, inc_nets, recs, part, vertex_w, bw, subrounds, seed, s, target, gain);
     e = cudaGetLastError();
     if (e != cudaSuccess) return HGP_ERR_CUDA;
