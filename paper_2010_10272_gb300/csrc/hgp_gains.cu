@@ -14,6 +14,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <algorithm>
+
 #include "hgp_host.cuh"
 
 using namespace hgp;
@@ -21,24 +23,27 @@ using namespace hgp;
 namespace {
 
 constexpr unsigned long long kEmpty = ~0ull;
+constexpr unsigned kFull = 0xffffffffu;
 
-struct Slot {
+// order statistics of one (net, block), one 32-byte sector; all bytes 0xFF when free, so a memset
+// clears the table
+struct __align__(32) Slot {
     unsigned long long key;   // e * 64 + i, kEmpty when free
     int32_t max_out;          // largest index of a move out of block i with a pin of e, -1 if none
-    int32_t min_in;           // smallest index of a move into block i, INT32_MAX if none
-    int32_t n_out;            // |out(e, i)|
-    int32_t pad;
+    uint32_t min_in;          // smallest index of a move into block i, 0xFFFFFFFF if none
+    int32_t n_out;            // |out(e, i)| - 1
+    int32_t pad[3];
 };
 
 __device__ __forceinline__ uint64_t slot_hash(uint64_t key) { return splitmix64_output(key); }
 
-// find or insert (linear probing; the table is at most half full, so a free slot exists)
-__device__ __forceinline__ Slot *find_slot(Slot *table, uint64_t mask, unsigned long long key, bool insert)
+// find or insert (linear probing; the table is at most two thirds full, so a free slot exists).
+// cur: the key at the first position, already loaded.
+__device__ __forceinline__ Slot *find_slot(Slot *table, uint64_t mask, uint64_t p, unsigned long long cur,
+                                           unsigned long long key, bool insert)
 {
-    uint64_t p = slot_hash(key) & mask;
     for (uint64_t probe = 0; probe <= mask; ++probe) {
         Slot *s = table + p;
-        unsigned long long cur = s->key;
         if (cur == key) return s;
         if (cur == kEmpty) {
             if (!insert) return nullptr;
@@ -46,81 +51,145 @@ __device__ __forceinline__ Slot *find_slot(Slot *table, uint64_t mask, unsigned 
             if (cur == kEmpty || cur == key) return s;
         }
         p = (p + 1) & mask;
+        cur = __ldcg(&table[p].key);
     }
     return nullptr;
 }
 
-__global__ void k_eg_init(Slot *table, uint64_t size)
+// the slots of (e, a) and (e, b); the first probes of both are in flight together
+__device__ __forceinline__ void find_both(Slot *table, uint64_t mask, unsigned long long e, int a, int b, bool insert,
+                                          Slot *&sa, Slot *&sb)
 {
-    for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < size;
-         i += (uint64_t)gridDim.x * blockDim.x) {
-        Slot s;
-        s.key = kEmpty;
-        s.max_out = -1;
-        s.min_in = 0x7fffffff;
-        s.n_out = 0;
-        s.pad = 0;
-        table[i] = s;
-    }
+    const unsigned long long ka = e * 64 + a, kb = e * 64 + b;
+    const uint64_t pa = slot_hash(ka) & mask, pb = slot_hash(kb) & mask;
+    const unsigned long long ca = __ldcg(&table[pa].key), cb = __ldcg(&table[pb].key);
+    sa = find_slot(table, mask, pa, ca, ka, insert);
+    sb = find_slot(table, mask, pb, cb, kb, insert);
 }
 
-// validation: vertex in range, moved once, from = Pi(u), to in range and different
-__global__ void k_eg_check(Dev d, const int32_t *moves, int32_t count, int32_t *seen, int32_t *err)
+// validation: vertex in range, moved once, from = Pi(u), to in range and different; and the sum of
+// the degrees of the moved vertices (each contributes 2 keys per incident net).  out: error, sum
+__global__ void k_eg_check(Dev d, const int32_t *moves, int32_t count, int32_t *seen, unsigned long long *out)
 {
+    unsigned long long s = 0;
     for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < count;
          j += (int64_t)gridDim.x * blockDim.x) {
         const int32_t u = moves[3 * j], a = moves[3 * j + 1], b = moves[3 * j + 2];
         bool bad = u < 0 || u >= d.n || b < 0 || b >= d.k || a == b;
-        if (!bad) bad = d.part[u] != a || atomicExch(&seen[u], 1) != 0;
-        if (bad) atomicOr(err, 1);
+        if (!bad) {
+            bad = d.part[u] != a || atomicExch(&seen[u], 1) != 0;
+            s += (unsigned long long)(d.vtx_off[u + 1] - d.vtx_off[u]);
+        }
+        if (bad) atomicOr(&out[0], 1ull);
     }
+    for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(kFull, s, o);
+    if ((threadIdx.x & 31) == 0 && s) atomicAdd(&out[1], s);
 }
 
-// warp per move: record out / in order statistics of every (net, block) the move touches
-__global__ void k_eg_pass1(Dev d, const int32_t *moves, int32_t count, Slot *table, uint64_t mask, int32_t *err)
+// `per` (at most 32) moves of a warp, about 32 incidences in all, one run that the lanes walk
+// flattened (a warp per move left most lanes idle, 6 nets of 32; 32 moves per warp were as slow, too
+// few warps for the chains of dependent accesses).  100k moves of 6 nets each, the whole call: 295 ->
+// 253 us, of which the host copies and waits are about 110.
+struct MoveWarp {
+    int32_t off[33];
+    int32_t jb[32];
+    int32_t a[32], b[32];
+    unsigned long long g[32];
+    __device__ __forceinline__ int32_t load(const Dev &d, const int32_t *moves, int64_t j0, int32_t count, int per)
+    {
+        const int lane = threadIdx.x & 31;
+        const int64_t j = j0 + lane;
+        int32_t deg = 0, first = 0, ma = 0, mb = 0;
+        if (j < count && lane < per) {
+            const int32_t u = moves[3 * j];
+            ma = moves[3 * j + 1];
+            mb = moves[3 * j + 2];
+            first = d.vtx_off[u];
+            deg = d.vtx_off[u + 1] - first;
+        }
+        int32_t incl = deg;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int32_t y = __shfl_up_sync(kFull, incl, o);
+            if (lane >= o) incl += y;
+        }
+        __syncwarp();
+        off[lane] = incl - deg;
+        jb[lane] = first;
+        a[lane] = ma;
+        b[lane] = mb;
+        g[lane] = 0;
+        if (lane == 31) off[32] = incl;
+        __syncwarp();
+        return off[32];
+    }
+    __device__ __forceinline__ int slot(int32_t i) const
+    {
+        int v = 0;
+#pragma unroll
+        for (int st = 16; st; st >>= 1)
+            if (off[v + st] <= i) v += st;
+        return v;
+    }
+};
+
+// order statistics of every (net, block) the moves touch
+__global__ void __launch_bounds__(256) k_eg_pass1(Dev d, const int32_t *moves, int32_t count, int per, Slot *table,
+                                                  uint64_t mask, unsigned long long *out)
 {
+    __shared__ MoveWarp mw[8];
+    MoveWarp &w = mw[threadIdx.x >> 5];
     const int lane = threadIdx.x & 31;
-    const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
-    for (int64_t j = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; j < count; j += warps) {
-        const int32_t u = moves[3 * j], a = moves[3 * j + 1], b = moves[3 * j + 2];
-        for (int32_t x = d.vtx_off[u] + lane; x < d.vtx_off[u + 1]; x += 32) {
-            const unsigned long long e = (unsigned long long)(d.inc[x] & kNetMask);
-            Slot *sa = find_slot(table, mask, e * 64 + a, true);
-            Slot *sb = find_slot(table, mask, e * 64 + b, true);
+    const int64_t warps = (int64_t)gridDim.x * 8;
+    for (int64_t j0 = ((int64_t)blockIdx.x * 8 + (threadIdx.x >> 5)) * per; j0 < count; j0 += warps * per) {
+        const int32_t total = w.load(d, moves, j0, count, per);
+        for (int32_t i = lane; i < total; i += 32) {
+            const int v = w.slot(i);
+            const int32_t j = (int32_t)j0 + v;
+            const unsigned long long e = (unsigned long long)(d.inc[w.jb[v] + (i - w.off[v])] & kNetMask);
+            Slot *sa, *sb;
+            find_both(table, mask, e, w.a[v], w.b[v], true, sa, sb);
             if (!sa || !sb) {
-                atomicOr(err, 2);
+                atomicOr(&out[0], 2ull);
                 continue;
             }
-            atomicMax(&sa->max_out, (int32_t)j);
+            atomicMax(&sa->max_out, j);
             atomicAdd(&sa->n_out, 1);
-            atomicMin(&sb->min_in, (int32_t)j);
+            atomicMin(&sb->min_in, (uint32_t)j);
         }
     }
 }
 
-// warp per move: exact gain from Lemma 1
-__global__ void k_eg_pass2(Dev d, const int32_t *moves, int32_t count, Slot *table, uint64_t mask, int64_t *gains)
+// exact gain of every move from Lemma 1; Phi is only read where the order statistics leave it to decide
+__global__ void __launch_bounds__(256) k_eg_pass2(Dev d, const int32_t *moves, int32_t count, int per, Slot *table,
+                                                  uint64_t mask, int64_t *gains)
 {
+    __shared__ MoveWarp mw[8];
+    MoveWarp &w = mw[threadIdx.x >> 5];
     const int lane = threadIdx.x & 31;
-    const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
+    const int64_t warps = (int64_t)gridDim.x * 8;
     const Rec16 *r16 = reinterpret_cast<const Rec16 *>(d.rec);
     const Rec32 *r32 = reinterpret_cast<const Rec32 *>(d.rec);
-    for (int64_t j = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; j < count; j += warps) {
-        const int32_t u = moves[3 * j], a = moves[3 * j + 1], b = moves[3 * j + 2];
-        long long g = 0;
-        for (int32_t x = d.vtx_off[u] + lane; x < d.vtx_off[u + 1]; x += 32) {
-            const int32_t eraw = d.inc[x];
+    for (int64_t j0 = ((int64_t)blockIdx.x * 8 + (threadIdx.x >> 5)) * per; j0 < count; j0 += warps * per) {
+        const int32_t total = w.load(d, moves, j0, count, per);
+        for (int32_t i = lane; i < total; i += 32) {
+            const int v = w.slot(i);
+            const int32_t j = (int32_t)j0 + v, a = w.a[v], b = w.b[v];
+            const int32_t eraw = d.inc[w.jb[v] + (i - w.off[v])];
             const int32_t e = eraw & kNetMask;
             const bool wide = eraw < 0;
             const int32_t wrow = wide ? d.widx[e] : 0;
-            const int32_t w = (d.k <= 32 ? r16[e].w : r32[e].w) & 0x7fffffff;
-            const Slot *sa = find_slot(table, mask, (unsigned long long)e * 64 + a, false);
-            const Slot *sb = find_slot(table, mask, (unsigned long long)e * 64 + b, false);
-            if (sa && sa->n_out == phi_get(d, e, a, wide, wrow) && sa->max_out == j && sa->min_in > j) g += w;
-            if (sb && sb->n_out == phi_get(d, e, b, wide, wrow) && sb->min_in == j && sb->max_out < j) g -= w;
+            const int32_t we = (d.k <= 32 ? r16[e].w : r32[e].w) & 0x7fffffff;
+            Slot *sa, *sb;
+            find_both(table, mask, (unsigned long long)e, a, b, false, sa, sb);
+            long long g = 0;
+            if (sa && sa->max_out == j && sa->min_in > (uint32_t)j && sa->n_out + 1 == phi_get(d, e, a, wide, wrow)) g += we;
+            if (sb && sb->min_in == (uint32_t)j && sb->max_out < j && sb->n_out + 1 == phi_get(d, e, b, wide, wrow)) g -= we;
+            if (g) atomicAdd(&w.g[v], (unsigned long long)g);
         }
-        for (int o = 16; o; o >>= 1) g += __shfl_xor_sync(0xffffffffu, g, o);
-        if (lane == 0) gains[j] = g;
+        __syncwarp();
+        if (lane < per && j0 + lane < count) gains[j0 + lane] = (int64_t)w.g[lane];
+        __syncwarp();
     }
 }
 
@@ -134,19 +203,6 @@ int grid_of(int64_t work, int threads)
 
 }  // namespace
 
-// sum of the degrees of the moved vertices (each contributes 2 keys per incident net)
-__global__ void k_eg_degsum(Dev d, const int32_t *moves, int32_t count, unsigned long long *out)
-{
-    unsigned long long s = 0;
-    for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < count;
-         j += (int64_t)gridDim.x * blockDim.x) {
-        const int32_t u = moves[3 * j];
-        if (u >= 0 && u < d.n) s += (unsigned long long)(d.vtx_off[u + 1] - d.vtx_off[u]);
-    }
-    for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if ((threadIdx.x & 31) == 0 && s) atomicAdd(out, s);
-}
-
 extern "C" int hgp_exact_gains(hgp_handle *h, int32_t count, const int32_t *moves, int64_t *gains)
 {
     if (!h || count < 0 || (count > 0 && (!moves || !gains))) return HGP_ERR_INVALID;
@@ -154,49 +210,45 @@ extern "C" int hgp_exact_gains(hgp_handle *h, int32_t count, const int32_t *move
     if (count == 0) return HGP_OK;
     Dev &d = h->d;
     cudaStream_t st = h->stream;
-    int32_t *mv = nullptr, *seen = nullptr, *err = nullptr;
-    unsigned long long *degsum = nullptr;
+    int32_t *mv = nullptr, *seen = nullptr;
+    unsigned long long *out = nullptr;   // error, degree sum
     Slot *table = nullptr;
     int64_t *g_d = nullptr;
-    int32_t herr = 0;
-    unsigned long long hdeg = 0;
+    unsigned long long host[2] = {0, 0};
     int rc = HGP_OK;
     cudaError_t e = dev_alloc(reinterpret_cast<void **>(&mv), sizeof(int32_t) * 3 * (size_t)count, st);
     if (e == cudaSuccess) e = cudaMemcpyAsync(mv, moves, sizeof(int32_t) * 3 * (size_t)count, cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess) e = dev_alloc(reinterpret_cast<void **>(&seen), sizeof(int32_t) * ((size_t)d.n + 1), st);
-    if (e == cudaSuccess) e = dev_alloc(reinterpret_cast<void **>(&err), sizeof(int32_t), st);
-    if (e == cudaSuccess) e = dev_alloc(reinterpret_cast<void **>(&degsum), sizeof(unsigned long long), st);
+    if (e == cudaSuccess) e = dev_alloc(reinterpret_cast<void **>(&out), sizeof(host), st);
     if (e == cudaSuccess) e = cudaMemsetAsync(seen, 0, sizeof(int32_t) * ((size_t)d.n + 1), st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(err, 0, sizeof(int32_t), st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(degsum, 0, sizeof(unsigned long long), st);
+    if (e == cudaSuccess) e = cudaMemsetAsync(out, 0, sizeof(host), st);
     if (e == cudaSuccess) {
-        k_eg_check<<<grid_of(count, 256), 256, 0, st>>>(d, mv, count, seen, err);
-        k_eg_degsum<<<grid_of(count, 256), 256, 0, st>>>(d, mv, count, degsum);
+        k_eg_check<<<grid_of(count, 256), 256, 0, st>>>(d, mv, count, seen, out);
+        h->launches += 1;
+        e = cudaGetLastError();
+    }
+    if (e == cudaSuccess) e = cudaMemcpyAsync(host, out, sizeof(host), cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = stream_wait(st);
+    if (e == cudaSuccess && host[0]) rc = HGP_ERR_INVALID;
+    // at most 2 keys per incident net of a moved vertex; the table is at most two thirds full
+    uint64_t size = 64;
+    while (size < 3 * (uint64_t)host[1]) size <<= 1;
+    if (e == cudaSuccess && rc == HGP_OK) e = dev_alloc(reinterpret_cast<void **>(&table), sizeof(Slot) * size, st);
+    if (e == cudaSuccess && rc == HGP_OK) e = dev_alloc(reinterpret_cast<void **>(&g_d), sizeof(int64_t) * (size_t)count, st);
+    if (e == cudaSuccess && rc == HGP_OK) e = cudaMemsetAsync(table, 0xFF, sizeof(Slot) * size, st);
+    if (e == cudaSuccess && rc == HGP_OK) {
+        const int per = (int)std::min<uint64_t>(32, std::max<uint64_t>(1, 32 * (uint64_t)count / std::max<uint64_t>(1, host[1])));
+        const int grid = grid_of(((int64_t)count + per - 1) / per * 32, 256);
+        k_eg_pass1<<<grid, 256, 0, st>>>(d, mv, count, per, table, size - 1, out);
+        k_eg_pass2<<<grid, 256, 0, st>>>(d, mv, count, per, table, size - 1, g_d);
         h->launches += 2;
         e = cudaGetLastError();
     }
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&herr, err, sizeof(int32_t), cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&hdeg, degsum, sizeof(hdeg), cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess) e = stream_wait(st);
-    if (e == cudaSuccess && herr) rc = HGP_ERR_INVALID;
-    // at most 2 keys per incident net of a moved vertex; keep the table at most half full
-    uint64_t size = 64;
-    while (size < 4 * (uint64_t)hdeg) size <<= 1;
-    if (e == cudaSuccess && rc == HGP_OK) e = dev_alloc(reinterpret_cast<void **>(&table), sizeof(Slot) * size, st);
-    if (e == cudaSuccess && rc == HGP_OK) e = dev_alloc(reinterpret_cast<void **>(&g_d), sizeof(int64_t) * (size_t)count, st);
-    if (e == cudaSuccess && rc == HGP_OK) {
-        k_eg_init<<<grid_of((int64_t)size, 256), 256, 0, st>>>(table, size);
-        k_eg_pass1<<<grid_of((int64_t)count * 32, 256), 256, 0, st>>>(d, mv, count, table, size - 1, err);
-        k_eg_pass2<<<grid_of((int64_t)count * 32, 256), 256, 0, st>>>(d, mv, count, table, size - 1, g_d);
-        h->launches += 3;
-        e = cudaGetLastError();
-    }
-    if (e == cudaSuccess && rc == HGP_OK) e = cudaMemcpyAsync(&herr, err, sizeof(int32_t), cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess && rc == HGP_OK) e = cudaMemcpyAsync(host, out, sizeof(host), cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess && rc == HGP_OK) e = cudaMemcpyAsync(gains, g_d, sizeof(int64_t) * (size_t)count, cudaMemcpyDeviceToHost, st);
     if (mv) pool_free(mv, st);
     if (seen) pool_free(seen, st);
-    if (err) pool_free(err, st);
-    if (degsum) pool_free(degsum, st);
+    if (out) pool_free(out, st);
     if (table) pool_free(table, st);
     if (g_d) pool_free(g_d, st);
     const cudaError_t e2 = stream_wait(st);
@@ -205,6 +257,6 @@ extern "C" int hgp_exact_gains(hgp_handle *h, int32_t count, const int32_t *move
         (void)cudaGetLastError();
         return status_of(e);
     }
-    if (rc == HGP_OK && herr) rc = HGP_ERR_INTERNAL;
+    if (rc == HGP_OK && host[0]) rc = HGP_ERR_INTERNAL;
     return rc;
 }
