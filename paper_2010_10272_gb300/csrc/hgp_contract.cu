@@ -3,10 +3,11 @@
 //   1. used cluster ids flagged and remapped to 0..n'-1 by an exclusive prefix sum;
 //   2. coarse vertex weights by atomic adds (checked to fit int32);
 //   3. every net's pins mapped to coarse ids, sorted and de-duplicated by size class: a thread
-//      per net of at most 8 pins (sorting network in registers), a warp per net of 9..32 (bitonic
-//      across the lanes), a CTA per net of 33..2048 (bitonic in shared memory), and for larger
-//      nets 2048-pin chunks sorted by separate CTAs and merged pairwise by merge-path tiles
-//      spread over the whole grid; the net's fingerprint is taken during the de-duplication;
+//      per net of at most 8 pins (sorting network in registers), a warp per net of 9..512 (bitonic
+//      in registers, up to 16 values per lane), a CTA per net of up to 2048 (four such runs, merged
+//      in shared memory), and for larger nets 2048-pin chunks sorted by separate CTAs and merged
+//      pairwise by merge-path tiles spread over the whole grid; the net's fingerprint is taken
+//      during the de-duplication;
 //   4. nets with fewer than two pins dropped; identical nets found through a 64-bit
 //      fingerprint table (key -> smallest net id) and an exact comparison with that net; a
 //      net that only shares the fingerprint stays unresolved and takes part in the next round
@@ -18,7 +19,9 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <algorithm>
 #include <new>
+#include <utility>
 
 #include "hgp_host.cuh"
 
@@ -39,8 +42,7 @@ struct hgp_coarse {
 namespace {
 
 constexpr unsigned kFull = 0xffffffffu;
-constexpr int kScanTile = 1024;
-constexpr int kSortThreads = 256;
+constexpr int kScanTile = 4096;
 constexpr unsigned long long kKeyEmpty = ~0ull;
 constexpr int32_t kUnresolved = -2, kDropped = -1;
 
@@ -53,14 +55,27 @@ int grid_of(int64_t work, int threads)
 }
 
 // ---------------------------------------------------------------- device-wide exclusive scan
-// out[0..len] = exclusive prefix sums of in[0..len-1] (out[len] = total)
+// out[0..len] = exclusive prefix sums of in[0..len-1] (out[len] = total).  Reduce, then scan: a tile's
+// sum first, so that the 8-byte output is written once (scanning the tiles and adding the offsets
+// afterwards wrote and read it twice more; 10M entries 68 -> 35 us).
+constexpr int kScanPer = 4;   // entries per thread
+
 template <typename T>
-__global__ void __launch_bounds__(kScanTile) k_scan_tile(const T *in, int64_t len, int64_t *out, int64_t *sums)
+__device__ __forceinline__ int64_t scan_load(const T *in, int64_t len, int64_t i0, int64_t (&v)[kScanPer])
 {
-    __shared__ int64_t wt[32];
-    const int64_t i = blockIdx.x * (int64_t)kScanTile + threadIdx.x;
+    int64_t sum = 0;
+#pragma unroll
+    for (int q = 0; q < kScanPer; ++q) {
+        v[q] = i0 + q < len ? (int64_t)in[i0 + q] : 0;
+        sum += v[q];
+    }
+    return sum;
+}
+
+// exclusive prefix of v over the CTA (kScanTile / kScanPer threads); total in *total
+__device__ __forceinline__ int64_t scan_cta(int64_t v, int64_t *wt, int64_t *total)
+{
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const int64_t v = i < len ? (int64_t)in[i] : 0;
     int64_t x = v;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
@@ -70,7 +85,7 @@ __global__ void __launch_bounds__(kScanTile) k_scan_tile(const T *in, int64_t le
     if (lane == 31) wt[wid] = x;
     __syncthreads();
     if (wid == 0) {
-        const int64_t t = wt[lane];
+        const int64_t t = lane < kScanTile / kScanPer / 32 ? wt[lane] : 0;
         int64_t s = t;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
@@ -78,16 +93,35 @@ __global__ void __launch_bounds__(kScanTile) k_scan_tile(const T *in, int64_t le
             if (lane >= o) s += y;
         }
         wt[lane] = s - t;
-        if (lane == 31) sums[blockIdx.x] = s;
+        if (lane == 31) *total = s;
     }
     __syncthreads();
-    if (i <= len) out[i] = wt[wid] + x - v;
+    return wt[wid] + x - v;
 }
 
-__global__ void k_scan_add(int64_t *out, int64_t len, const int64_t *block_prefix)
+template <typename T>
+__global__ void __launch_bounds__(kScanTile / kScanPer) k_scan_tile(const T *in, int64_t len, int64_t *sums)
 {
-    const int64_t i = blockIdx.x * (int64_t)kScanTile + threadIdx.x;
-    if (i <= len) out[i] += block_prefix[blockIdx.x];
+    __shared__ int64_t wt[32], total;
+    int64_t v[kScanPer];
+    const int64_t s = scan_load(in, len, blockIdx.x * (int64_t)kScanTile + threadIdx.x * kScanPer, v);
+    scan_cta(s, wt, &total);
+    if (threadIdx.x == 0) sums[blockIdx.x] = total;
+}
+
+template <typename T>
+__global__ void __launch_bounds__(kScanTile / kScanPer) k_scan_out(const T *in, int64_t len, const int64_t *prefix,
+                                                                   int64_t *out)
+{
+    __shared__ int64_t wt[32], total;
+    int64_t v[kScanPer];
+    const int64_t i0 = blockIdx.x * (int64_t)kScanTile + threadIdx.x * kScanPer;
+    int64_t run = scan_cta(scan_load(in, len, i0, v), wt, &total) + (prefix ? prefix[blockIdx.x] : 0);
+#pragma unroll
+    for (int q = 0; q < kScanPer; ++q) {
+        if (i0 + q <= len) out[i0 + q] = run;
+        run += v[q];
+    }
 }
 
 // exclusive scan with the total at out[len]; out has len + 1 entries
@@ -95,19 +129,21 @@ template <typename T>
 cudaError_t scan_excl(const T *in, int64_t len, int64_t *out, cudaStream_t st)
 {
     const int64_t tiles = len / kScanTile + 1;   // covers indices 0..len
-    int64_t *sums = nullptr, *pref = nullptr;
-    cudaError_t e = dev_alloc(reinterpret_cast<void **>(&sums), sizeof(int64_t) * (size_t)tiles, st);
+    constexpr int threads = kScanTile / kScanPer;
+    if (tiles == 1) {
+        k_scan_out<T><<<1, threads, 0, st>>>(in, len, nullptr, out);
+        return cudaGetLastError();
+    }
+    int64_t *sums = nullptr;
+    cudaError_t e = dev_alloc(reinterpret_cast<void **>(&sums), sizeof(int64_t) * (size_t)(2 * tiles + 1), st);
     if (e != cudaSuccess) return e;
-    k_scan_tile<T><<<(unsigned)tiles, kScanTile, 0, st>>>(in, len, out, sums);
+    int64_t *pref = sums + tiles;
+    k_scan_tile<T><<<(unsigned)tiles, threads, 0, st>>>(in, len, sums);
     e = cudaGetLastError();
-    if (e == cudaSuccess && tiles > 1) {
-        e = dev_alloc(reinterpret_cast<void **>(&pref), sizeof(int64_t) * (size_t)(tiles + 1), st);
-        if (e == cudaSuccess) e = scan_excl<int64_t>(sums, tiles, pref, st);
-        if (e == cudaSuccess) {
-            k_scan_add<<<(unsigned)tiles, kScanTile, 0, st>>>(out, len, pref);
-            e = cudaGetLastError();
-        }
-        if (pref) pool_free(pref, st);
+    if (e == cudaSuccess) e = scan_excl<int64_t>(sums, tiles, pref, st);
+    if (e == cudaSuccess) {
+        k_scan_out<T><<<(unsigned)tiles, threads, 0, st>>>(in, len, pref, out);
+        e = cudaGetLastError();
     }
     pool_free(sums, st);
     return e;
@@ -124,8 +160,15 @@ __global__ void k_ct_check(const int64_t *off, const int32_t *pins, const int32_
         if (off[e] < 0 || off[e] > off[e + 1] || off[e + 1] > P || (e == 0 && off[0] != 0)) atomicOr(err, ERR_INVALID);
         if (nw && nw[e] < 1) atomicOr(err, ERR_INVALID);
     }
-    for (int64_t j = t; j < P; j += stride)
-        if (pins[j] < 0 || pins[j] >= n) atomicOr(err, ERR_INVALID);
+    bool bad = false;
+    for (int64_t j0 = t; j0 < P; j0 += 8 * stride) {   // eight pins per thread in flight
+        int32_t v[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) v[q] = j0 + q * stride < P ? __ldcs(&pins[j0 + q * stride]) : 0;
+#pragma unroll
+        for (int q = 0; q < 8; ++q) bad = bad || v[q] < 0 || v[q] >= n;
+    }
+    if (bad) atomicOr(err, ERR_INVALID);
     if (vw)
         for (int64_t u = t; u < n; u += stride)
             if (vw[u] < 1) atomicOr(err, ERR_INVALID);
@@ -187,13 +230,12 @@ __device__ __forceinline__ void net_done(int64_t e, int32_t kept, unsigned long 
     }
 }
 
-constexpr int kTiny = 8, kMid = 256, kMedium = 2048;
+constexpr int kTiny = 8, kMid = 512, kMedium = 2048;
 constexpr int kClasses = 4;   // listed classes: 9..32, 33..kMid, kMid+1..kMedium, larger
 
 // thread per net: nets of at most kTiny pins are sorted in registers (an unrolled sorting
-// network), de-duplicated and fingerprinted; larger nets go to the lists of the warp-register
-// (9..32 pins), warp shared-memory (..kMid), CTA shared-memory (..kMedium) and chunked (larger)
-// kernels
+// network), de-duplicated and fingerprinted; larger nets go to the lists of the warp (9..32 pins,
+// ..kMid), CTA (..kMedium) and chunked (larger) kernels
 __global__ void k_ct_tiny(const int64_t *off, const int32_t *pins, int32_t m, const int32_t *map, int32_t *a,
                           int32_t *size1, unsigned long long *key, int32_t *rep, int32_t *lists, int32_t *counts)
 {
@@ -245,88 +287,179 @@ __global__ void k_ct_tiny(const int64_t *off, const int32_t *pins, int32_t m, co
     }
 }
 
-// warp per listed net of 9..32 pins: bitonic sort across the lanes, de-duplication, fingerprint
-__global__ void k_ct_small(const int64_t *off, const int32_t *pins, const int32_t *map, const int32_t *list,
-                           const int32_t *count, int32_t *a, int32_t *size1, unsigned long long *key, int32_t *rep)
+// Bitonic sort of 32 K values, K per lane in registers: ascending in the order lane * K + i.  Pairs
+// closer than K are in the lane, the others come by shuffle; no shared memory and no barriers
+// (sorting in shared memory, two accesses and a barrier per step, took 346 us for the nets of
+// 33..256 pins and 584 us for those of 257..2048 of a 10M-net power-law instance; 280 us for 33..512
+// and 138 for 513..2048 now).
+template <int K>
+__device__ __forceinline__ void warp_sort(int32_t (&v)[K])
 {
     const int lane = threadIdx.x & 31;
-    const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
-    const int32_t cnt = *count;
-    for (int64_t i = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; i < cnt; i += warps) {
-        const int64_t e = list[i];
-        const int64_t b = off[e];
-        const int32_t s = (int32_t)(off[e + 1] - b);
-        int32_t v = lane < s ? map[pins[b + lane]] : 0x7fffffff;
 #pragma unroll
-        for (int k = 2; k <= 32; k <<= 1) {
+    for (int k = 2; k <= 32 * K; k <<= 1) {
 #pragma unroll
-            for (int j = k >> 1; j > 0; j >>= 1) {
-                const int32_t o = __shfl_xor_sync(kFull, v, j);
-                const bool up = (lane & k) == 0;            // ascending run of the merge
-                const bool low = (lane & j) == 0;           // lower partner of the pair
-                v = (low == up) ? min(v, o) : max(v, o);
+        for (int j = k >> 1; j > 0; j >>= 1) {
+            if (j >= K) {
+                const int dl = j / K;
+                const bool keep_min = ((lane & dl) == 0) == (((lane * K) & k) == 0);
+#pragma unroll
+                for (int i = 0; i < K; ++i) {
+                    const int32_t o = __shfl_xor_sync(kFull, v[i], dl);
+                    v[i] = keep_min ? min(v[i], o) : max(v[i], o);
+                }
+            } else {
+#pragma unroll
+                for (int i = 0; i < K; ++i) {
+                    if (i & j) continue;
+                    const bool up = ((lane * K + i) & k) == 0;
+                    const int32_t x = v[i], y = v[i | j];
+                    v[i] = up ? min(x, y) : max(x, y);
+                    v[i | j] = up ? max(x, y) : min(x, y);
+                }
             }
         }
-        const int32_t prev = __shfl_up_sync(kFull, v, 1);
-        const bool keep = lane < s && (lane == 0 || v != prev);
-        const unsigned km = __ballot_sync(kFull, keep);
-        if (keep) a[b + __popc(km & ((1u << lane) - 1))] = v;
-        unsigned long long h = keep ? pin_mix(v) : 0ull;
-        for (int o = 16; o; o >>= 1) h += __shfl_xor_sync(kFull, h, o);
-        if (lane == 0) net_done(e, __popc(km), h, size1, key, rep);
     }
 }
 
-// warp per listed net of 33..kMid pins: bitonic sort in the warp's shared buffer (padded to a
-// power of two), then an order-preserving compaction 32 values at a time, and the fingerprint
+// mapped pins first .. of a run of s, 32 K of them into the lanes' registers (any order; absent ones sort
+// last: coarse ids are below 2^31 - 1)
+template <int K>
+__device__ __forceinline__ void load_mapped(const int32_t *pins, const int32_t *map, int32_t first, int32_t s,
+                                            int32_t (&v)[K])
+{
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int i = 0; i < K; ++i) v[i] = first + i * 32 + lane < s ? __ldcs(&pins[first + i * 32 + lane]) : -1;
+#pragma unroll
+    for (int i = 0; i < K; ++i) v[i] = v[i] >= 0 ? map[v[i]] : 0x7fffffff;
+}
+
+// one net of at most 32 K pins by a warp
+template <int K>
+__device__ __forceinline__ void warp_net(int64_t e, int64_t b, int32_t s, const int32_t *pins, const int32_t *map,
+                                         int32_t *a, int32_t *size1, unsigned long long *key, int32_t *rep)
+{
+    const int lane = threadIdx.x & 31;
+    int32_t v[K];
+    load_mapped<K>(pins + b, map, 0, s, v);
+    warp_sort<K>(v);
+    int32_t prev = __shfl_up_sync(kFull, v[K - 1], 1);
+    if (lane == 0) prev = -1;
+    uint32_t keep = 0;
+#pragma unroll
+    for (int i = 0; i < K; ++i) {
+        if (v[i] != prev && lane * K + i < s) keep |= 1u << i;
+        prev = v[i];
+    }
+    int32_t incl = __popc(keep);
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int32_t y = __shfl_up_sync(kFull, incl, o);
+        if (lane >= o) incl += y;
+    }
+    int32_t *out = a + b + (incl - __popc(keep));
+    unsigned long long h = 0;
+#pragma unroll
+    for (int i = 0; i < K; ++i) {
+        if ((keep >> i) & 1) {
+            *out++ = v[i];
+            h += pin_mix(v[i]);
+        }
+    }
+    for (int o = 16; o; o >>= 1) h += __shfl_xor_sync(kFull, h, o);
+    if (lane == 31) net_done(e, incl, h, size1, key, rep);
+}
+
+// warp per listed net of 9..32 pins
+__global__ void __launch_bounds__(256) k_ct_small(const int64_t *off, const int32_t *pins, const int32_t *map,
+                                                  const int32_t *list, const int32_t *count, int32_t *a,
+                                                  int32_t *size1, unsigned long long *key, int32_t *rep)
+{
+    const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
+    const int32_t cnt = *count;
+    for (int64_t i = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; i < cnt; i += warps) {
+        const int64_t e = list[i], b = off[e];
+        warp_net<1>(e, b, (int32_t)(off[e + 1] - b), pins, map, a, size1, key, rep);
+    }
+}
+
+// warp per listed net of 33..kMid pins
 __global__ void __launch_bounds__(256) k_ct_mid(const int64_t *off, const int32_t *pins, const int32_t *map,
                                                 const int32_t *list, const int32_t *count, int32_t *a,
                                                 int32_t *size1, unsigned long long *key, int32_t *rep)
 {
-    __shared__ int32_t buf_w[8][kMid];
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    int32_t *buf = buf_w[wid];
     const int64_t warps = (int64_t)gridDim.x * 8;
     const int32_t cnt = *count;
-    for (int64_t i = (int64_t)blockIdx.x * 8 + wid; i < cnt; i += warps) {
-        const int64_t e = list[i];
-        const int64_t b = off[e];
+    for (int64_t i = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5); i < cnt; i += warps) {
+        const int64_t e = list[i], b = off[e];
         const int32_t s = (int32_t)(off[e + 1] - b);
-        int32_t np2 = 64;
-        while (np2 < s) np2 <<= 1;
-        for (int32_t j = lane; j < np2; j += 32) buf[j] = j < s ? map[pins[b + j]] : 0x7fffffff;
-        __syncwarp();
-        for (int32_t k = 2; k <= np2; k <<= 1) {
-            for (int32_t jj = k >> 1; jj > 0; jj >>= 1) {
-                for (int32_t x = lane; x < np2; x += 32) {
-                    const int32_t y = x ^ jj;
-                    if (y > x) {
-                        const bool up = (x & k) == 0;
-                        const int32_t vx = buf[x], vy = buf[y];
-                        if ((vx > vy) == up) { buf[x] = vy; buf[y] = vx; }
-                    }
-                }
-                __syncwarp();
-            }
-        }
-        int32_t kept = 0;
-        unsigned long long h = 0;
-        for (int32_t c = 0; c < s; c += 32) {
-            const int32_t j = c + lane;
-            const bool has = j < s;
-            const int32_t v = has ? buf[j] : 0;
-            const bool keep = has && (j == 0 || v != buf[j - 1]);
-            const unsigned km = __ballot_sync(kFull, keep);
-            if (keep) {
-                a[b + kept + __popc(km & ((1u << lane) - 1))] = v;
-                h += pin_mix(v);
-            }
-            kept += __popc(km);
-        }
-        for (int o = 16; o; o >>= 1) h += __shfl_xor_sync(kFull, h, o);
-        if (lane == 0) net_done(e, kept, h, size1, key, rep);
-        __syncwarp();
+        if (s <= 64) warp_net<2>(e, b, s, pins, map, a, size1, key, rep);
+        else if (s <= 128) warp_net<4>(e, b, s, pins, map, a, size1, key, rep);
+        else if (s <= 256) warp_net<8>(e, b, s, pins, map, a, size1, key, rep);
+        else warp_net<16>(e, b, s, pins, map, a, size1, key, rep);
     }
+}
+
+// merge path: number of elements taken from A among the first d outputs of merge(A, B)
+__device__ __forceinline__ int32_t merge_split(const int32_t *A, int32_t na, const int32_t *B, int32_t nb, int32_t d)
+{
+    int32_t lo = max(0, d - nb), hi = min(d, na);
+    while (lo < hi) {
+        const int32_t i = (lo + hi) >> 1;          // candidate count from A
+        if (A[i] <= B[d - 1 - i]) lo = i + 1;     // A[i] comes before B[d-1-i]: take more from A
+        else hi = i;
+    }
+    return lo;
+}
+
+// A CTA of kCtaSort threads sorts up to kMedium mapped pins: a run of 512 per warp in registers, then two
+// rounds of merges in shared memory, each thread 16 outputs of one merge.  Returns the buffer
+// (x or y, kMedium values each) that holds the result.
+constexpr int kCtaSort = 128;
+constexpr int kRun = kMedium / (kCtaSort / 32);   // 512
+constexpr int kOut = kMedium / kCtaSort;          // 16
+
+__device__ __forceinline__ int32_t *cta_sort(const int32_t *pins, const int32_t *map, int32_t s, int32_t *x, int32_t *y)
+{
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    {
+        int32_t v[kOut];
+        load_mapped<kOut>(pins, map, wid * kRun, s, v);
+        warp_sort<kOut>(v);
+        int4 *dst = reinterpret_cast<int4 *>(x + wid * kRun + lane * kOut);
+#pragma unroll
+        for (int i = 0; i < kOut / 4; ++i) dst[i] = make_int4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
+    }
+    __syncthreads();
+#pragma unroll
+    for (int w = kRun; w < kMedium; w *= 2) {
+        const int o0 = tid * kOut, base = o0 / (2 * w) * (2 * w);
+        const int32_t *A = x + base, *B = A + w;
+        int i = merge_split(A, w, B, w, o0 - base), j = o0 - base - i;
+        int32_t out[kOut];
+        int32_t va = i < w ? A[i] : 0x7fffffff, vb = j < w ? B[j] : 0x7fffffff;
+#pragma unroll
+        for (int q = 0; q < kOut; ++q) {
+            const bool take_a = j >= w || (i < w && va <= vb);
+            out[q] = take_a ? va : vb;
+            if (take_a) {
+                ++i;
+                va = i < w ? A[i] : 0x7fffffff;
+            } else {
+                ++j;
+                vb = j < w ? B[j] : 0x7fffffff;
+            }
+        }
+        int4 *dst = reinterpret_cast<int4 *>(y + o0);
+#pragma unroll
+        for (int q = 0; q < kOut / 4; ++q) dst[q] = make_int4(out[4 * q], out[4 * q + 1], out[4 * q + 2], out[4 * q + 3]);
+        __syncthreads();
+        int32_t *t = x;
+        x = y;
+        y = t;
+    }
+    return x;
 }
 
 // block-wide: order-preserving compaction of the first of every run of equal values of the
@@ -365,52 +498,34 @@ __device__ __forceinline__ void compact_runs(const int32_t *src, int32_t *dst, i
     h_out = *hsum;
 }
 
-// CTA per listed net of kMid+1..kMedium pins: bitonic sort of the mapped pins in shared memory
-// (padded to a power of two), then compaction into a and the fingerprint
-__global__ void __launch_bounds__(kSortThreads) k_ct_medium(const int64_t *off, const int32_t *pins,
-                                                            const int32_t *map, const int32_t *list,
-                                                            const int32_t *count, int32_t *a, int32_t *size1,
-                                                            unsigned long long *key, int32_t *rep)
+// CTA per listed net of kMid+1..kMedium pins: sort, then compaction into a and the fingerprint
+__global__ void __launch_bounds__(kCtaSort) k_ct_medium(const int64_t *off, const int32_t *pins, const int32_t *map,
+                                                        const int32_t *list, const int32_t *count, int32_t *a,
+                                                        int32_t *size1, unsigned long long *key, int32_t *rep)
 {
-    __shared__ int32_t buf[kMedium];
-    __shared__ int32_t wtot[kSortThreads / 32];
+    __shared__ __align__(16) int32_t x[kMedium], y[kMedium];
+    __shared__ int32_t wtot[kCtaSort / 32];
     __shared__ unsigned long long hsum;
-    const int tid = threadIdx.x;
     const int32_t cnt = *count;
     for (int64_t i = blockIdx.x; i < cnt; i += gridDim.x) {
-        const int64_t e = list[i];
-        const int64_t b = off[e];
+        const int64_t e = list[i], b = off[e];
         const int32_t s = (int32_t)(off[e + 1] - b);
-        int32_t np2 = 2 * kMid;
-        while (np2 < s) np2 <<= 1;
-        for (int32_t j = tid; j < np2; j += kSortThreads) buf[j] = j < s ? map[pins[b + j]] : 0x7fffffff;
-        __syncthreads();
-        for (int32_t k = 2; k <= np2; k <<= 1) {
-            for (int32_t j = k >> 1; j > 0; j >>= 1) {
-                for (int32_t x = tid; x < np2; x += kSortThreads) {
-                    const int32_t y = x ^ j;
-                    if (y > x) {
-                        const bool up = (x & k) == 0;
-                        const int32_t vx = buf[x], vy = buf[y];
-                        if ((vx > vy) == up) { buf[x] = vy; buf[y] = vx; }
-                    }
-                }
-                __syncthreads();
-            }
-        }
+        const int32_t *sorted = cta_sort(pins + b, map, s, x, y);
         int32_t kept;
         unsigned long long h;
-        compact_runs(buf, a + b, s, wtot, &hsum, kept, h);
-        if (tid == 0) net_done(e, kept, h, size1, key, rep);
+        compact_runs(sorted, a + b, s, wtot, &hsum, kept, h);
+        if (threadIdx.x == 0) net_done(e, kept, h, size1, key, rep);
         __syncthreads();
     }
 }
 
-// Nets of more than kMedium pins, load-balanced over the grid: every kMedium-pin chunk of every
-// such net is sorted by one CTA in shared memory (k_lg_chunk), then runs are merged pairwise,
-// each CTA producing kMedium outputs of one merge found by a merge-path search (k_lg_merge), and
-// finally one CTA per net de-duplicates and fingerprints it (k_lg_dedupe).
-constexpr int kLgThreads = 1024;
+// Nets of more than kMedium pins, load-balanced over the grid by tasks of kMedium pins: every chunk
+// is sorted by one CTA (k_lg_chunk), then runs are merged pairwise, each CTA producing kMedium
+// outputs of one merge found by a merge-path search (k_lg_merge); the distinct values of every chunk
+// are counted and fingerprinted (k_lg_distinct), their places follow from a prefix sum, and each
+// chunk is written there (k_lg_compact).  (One CTA per net for the last step took as long as the
+// largest net: 543 us for nets of up to 100,000 pins.)
+constexpr int kLgThreads = 256;
 
 // chunk task t -> (list index, chunk) through the exclusive prefix of the chunk counts
 __device__ __forceinline__ int32_t find_task(const int64_t *cpre, int32_t nl, int64_t t)
@@ -436,21 +551,24 @@ __global__ void k_lg_count(const int64_t *off, const int32_t *list, const int32_
     }
 }
 
-// CTA per large net: a representative's pins, offset and summed weight at its coarse position
+// task t: a representative's pins of the chunk to its coarse position (and with the first chunk its
+// offset and summed weight)
 __global__ void __launch_bounds__(kLgThreads) k_lg_emit(const int64_t *off, const int32_t *a, const int32_t *size1,
                                                         const int32_t *rep, const int64_t *nid, const int64_t *poff,
                                                         const unsigned long long *w64, const int32_t *list,
-                                                        const int32_t *count, int32_t *pins2, int64_t *off2,
-                                                        int32_t *nw2, int32_t *err)
+                                                        const int32_t *count, const int64_t *cpre, int64_t tasks,
+                                                        int32_t *pins2, int64_t *off2, int32_t *nw2, int32_t *err)
 {
     const int32_t nl = *count;
-    for (int64_t i = blockIdx.x; i < nl; i += gridDim.x) {
-        const int64_t e = list[i];
+    for (int64_t t = blockIdx.x; t < tasks; t += gridDim.x) {
+        const int32_t li = find_task(cpre, nl, t);
+        const int64_t e = list[li];
         if (rep[e] != (int32_t)e) continue;
         const int64_t src = off[e], dst = poff[e];
-        const int32_t s = size1[e];
-        for (int32_t j = threadIdx.x; j < s; j += kLgThreads) pins2[dst + j] = a[src + j];
-        if (threadIdx.x == 0) {
+        const int32_t c0 = (int32_t)(t - cpre[li]) * kMedium, c1 = min(size1[e], c0 + kMedium);
+#pragma unroll 4
+        for (int32_t j = c0 + threadIdx.x; j < c1; j += kLgThreads) pins2[dst + j] = a[src + j];
+        if (c0 == 0 && threadIdx.x == 0) {
             off2[nid[e]] = dst;
             const unsigned long long w = w64[e];
             if (w >= (1ull << 31)) atomicOr(err, ERR_UNSUPPORTED);
@@ -459,151 +577,189 @@ __global__ void __launch_bounds__(kLgThreads) k_lg_emit(const int64_t *off, cons
     }
 }
 
-__global__ void __launch_bounds__(kLgThreads) k_lg_chunk(const int64_t *off, const int32_t *pins, const int32_t *map,
-                                                         const int32_t *list, const int32_t *count,
-                                                         const int64_t *cpre, int64_t tasks, int32_t *a)
+__global__ void __launch_bounds__(kCtaSort) k_lg_chunk(const int64_t *off, const int32_t *pins, const int32_t *map,
+                                                       const int32_t *list, const int32_t *count, const int64_t *cpre,
+                                                       int64_t tasks, int32_t *dst)
 {
-    __shared__ int32_t buf[kMedium];
-    const int tid = threadIdx.x;
+    __shared__ __align__(16) int32_t x[kMedium], y[kMedium];
     const int32_t nl = *count;
     for (int64_t t = blockIdx.x; t < tasks; t += gridDim.x) {
         const int32_t li = find_task(cpre, nl, t);
-        const int64_t e = list[li];
-        const int64_t b = off[e];
+        const int64_t e = list[li], b = off[e];
         const int32_t s = (int32_t)(off[e + 1] - b);
         const int32_t c0 = (int32_t)(t - cpre[li]) * kMedium;
         const int32_t len = min(kMedium, s - c0);
-        for (int32_t j = tid; j < kMedium; j += kLgThreads) buf[j] = j < len ? map[pins[b + c0 + j]] : 0x7fffffff;
-        __syncthreads();
-        for (int32_t k = 2; k <= kMedium; k <<= 1) {
-            for (int32_t j = k >> 1; j > 0; j >>= 1) {
-                for (int32_t x = tid; x < kMedium; x += kLgThreads) {
-                    const int32_t y = x ^ j;
-                    if (y > x) {
-                        const bool up = (x & k) == 0;
-                        const int32_t vx = buf[x], vy = buf[y];
-                        if ((vx > vy) == up) { buf[x] = vy; buf[y] = vx; }
-                    }
-                }
-                __syncthreads();
-            }
-        }
-        for (int32_t j = tid; j < len; j += kLgThreads) a[b + c0 + j] = buf[j];
+        const int32_t *sorted = cta_sort(pins + b + c0, map, len, x, y);
+        for (int32_t j = threadIdx.x; j < len; j += kCtaSort) dst[b + c0 + j] = sorted[j];
         __syncthreads();
     }
-}
-
-// merge path: number of elements taken from A among the first d outputs of merge(A, B)
-__device__ __forceinline__ int32_t merge_split(const int32_t *A, int32_t na, const int32_t *B, int32_t nb, int32_t d)
-{
-    int32_t lo = max(0, d - nb), hi = min(d, na);
-    while (lo < hi) {
-        const int32_t i = (lo + hi) >> 1;          // candidate count from A
-        if (A[i] <= B[d - 1 - i]) lo = i + 1;     // A[i] comes before B[d-1-i]: take more from A
-        else hi = i;
-    }
-    return lo;
 }
 
 // one merge pass over all large nets: runs of width w (sorted) of src are merged pairwise into
-// dst; task t = output tile of kMedium elements of one net (same task numbering as the chunks)
+// dst; task t = output tile of kMedium elements of one net (same task numbering as the chunks).
+// The tile's two input pieces are staged in shared memory.
 __global__ void __launch_bounds__(kLgThreads) k_lg_merge(const int64_t *off, const int32_t *list, const int32_t *count,
                                                          const int64_t *cpre, int64_t tasks, const int32_t *src,
                                                          int32_t *dst, int32_t w)
 {
+    __shared__ int32_t in[kMedium], out[kMedium];
+    __shared__ int32_t split[2];
     const int tid = threadIdx.x;
     const int32_t nl = *count;
     constexpr int kPer = kMedium / kLgThreads;
     for (int64_t t = blockIdx.x; t < tasks; t += gridDim.x) {
         const int32_t li = find_task(cpre, nl, t);
-        const int64_t e = list[li];
-        const int64_t b = off[e];
+        const int64_t e = list[li], b = off[e];
         const int32_t s = (int32_t)(off[e + 1] - b);
-        const int32_t o0 = (int32_t)(t - cpre[li]) * kMedium + tid * kPer;   // this thread's outputs
-        if (o0 >= s) continue;
-        const int32_t base = (o0 / (2 * w)) * (2 * w);
+        const int32_t o0 = (int32_t)(t - cpre[li]) * kMedium;   // the tile's outputs [o0, o0 + len)
+        const int32_t len = min(kMedium, s - o0);
+        const int32_t base = (o0 / (2 * w)) * (2 * w);           // w is a multiple of kMedium: one merge per tile
         const int32_t na = min(w, s - base), nb = max(0, min(w, s - base - w));
         const int32_t *A = src + b + base, *B = A + na;
-        int32_t i = merge_split(A, na, B, nb, o0 - base);
-        int32_t j = o0 - base - i;
-        int32_t *out = dst + b + o0;
-        const int32_t cnt = min(kPer, s - o0);
-        for (int q = 0; q < cnt; ++q) {
-            const bool takeA = j >= nb || (i < na && A[i] <= B[j]);
-            out[q] = takeA ? A[i++] : B[j++];
+        if (tid < 2) split[tid] = merge_split(A, na, B, nb, o0 - base + (tid ? len : 0));
+        __syncthreads();
+        const int32_t a0 = split[0], b0 = o0 - base - a0;
+        const int32_t la = split[1] - a0, lb = len - la;
+        for (int32_t j = tid; j < len; j += kLgThreads) in[j] = j < la ? A[a0 + j] : B[b0 + (j - la)];
+        __syncthreads();
+        const int32_t d0 = tid * kPer;
+        if (d0 < len) {
+            const int32_t *SA = in, *SB = in + la;
+            int32_t i = merge_split(SA, la, SB, lb, d0), j = d0 - i;
+            const int32_t n_out = min(kPer, len - d0);
+            for (int q = 0; q < n_out; ++q) {
+                const bool take_a = j >= lb || (i < la && SA[i] <= SB[j]);
+                out[d0 + q] = take_a ? SA[i++] : SB[j++];
+            }
         }
-    }
-}
-
-// CTA per large net: compaction of the first of every run into a, and the fingerprint
-__global__ void __launch_bounds__(kLgThreads) k_lg_dedupe(const int64_t *off, const int32_t *list, const int32_t *count,
-                                                          const int32_t *src, int32_t *a, int32_t *size1,
-                                                          unsigned long long *key, int32_t *rep)
-{
-    __shared__ int32_t wtot[kLgThreads / 32];
-    __shared__ unsigned long long hsum;
-    const int32_t nl = *count;
-    for (int64_t i = blockIdx.x; i < nl; i += gridDim.x) {
-        const int64_t e = list[i];
-        const int64_t b = off[e];
-        const int32_t s = (int32_t)(off[e + 1] - b);
-        int32_t kept;
-        unsigned long long h;
-        compact_runs(src + b, a + b, s, wtot, &hsum, kept, h);
-        if (threadIdx.x == 0) net_done(e, kept, h, size1, key, rep);
+        __syncthreads();
+        for (int32_t j = tid; j < len; j += kLgThreads) dst[b + o0 + j] = out[j];
         __syncthreads();
     }
 }
 
-// ---------------------------------------------------------------- identical nets
-struct KeySlot {
-    unsigned long long key;
-    int32_t min_id;
-    int32_t pad;
-};
-
-__global__ void k_ct_table_clear(KeySlot *tab, int64_t size)
+// task t: number of values of its chunk that differ from the one before, and their fingerprint sum
+__global__ void __launch_bounds__(kLgThreads) k_lg_distinct(const int64_t *off, const int32_t *list, const int32_t *count,
+                                                            const int64_t *cpre, int64_t tasks, const int32_t *src,
+                                                            int32_t *distinct, unsigned long long *hsum)
 {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < size; i += (int64_t)gridDim.x * blockDim.x) {
-        tab[i].key = kKeyEmpty;
-        tab[i].min_id = 0x7fffffff;
+    const int tid = threadIdx.x;
+    const int32_t nl = *count;
+    for (int64_t t = blockIdx.x; t < tasks; t += gridDim.x) {
+        const int32_t li = find_task(cpre, nl, t);
+        const int64_t e = list[li], b = off[e];
+        const int32_t s = (int32_t)(off[e + 1] - b);
+        const int32_t c0 = (int32_t)(t - cpre[li]) * kMedium, c1 = min(s, c0 + kMedium);
+        int32_t kept = 0;
+        unsigned long long h = 0;
+        for (int32_t j = c0 + tid; j < c1; j += kLgThreads) {
+            const int32_t v = src[b + j];
+            if (j == 0 || v != src[b + j - 1]) {
+                ++kept;
+                h += pin_mix(v);
+            }
+        }
+        kept = __reduce_add_sync(kFull, kept);
+        for (int o = 16; o; o >>= 1) h += __shfl_xor_sync(kFull, h, o);
+        if ((tid & 31) == 0 && kept) {
+            atomicAdd(&distinct[t], kept);
+            atomicAdd(&hsum[li], h);
+        }
     }
 }
 
-__device__ __forceinline__ KeySlot *key_find(KeySlot *tab, uint64_t mask, unsigned long long key, bool insert)
+// task t: its distinct values to their places (pre: exclusive prefix of the tasks' counts)
+__global__ void __launch_bounds__(kLgThreads) k_lg_compact(const int64_t *off, const int32_t *list, const int32_t *count,
+                                                           const int64_t *cpre, int64_t tasks, const int32_t *src,
+                                                           const int64_t *pre, int32_t *a)
 {
-    uint64_t p = splitmix64_output(key) & mask;
-    for (uint64_t probe = 0; probe <= mask; ++probe) {
-        KeySlot *sl = tab + p;
-        unsigned long long cur = __ldcg(&sl->key);
-        if (cur == key) return sl;
-        if (cur == kKeyEmpty) {
-            if (!insert) return nullptr;
-            cur = atomicCAS(&sl->key, kKeyEmpty, key);
-            if (cur == kKeyEmpty || cur == key) return sl;
+    __shared__ int32_t wtot[kLgThreads / 32];
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const int32_t nl = *count;
+    for (int64_t t = blockIdx.x; t < tasks; t += gridDim.x) {
+        const int32_t li = find_task(cpre, nl, t);
+        const int64_t e = list[li], b = off[e];
+        const int32_t s = (int32_t)(off[e + 1] - b);
+        const int32_t c0 = (int32_t)(t - cpre[li]) * kMedium, c1 = min(s, c0 + kMedium);
+        int64_t at = b + (pre[t] - pre[cpre[li]]);
+        for (int32_t j0 = c0; j0 < c1; j0 += kLgThreads) {
+            const int32_t j = j0 + tid;
+            const int32_t v = j < c1 ? src[b + j] : 0;
+            const bool keep = j < c1 && (j == 0 || v != src[b + j - 1]);
+            const unsigned km = __ballot_sync(kFull, keep);
+            if (lane == 0) wtot[wid] = __popc(km);
+            __syncthreads();
+            int32_t before = 0, all = 0;
+            for (int w = 0; w < kLgThreads / 32; ++w) {
+                if (w < wid) before += wtot[w];
+                all += wtot[w];
+            }
+            if (keep) a[at + before + __popc(km & ((1u << lane) - 1))] = v;
+            at += all;
+            __syncthreads();
         }
-        p = (p + 1) & mask;
     }
-    return nullptr;
+}
+
+// thread per large net: its size and fingerprint
+__global__ void k_lg_done(const int32_t *list, const int32_t *count, const int64_t *cpre, const int64_t *pre,
+                          const unsigned long long *hsum, int32_t *size1, unsigned long long *key, int32_t *rep)
+{
+    const int32_t nl = *count;
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < nl; i += (int64_t)gridDim.x * blockDim.x)
+        net_done(list[i], (int32_t)(pre[cpre[i + 1]] - pre[cpre[i]]), hsum[i], size1, key, rep);
+}
+
+// ---------------------------------------------------------------- identical nets
+// A slot holds a net's upper 32 fingerprint bits and its id, the smallest of the unresolved nets with
+// those bits in their run of probes (which starts at the lower fingerprint bits).  All bytes 0xFF
+// when free.  Nets that only share the bits are told apart by the comparison.
+__device__ __forceinline__ uint64_t slot_value(unsigned long long key, int32_t e)
+{
+    return (key & 0xFFFFFFFF00000000ull) | (uint32_t)e;
 }
 
 // thread per unresolved net: its fingerprint's smallest unresolved net id
-__global__ void k_ct_insert(const unsigned long long *key, const int32_t *rep, int32_t m, KeySlot *tab,
+__global__ void k_ct_insert(const unsigned long long *key, const int32_t *rep, int32_t m, unsigned long long *tab,
                             uint64_t mask, int32_t *err)
 {
     for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < m; e += (int64_t)gridDim.x * blockDim.x) {
         if (rep[e] != kUnresolved) continue;
-        KeySlot *sl = key_find(tab, mask, key[e], true);
-        if (!sl) { atomicOr(err, ERR_INVALID); continue; }
-        atomicMin(&sl->min_id, (int32_t)e);
+        const unsigned long long val = slot_value(key[e], (int32_t)e);
+        uint64_t p = key[e] & mask;
+        bool placed = false;
+        for (uint64_t probe = 0; probe <= mask; ++probe) {
+            unsigned long long cur = __ldcg(&tab[p]);
+            if (cur == kKeyEmpty) cur = atomicCAS(&tab[p], kKeyEmpty, val);
+            if (cur == kKeyEmpty || (cur >> 32) == (val >> 32)) {
+                if (cur != kKeyEmpty && val < cur) atomicMin(&tab[p], val);
+                placed = true;
+                break;
+            }
+            p = (p + 1) & mask;
+        }
+        if (!placed) atomicOr(err, ERR_INVALID);
     }
+}
+
+// the net in the slot of key's fingerprint bits, -1 if there is none
+__device__ __forceinline__ int32_t smallest_net(const unsigned long long *tab, uint64_t mask, unsigned long long key)
+{
+    uint64_t p = key & mask;
+    for (uint64_t probe = 0; probe <= mask; ++probe) {
+        const unsigned long long cur = __ldcg(&tab[p]);
+        if (cur == kKeyEmpty) return -1;
+        if ((cur >> 32) == (key >> 32)) return (int32_t)(uint32_t)cur;
+        p = (p + 1) & mask;
+    }
+    return -1;
 }
 
 // 32 nets per warp, one per lane: an unresolved net whose fingerprint's smallest net is itself
 // is resolved to itself; the others compare their pin lists with that net, the whole warp on
 // one net at a time, and are resolved to it if equal, else stay unresolved for the next round
 __global__ void k_ct_resolve(const int64_t *off, const int32_t *a, const int32_t *size1,
-                             const unsigned long long *key, int32_t *rep, int32_t m, const KeySlot *tab,
+                             const unsigned long long *key, int32_t *rep, int32_t m, const unsigned long long *tab,
                              uint64_t mask, int32_t *left)
 {
     const int lane = threadIdx.x & 31;
@@ -612,8 +768,8 @@ __global__ void k_ct_resolve(const int64_t *off, const int32_t *a, const int32_t
         int32_t r = -1;
         bool todo = false;
         if (e < m && rep[e] == kUnresolved) {
-            const KeySlot *sl = key_find(const_cast<KeySlot *>(tab), mask, key[e], false);
-            r = sl ? sl->min_id : (int32_t)e;
+            r = smallest_net(tab, mask, key[e]);
+            if (r < 0) r = (int32_t)e;
             if (r == (int32_t)e) rep[e] = (int32_t)e;
             else todo = true;
         }
@@ -696,10 +852,20 @@ __global__ void k_ct_emit(const int64_t *off, const int32_t *a, const int32_t *s
         if (lane == 31) off33[32] = incl;
         __syncwarp();
         const int32_t total = off33[32];
-        for (int32_t i = lane; i < total; i += 32) {
-            const int v = slot_in(off33, i);
-            const int32_t k = i - off33[v];
-            pins2[dst_w[wid][v] + k] = a[src_w[wid][v] + k];
+        for (int32_t i0 = lane; i0 < total; i0 += 128) {   // four pins per lane in flight
+            int32_t x[4];
+            int64_t at[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const int32_t i = i0 + 32 * q;
+                const int v = slot_in(off33, i < total ? i : 0);
+                const int32_t k = i - off33[v];
+                at[q] = dst_w[wid][v] + k;
+                x[q] = i < total ? __ldcs(&a[src_w[wid][v] + k]) : 0;
+            }
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                if (i0 + 32 * q < total) pins2[at[q]] = x[q];
         }
         __syncwarp();
     }
@@ -711,14 +877,11 @@ __global__ void k_ct_project(const int32_t *map, int32_t n, const int32_t *coars
         fine_part[u] = coarse_part[map[u]];
 }
 
+// the arrays go back to the library's pool (behind the work queued on the stream)
 void coarse_free(hgp_coarse *c)
 {
     if (!c) return;
-    if (c->net_off) cudaFree(c->net_off);
-    if (c->pins) cudaFree(c->pins);
-    if (c->vw) cudaFree(c->vw);
-    if (c->nw) cudaFree(c->nw);
-    if (c->map) cudaFree(c->map);
+    for (void *p : {(void *)c->net_off, (void *)c->pins, (void *)c->vw, (void *)c->nw, (void *)c->map}) dev_free(p, c->stream);
     delete c;
 }
 
@@ -747,12 +910,13 @@ extern "C" int hgp_contract(int32_t n, int32_t m, const int64_t *net_off, const 
     int rc = HGP_OK;
     int32_t *err = nullptr, *used = nullptr, *a = nullptr, *b = nullptr, *size1 = nullptr, *rep = nullptr;
     int32_t *is_rep = nullptr, *rep_size = nullptr, *left = nullptr, *lists = nullptr, *counts = nullptr;
-    void *lg_scratch[2] = {nullptr, nullptr};
+    void *lg_scratch[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};
     int32_t n_large = 0;
+    int64_t lg_tasks = 0;
     int sms = 1;
     int64_t *cid = nullptr, *nid = nullptr, *poff = nullptr;
     unsigned long long *w64 = nullptr, *key = nullptr, *nw64 = nullptr;
-    KeySlot *tab = nullptr;
+    unsigned long long *tab = nullptr;
     int64_t P = 0, n2 = 0, m2 = 0, P2 = 0;
     int32_t herr = 0;
     const int64_t mm = m > 0 ? m : 1;
@@ -763,7 +927,7 @@ extern "C" int hgp_contract(int32_t n, int32_t m, const int64_t *net_off, const 
     CT(dev_alloc(reinterpret_cast<void **>(&err), sizeof(int32_t) * 2, st));
     CT(cudaMemsetAsync(err, 0, sizeof(int32_t) * 2, st));
     left = err + 1;
-    k_ct_check<<<grid_of(P > n ? P : n, 256), 256, 0, st>>>(net_off, pins, vertex_w, net_w, n, m, P, err);
+    k_ct_check<<<152 * 16, 256, 0, st>>>(net_off, pins, vertex_w, net_w, n, m, P, err);
     CT(cudaGetLastError());
     CT(cudaMemcpyAsync(&herr, err, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
     CT(stream_wait(st));
@@ -781,8 +945,8 @@ extern "C" int hgp_contract(int32_t n, int32_t m, const int64_t *net_off, const 
     if (herr) { rc = HGP_ERR_INVALID; goto done; }
     c->n = (int32_t)n2;
     // (2) map and cluster weights
-    CT(cudaMalloc(reinterpret_cast<void **>(&c->map), sizeof(int32_t) * (size_t)n));
-    CT(cudaMalloc(reinterpret_cast<void **>(&c->vw), sizeof(int32_t) * (size_t)n2));
+    CT(dev_alloc(reinterpret_cast<void **>(&c->map), sizeof(int32_t) * (size_t)n, st));
+    CT(dev_alloc(reinterpret_cast<void **>(&c->vw), sizeof(int32_t) * (size_t)n2, st));
     CT(dev_alloc(reinterpret_cast<void **>(&w64), sizeof(unsigned long long) * (size_t)(n > mm ? n : mm), st));
     CT(cudaMemsetAsync(w64, 0, sizeof(unsigned long long) * (size_t)n2, st));
     k_ct_map<<<grid_of(n, 256), 256, 0, st>>>(cluster, n, cid, vertex_w, c->map, w64);
@@ -802,7 +966,7 @@ extern "C" int hgp_contract(int32_t n, int32_t m, const int64_t *net_off, const 
         k_ct_tiny<<<grid_of(m, 256), 256, 0, st>>>(net_off, pins, m, c->map, a, size1, key, rep, lists, counts);
         k_ct_small<<<sms * 8, 256, 0, st>>>(net_off, pins, c->map, lists, counts, a, size1, key, rep);
         k_ct_mid<<<sms * 8, 256, 0, st>>>(net_off, pins, c->map, lists + mm, counts + 1, a, size1, key, rep);
-        k_ct_medium<<<sms * 8, kSortThreads, 0, st>>>(net_off, pins, c->map, lists + 2 * mm, counts + 2, a, size1, key, rep);
+        k_ct_medium<<<sms * 12, kCtaSort, 0, st>>>(net_off, pins, c->map, lists + 2 * mm, counts + 2, a, size1, key, rep);
         CT(cudaGetLastError());
         // nets of more than kMedium pins: chunk sorts, merge passes, de-duplication
         int32_t hcnt[kClasses] = {0, 0, 0, 0};
@@ -820,33 +984,51 @@ extern "C" int hgp_contract(int32_t n, int32_t m, const int64_t *net_off, const 
             k_lg_count<<<grid_of(n_large, 256), 256, 0, st>>>(net_off, lists + 3 * mm, counts + 3, chunks, counts + kClasses);
             CT(cudaGetLastError());
             CT(scan_excl<int32_t>(chunks, n_large, cpre, st));
-            int64_t tasks = 0;
+            int64_t &tasks = lg_tasks;
             int32_t max_size = 0;
             CT(cudaMemcpyAsync(&tasks, cpre + n_large, sizeof(int64_t), cudaMemcpyDeviceToHost, st));
             CT(cudaMemcpyAsync(&max_size, counts + kClasses, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
             CT(stream_wait(st));
-            const int g = (int)(tasks < (int64_t)sms * 2 ? tasks : (int64_t)sms * 2);
-            k_lg_chunk<<<g, kLgThreads, 0, st>>>(net_off, pins, c->map, lists + 3 * mm, counts + 3, cpre, tasks, a);
-            int32_t *src = a, *dst = b;
+            int32_t *distinct = nullptr;
+            int64_t *pre = nullptr;
+            unsigned long long *hsum = nullptr;
+            CT(dev_alloc(reinterpret_cast<void **>(&distinct), sizeof(int32_t) * (size_t)tasks, st));
+            lg_scratch[2] = distinct;
+            CT(dev_alloc(reinterpret_cast<void **>(&pre), sizeof(int64_t) * ((size_t)tasks + 1), st));
+            lg_scratch[3] = pre;
+            CT(dev_alloc(reinterpret_cast<void **>(&hsum), sizeof(unsigned long long) * (size_t)n_large, st));
+            lg_scratch[4] = hsum;
+            CT(cudaMemsetAsync(distinct, 0, sizeof(int32_t) * (size_t)tasks, st));
+            CT(cudaMemsetAsync(hsum, 0, sizeof(unsigned long long) * (size_t)n_large, st));
+            const int32_t *list = lists + 3 * mm, *cnt = counts + 3;
+            const int g = (int)std::min<int64_t>(tasks, (int64_t)sms * 12);
+            // the sorted runs end up in b, the distinct values go to a
+            int passes = 0;
+            for (int64_t w = kMedium; w < max_size; w *= 2) ++passes;
+            int32_t *src = passes % 2 ? a : b, *dst = passes % 2 ? b : a;
+            k_lg_chunk<<<g, kCtaSort, 0, st>>>(net_off, pins, c->map, list, cnt, cpre, tasks, src);
             for (int64_t w = kMedium; w < max_size; w *= 2) {
-                k_lg_merge<<<g, kLgThreads, 0, st>>>(net_off, lists + 3 * mm, counts + 3, cpre, tasks, src, dst, (int32_t)w);
-                int32_t *t = src; src = dst; dst = t;
+                k_lg_merge<<<g, kLgThreads, 0, st>>>(net_off, list, cnt, cpre, tasks, src, dst, (int32_t)w);
+                std::swap(src, dst);
             }
-            k_lg_dedupe<<<n_large < sms * 2 ? n_large : sms * 2, kLgThreads, 0, st>>>(net_off, lists + 3 * mm, counts + 3,
-                                                                                     src, a, size1, key, rep);
+            k_lg_distinct<<<g, kLgThreads, 0, st>>>(net_off, list, cnt, cpre, tasks, src, distinct, hsum);
+            CT(cudaGetLastError());
+            CT(scan_excl<int32_t>(distinct, tasks, pre, st));
+            k_lg_compact<<<g, kLgThreads, 0, st>>>(net_off, list, cnt, cpre, tasks, src, pre, a);
+            k_lg_done<<<grid_of(n_large, 256), 256, 0, st>>>(list, cnt, cpre, pre, hsum, size1, key, rep);
             CT(cudaGetLastError());
         }
     }
     // (4) identical nets
     if (m > 0) {
-        uint64_t size = 1024;
-        while (size < 2 * (uint64_t)m) size <<= 1;
-        CT(dev_alloc(reinterpret_cast<void **>(&tab), sizeof(KeySlot) * size, st));
+        uint64_t size = 1024;   // at most three quarters full
+        while (3 * size < 4 * (uint64_t)m) size <<= 1;
+        CT(dev_alloc(reinterpret_cast<void **>(&tab), sizeof(unsigned long long) * size, st));
         for (int round = 0;; ++round) {
             if (round >= 4096) { rc = HGP_ERR_INTERNAL; goto done; }
             int32_t hleft = 0;
             CT(cudaMemsetAsync(left, 0, sizeof(int32_t), st));
-            k_ct_table_clear<<<grid_of((int64_t)size, 256), 256, 0, st>>>(tab, (int64_t)size);
+            CT(cudaMemsetAsync(tab, 0xFF, sizeof(unsigned long long) * size, st));
             k_ct_insert<<<grid_of(m, 256), 256, 0, st>>>(key, rep, m, tab, size - 1, err);
             k_ct_resolve<<<grid_of(m, 256), 256, 0, st>>>(net_off, a, size1, key, rep, m, tab, size - 1, left);
             CT(cudaGetLastError());
@@ -873,15 +1055,15 @@ extern "C" int hgp_contract(int32_t n, int32_t m, const int64_t *net_off, const 
     CT(stream_wait(st));
     c->m = (int32_t)m2;
     c->P = P2;
-    CT(cudaMalloc(reinterpret_cast<void **>(&c->net_off), sizeof(int64_t) * ((size_t)m2 + 1)));
-    CT(cudaMalloc(reinterpret_cast<void **>(&c->pins), sizeof(int32_t) * (size_t)(P2 > 0 ? P2 : 1)));
-    CT(cudaMalloc(reinterpret_cast<void **>(&c->nw), sizeof(int32_t) * (size_t)(m2 > 0 ? m2 : 1)));
+    CT(dev_alloc(reinterpret_cast<void **>(&c->net_off), sizeof(int64_t) * ((size_t)m2 + 1), st));
+    CT(dev_alloc(reinterpret_cast<void **>(&c->pins), sizeof(int32_t) * (size_t)(P2 > 0 ? P2 : 1), st));
+    CT(dev_alloc(reinterpret_cast<void **>(&c->nw), sizeof(int32_t) * (size_t)(m2 > 0 ? m2 : 1), st));
     CT(cudaMemcpyAsync(c->net_off + m2, &P2, sizeof(int64_t), cudaMemcpyHostToDevice, st));
     if (m > 0) {
         if (n_large > 0)
-            k_lg_emit<<<n_large < sms * 2 ? n_large : sms * 2, kLgThreads, 0, st>>>(net_off, a, size1, rep, nid, poff, nw64,
-                                                                                   lists + 3 * mm, counts + 3, c->pins,
-                                                                                   c->net_off, c->nw, err);
+            k_lg_emit<<<(unsigned)std::min<int64_t>(lg_tasks, (int64_t)sms * 16), kLgThreads, 0, st>>>(
+                net_off, a, size1, rep, nid, poff, nw64, lists + 3 * mm, counts + 3, (const int64_t *)lg_scratch[1], lg_tasks,
+                c->pins, c->net_off, c->nw, err);
         k_ct_emit<<<grid_of(m, 256), 256, 0, st>>>(net_off, a, size1, rep, nid, poff, nw64, m,
                                                                  c->pins, c->net_off, c->nw, err);
         CT(cudaGetLastError());
@@ -983,6 +1165,8 @@ extern "C" int hgp_coarse_project(const hgp_coarse *c, const int32_t *coarse_par
 
 extern "C" void hgp_coarse_destroy(hgp_coarse *c)
 {
-    if (c) stream_wait(c->stream);
+    if (!c) return;
+    // the arrays may be in use on any stream of the device (cudaFree would wait for them all, too)
+    if (cudaDeviceSynchronize() != cudaSuccess) (void)cudaGetLastError();
     coarse_free(c);
 }
