@@ -320,7 +320,8 @@ __device__ __forceinline__ Lam with_room(Lam T, const GainWarp &g, int32_t cu)
 // in NP bit planes held in registers (bit t of plane p is bit p of conn_t): adding omega(e) to
 // every block of Lambda(e) is a ripple-carry addition on whole bitsets, O(NP) word operations
 // whatever the number of blocks.  W(u) is known from creation, so NP is too (conn_t <= W(u) <
-// 2^NP).  kAhead records are in flight per lane.  Then the block of T with room with the largest
+// 2^NP).  kAhead records are in flight per lane, and the net ids of the next ones (32-byte records, 3
+// ahead on 3 CTAs per SM: 30.2 ms per power-law step, 2 on 4: 31.8, 4 on 3: 32.0, 1 on 4: 34.0).  Then the block of T with room with the largest
 // conn_t (smallest id among equals).  Against incidences spread over the lanes (a binary search
 // and three shared-memory atomics each, (Lambda, omega) kept for a second pass over the nets):
 // row-net 2M, k = 8, records in L2: 93 -> 56 us per launch of 5 M gathers; power-law 50M, k = 64,
@@ -330,24 +331,32 @@ __device__ __forceinline__ void lane_best(const Rec *recs, const int32_t *inc, i
                                           const GainWarp &g, int32_t cu, Lam kall, int32_t eq_value, Nets<Lam> &x,
                                           Lam &T_all, Lam &T, int &t_out, int32_t &conn_out, Lam &eq_out)
 {
-    constexpr int kAhead = sizeof(Lam) == 8 ? 2 : 4;
+    constexpr int kAhead = RB ? 2 : 3;
     Lam c[NP];
 #pragma unroll
     for (int p = 0; p < NP; ++p) c[p] = 0;
+    int32_t e[kAhead];
+#pragma unroll
+    for (int q = 0; q < kAhead; ++q) e[q] = jb + q < je ? (__ldg(&inc[jb + q]) & kNetMask) : -1;
     for (int32_t j = jb; j < je; j += kAhead) {
-        int32_t e[kAhead];
         Lam s1[kAhead], lam[kAhead];
         int32_t w[kAhead], mv[kAhead];
-#pragma unroll
-        for (int q = 0; q < kAhead; ++q) e[q] = j + q < je ? (__ldg(&inc[j + q]) & kNetMask) : -1;
+        bool on[kAhead];
 #pragma unroll
         for (int q = 0; q < kAhead; ++q) {
             s1[q] = 0; lam[q] = 0; w[q] = 0; mv[q] = 0;
-            if (e[q] >= 0) RecIO<Rec>::template load_full<COH>(recs + e[q], s1[q], w[q], mv[q], lam[q]);
+            on[q] = e[q] >= 0;
+            if (on[q]) RecIO<Rec>::template load_full<COH>(recs + e[q], s1[q], w[q], mv[q], lam[q]);
+        }
+        // the next records' net ids, while these are on their way
+#pragma unroll
+        for (int q = 0; q < kAhead; ++q) {
+            const int32_t jn = j + kAhead + q;
+            e[q] = jn < je ? (__ldg(&inc[jn]) & kNetMask) : -1;
         }
 #pragma unroll
         for (int q = 0; q < kAhead; ++q) {
-            if (e[q] < 0) continue;
+            if (!on[q]) continue;
             const int32_t we = UNIT ? 1 : w[q] & 0x7fffffff;
             take_net(x, s1[q], lam[q], we, mv[q], a, r);
             if (UNIT) {
@@ -675,7 +684,7 @@ __device__ __forceinline__ void load_dev(Dev &dst, const Dev *src)
 // ones come from a per-launch device counter, `take` of them at a time (so that a large
 // instance's 10^5 items do not queue at one address), fetched while the items before are worked on.
 template <typename Rec, bool B, bool RB = false>
-__global__ void __launch_bounds__(kThreads, 4) k_gain(const Dev d0, const Dev *devs, const int2 *items,
+__global__ void __launch_bounds__(kThreads, sizeof(Rec) == 16 || RB ? 4 : 3) k_gain(const Dev d0, const Dev *devs, const int2 *items,
                                                       int32_t n_items, int32_t per_tile, int32_t take, int32_t s,
                                                       int32_t rr, RbArgs rb = RbArgs{0, 0, 0})
 {
