@@ -202,14 +202,14 @@ template <> struct RecIO<Rec16> {
     {
         const uint4 *p = reinterpret_cast<const uint4 *>(r);
         const uint4 q = COH ? __ldcg(p) : __ldg(p);
-        s1 = q.x; w = (int32_t)q.y; mv = (int32_t)q.z; lam = q.w;
+        s1 = q.x; lam = q.y; w = (int32_t)q.z; mv = (int32_t)q.w;
     }
     template <bool COH>
     __device__ static void load_b(const Rec16 *r, Lam &lam, int32_t &w)
     {
         const uint4 *p = reinterpret_cast<const uint4 *>(r);
         const uint4 q = COH ? __ldcg(p) : __ldg(p);
-        lam = q.w; w = (int32_t)q.y;
+        lam = q.y; w = (int32_t)q.z;
     }
 };
 
@@ -220,22 +220,23 @@ template <> struct RecIO<Rec32> {
     __device__ static void load_full(const Rec32 *r, Lam &s1, int32_t &w, int32_t &mv, Lam &lam)
     {
         if (COH) {
-            const uint4 q = __ldcg(reinterpret_cast<const uint4 *>(r)), l = __ldcg(reinterpret_cast<const uint4 *>(r) + 1);
-            s1 = (uint64_t)q.x | ((uint64_t)q.y << 32); w = (int32_t)q.z; mv = (int32_t)q.w;
-            lam = (uint64_t)l.x | ((uint64_t)l.y << 32);
+            const uint4 q = __ldcg(reinterpret_cast<const uint4 *>(r));
+            const int2 l = __ldcg(reinterpret_cast<const int2 *>(&r->w));
+            s1 = (uint64_t)q.x | ((uint64_t)q.y << 32); lam = (uint64_t)q.z | ((uint64_t)q.w << 32);
+            w = l.x; mv = l.y;
             return;
         }
         uint64_t wm;
         [[maybe_unused]] uint64_t tail;
-        asm("ld.global.nc.v4.b64 {%0, %1, %2, %3}, [%4];" : "=l"(s1), "=l"(wm), "=l"(lam), "=l"(tail) : "l"(r));
+        asm("ld.global.nc.v4.b64 {%0, %1, %2, %3}, [%4];" : "=l"(s1), "=l"(lam), "=l"(wm), "=l"(tail) : "l"(r));
         w = (int32_t)(uint32_t)wm; mv = (int32_t)(uint32_t)(wm >> 32);
     }
     template <bool COH>
     __device__ static void load_b(const Rec32 *r, Lam &lam, int32_t &w)
     {
-        const uint4 *p = reinterpret_cast<const uint4 *>(&r->lam);
-        const uint4 q = COH ? __ldcg(p) : __ldg(p);
-        lam = (uint64_t)q.x | ((uint64_t)q.y << 32); w = (int32_t)q.z;
+        const unsigned long long *p = reinterpret_cast<const unsigned long long *>(&r->lam);
+        lam = COH ? __ldcg(p) : __ldg(p);
+        w = __ldg(&r->w);
     }
 };
 
@@ -1148,6 +1149,52 @@ struct alignas(16) MoveQueue {
 // result is used, so their latencies overlap.
 constexpr int kPins = 4;
 
+// Lambda and S1 of a tiny net (Dev::tiny) after one pin went a -> t, by compare-and-swap (at most
+// three other movers can come between); whether a left Lambda and whether t entered it.
+__device__ __forceinline__ void tiny_step(uint64_t &s1, uint64_t &lam, int a, int t, int size, bool &left, bool &entered)
+{
+    const int ca = tiny_count<uint64_t>(s1, lam, size, a), ct = tiny_count<uint64_t>(s1, lam, size, t);
+    const uint64_t ba = 1ull << a, bt = 1ull << t;
+    left = ca == 1;
+    entered = ct == 0;
+    lam = (lam & ~(left ? ba : 0ull)) | bt;
+    s1 = (s1 & ~(ba | bt)) | (ca == 2 ? ba : 0ull) | (entered ? bt : 0ull);
+}
+
+__device__ __forceinline__ void tiny_move(Rec16 *rc, int a, int t, int size, bool &left, bool &entered)
+{
+    unsigned long long *p = reinterpret_cast<unsigned long long *>(rc);   // s1 | lam << 32
+    unsigned long long cur = __ldcg(p);
+    while (true) {
+        uint64_t s1 = (uint32_t)cur, lam = cur >> 32;
+        tiny_step(s1, lam, a, t, size, left, entered);
+        const unsigned long long old = atomicCAS(p, cur, s1 | (lam << 32));
+        if (old == cur) return;
+        cur = old;
+    }
+}
+
+__device__ __forceinline__ void tiny_move(Rec32 *rc, int a, int t, int size, bool &left, bool &entered)
+{
+    ulonglong2 cur = __ldcg(reinterpret_cast<const ulonglong2 *>(rc));
+    while (true) {
+        uint64_t s1 = cur.x, lam = cur.y;
+        tiny_step(s1, lam, a, t, size, left, entered);
+        ulonglong2 old;
+        asm volatile(
+            "{\n\t.reg .b128 c, n, o;\n\t"
+            "mov.b128 c, {%2, %3};\n\t"
+            "mov.b128 n, {%4, %5};\n\t"
+            "atom.relaxed.gpu.global.cas.b128 o, [%6], c, n;\n\t"
+            "mov.b128 {%0, %1}, o;\n\t}"
+            : "=l"(old.x), "=l"(old.y)
+            : "l"(cur.x), "l"(cur.y), "l"(s1), "l"(lam), "l"(rc)
+            : "memory");
+        if (old.x == cur.x && old.y == cur.y) return;
+        cur = old;
+    }
+}
+
 // RVC (LP apply with the revert variant on): also counts the movers of every net (d.rv_net)
 // and, in `shared`, the moved incidences on nets with several movers (a second mover adds its
 // own incidence and the first one's, later movers their own).
@@ -1179,8 +1226,10 @@ __device__ __forceinline__ long long apply_pins(const Dev &d, Rec *recs, const A
         Rec *rc = recs + ee;
         mv[q] = STAMP ? __ldcg(&rc->mv) : 0;
         w[q] = __ldg(&rc->w) & 0x7fffffff;
-        oa[q] = phi_add(d, ee, a[q], -1, wide, wrow);
-        ot[q] = phi_add(d, ee, t[q], +1, wide, wrow);
+        if (ee < d.tiny[0]) {
+            oa[q] = phi_add(d, ee, a[q], -1, wide, wrow);
+            ot[q] = phi_add(d, ee, t[q], +1, wide, wrow);
+        }
         if (RVC && d.rv_net) {
             const int32_t before = atomicAdd(&d.rv_net[ee], 1);
             *shared += before == 1 ? 2 : (before >= 2 ? 1 : 0);
@@ -1191,15 +1240,22 @@ __device__ __forceinline__ long long apply_pins(const Dev &d, Rec *recs, const A
     for (int q = 0; q < kPins; ++q) {
         if (!ok[q]) continue;
         Rec *rc = recs + (e[q] & kNetMask);
-        const Lam ba = (Lam)1 << a[q], bt = (Lam)1 << t[q];
-        const Lam lx = (oa[q] == 1 ? ba : (Lam)0) | (ot[q] == 0 ? bt : (Lam)0);
-        const Lam sx = ((oa[q] == 1 || oa[q] == 2) ? ba : (Lam)0) | ((ot[q] == 0 || ot[q] == 1) ? bt : (Lam)0);
-        if (sizeof(Lam) == 8) {
-            if (lx) atomicXor(reinterpret_cast<unsigned long long *>(&rc->lam), (unsigned long long)lx);
-            if (sx) atomicXor(reinterpret_cast<unsigned long long *>(&rc->s1), (unsigned long long)sx);
+        const int32_t ee = e[q] & kNetMask;
+        bool left, entered;
+        if (ee >= d.tiny[0]) {
+            tiny_move(rc, a[q], t[q], tiny_size(d, ee), left, entered);
         } else {
-            if (lx) atomicXor(reinterpret_cast<unsigned int *>(&rc->lam), (unsigned int)lx);
-            if (sx) atomicXor(reinterpret_cast<unsigned int *>(&rc->s1), (unsigned int)sx);
+            const Lam ba = (Lam)1 << a[q], bt = (Lam)1 << t[q];
+            left = oa[q] == 1;
+            entered = ot[q] == 0;
+            const Lam lx = (left ? ba : (Lam)0) | (entered ? bt : (Lam)0);
+            const Lam sx = ((oa[q] == 1 || oa[q] == 2) ? ba : (Lam)0) | ((ot[q] == 0 || ot[q] == 1) ? bt : (Lam)0);
+            if (sizeof(Lam) == 8) {
+                if (lx) atomicXor(reinterpret_cast<unsigned long long *>(&rc->lam), (unsigned long long)lx);
+                if (sx) atomicXor(reinterpret_cast<unsigned long long *>(&rc->s1), (unsigned long long)sx);
+            } else if (sx) {   // a Lambda flip is an S1 flip, too
+                atomicXor(reinterpret_cast<unsigned long long *>(rc), (unsigned long long)sx | ((unsigned long long)lx << 32));
+            }
         }
         // stamp: every writer of round r derives the same value from the pre-round stamp,
         // and one that already sees round r leaves it alone
@@ -1207,7 +1263,7 @@ __device__ __forceinline__ long long apply_pins(const Dev &d, Rec *recs, const A
             const int32_t last = mv[q] >> 1;
             if (last != r) rc->mv = (r << 1) | (last == r - 1 ? 1 : 0);
         }
-        dobj += (long long)(ot[q] == 0 ? w[q] : 0) - (long long)(oa[q] == 1 ? w[q] : 0);
+        dobj += (long long)(entered ? w[q] : 0) - (long long)(left ? w[q] : 0);
     }
     return dobj;
 }

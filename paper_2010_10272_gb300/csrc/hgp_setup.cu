@@ -210,12 +210,15 @@ __global__ void __launch_bounds__(256) k_check_pins(const int32_t *off, const in
 // On skewed instances a few large nets take most record gathers (each incidence reads its net's
 // record); stored first, their records and Phi rows share L2 lines and stay resident there.
 // Gains, objective and every move are sums over nets, so results do not depend on the order.
-constexpr int kNrRanks = 32;        // rank 0: the largest size class (2^30 pins and up)
+// Nets of at most 4 pins (Dev::tiny) come last, a class per size.
+constexpr int kNrRanks = 34;        // rank 0: the largest size class (2^30 pins and up)
+constexpr int kNrTiny = 30;         // rank of the nets of 4 pins
 constexpr int kNrThreads = 256;
 
 __device__ __forceinline__ int nr_rank(int32_t size)
 {
-    return size <= 1 ? kNrRanks - 1 : __clz(size);   // sizes [2^c, 2^(c+1)) -> 31 - c
+    // sizes [2^c, 2^(c+1)) -> 31 - c; 5..7 -> 29; 4, 3, 2, at most 1 -> 30 .. 33
+    return size > 4 ? __clz(size) : kNrTiny + 4 - max(size, 1);
 }
 
 // per CTA (a contiguous chunk of per_cta nets): nets per rank, written rank-major so that one
@@ -777,10 +780,10 @@ __device__ __forceinline__ void write_record(const Dev &d, int64_t e, uint64_t l
 {
     uint4 *rec = reinterpret_cast<uint4 *>(reinterpret_cast<Rec *>(d.rec) + e);
     if constexpr (sizeof(Rec) == 16) {
-        __stcs(rec, make_uint4((uint32_t)s1, (uint32_t)wf, (uint32_t)(kNever * 2), (uint32_t)lam));
+        __stcs(rec, make_uint4((uint32_t)s1, (uint32_t)lam, (uint32_t)wf, (uint32_t)(kNever * 2)));
     } else {
-        __stcs(rec, make_uint4((uint32_t)s1, (uint32_t)(s1 >> 32), (uint32_t)wf, (uint32_t)(kNever * 2)));
-        __stcs(rec + 1, make_uint4((uint32_t)lam, (uint32_t)(lam >> 32), (uint32_t)wf, 0u));
+        __stcs(rec, make_uint4((uint32_t)s1, (uint32_t)(s1 >> 32), (uint32_t)lam, (uint32_t)(lam >> 32)));
+        __stcs(rec + 1, make_uint4((uint32_t)wf, (uint32_t)(kNever * 2), 0u, 0u));
     }
 }
 
@@ -822,7 +825,7 @@ __device__ __forceinline__ long long init_net_cta(const Dev &d, const uint8_t *p
     __syncthreads();
     const bool wide = d.widx != nullptr && sz > narrow_max_of(d);
     uint8_t *row = reinterpret_cast<uint8_t *>(d.phi) + e * (int64_t)(d.k * w);
-    for (int i = threadIdx.x; i < d.k; i += blockDim.x) {
+    for (int i = threadIdx.x; i < d.k && e < d.tiny[0]; i += blockDim.x) {
         const int32_t v = wide ? 0 : cnt[i];
         if (w == 1) row[i] = (uint8_t)v;
         else if (w == 2) reinterpret_cast<uint16_t *>(row)[i] = (uint16_t)v;
@@ -969,7 +972,8 @@ __global__ void __launch_bounds__(kInitWarps * 32, 4) k_init_nets(Dev d, const u
     };
     for (int64_t c0 = e_begin + (int64_t)blockIdx.x * kPerCta; c0 < d.m; c0 += (int64_t)gridDim.x * kPerCta) {
         const int64_t e0 = c0 + wid * 32, e = e0 + lane;
-        const int32_t rows = (int32_t)max((int64_t)0, min((int64_t)32, (int64_t)d.m - e0));
+        // rows of the table: none of tiny nets
+        const int32_t rows = (int32_t)max((int64_t)0, min((int64_t)32, min((int64_t)d.m, (int64_t)d.tiny[0]) - e0));
         int32_t b = 0, size = 0;
         if (e < d.m) {
             b = d.net_off[e];
@@ -982,6 +986,7 @@ __global__ void __launch_bounds__(kInitWarps * 32, 4) k_init_nets(Dev d, const u
         auto in_registers = [&](auto net) {
             net.count(d.pins, part, b, size);
             net.sets(lam, s1);
+            if (rows == 0) return;
             net.template stage<false>(stage, lane, w, wb);
             __syncwarp();
             store_rows(e0, rows);
@@ -1090,7 +1095,11 @@ __global__ void k_obj_from_phi(Dev d, unsigned long long *out)
         const bool wide = d.widx != nullptr && size > (d.phi_w == 1 ? 255 : (d.phi_w == 2 ? 65535 : 0x7fffffff));
         const int32_t wrow = wide ? d.widx[e] : 0;
         int lambda = 0;
-        for (int i = 0; i < d.k; ++i) lambda += phi_get(d, (int32_t)e, i, wide, wrow) > 0;
+        if (e >= d.tiny[0])
+            lambda = d.k <= 32 ? __popc(reinterpret_cast<const Rec16 *>(d.rec)[e].lam)
+                               : __popcll((long long)reinterpret_cast<const Rec32 *>(d.rec)[e].lam);
+        else
+            for (int i = 0; i < d.k; ++i) lambda += phi_get(d, (int32_t)e, i, wide, wrow) > 0;
         if (lambda > 0) s += (long long)(lambda - 1) * (d.nw ? d.nw[e] : 1);
     }
     for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(kFull, s, o);
@@ -1450,6 +1459,7 @@ int create_impl(int32_t n, int32_t m, const int64_t *net_offsets, const int32_t 
     d.k = k;
     d.P = (int32_t)P;
     d.S = o.subrounds;
+    for (int32_t &t : d.tiny) t = 0x7fffffff;
     d.n_tiles = (int32_t)(((int64_t)n + kTile - 1) / kTile);
     d.nseg = segments_of(d.S);
 
@@ -1582,14 +1592,19 @@ int create_impl(int32_t n, int32_t m, const int64_t *net_offsets, const int32_t 
         if (nw_d) CKF(dalloc(h, &nw_int, m));
         k_nr_count<<<(unsigned)nr_ctas, kNrThreads, 0, st>>>(net_off, m, per_cta, cnt); h->launches++;
         CKF(scan(cnt, base, nslots));
-        int big_rank = 0;   // first rank of the nets below kBigNet pins
-        while (((int64_t)1 << (31 - big_rank)) >= kBigNet) ++big_rank;
-        int huge_rank = 0;
-        while (((int64_t)1 << (31 - huge_rank)) >= kHugeNet) ++huge_rank;
-        int32_t mb = 0;
-        CKF(cudaMemcpyAsync(&h->m_huge, base + (int64_t)huge_rank * nr_ctas, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
-        CKF(cudaMemcpyAsync(&mb, base + (int64_t)big_rank * nr_ctas, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
+        // first internal id of every rank
+        int32_t first[kNrRanks];
+        CKF(cudaMemcpy2DAsync(first, sizeof(int32_t), base, sizeof(int32_t) * (size_t)nr_ctas, sizeof(int32_t), kNrRanks,
+                              cudaMemcpyDeviceToHost, st));
         CKF(stream_wait(st));
+        auto below = [&](int32_t size) {   // nets of at least `size` pins (a power of two)
+            int rank = 0;
+            while (((int64_t)1 << (31 - rank)) >= size) ++rank;
+            return first[rank];
+        };
+        const int32_t mb = below(kBigNet);
+        h->m_huge = below(kHugeNet);
+        for (int i = 0; i < 4; ++i) d.tiny[i] = first[kNrTiny + i];
         int32_t *src_big = nullptr;   // where the pins of the large-net prefix come from
         if (mb > 0) CKF(dev_alloc(reinterpret_cast<void **>(&src_big), sizeof(int32_t) * (size_t)mb, st));
         k_nr_place<<<(unsigned)nr_ctas, kNrThreads, 0, st>>>(net_off, m, per_cta, base, perm, tmp, mb, src_big);
@@ -1630,6 +1645,7 @@ int create_impl(int32_t n, int32_t m, const int64_t *net_offsets, const int32_t 
     const int32_t narrow_max = w == 1 ? 255 : (w == 2 ? 65535 : 0x7fffffff);
 
     // ---- wide nets
+    const int32_t phi_rows = std::min(m, d.tiny[0]);
     if (max_size > narrow_max) {
         int32_t *widx = nullptr;
         CKF(dalloc(h, &widx, (int64_t)m + 1));
@@ -1712,7 +1728,7 @@ int create_impl(int32_t n, int32_t m, const int64_t *net_offsets, const int32_t 
 
     // ---- state (Pi was stored by the input check)
     d.part = part;
-    const int64_t entries = (int64_t)m * k;
+    const int64_t entries = (int64_t)phi_rows * k;
     const int64_t words = (entries * w + 3) / 4;
     uint32_t *phi = nullptr;
     CKF(dalloc(h, &phi, words));
