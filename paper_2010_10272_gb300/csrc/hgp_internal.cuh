@@ -215,16 +215,6 @@ __device__ __forceinline__ bool moved_in_prev_round(int32_t mv, int32_t r)
     return last == r - 1 || (last == r && (mv & 1));
 }
 
-// Stamp net e as moved in round r.  Every writer of round r computes the same value from
-// the pre-round stamp, and a writer that already sees round r leaves it alone, so plain
-// stores suffice.
-__device__ __forceinline__ void stamp_moved(int32_t *mv_ptr, int32_t r)
-{
-    const int32_t v = *reinterpret_cast<volatile int32_t *>(mv_ptr);
-    const int32_t last = v >> 1;
-    if (last != r) *mv_ptr = (r << 1) | (last == r - 1 ? 1 : 0);
-}
-
 __device__ __forceinline__ uint64_t splitmix64_output(uint64_t z)
 {
     // SplitMix64 output function (Steele, Lea, Flood, OOPSLA 2014)
