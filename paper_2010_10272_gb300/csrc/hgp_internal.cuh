@@ -102,7 +102,7 @@ struct Dev {
     int32_t bins;           // gains lie below this (a multiple of kThreads), or it is kBins
     int32_t pad1;
     uint8_t *part;
-    uint32_t *phi;
+    uint32_t *phi;          // a whole number of 8-byte words
     int32_t *phi_wide;
     const int32_t *widx;    // [m] row index in phi_wide (valid where the wide flag is set)
     const int32_t *net_perm;  // [m] internal id of input net e (nullptr: input order kept);
@@ -171,6 +171,28 @@ __device__ __forceinline__ int32_t phi_add(const Dev &d, int32_t e, int32_t i, i
     const uint32_t sh = (uint32_t)(x & 3) * 8u;
     const uint32_t old = atomicAdd(&d.phi[x >> 2], (uint32_t)delta << sh);
     return (int32_t)((old >> sh) & 0xFFu);
+}
+
+// One pin of net e from block a to block t: Phi(e, a)--, Phi(e, t)++, and the values before.  With few
+// blocks both entries mostly share an aligned 8-byte word (always up to k = 8 with 1-byte
+// entries), which one 64-bit atomic changes; exact for the same reason as above.
+__device__ __forceinline__ void phi_move(const Dev &d, int32_t e, int32_t a, int32_t t, bool wide, int32_t wrow,
+                                         int32_t &old_a, int32_t &old_t)
+{
+    if (!wide) {
+        const int64_t ba = ((int64_t)e * d.k + a) * d.phi_w, bt = ((int64_t)e * d.k + t) * d.phi_w;
+        if ((ba >> 3) == (bt >> 3)) {
+            const int sa = (int)(ba & 7) * 8, st = (int)(bt & 7) * 8;
+            const unsigned long long old = atomicAdd(reinterpret_cast<unsigned long long *>(d.phi) + (ba >> 3),
+                                                     (1ull << st) - (1ull << sa));
+            const uint32_t mask = d.phi_w == 1 ? 0xFFu : (d.phi_w == 2 ? 0xFFFFu : 0xFFFFFFFFu);
+            old_a = (int32_t)((uint32_t)(old >> sa) & mask);
+            old_t = (int32_t)((uint32_t)(old >> st) & mask);
+            return;
+        }
+    }
+    old_a = phi_add(d, e, a, -1, wide, wrow);
+    old_t = phi_add(d, e, t, +1, wide, wrow);
 }
 
 // pins of a tiny net

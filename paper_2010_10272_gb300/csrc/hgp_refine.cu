@@ -1242,12 +1242,10 @@ __device__ __forceinline__ long long apply_pins(const Dev &d, Rec *recs, const A
         const int32_t ee = e[q] & kNetMask;
         const int32_t wrow = wide ? d.widx[ee] : 0;
         Rec *rc = recs + ee;
-        mv[q] = STAMP ? __ldcg(&rc->mv) : 0;
-        w[q] = __ldg(&rc->w) & 0x7fffffff;
-        if (ee < d.tiny[0]) {
-            oa[q] = phi_add(d, ee, a[q], -1, wide, wrow);
-            ot[q] = phi_add(d, ee, t[q], +1, wide, wrow);
-        }
+        const int2 wm = __ldcg(reinterpret_cast<const int2 *>(&rc->w));   // omega and stamp
+        mv[q] = STAMP ? wm.y : 0;
+        w[q] = wm.x & 0x7fffffff;
+        if (ee < d.tiny[0]) phi_move(d, ee, a[q], t[q], wide, wrow, oa[q], ot[q]);
         if (RVC && d.rv_net) {
             const int32_t before = atomicAdd(&d.rv_net[ee], 1);
             *shared += before == 1 ? 2 : (before >= 2 ? 1 : 0);

@@ -1378,7 +1378,7 @@ size_t small_handle_bytes(int32_t n, int32_t m, int64_t P, int32_t k, const hgp_
     if (has_nw) b += A(4 * (int64_t)m) + A(4 * (int64_t)n);                           // and W(u)
     b += A(4 * (nb + 1)) + A(4 * (nm + 1));                                          // scan scratch
     b += A(4 * ((int64_t)n + 1)) + A(4 * P);                                         // vtx_off, inc
-    b += 2 * A(n) + A(4 * (((int64_t)m * k * w + 3) / 4)) + A((int64_t)m * (k <= 32 ? 16 : 32)) + A(8 * kSmallN);
+    b += 2 * A(n) + A(4 * (((int64_t)m * k * w + 7) / 8 * 2)) + A((int64_t)m * (k <= 32 ? 16 : 32)) + A(8 * kSmallN);
     b += A(2 * n_tiles * kTile) + A(2 * n_tiles * (S + 1)) + A(8 * n_tiles * kTile) + A(4 * n_tiles * nseg);
     b += A(8 * 64) + A(8 * (int64_t)k * kBins) + A((int64_t)sizeof(Sel) * 64) + A(8 * (int64_t)k * n_tiles);
     if (o.revert_negative) {
@@ -1729,7 +1729,7 @@ int create_impl(int32_t n, int32_t m, const int64_t *net_offsets, const int32_t 
     // ---- state (Pi was stored by the input check)
     d.part = part;
     const int64_t entries = (int64_t)phi_rows * k;
-    const int64_t words = (entries * w + 3) / 4;
+    const int64_t words = (entries * w + 7) / 8 * 2;
     uint32_t *phi = nullptr;
     CKF(dalloc(h, &phi, words));
     d.phi = phi;   // written whole by init_state
