@@ -255,6 +255,13 @@ __device__ __forceinline__ int slot_of(const int32_t *off, int32_t i)
     return v;
 }
 
+// COH: the list may be a copy in shared memory
+template <bool COH>
+__device__ __forceinline__ int32_t load_inc(const int32_t *inc, int32_t j)
+{
+    return COH ? inc[j] : __ldg(&inc[j]);
+}
+
 constexpr int32_t kPlaneMaxW = 2047;   // W(u) up to this uses bit planes (NP <= 11)
 // degrees above this are walked by the whole warp: its two passes cost about as many issue slots
 // as a lane's walk of this length with the other lanes idle
@@ -338,7 +345,7 @@ __device__ __forceinline__ void lane_best(const Rec *recs, const int32_t *inc, i
     for (int p = 0; p < NP; ++p) c[p] = 0;
     int32_t e[kAhead];
 #pragma unroll
-    for (int q = 0; q < kAhead; ++q) e[q] = jb + q < je ? (__ldg(&inc[jb + q]) & kNetMask) : -1;
+    for (int q = 0; q < kAhead; ++q) e[q] = jb + q < je ? (load_inc<COH>(inc, jb + q) & kNetMask) : -1;
     for (int32_t j = jb; j < je; j += kAhead) {
         Lam s1[kAhead], lam[kAhead];
         int32_t w[kAhead], mv[kAhead];
@@ -353,7 +360,7 @@ __device__ __forceinline__ void lane_best(const Rec *recs, const int32_t *inc, i
 #pragma unroll
         for (int q = 0; q < kAhead; ++q) {
             const int32_t jn = j + kAhead + q;
-            e[q] = jn < je ? (__ldg(&inc[jn]) & kNetMask) : -1;
+            e[q] = jn < je ? (load_inc<COH>(inc, jn) & kNetMask) : -1;
         }
 #pragma unroll
         for (int q = 0; q < kAhead; ++q) {
@@ -408,10 +415,11 @@ __device__ __forceinline__ void lane_best(const Rec *recs, const int32_t *inc, i
 }
 
 // The best target of the vertex in this lane (a = its block, cu its weight, [jb, je) its nets, W their
-// weight): block t_best (-1: none) and its gain; returns eligibility.  The warp calls it together.
+// weight, inc the incidence lists): block t_best (-1: none) and its gain; returns eligibility.  The
+// warp calls it together.
 template <typename Rec, bool RB, bool COH>
-__device__ __forceinline__ bool gain_vertex(const Dev &d, const GainWarp &g, const GainInst<typename RecIO<Rec>::Lam> &gi,
-                                            const RbArgs &rb, bool valid, int32_t a, int32_t cu, int32_t jb, int32_t je,
+__device__ __forceinline__ bool gain_vertex(const Dev &d, const int32_t *inc, const GainWarp &g,
+                                            const GainInst<typename RecIO<Rec>::Lam> &gi, const RbArgs &rb, bool valid, int32_t a, int32_t cu, int32_t jb, int32_t je,
                                             int32_t W, int &t_best, int32_t &g_best)
 {
     typedef typename RecIO<Rec>::Lam Lam;
@@ -434,7 +442,7 @@ __device__ __forceinline__ bool gain_vertex(const Dev &d, const GainWarp &g, con
     if (light) {
         const int np = 32 - __clz((int)wmax);   // 2^np > wmax >= conn_t
         const int32_t eqv = balance ? W : -1;
-#define HGP_LANE(NP, U) lane_best<Lam, Rec, NP, U, RB, COH>(recs, d.inc, jb, je, a, r, g, cu, kall, eqv, x, T_all, T, t_best, conn, zero_in)
+#define HGP_LANE(NP, U) lane_best<Lam, Rec, NP, U, RB, COH>(recs, inc, jb, je, a, r, g, cu, kall, eqv, x, T_all, T, t_best, conn, zero_in)
         if (unit) {
             if (np <= 4) HGP_LANE(4, true);
             else HGP_LANE(7, true);             // at most kLaneDeg nets
@@ -465,7 +473,7 @@ __device__ __forceinline__ bool gain_vertex(const Dev &d, const GainWarp &g, con
         for (int32_t j = hjb + lane; j < hje; j += 32) {
             Lam s1, lam;
             int32_t w, mv;
-            RecIO<Rec>::template load_full<COH>(recs + (__ldg(&d.inc[j]) & kNetMask), s1, w, mv, lam);
+            RecIO<Rec>::template load_full<COH>(recs + (load_inc<COH>(inc, j) & kNetMask), s1, w, mv, lam);
             take_net(y, s1, lam, w & 0x7fffffff, mv, ha, r);
         }
         y.b = __reduce_add_sync(kFull, y.b);
@@ -491,7 +499,7 @@ __device__ __forceinline__ bool gain_vertex(const Dev &d, const GainWarp &g, con
             Lam lam = 0;
             int32_t w = 0;
             if (j < hje) {
-                RecIO<Rec>::template load_b<COH>(recs + (__ldg(&d.inc[j]) & kNetMask), lam, w);
+                RecIO<Rec>::template load_b<COH>(recs + (load_inc<COH>(inc, j) & kNetMask), lam, w);
                 w &= 0x7fffffff;
             }
             const int nn = min(32, hje - j0);
@@ -610,7 +618,7 @@ __device__ __forceinline__ int32_t gain_seg(const Dev &d, int32_t tile, int32_t 
         }
         int t_best;
         int32_t g_best;
-        const bool elig = gain_vertex<Rec, RB, false>(d, g, gi, rb, valid, a, cu, jb, je, W, t_best, g_best);
+        const bool elig = gain_vertex<Rec, RB, false>(d, d.inc, g, gi, rb, valid, a, cu, jb, je, W, t_best, g_best);
         nel += __popc(__ballot_sync(kFull, elig));
         const unsigned cm = __ballot_sync(kFull, t_best >= 0);
         const bool small_c = __all_sync(kFull, cu < (1 << 26));   // 32 of them fit 32 bits
@@ -1217,7 +1225,7 @@ __device__ __forceinline__ void tiny_move(Rec32 *rc, int a, int t, int size, boo
 // and, in `shared`, the moved incidences on nets with several movers (a second mover adds its
 // own incidence and the first one's, later movers their own).
 template <typename Rec, bool STAMP = true, bool RVC = false>
-__device__ __forceinline__ long long apply_pins(const Dev &d, Rec *recs, const ApplyWarp &w_,
+__device__ __forceinline__ long long apply_pins(const Dev &d, const int32_t *inc, Rec *recs, const ApplyWarp &w_,
                                                 int32_t i0, int32_t total, int32_t r, int32_t *shared = nullptr)
 {
     typedef typename RecIO<Rec>::Lam Lam;
@@ -1232,7 +1240,7 @@ __device__ __forceinline__ long long apply_pins(const Dev &d, Rec *recs, const A
             const int v = slot_of(w_.off, i);
             a[q] = w_.a[v];
             t[q] = w_.t[v];
-            e[q] = d.inc[w_.jb[v] + (i - w_.off[v])];
+            e[q] = inc[w_.jb[v] + (i - w_.off[v])];
         }
     }
 #pragma unroll
@@ -1326,7 +1334,7 @@ __device__ __forceinline__ bool approve(uint64_t c, int32_t slot, const ApplyIns
 // Applies the queued moves [first, first + 32) (at most `queued` in all) over their incidences,
 // flattened across the lanes.
 template <typename Rec, int KEY>
-__device__ __forceinline__ void apply_queue(const Dev &d, const int32_t *qu, const uint16_t *qat, int32_t first,
+__device__ __forceinline__ void apply_queue(const Dev &d, const int32_t *vtx_off, const int32_t *inc, const int32_t *qu, const uint16_t *qat, int32_t first,
                                             int32_t queued, int32_t r, ApplyWarp &w_,
                                             long long &dobj, int32_t &npins, int32_t &nshared)
 {
@@ -1337,8 +1345,8 @@ __device__ __forceinline__ void apply_queue(const Dev &d, const int32_t *qu, con
         const int32_t u = qu[first + lane], at = qat[first + lane];
         a = at & 0xFF;
         t = at >> 8;
-        jb = d.vtx_off[u];
-        deg = d.vtx_off[u + 1] - jb;
+        jb = vtx_off[u];
+        deg = vtx_off[u + 1] - jb;
         npins += deg;
     }
     int32_t incl = deg;
@@ -1355,7 +1363,7 @@ __device__ __forceinline__ void apply_queue(const Dev &d, const int32_t *qu, con
     if (lane == 31) w_.off[32] = total;
     __syncwarp();
     for (int32_t i0 = 0; i0 < total; i0 += 32 * kPins)
-        dobj += apply_pins<Rec, KEY == KEY_T, KEY == KEY_T>(d, recs, w_, i0 + lane, total, r, &nshared);
+        dobj += apply_pins<Rec, KEY == KEY_T, KEY == KEY_T>(d, inc, recs, w_, i0 + lane, total, r, &nshared);
     __syncwarp();
 }
 
@@ -1414,7 +1422,7 @@ __device__ __forceinline__ void apply_segs(const Dev &d, int32_t tile, int32_t s
         __syncwarp();
         int32_t first = 0;
         for (; queued - first >= 32; first += 32)
-            apply_queue<Rec, KEY>(d, mq.u, mq.at, first, queued, r, w_, dobj, npins, nshared);
+            apply_queue<Rec, KEY>(d, d.vtx_off, d.inc, mq.u, mq.at, first, queued, r, w_, dobj, npins, nshared);
         if (first && queued - first > 0) {   // the rest moves to the front
             int32_t u2 = 0;
             uint16_t at2 = 0;
@@ -1441,7 +1449,7 @@ __device__ __forceinline__ void apply_segs(const Dev &d, int32_t tile, int32_t s
 // a chain of loads for every 32, was slower than no queue, 42 us and 1.19 ms.)
 // B as for k_gain.
 template <typename Rec, bool B, int KEY = KEY_T>
-__global__ void __launch_bounds__(kThreads, 4) k_apply(const Dev d0, const Dev *devs, const int2 *items,
+__global__ void __launch_bounds__(kThreads, B ? 3 : 4) k_apply(const Dev d0, const Dev *devs, const int2 *items,
                                                        int32_t n_items, int32_t nseg, int32_t per, int32_t rr)
 {
     after_previous();
@@ -1465,7 +1473,7 @@ __global__ void __launch_bounds__(kThreads, 4) k_apply(const Dev d0, const Dev *
     const int32_t n_it = (B ? n_items : d0.n_tiles) * groups;
     // a batch instance's queue, block weights and counters, before the warp turns to another one
     auto leave = [&](const Dev &d) {
-        if (queued) apply_queue<Rec, KEY>(d, mq_w[wid].u, mq_w[wid].at, 0, queued, r, aw[wid], dobj, npins, nshared);
+        if (queued) apply_queue<Rec, KEY>(d, d.vtx_off, d.inc, mq_w[wid].u, mq_w[wid].at, 0, queued, r, aw[wid], dobj, npins, nshared);
         queued = 0;
         for (int o = 16; o; o >>= 1) {
             dobj += __shfl_xor_sync(kFull, dobj, o);
@@ -1521,7 +1529,7 @@ __global__ void __launch_bounds__(kThreads, 4) k_apply(const Dev d0, const Dev *
         if (inst_prev >= 0) leave(dsm[wid]);
         return;
     }
-    if (queued) apply_queue<Rec, KEY>(d0, mq_w[wid].u, mq_w[wid].at, 0, queued, r, aw[wid], dobj, npins, nshared);
+    if (queued) apply_queue<Rec, KEY>(d0, d0.vtx_off, d0.inc, mq_w[wid].u, mq_w[wid].at, 0, queued, r, aw[wid], dobj, npins, nshared);
     if (!B && KEY == KEY_T && d0.rv_cnt) {
         // revert variant: moved incidences on nets with several movers (sizes the order-statistics table)
         nshared = __reduce_add_sync(kFull, nshared);
@@ -1803,7 +1811,7 @@ __global__ void __launch_bounds__(kThreads) k_rv_revert(const Dev d, int32_t rr)
         if (lane == 31) aw[wid].off[32] = total;
         __syncwarp();
         for (int32_t i0 = 0; i0 < total; i0 += 32 * kPins)
-            dobj += apply_pins<Rec>(d, recs, aw[wid], i0 + lane, total, r);
+            dobj += apply_pins<Rec>(d, d.inc, recs, aw[wid], i0 + lane, total, r);
         __syncwarp();
     }
     for (int o = 16; o; o >>= 1) {
@@ -2179,7 +2187,10 @@ bool small_plan(const Plan &p, int device, int32_t debug)
     if (r == 0) {
         auto kernel = p.rec32 ? k_small<Rec32> : k_small<Rec16>;
         cudaLaunchAttribute at;
-        cudaLaunchConfig_t cfg = small_config(kSmallVertices, nullptr, &at);
+        bool cached;
+        int32_t inc_room;
+        cudaLaunchConfig_t cfg = small_config(p.d0, nullptr, &at, cached, inc_room);
+        cfg.dynamicSmemBytes = kSmMaxBytes;   // the largest of any handle
         int clusters = 0;
         cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
         if (e == cudaSuccess)
@@ -2196,10 +2207,12 @@ cudaError_t launch_small(const Plan &p, int32_t rounds, int64_t max_netweight)
     int nd = 1;
     while (nd < 4 && (max_netweight >> (kSmDigit * nd)) > 0) ++nd;
     cudaLaunchAttribute at;
-    const cudaLaunchConfig_t cfg = small_config(p.d0.n, p.st, &at);
+    bool cached;
+    int32_t inc_room;
+    const cudaLaunchConfig_t cfg = small_config(p.d0, p.st, &at, cached, inc_room);
     *p.launches += 1;
-    return p.rec32 ? cudaLaunchKernelEx(&cfg, k_small<Rec32>, p.d0, rounds, (int32_t)nd)
-                   : cudaLaunchKernelEx(&cfg, k_small<Rec16>, p.d0, rounds, (int32_t)nd);
+    return p.rec32 ? cudaLaunchKernelEx(&cfg, k_small<Rec32>, p.d0, rounds, (int32_t)nd, cached, inc_room)
+                   : cudaLaunchKernelEx(&cfg, k_small<Rec16>, p.d0, rounds, (int32_t)nd, cached, inc_room);
 }
 
 cudaError_t enqueue_rounds(const Plan &p, int64_t *stats, int32_t rounds, bool small, int64_t max_netweight)

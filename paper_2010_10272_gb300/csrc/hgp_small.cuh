@@ -7,6 +7,9 @@
 // between the launches of the general path stays on the chip:
 //   * a warp owns a contiguous range of vertices, hashes its sub-rounds once per round, and keeps
 //     its candidates in shared memory between the gain and the apply step;
+//   * the vertices' blocks, weights and list offsets are kept in shared memory, and as much of the
+//     lists as fits: a cluster barrier drops the L1 lines, so each of them would cost an L2 round
+//     trip in every phase (10k vertices 255 -> 239 us a call, 30k 381 -> 373 us);
 //   * block weights are a copy per CTA, updated through distributed shared memory;
 //   * the approval is a radix select on the key (gain desc, id asc): the candidates' weights are
 //     summed per target block and key digit in the shared memory of the block's home CTA, and the
@@ -15,7 +18,7 @@
 // The records and pin counts live in global memory as in the general path; another SM's updates
 // are read from L2 (RecIO<..>::load_full<true>, atomics), ordered by the cluster barriers.
 //
-// 10k vertices (k = 2, 60k pins, 5 rounds): 740 -> 210 us a call.
+// 10k vertices (k = 2, 60k pins, 5 rounds): 740 -> 200 us a call.
 
 constexpr int kSmWarps = 16;
 constexpr int kSmThreads = 32 * kSmWarps;
@@ -40,7 +43,12 @@ __host__ __device__ inline int small_per_warp(int32_t n)
     const int32_t v = (n + kSmCtas * kSmWarps - 1) / (kSmCtas * kSmWarps);
     return (v + 7) / 8 * 8;
 }
-__host__ __device__ inline int small_warp_bytes(int per_warp) { return per_warp * (8 + 2 + 1); }
+// and, with `cached`, their list offsets, blocks, and weights c and W where they are not one
+__host__ __device__ inline int small_warp_bytes(int per_warp, bool cached, bool vw, bool nw)
+{
+    return per_warp * (8 + 2 + 1) + (cached ? (per_warp + 2) * 4 + per_warp * (1 + 4 * vw + 4 * nw) : 0) + 7 & ~7;
+}
+constexpr int kSmMaxBytes = 226 << 10;   // dynamic shared memory of a CTA
 
 struct SmallShared {
     unsigned long long row[kSmPerHome][kSmRow];   // home CTA: weight per key digit of a block
@@ -161,21 +169,32 @@ __device__ __forceinline__ void small_select(SmallShared &sh, const Dev &d, unsi
 }
 
 template <typename Rec>
-__global__ void __launch_bounds__(kSmThreads, 1) k_small(const Dev d, int32_t rounds, int32_t nd)
+__global__ void __launch_bounds__(kSmThreads, 1) k_small(const Dev d, int32_t rounds, int32_t nd, bool cached, int32_t inc_room)
 {
     extern __shared__ __align__(16) unsigned char small_dyn[];
     SmallShared &sh = *reinterpret_cast<SmallShared *>(small_dyn);
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const unsigned rank = blockIdx.x;   // one cluster: the CTA's rank in it
     const int per_warp = small_per_warp(d.n);
-    unsigned char *mine = small_dyn + sizeof(SmallShared) + wid * small_warp_bytes(per_warp);
+    const int warp_bytes = small_warp_bytes(per_warp, cached, d.vw != nullptr, d.nw != nullptr);
+    unsigned char *mine = small_dyn + sizeof(SmallShared) + wid * warp_bytes;
     SmallCand *cand = reinterpret_cast<SmallCand *>(mine);
-    uint16_t *list = reinterpret_cast<uint16_t *>(mine + per_warp * 8);
-    uint8_t *sub = mine + per_warp * 10;
+    // per_warp is a multiple of 8, so every array is aligned
+    int32_t *offs = reinterpret_cast<int32_t *>(mine + per_warp * 8);            // [per_warp + 2] if cached
+    unsigned char *rest = mine + per_warp * 8 + (cached ? (per_warp + 2) * 4 : 0);
+    int32_t *vws = reinterpret_cast<int32_t *>(rest);                            // [per_warp] if cached, weighted
+    rest += cached && d.vw ? per_warp * 4 : 0;
+    int32_t *vnws = reinterpret_cast<int32_t *>(rest);                           // the same
+    rest += cached && d.nw ? per_warp * 4 : 0;
+    uint16_t *list = reinterpret_cast<uint16_t *>(rest);
+    uint8_t *sub = rest + per_warp * 2;
+    uint8_t *blocks = rest + per_warp * 3;                                       // [per_warp] if cached
+    int32_t *incs = reinterpret_cast<int32_t *>(small_dyn + sizeof(SmallShared) + kSmWarps * warp_bytes);   // [inc_room]
     int32_t *qu = sh.qu[wid];
     uint16_t *qat = sh.qat[wid];
     const int32_t v0 = ((int32_t)rank * kSmWarps + wid) * per_warp;
     const int32_t nv = max(0, min(per_warp, d.n - v0));
+    const int32_t c0 = min(d.n, (int32_t)rank * kSmWarps * per_warp), c1 = min(d.n, c0 + kSmWarps * per_warp);
     const int passes = nd + 2;
     const bool unit = d.nw == nullptr;
     const int32_t S = d.S;
@@ -190,6 +209,21 @@ __global__ void __launch_bounds__(kSmThreads, 1) k_small(const Dev d, int32_t ro
         sh.open[tid] = 0;
     }
     if (tid < 6) sh.sum[tid] = 0;
+    // the CTA's lists from the first on, and the warp's vertices
+    const int32_t inc0 = d.vtx_off[c0], inc_n = min(inc_room, d.vtx_off[c1] - inc0);
+    for (int32_t i = tid; i < inc_n; i += kSmThreads) incs[i] = __ldg(&d.inc[inc0 + i]);
+    const int32_t *vtx = d.vtx_off, *inc = d.inc;   // indexed by vertex / incidence, wherever they are
+    if (cached) {
+        for (int32_t i = lane; i < nv; i += 32) {
+            blocks[i] = d.part[v0 + i];
+            if (d.vw) vws[i] = d.vw[v0 + i];
+            if (!unit) vnws[i] = d.vnw[v0 + i];
+        }
+        for (int32_t i = lane; i <= nv; i += 32) offs[i] = nv ? d.vtx_off[v0 + i] : 0;
+        __syncwarp();
+        vtx = offs - v0;
+        if (nv && offs[nv] - inc0 <= inc_n) inc = incs - inc0;
+    }
     long long obj = rank == 0 && tid == 0 ? *d.obj : 0;
     cluster_sync();
     for (int32_t rr = 0; rr < rounds; ++rr) {
@@ -220,15 +254,15 @@ __global__ void __launch_bounds__(kSmThreads, 1) k_small(const Dev d, int32_t ro
                 if (valid) {
                     ul = list[c0 + lane];
                     const int32_t u = v0 + ul;
-                    a = d.part[u];   // only this warp reads or changes it here
-                    cu = d.vw ? d.vw[u] : 1;
-                    jb = d.vtx_off[u];
-                    je = d.vtx_off[u + 1];
-                    W = unit ? je - jb : d.vnw[u];
+                    a = cached ? blocks[ul] : d.part[u];   // only this warp reads or changes it here
+                    cu = d.vw ? (cached ? vws[ul] : d.vw[u]) : 1;
+                    jb = vtx[u];
+                    je = vtx[u + 1];
+                    W = unit ? je - jb : (cached ? vnws[ul] : d.vnw[u]);
                 }
                 int t_best;
                 int32_t g_best;
-                const bool elig = gain_vertex<Rec, false, true>(d, sh.g[wid], gi, RbArgs{0, 0, 0}, valid, a, cu, jb, je, W,
+                const bool elig = gain_vertex<Rec, false, true>(d, inc, sh.g[wid], gi, RbArgs{0, 0, 0}, valid, a, cu, jb, je, W,
                                                                 t_best, g_best);
                 nelig += elig;
                 const unsigned cm = __ballot_sync(kFull, t_best >= 0);
@@ -261,7 +295,7 @@ __global__ void __launch_bounds__(kSmThreads, 1) k_small(const Dev d, int32_t ro
                         const unsigned long long key = small_key(c.g, u, nd);
                         in = sh.open[t] && (key >> (shift + kSmDigit)) == sh.key[t];
                         digit = (int)(key >> shift) & (kSmBins - 1);
-                        if (in && d.vw) cu = d.vw[u];
+                        if (in && d.vw) cu = cached ? vws[c.uat >> 12] : d.vw[u];
                     }
                     small_count(sh, in, t, digit, cu);
                 }
@@ -285,7 +319,8 @@ __global__ void __launch_bounds__(kSmThreads, 1) k_small(const Dev d, int32_t ro
                 const unsigned am = __ballot_sync(kFull, appr);
                 if (appr) {
                     d.part[u] = (uint8_t)t;
-                    const unsigned long long cw = d.vw ? (unsigned long long)d.vw[u] : 1ull;
+                    if (cached) blocks[u - v0] = (uint8_t)t;
+                    const unsigned long long cw = d.vw ? (unsigned long long)(cached ? vws[u - v0] : d.vw[u]) : 1ull;
                     atomicAdd(&sh.dbw[a], (unsigned long long)(-(long long)cw));
                     atomicAdd(&sh.dbw[t], cw);
                     ++nappr;
@@ -296,7 +331,7 @@ __global__ void __launch_bounds__(kSmThreads, 1) k_small(const Dev d, int32_t ro
                 queued += __popc(am);
                 __syncwarp();
                 if (queued >= 32) {
-                    apply_queue<Rec, KEY_T>(d, qu, qat, 0, queued, r, sh.aw[wid], dobj, npins, nshared);
+                    apply_queue<Rec, KEY_T>(d, vtx, inc, qu, qat, 0, queued, r, sh.aw[wid], dobj, npins, nshared);
                     int32_t u2 = 0;
                     uint16_t at2 = 0;
                     if (32 + lane < queued) {
@@ -310,7 +345,7 @@ __global__ void __launch_bounds__(kSmThreads, 1) k_small(const Dev d, int32_t ro
                     __syncwarp();
                 }
             }
-            if (queued) apply_queue<Rec, KEY_T>(d, qu, qat, 0, queued, r, sh.aw[wid], dobj, npins, nshared);
+            if (queued) apply_queue<Rec, KEY_T>(d, vtx, inc, qu, qat, 0, queued, r, sh.aw[wid], dobj, npins, nshared);
             __syncthreads();
             // this CTA's block weight changes into every CTA's copy
             for (int i = tid; i < 64 * kSmCtas; i += kSmThreads) {
@@ -364,13 +399,21 @@ __global__ void __launch_bounds__(kSmThreads, 1) k_small(const Dev d, int32_t ro
     cluster_sync();   // no CTA leaves while others may still reach into its shared memory
 }
 
-// launch of k_small for n vertices: one cluster
-inline cudaLaunchConfig_t small_config(int32_t n, cudaStream_t st, cudaLaunchAttribute *at)
+// launch of k_small: one cluster.  cached / inc_room: what its shared memory has room for.
+inline cudaLaunchConfig_t small_config(const Dev &d, cudaStream_t st, cudaLaunchAttribute *at, bool &cached, int32_t &inc_room)
 {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(kSmCtas);
     cfg.blockDim = dim3(kSmThreads);
-    cfg.dynamicSmemBytes = sizeof(SmallShared) + (size_t)kSmWarps * small_warp_bytes(small_per_warp(n));
+    const int per_warp = small_per_warp(d.n);
+    auto bytes = [&](bool c) {
+        return (int)sizeof(SmallShared) + kSmWarps * small_warp_bytes(per_warp, c, d.vw != nullptr, d.nw != nullptr);
+    };
+    cached = bytes(true) <= kSmMaxBytes;
+    // the lists of a CTA's vertices, twice their average, as far as they fit
+    const int64_t want = 2 * ((int64_t)d.P / kSmCtas + 256);
+    inc_room = cached ? (int32_t)std::min<int64_t>(want, (kSmMaxBytes - bytes(true)) / 4) : 0;
+    cfg.dynamicSmemBytes = (size_t)bytes(cached) + 4 * (size_t)inc_room;
     cfg.stream = st;
     at->id = cudaLaunchAttributeClusterDimension;
     at->val.clusterDim.x = kSmCtas;
