@@ -529,6 +529,9 @@ constexpr int32_t kReorderMinNets = 1 << 20;
 constexpr int64_t kReorderSkew = 8;
 // host inputs with fewer nets than this: the host reads the net sizes (see create_impl)
 constexpr int32_t kHostSizesMaxNets = 1 << 20;
+// device inputs with fewer nets than this carve their buffers from one allocation, too (about 30 pool
+// calls at creation otherwise: 256 handles of 1k to 200k vertices 900 -> 55-154 ms)
+constexpr int32_t kDeviceArenaMaxNets = 1 << 18;
 // in internal order, nets of at least kBigNet pins (a prefix) get their own CTAs at creation and
 // initialisation (a power of two: size classes are powers of two)
 
@@ -1358,8 +1361,8 @@ int init_state(hgp_handle *h, const uint8_t *part, const int32_t *guard)
 
 constexpr int kSmallN = 72 + kAccN;   // int64 entries of a handle's small state (see create_impl)
 
-// Device bytes of every buffer create_impl (and the first refine) allocates for a handle made
-// from host inputs of fewer than kHostSizesMaxNets nets, each rounded up to 256 bytes: the arena
+// Device bytes of every buffer create_impl (and the first refine) allocates for a handle of few
+// nets (see kHostSizesMaxNets, kDeviceArenaMaxNets), each rounded up to 256 bytes: the arena
 // those buffers are carved from.  It covers the direct transpose in input net order without
 // wide nets; buffers of any other path (or beyond a miscount) come from the pool instead.
 size_t small_handle_bytes(int32_t n, int32_t m, int64_t P, int32_t k, const hgp_options &o, int32_t max_size,
@@ -1490,7 +1493,11 @@ int create_impl(int32_t n, int32_t m, const int64_t *net_offsets, const int32_t 
         }
         if (lo < 0) return fail(HGP_ERR_INVALID);   // then every size is at most P < 2^31
         max_size = (int32_t)hi;
-        const size_t bytes = small_handle_bytes(n, m, P, k, o, max_size, vertex_w != nullptr, net_w != nullptr);
+    }
+    if (host_sizes || m < kDeviceArenaMaxNets) {
+        // device inputs: the largest net is not known yet, so Phi gets room for 2-byte entries
+        const size_t bytes = small_handle_bytes(n, m, P, k, o, host_sizes ? max_size : 65535, vertex_w != nullptr,
+                                                net_w != nullptr);
         void *a = nullptr;
         if (dev_alloc(&a, bytes, st) == cudaSuccess) {   // else every buffer comes from the pool
             h->allocs[h->n_allocs++] = a;
