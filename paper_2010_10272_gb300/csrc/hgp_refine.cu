@@ -1825,11 +1825,21 @@ __global__ void __launch_bounds__(kThreads) k_rv_revert(const Dev d, int32_t rr)
     }
 }
 
-// Pi of one handle widened to int32 (batch partition read-back)
-__global__ void k_part_widen(const uint8_t *part, int32_t n, int32_t *out)
+// The 1-byte partitions of up to kGather members one after another (batch read-back): grid row i
+// copies member i.  One launch for 120 of them; a launch each cost the host 1 ms for 256.
+constexpr int kGather = 120;
+struct GatherArgs {
+    const uint8_t *part[kGather];
+    int64_t off[kGather + 1];
+};
+__global__ void __launch_bounds__(256) k_part_gather(const GatherArgs g, uint8_t *out)
 {
+    const int i = blockIdx.y;
+    const uint8_t *src = g.part[i];
+    const int64_t n = g.off[i + 1] - g.off[i];
+    uint8_t *dst = out + g.off[i];
     for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < n; v += (int64_t)gridDim.x * blockDim.x)
-        out[v] = part[v];
+        dst[v] = src[v];
 }
 
 // thread per instance: per-round objective and heaviest block; advance the round state
@@ -2936,20 +2946,29 @@ int hgp_batch_get_partitions(hgp_batch *b, const int32_t *members, int32_t count
         if (e != cudaSuccess) b->aux = nullptr;
     }
     if (e == cudaSuccess) e = cudaStreamWaitEvent(b->aux, b->ev_end, 0);
-    int32_t *stage = nullptr;
-    if (e == cudaSuccess) e = dev_alloc(reinterpret_cast<void **>(&stage), sizeof(int32_t) * (size_t)total, b->aux);
+    uint8_t *stage = nullptr;
+    if (e == cudaSuccess) e = dev_alloc(reinterpret_cast<void **>(&stage), (size_t)total, b->aux);
     int64_t off = 0;
-    for (int32_t i = 0; i < count && e == cudaSuccess; ++i) {
-        const Dev &d = b->hs[members[i]]->d;
-        const int grid = (int)std::min<int64_t>((d.n + 255) / 256, 152 * 8);
-        k_part_widen<<<grid, 256, 0, b->aux>>>(d.part, d.n, stage + off);
+    for (int32_t i = 0; i < count && e == cudaSuccess;) {
+        GatherArgs g;
+        int64_t most = 0;
+        int32_t rows = 0;
+        for (; rows < kGather && i < count; ++rows, ++i) {
+            const Dev &d = b->hs[members[i]]->d;
+            g.part[rows] = d.part;
+            g.off[rows] = off;
+            off += d.n;
+            most = std::max<int64_t>(most, d.n);
+        }
+        g.off[rows] = off;
+        const dim3 grid((unsigned)std::min<int64_t>((most + 1023) / 1024, 152), (unsigned)rows);
+        k_part_gather<<<grid, 256, 0, b->aux>>>(g, stage);
         e = cudaGetLastError();
-        off += d.n;
         b->launches++;
     }
     // through a page-locked staging buffer of the library (grown when needed), so the copy runs
-    // at the link's rate whatever memory `out` is
-    const size_t bytes = sizeof(int32_t) * (size_t)total;
+    // at the link's rate whatever memory `out` is; the bytes are widened on the way out of it
+    const size_t bytes = (size_t)total;
     std::lock_guard<std::mutex> lk(g_stage_mu);
     if (e == cudaSuccess && g_stage_cap < bytes) {
         if (g_stage) cudaFreeHost(g_stage);
@@ -2967,7 +2986,8 @@ int hgp_batch_get_partitions(hgp_batch *b, const int32_t *members, int32_t count
         (void)cudaGetLastError();
         return status_of(e);
     }
-    memcpy(out, g_stage, bytes);
+    const uint8_t *from = static_cast<const uint8_t *>(g_stage);
+    for (int64_t v = 0; v < total; ++v) out[v] = from[v];
     return HGP_OK;
 }
 
