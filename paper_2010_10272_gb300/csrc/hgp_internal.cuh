@@ -123,7 +123,6 @@ struct Dev {
     uint64_t *cand;         // [n_tiles * kTile] (gain << 32 | offset << 8 | target); a segment's
                             // candidates start at slot kSeg * segment of its tile
     int32_t *cand_cnt;      // [n_tiles * nseg]
-    int64_t *tot;           // [k] candidate weight per key block (rebalancing)
     unsigned long long *hist;  // [k * kBins]
     Sel *sel;               // [k]
     int64_t *tie;           // [k * n_tiles] weight of the candidates at the threshold gain

@@ -414,6 +414,21 @@ __device__ __forceinline__ void lane_best(const Rec *recs, const int32_t *inc, i
     }
 }
 
+// Level-0 histogram of an approval stage: each lane's weight cu (ok lanes) by key block and gain (or
+// priority) bin, a reduction in L2.  Gains are small numbers, so a warp's candidates share bins: one
+// reduction per distinct (block, bin).  The warp calls it together.
+__device__ __forceinline__ void count_gain(const Dev &d, bool ok, int key, int32_t g, int32_t cu)
+{
+    const unsigned mask = __ballot_sync(kFull, ok);
+    if (!ok) return;
+    const int bin = g < kBins - 1 ? g : kBins - 1;
+    const unsigned peers = __match_any_sync(mask, key * kBins + bin);
+    // two halves: 32 sums of either fit 32 bits
+    const unsigned long long sum = (unsigned long long)__reduce_add_sync(peers, (uint32_t)cu & 0xFFFFu) +
+                                   ((unsigned long long)__reduce_add_sync(peers, (uint32_t)cu >> 16) << 16);
+    if ((int)(threadIdx.x & 31) == __ffs(peers) - 1) atomicAdd(&d.hist[(int64_t)key * kBins + bin], sum);
+}
+
 // The best target of the vertex in this lane (a = its block, cu its weight, [jb, je) its nets, W their
 // weight, inc the incidence lists): block t_best (-1: none) and its gain; returns eligibility.  The
 // warp calls it together.
@@ -570,10 +585,10 @@ __device__ __forceinline__ bool gain_vertex(const Dev &d, const int32_t *inc, co
 // candidates written, to the slots of segment seg.
 // RB: a rebalancing pass (Sec. 8): only vertices of overloaded blocks take part, their target
 // is the block with room of highest gain (any sign), and the candidate records its source
-// block (bits 19..24) and the priority gain + off; the per-block totals are by source block.
+// block (bits 19..24) and the priority gain + off, by which it is counted.
 template <typename Rec, bool RB>
 __device__ __forceinline__ int32_t gain_seg(const Dev &d, int32_t tile, int32_t seg, int32_t seg_end, int32_t s,
-                                            const GainWarp &g, uint16_t *picked, unsigned long long *tot,
+                                            const GainWarp &g, uint16_t *picked,
                                             const GainInst<typename RecIO<Rec>::Lam> &gi, int32_t &nel, const RbArgs &rb)
 {
     const int lane = threadIdx.x & 31;
@@ -621,29 +636,15 @@ __device__ __forceinline__ int32_t gain_seg(const Dev &d, int32_t tile, int32_t 
         const bool elig = gain_vertex<Rec, RB, false>(d, d.inc, g, gi, rb, valid, a, cu, jb, je, W, t_best, g_best);
         nel += __popc(__ballot_sync(kFull, elig));
         const unsigned cm = __ballot_sync(kFull, t_best >= 0);
-        const bool small_c = __all_sync(kFull, cu < (1 << 26));   // 32 of them fit 32 bits
         if (t_best >= 0) {
             const int pos = nout + __popc(cm & lanemask_lt());
-            if (RB) {
+            if (RB)
                 out[pos] = ((uint64_t)(uint32_t)(g_best + rb.off) << 32) | ((uint32_t)a << 19) |
                            ((uint32_t)ul << 8) | (uint32_t)t_best;
-                atomicAdd(&tot[a], (unsigned long long)cu);
-            } else {
+            else
                 out[pos] = ((uint64_t)(uint32_t)g_best << 32) | ((uint32_t)ul << 8) | (uint32_t)t_best;
-                // level-0 histogram of the approval step: candidate weight by target block and
-                // gain bin (a reduction in L2).  Gains are small numbers, so a warp's candidates
-                // share bins: one reduction per distinct (block, bin)
-                const int bin = g_best < kBins - 1 ? g_best : kBins - 1;
-                unsigned long long *slot = &d.hist[(int64_t)t_best * kBins + bin];
-                if (small_c) {
-                    const unsigned peers = __match_any_sync(cm, t_best * kBins + bin);
-                    const unsigned sum = __reduce_add_sync(peers, (unsigned)cu);
-                    if (lane == __ffs(peers) - 1) atomicAdd(slot, (unsigned long long)sum);
-                } else {
-                    atomicAdd(slot, (unsigned long long)cu);
-                }
-            }
         }
+        count_gain(d, t_best >= 0, RB ? a : t_best, RB ? g_best + rb.off : g_best, cu);
         nout += __popc(cm);
         __syncwarp();
     }
@@ -700,13 +701,11 @@ __global__ void __launch_bounds__(kThreads, sizeof(Rec) == 16 || RB ? 4 : 3) k_g
     after_previous();
     typedef typename RecIO<Rec>::Lam Lam;
     __shared__ GainWarp ws[kWarps];
-    __shared__ unsigned long long tot_s[RB ? 64 : 1];
     __shared__ uint16_t picked[RB ? kWarps : 1][RB ? kTile : 1];
     __shared__ Dev dsm[B ? kWarps : 1];
     __shared__ unsigned long long cnt_s[2];
     __shared__ int warps_done;
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-    if (RB && tid < 64) tot_s[tid] = 0;
     if (tid == 0) { cnt_s[0] = 0; cnt_s[1] = 0; warps_done = 0; }
     __syncthreads();   // before any warp adds into them
     GainInst<Lam> gi;
@@ -736,7 +735,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(Rec) == 16 || RB ? 4 : 3) k_g
                 }
                 const Dev &d = dsm[wid];
                 if (seg >= d.nseg) continue;
-                const int32_t nout = gain_seg<Rec, false>(d, tile, seg, seg + 1, s, ws[wid], nullptr, tot_s, gi, nel, rb);
+                const int32_t nout = gain_seg<Rec, false>(d, tile, seg, seg + 1, s, ws[wid], nullptr, gi, nel, rb);
                 if (lane == 0) {
                     d.cand_cnt[(int64_t)tile * d.nseg + seg] = nout;
                     unsigned long long *row = reinterpret_cast<unsigned long long *>(d.stats + (int64_t)rr * ST_N);
@@ -751,8 +750,8 @@ __global__ void __launch_bounds__(kThreads, sizeof(Rec) == 16 || RB ? 4 : 3) k_g
                     inst_prev = 0;
                 }
                 const int32_t seg_end = RB ? min(d0.nseg, seg + kRbSegs) : seg + 1;
-                const int32_t nout = gain_seg<Rec, RB>(d0, tile, seg, seg_end, s, ws[wid], picked[RB ? wid : 0], tot_s,
-                                                       gi, nel, rb);
+                const int32_t nout = gain_seg<Rec, RB>(d0, tile, seg, seg_end, s, ws[wid], picked[RB ? wid : 0], gi, nel,
+                                                       rb);
                 int32_t *cnt = d0.cand_cnt + (int64_t)tile * d0.nseg + seg;
                 if (RB) {
                     // the item's candidates lie together, filled segments first
@@ -782,12 +781,6 @@ __global__ void __launch_bounds__(kThreads, sizeof(Rec) == 16 || RB ? 4 : 3) k_g
         last = __shfl_sync(kFull, last, 0);
         if (last) {
             __threadfence_block();
-            if (RB) {
-                for (int t = lane; t < 64 && t < d0.k; t += 32) {
-                    const unsigned long long v = atomicAdd(&tot_s[t], 0ull);
-                    if (v) atomicAdd(reinterpret_cast<unsigned long long *>(&d0.tot[t]), v);
-                }
-            }
             if (lane == 0) {
                 unsigned long long *row = reinterpret_cast<unsigned long long *>(d0.stats + (int64_t)rr * ST_N);
                 const unsigned long long c0 = atomicAdd(&cnt_s[0], 0ull), c1 = atomicAdd(&cnt_s[1], 0ull);
@@ -840,7 +833,8 @@ __device__ __forceinline__ int refine_digit(int32_t v, int level, int64_t prefix
     return v & 1023;
 }
 
-// CTA per tile item: histogram of candidate weight by gain for saturated key blocks
+// CTA per tile item: histogram of candidate weight by digit (level 1..3) for the key blocks whose
+// threshold lies in the overflow bin
 template <int KEY = KEY_T>
 __global__ void __launch_bounds__(kThreads) k_hist(const Dev *devs, const int2 *items, int32_t n_items, int level)
 {
@@ -854,13 +848,9 @@ __global__ void __launch_bounds__(kThreads) k_hist(const Dev *devs, const int2 *
     const Dev &d = item_of(devs, items, blockIdx.x, tile);
     int a = 0;
     if (tid < d.k) {
-        if (level == 0) {
-            a = d.tot[tid] > 0 && d.tot[tid] > stage_cap<KEY>(d, tid);
-        } else {
-            const Sel sl = d.sel[tid];
-            a = sl.mode == SEL_REFINE && sl.level == level;
-            prefix[tid] = sl.g;
-        }
+        const Sel sl = d.sel[tid];
+        a = sl.mode == SEL_REFINE && sl.level == level;
+        prefix[tid] = sl.g;
     }
     if (tid < 64) active[tid] = a;
     if (!__syncthreads_or(a)) return;
@@ -876,15 +866,10 @@ __global__ void __launch_bounds__(kThreads) k_hist(const Dev *devs, const int2 *
         if (!decode_key<KEY>(d.cand[slot], key, t, g, ul) || !active[key]) continue;
         t = key;
         const unsigned long long c = d.vw ? (unsigned long long)d.vw[cand_vertex(slot, ul)] : 1ull;
-        int bin;
-        if (level == 0) {
-            bin = g < kBins - 1 ? g : kBins - 1;
-        } else {
-            if (g < kBins - 1) continue;
-            bool match;
-            bin = refine_digit(g - (kBins - 1), level, prefix[t], match);
-            if (!match) continue;
-        }
+        if (g < kBins - 1) continue;
+        bool match;
+        const int bin = refine_digit(g - (kBins - 1), level, prefix[t], match);
+        if (!match) continue;
         atomicAdd(&d.hist[(int64_t)t * kBins + bin], c);
     }
 }
@@ -918,8 +903,11 @@ __device__ __forceinline__ unsigned long long block_scan_u64(unsigned long long 
 }
 
 // one CTA per block item (instance, t): threshold of the (gain desc, id asc) prefix that fits
+// (the level-0 histogram was filled by the gain step, or by k_rb_mark for the target side; bins: how
+// many of its bins are in use, 0: Dev::bins)
 template <int KEY = KEY_T>
-__global__ void __launch_bounds__(kThreads) k_select(const Dev *devs, const int2 *items, int32_t n_items, int level)
+__global__ void __launch_bounds__(kThreads) k_select(const Dev *devs, const int2 *items, int32_t n_items, int level,
+                                                     int32_t bins)
 {
     after_previous();
     __shared__ unsigned long long wt[32];
@@ -929,42 +917,12 @@ __global__ void __launch_bounds__(kThreads) k_select(const Dev *devs, const int2
     const int tid = threadIdx.x;
     if ((int32_t)blockIdx.x >= item_count(devs, items, n_items, ITEM_BLOCK)) return;
     int32_t t;
-    const Dev d = item_of(devs, items, blockIdx.x, t);
-    Sel sl = d.sel[t];
-    long long cap;
-    int nbins;
+    const Dev &d = item_of(devs, items, blockIdx.x, t);
+    const Sel sl = d.sel[t];
+    if (level > 0 && (sl.mode != SEL_REFINE || sl.level != level)) return;
+    const int nbins = level == 0 ? (bins ? bins : d.bins) : (level == 1 ? 2048 : 1024);
+    const long long cap = level == 0 ? stage_cap<KEY>(d, t) : (long long)sl.rem;
     unsigned long long *row = d.hist + (int64_t)t * kBins;
-    if (level == 0) {
-        // LP: the gain step filled the level-0 row of every target block, the total is its sum
-        nbins = KEY == KEY_T ? d.bins : kBins;
-        long long tot = 0;
-        if (KEY == KEY_T) {
-            unsigned long long part = 0;
-            for (int b = tid; b < nbins; b += kThreads) part += row[b];
-            const unsigned long long before = block_scan_u64(part, wt);
-            if (tid == kThreads - 1) tot_s = before + part;
-            __syncthreads();
-            tot = (long long)tot_s;
-        } else {
-            tot = d.tot[t];
-        }
-        cap = stage_cap<KEY>(d, t);
-        if (tot == 0 || tot <= cap) {
-            if (KEY == KEY_T && tot)
-                for (int b = tid; b < nbins; b += kThreads) row[b] = 0;
-            if (tid == 0) {
-                Sel o;
-                o.mode = SEL_ALL; o.level = 0; o.g = 0; o.rem = 0; o.cut = 0;
-                d.sel[t] = o;
-                if (KEY != KEY_T) d.tot[t] = 0;
-            }
-            return;
-        }
-    } else {
-        if (sl.mode != SEL_REFINE || sl.level != level) return;
-        cap = sl.rem;
-        nbins = level == 1 ? 2048 : 1024;
-    }
     // thread i owns bins [nbins - per*(i+1), nbins - per*i), visited from high to low
     const int per = nbins / kThreads;
     const int hi = nbins - per * tid;
@@ -972,6 +930,21 @@ __global__ void __launch_bounds__(kThreads) k_select(const Dev *devs, const int2
     for (int b = hi - 1; b >= hi - per; --b) sum += row[b];
     if (tid == 0) { found_bin = -1; found_before = 0; }
     const unsigned long long before = block_scan_u64(sum, wt);
+    if (level == 0) {
+        if (tid == kThreads - 1) tot_s = before + sum;
+        __syncthreads();
+        const long long tot = (long long)tot_s;
+        if (tot == 0 || tot <= cap) {   // every candidate passes
+            if (sum)
+                for (int b = hi - 1; b >= hi - per; --b) row[b] = 0;
+            if (tid == 0) {
+                Sel o;
+                o.mode = SEL_ALL; o.level = 0; o.g = 0; o.rem = 0; o.cut = 0;
+                d.sel[t] = o;
+            }
+            return;
+        }
+    }
     if ((long long)before <= cap && (long long)(before + sum) > cap) {
         unsigned long long c = before;
         for (int b = hi - 1; b >= hi - per; --b) {
@@ -991,7 +964,6 @@ __global__ void __launch_bounds__(kThreads) k_select(const Dev *devs, const int2
         Sel o;
         o.cut = 0;
         if (level == 0) {
-            if (KEY != KEY_T) d.tot[t] = 0;
             if (fb < kBins - 1) {
                 o.mode = SEL_THRESH; o.level = 0; o.g = fb; o.rem = rem;
             } else {
@@ -1862,37 +1834,36 @@ __global__ void k_round_end(const Dev *devs, int32_t n_inst, int32_t rr, int32_t
 
 // Rebalancing, source side (KEY_A): persistent, a CTA per tile with a grid stride (the
 // per-block thresholds are read once per warp); marks the candidates that may leave their block
-// (bit 25) and adds their weights to the per-target totals of the target-side stage.
+// (bit 25) and counts them by target block and priority for the target-side stage.
 __global__ void __launch_bounds__(kThreads) k_rb_mark(const Dev d)
 {
     after_previous();
     __shared__ ApplyInst ai_w[kWarps];
     __shared__ SegRun run_w[kWarps];
-    __shared__ unsigned long long tot_w[kWarps][64];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     int32_t r;
     apply_refresh(d, ai_w[wid], r);
-    tot_w[wid][lane] = 0;
-    tot_w[wid][lane + 32] = 0;
-    __syncwarp();
     int32_t s0, s1;
     warp_segments(d, wid, s0, s1);
     for (int32_t tile = blockIdx.x; tile < d.n_tiles && s0 < s1; tile += gridDim.x) {
         const int32_t ncand = run_w[wid].load(d, tile, s0, s1);
-        for (int32_t i = lane; i < ncand; i += 32) {
-            const int32_t slot = run_w[wid].at(i);
-            int t;
-            int32_t u;
-            const uint64_t c = d.cand[slot];
-            if (approve<KEY_A>(c, slot, ai_w[wid], t, u)) {
-                d.cand[slot] = c | kSelBit;
-                atomicAdd(&tot_w[wid][t], d.vw ? (unsigned long long)d.vw[u] : 1ull);
+        for (int32_t i0 = 0; i0 < ncand; i0 += 32) {
+            int t = 0;
+            int32_t u = 0, g = 0, cu = 1;
+            bool pass = false;
+            if (i0 + lane < ncand) {
+                const int32_t slot = run_w[wid].at(i0 + lane);
+                const uint64_t c = d.cand[slot];
+                pass = approve<KEY_A>(c, slot, ai_w[wid], t, u);
+                g = (int32_t)(c >> 32);
+                if (pass) {
+                    d.cand[slot] = c | kSelBit;
+                    if (d.vw) cu = d.vw[u];
+                }
             }
+            count_gain(d, pass, t, g, cu);
         }
     }
-    __syncwarp();
-    for (int t = lane; t < 64 && t < d.k; t += 32)
-        if (tot_w[wid][t]) atomicAdd(reinterpret_cast<unsigned long long *>(&d.tot[t]), tot_w[wid][t]);
 }
 
 __global__ void __launch_bounds__(kThreads) k_expand_candidates(const Dev *devs, int32_t *target, int64_t *gain)
@@ -2078,12 +2049,12 @@ cudaError_t launch_round(const Plan &p, int32_t rr)
         if (e != cudaSuccess) break;
         int32_t n = 0;
         // the level-0 histogram was filled by the gain step
-        launch(k_select<KEY_T>, p.n_blocks, kThreads, p.st, p.devs, p.blocks, p.n_blocks, 0);
+        launch(k_select<KEY_T>, p.n_blocks, kThreads, p.st, p.devs, p.blocks, p.n_blocks, 0, 0);
         n += 1;
         if (p.levels) {
             for (int level = 1; level <= 3; ++level) {
                 launch(k_hist<KEY_T>, p.n_tiles, kThreads, p.st, p.devs, p.tiles, p.n_tiles, level);
-                launch(k_select<KEY_T>, p.n_blocks, kThreads, p.st, p.devs, p.blocks, p.n_blocks, level);
+                launch(k_select<KEY_T>, p.n_blocks, kThreads, p.st, p.devs, p.blocks, p.n_blocks, level, 0);
                 n += 2;
             }
         }
@@ -2406,7 +2377,6 @@ int debug_candidates(hgp_handle *h, int32_t s, int32_t *target, int64_t *gain)
     if (e == cudaSuccess) e = launch_prep(p);
     if (e == cudaSuccess) e = cudaMemsetAsync(d.wq, 0, sizeof(int32_t) * kWqPerRow, st);
     if (e == cudaSuccess) e = launch_gain(p, s, 0);
-    if (e == cudaSuccess) e = cudaMemsetAsync(d.tot, 0, sizeof(int64_t) * 64, st);
     if (e == cudaSuccess) e = cudaMemsetAsync(d.hist, 0, sizeof(unsigned long long) * (size_t)d.k * kBins, st);
     if (e == cudaSuccess) {
         k_expand_candidates<<<d.n_tiles, kThreads, 0, st>>>(h->d_dev, t_d, g_d);
@@ -2454,16 +2424,15 @@ namespace {
 
 // one approval stage over all candidates of the sub-round, grouped by KEY
 template <int KEY>
-int64_t launch_stage(const Plan &p, bool levels)
+int64_t launch_stage(const Plan &p, bool levels, int32_t bins)
 {
     int64_t n = 0;
-    launch(k_hist<KEY>, p.n_tiles, kThreads, p.st, p.devs, p.tiles, p.n_tiles, 0);
-    launch(k_select<KEY>, p.n_blocks, kThreads, p.st, p.devs, p.blocks, p.n_blocks, 0);
-    n += 2;
+    launch(k_select<KEY>, p.n_blocks, kThreads, p.st, p.devs, p.blocks, p.n_blocks, 0, bins);
+    n += 1;
     if (levels) {
         for (int level = 1; level <= 3; ++level) {
             launch(k_hist<KEY>, p.n_tiles, kThreads, p.st, p.devs, p.tiles, p.n_tiles, level);
-            launch(k_select<KEY>, p.n_blocks, kThreads, p.st, p.devs, p.blocks, p.n_blocks, level);
+            launch(k_select<KEY>, p.n_blocks, kThreads, p.st, p.devs, p.blocks, p.n_blocks, level, 0);
             n += 2;
         }
     }
@@ -2475,7 +2444,7 @@ int64_t launch_stage(const Plan &p, bool levels)
 // one rebalancing pass: S sub-rounds of gain (vertices of overloaded blocks), source-side
 // selection, target-side approval and apply, then the pass's objective and heaviest block
 template <typename Rec>
-cudaError_t launch_rebalance_pass(const Plan &p, int32_t pass, RbArgs rb, bool levels)
+cudaError_t launch_rebalance_pass(const Plan &p, int32_t pass, RbArgs rb, bool levels, int32_t bins)
 {
     launch(k_round_prep, p.n_tiles, kThreads, p.st, p.devs, p.tiles, p.n_tiles, rb.r);
     *p.launches += 1;
@@ -2483,10 +2452,10 @@ cudaError_t launch_rebalance_pass(const Plan &p, int32_t pass, RbArgs rb, bool l
         launch(k_gain<Rec, false, true>, p.grid_gain, kThreads, p.st, p.d0, p.devs, p.tiles, p.n_tiles, (p.nseg + kRbSegs - 1) / kRbSegs, 1, s,
                                                                     pass, rb);
         *p.launches += 1;
-        *p.launches += launch_stage<KEY_A>(p, levels);
+        *p.launches += launch_stage<KEY_A>(p, levels, bins);
         launch(k_rb_mark, p.grid_apply, kThreads, p.st, p.d0);
         *p.launches += 1;
-        *p.launches += launch_stage<KEY_TS>(p, levels);
+        *p.launches += launch_stage<KEY_TS>(p, levels, bins);
         launch(k_apply<Rec, false, KEY_TS>, p.grid_apply, kThreads, p.st, p.d0, p.devs, p.tiles, p.n_tiles, p.nseg, p.per, pass);
         *p.launches += 1;
     }
@@ -2533,9 +2502,11 @@ extern "C" int hgp_rebalance(hgp_handle *h, int32_t max_passes, hgp_round_stats 
         rb.r = (1 << 30) + pass;
         rb.phase = phase;
         rb.off = phase == 2 ? (int32_t)off : 0;
-        const bool levels = (phase == 2 ? 2 * off : off) >= kBins - 1;
-        e = p.rec32 ? launch_rebalance_pass<Rec32>(p, pass, rb, levels)
-                    : launch_rebalance_pass<Rec16>(p, pass, rb, levels);
+        const int64_t top = phase == 2 ? 2 * off : off;   // largest priority
+        const bool levels = top >= kBins - 1;
+        const int32_t bins = (int32_t)std::min<int64_t>(kBins, (top + kThreads) / kThreads * kThreads);
+        e = p.rec32 ? launch_rebalance_pass<Rec32>(p, pass, rb, levels, bins)
+                    : launch_rebalance_pass<Rec16>(p, pass, rb, levels, bins);
         int64_t appr = 0;
         if (e == cudaSuccess)
             e = cudaMemcpyAsync(&appr, h->d.stats + (int64_t)pass * ST_N + ST_APPR, sizeof(int64_t),

@@ -1383,7 +1383,7 @@ size_t small_handle_bytes(int32_t n, int32_t m, int64_t P, int32_t k, const hgp_
     b += A(4 * ((int64_t)n + 1)) + A(4 * P);                                         // vtx_off, inc
     b += 2 * A(n) + A(4 * (((int64_t)m * k * w + 7) / 8 * 2)) + A((int64_t)m * (k <= 32 ? 16 : 32)) + A(8 * kSmallN);
     b += A(2 * n_tiles * kTile) + A(2 * n_tiles * (S + 1)) + A(8 * n_tiles * kTile) + A(4 * n_tiles * nseg);
-    b += A(8 * 64) + A(8 * (int64_t)k * kBins) + A((int64_t)sizeof(Sel) * 64) + A(8 * (int64_t)k * n_tiles);
+    b += A(8 * (int64_t)k * kBins) + A((int64_t)sizeof(Sel) * 64) + A(8 * (int64_t)k * n_tiles);
     if (o.revert_negative) {
         int64_t cap = 1024;
         while (cap < 2 * P) cap <<= 1;
@@ -1749,24 +1749,21 @@ int create_impl(int32_t n, int32_t m, const int64_t *net_offsets, const int32_t 
     uint16_t *sub_list = nullptr, *sub_start = nullptr;
     uint64_t *cand = nullptr;
     int32_t *cand_cnt = nullptr;
-    int64_t *tot = nullptr, *tie = nullptr;
+    int64_t *tie = nullptr;
     unsigned long long *hist = nullptr;
     Sel *sel = nullptr;
     CKF(dalloc(h, &sub_list, (int64_t)d.n_tiles * kTile));
     CKF(dalloc(h, &sub_start, (int64_t)d.n_tiles * (d.S + 1)));
     CKF(dalloc(h, &cand, (int64_t)d.n_tiles * kTile));
     CKF(dalloc(h, &cand_cnt, (int64_t)d.n_tiles * d.nseg));
-    CKF(dalloc(h, &tot, 64));
     CKF(dalloc(h, &hist, (int64_t)k * kBins));
     CKF(dalloc(h, &sel, 64));
     CKF(dalloc(h, &tie, (int64_t)k * d.n_tiles));
-    CKF(cudaMemsetAsync(tot, 0, sizeof(int64_t) * 64, st));
     CKF(cudaMemsetAsync(hist, 0, sizeof(unsigned long long) * (size_t)k * kBins, st));
     d.sub_list = sub_list;
     d.sub_start = sub_start;
     d.cand = cand;
     d.cand_cnt = cand_cnt;
-    d.tot = tot;
     d.hist = hist;
     d.sel = sel;
     d.tie = tie;
