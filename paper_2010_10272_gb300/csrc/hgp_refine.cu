@@ -339,7 +339,7 @@ __device__ __forceinline__ void lane_best(const Rec *recs, const int32_t *inc, i
                                           const GainWarp &g, int32_t cu, Lam kall, int32_t eq_value, Nets<Lam> &x,
                                           Lam &T_all, Lam &T, int &t_out, int32_t &conn_out, Lam &eq_out)
 {
-    constexpr int kAhead = RB ? 2 : 3;
+    constexpr int kAhead = RB || (COH && sizeof(Lam) == 8) ? 2 : 3;   // by registers
     Lam c[NP];
 #pragma unroll
     for (int p = 0; p < NP; ++p) c[p] = 0;

@@ -7,8 +7,8 @@
 // between the launches of the general path stays on the chip:
 //   * a warp owns a contiguous range of vertices, hashes its sub-rounds once per round, and keeps
 //     its candidates in shared memory between the gain and the apply step;
-//   * the vertices' blocks, weights and list offsets are kept in shared memory, and as much of the
-//     lists as fits: a cluster barrier drops the L1 lines, so each of them would cost an L2 round
+//   * the vertices' blocks, weights and list offsets are kept in shared memory, and the lists
+//     where they fit: a cluster barrier drops the L1 lines, so each of them would cost an L2 round
 //     trip in every phase (10k vertices 255 -> 239 us a call, 30k 381 -> 373 us);
 //   * block weights are a copy per CTA, updated through distributed shared memory;
 //   * the approval is a radix select on the key (gain desc, id asc): the candidates' weights are
@@ -29,9 +29,9 @@ constexpr int kSmRow = kSmBins + kSmBins / 16;       // padded: a lane sums 16 c
 constexpr int kSmIdBits = 2 * kSmDigit;
 constexpr int32_t kSmMaxN = 1 << kSmIdBits;
 // Instances that run this way.  Its time grows with the pins (16 SMs), that of the launches hardly
-// does at this size.  5 rounds, planted, k = 4: 286 / 362 / 487 / 605 us at 90 / 180 / 360 / 540
-// thousand pins against 526-553 us; row-net, k = 64: 470 / 653 / 951 us at 150 / 300 / 600 thousand
-// against 797-855 us.
+// does at this size.  5 rounds, planted, k = 4: 264 / 344 / 469 us at 90 / 180 / 360 thousand pins
+// against 522-526 us; power-law, k = 16: 360 / 470 / 632 us at 91 / 185 / 369 thousand against
+// 659-686 us; k = 64, 64-bit masks: 412 / 520 / 704 us at 87 / 178 / 358 thousand against 706-736 us.
 constexpr int32_t kSmallVertices = 1 << 17;
 constexpr int32_t kSmallPins = 7 << 16, kSmallPinsWide = 11 << 15;   // 459k for k <= 32, 360k for k > 32
 constexpr int kSmPerHome = (64 + kSmCtas - 1) / kSmCtas;
@@ -49,6 +49,9 @@ __host__ __device__ inline int small_warp_bytes(int per_warp, bool cached, bool 
     return per_warp * (8 + 2 + 1) + (cached ? (per_warp + 2) * 4 + per_warp * (1 + 4 * vw + 4 * nw) : 0) + 7 & ~7;
 }
 constexpr int kSmMaxBytes = 226 << 10;   // dynamic shared memory of a CTA
+// lists are copied only where all fit and this leaves enough L1 for the rest (with the copy filling
+// all of it, 60k vertices and k = 64 took 843 us instead of 704)
+constexpr int kSmListBytes = 150 << 10;
 
 struct SmallShared {
     unsigned long long row[kSmPerHome][kSmRow];   // home CTA: weight per key digit of a block
@@ -410,9 +413,9 @@ inline cudaLaunchConfig_t small_config(const Dev &d, cudaStream_t st, cudaLaunch
         return (int)sizeof(SmallShared) + kSmWarps * small_warp_bytes(per_warp, c, d.vw != nullptr, d.nw != nullptr);
     };
     cached = bytes(true) <= kSmMaxBytes;
-    // the lists of a CTA's vertices, twice their average, as far as they fit
+    // the lists of a CTA's vertices, twice their average
     const int64_t want = 2 * ((int64_t)d.P / kSmCtas + 256);
-    inc_room = cached ? (int32_t)std::min<int64_t>(want, (kSmMaxBytes - bytes(true)) / 4) : 0;
+    inc_room = cached && bytes(true) + 4 * want <= kSmListBytes ? (int32_t)want : 0;
     cfg.dynamicSmemBytes = (size_t)bytes(cached) + 4 * (size_t)inc_room;
     cfg.stream = st;
     at->id = cudaLaunchAttributeClusterDimension;
