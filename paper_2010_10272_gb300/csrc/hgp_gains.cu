@@ -39,6 +39,8 @@ __device__ __forceinline__ uint64_t slot_hash(uint64_t key) { return splitmix64_
 
 // find or insert (linear probing; the table is at most two thirds full, so a free slot exists).
 // cur: the key at the first position, already loaded.
+// Keys are read through L1: one that is there never changes, and a free slot read too late is settled by
+// the compare-and-swap (the slots of a large net are read by every move of its pins).
 __device__ __forceinline__ Slot *find_slot(Slot *table, uint64_t mask, uint64_t p, unsigned long long cur,
                                            unsigned long long key, bool insert)
 {
@@ -51,7 +53,7 @@ __device__ __forceinline__ Slot *find_slot(Slot *table, uint64_t mask, uint64_t 
             if (cur == kEmpty || cur == key) return s;
         }
         p = (p + 1) & mask;
-        cur = __ldcg(&table[p].key);
+        cur = table[p].key;
     }
     return nullptr;
 }
@@ -62,7 +64,7 @@ __device__ __forceinline__ void find_both(Slot *table, uint64_t mask, unsigned l
 {
     const unsigned long long ka = e * 64 + a, kb = e * 64 + b;
     const uint64_t pa = slot_hash(ka) & mask, pb = slot_hash(kb) & mask;
-    const unsigned long long ca = __ldcg(&table[pa].key), cb = __ldcg(&table[pb].key);
+    const unsigned long long ca = table[pa].key, cb = table[pb].key;
     sa = find_slot(table, mask, pa, ca, ka, insert);
     sb = find_slot(table, mask, pb, cb, kb, insert);
 }
@@ -86,10 +88,16 @@ __global__ void k_eg_check(Dev d, const int32_t *moves, int32_t count, int32_t *
     if ((threadIdx.x & 31) == 0 && s) atomicAdd(&out[1], s);
 }
 
+// Up to this many moves (all of whose warps run at once) a warp takes one each: the chain of dependent
+// accesses per 32 incidences is what a short sequence waits for (5k moves of 4 nets, 8 per warp: 144
+// us, one: 119 us).
+constexpr int kEgWarps = 152 * 32;
+constexpr uint64_t kEgDense = 1 << 20;   // slots (32 MB) from which a table may be two thirds full
+
 // `per` (at most 32) moves of a warp, about 32 incidences in all, one run that the lanes walk
 // flattened (a warp per move left most lanes idle, 6 nets of 32; 32 moves per warp were as slow, too
 // few warps for the chains of dependent accesses).  100k moves of 6 nets each, the whole call: 295 ->
-// 253 us, of which the host copies and waits are about 110.
+// 253 us, of which the host copies and waits are about 100; 218 us with keys read through L1.
 struct MoveWarp {
     int32_t off[33];
     int32_t jb[32];
@@ -210,18 +218,20 @@ extern "C" int hgp_exact_gains(hgp_handle *h, int32_t count, const int32_t *move
     if (count == 0) return HGP_OK;
     Dev &d = h->d;
     cudaStream_t st = h->stream;
-    int32_t *mv = nullptr, *seen = nullptr;
-    unsigned long long *out = nullptr;   // error, degree sum
     Slot *table = nullptr;
-    int64_t *g_d = nullptr;
+    char *buf = nullptr;
     unsigned long long host[2] = {0, 0};
     int rc = HGP_OK;
-    cudaError_t e = dev_alloc(reinterpret_cast<void **>(&mv), sizeof(int32_t) * 3 * (size_t)count, st);
+    // one buffer (five took 10 us more): error and degree sum, seen flags (both zeroed), gains, moves
+    const size_t zero_bytes = (sizeof(host) + sizeof(int32_t) * (size_t)d.n + 15) / 16 * 16;
+    const size_t g_bytes = sizeof(int64_t) * (size_t)count;
+    cudaError_t e = dev_alloc(reinterpret_cast<void **>(&buf), zero_bytes + g_bytes + sizeof(int32_t) * 3 * (size_t)count, st);
+    unsigned long long *out = reinterpret_cast<unsigned long long *>(buf);
+    int32_t *seen = reinterpret_cast<int32_t *>(buf + sizeof(host));
+    int64_t *g_d = reinterpret_cast<int64_t *>(buf + zero_bytes);
+    int32_t *mv = reinterpret_cast<int32_t *>(buf + zero_bytes + g_bytes);
     if (e == cudaSuccess) e = cudaMemcpyAsync(mv, moves, sizeof(int32_t) * 3 * (size_t)count, cudaMemcpyHostToDevice, st);
-    if (e == cudaSuccess) e = dev_alloc(reinterpret_cast<void **>(&seen), sizeof(int32_t) * ((size_t)d.n + 1), st);
-    if (e == cudaSuccess) e = dev_alloc(reinterpret_cast<void **>(&out), sizeof(host), st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(seen, 0, sizeof(int32_t) * ((size_t)d.n + 1), st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(out, 0, sizeof(host), st);
+    if (e == cudaSuccess) e = cudaMemsetAsync(buf, 0, zero_bytes, st);
     if (e == cudaSuccess) {
         k_eg_check<<<grid_of(count, 256), 256, 0, st>>>(d, mv, count, seen, out);
         h->launches += 1;
@@ -230,14 +240,15 @@ extern "C" int hgp_exact_gains(hgp_handle *h, int32_t count, const int32_t *move
     if (e == cudaSuccess) e = cudaMemcpyAsync(host, out, sizeof(host), cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = stream_wait(st);
     if (e == cudaSuccess && host[0]) rc = HGP_ERR_INVALID;
-    // at most 2 keys per incident net of a moved vertex; the table is at most two thirds full
+    // at most 2 keys per incident net of a moved vertex; the table is at most half full while it is small
+    // (long runs of probes are what few moves wait for: 5.4k moves 114 -> 96 us), two thirds above
     uint64_t size = 64;
-    while (size < 3 * (uint64_t)host[1]) size <<= 1;
+    while (size < (size < kEgDense ? 4 : 3) * (uint64_t)host[1]) size <<= 1;
     if (e == cudaSuccess && rc == HGP_OK) e = dev_alloc(reinterpret_cast<void **>(&table), sizeof(Slot) * size, st);
-    if (e == cudaSuccess && rc == HGP_OK) e = dev_alloc(reinterpret_cast<void **>(&g_d), sizeof(int64_t) * (size_t)count, st);
     if (e == cudaSuccess && rc == HGP_OK) e = cudaMemsetAsync(table, 0xFF, sizeof(Slot) * size, st);
     if (e == cudaSuccess && rc == HGP_OK) {
-        const int per = (int)std::min<uint64_t>(32, std::max<uint64_t>(1, 32 * (uint64_t)count / std::max<uint64_t>(1, host[1])));
+        const uint64_t fit = 32 * (uint64_t)count / std::max<uint64_t>(1, host[1]);   // moves of 32 incidences
+        const int per = (int)std::max<uint64_t>(1, std::min<uint64_t>({32, fit, (uint64_t)count / kEgWarps}));
         const int grid = grid_of(((int64_t)count + per - 1) / per * 32, 256);
         k_eg_pass1<<<grid, 256, 0, st>>>(d, mv, count, per, table, size - 1, out);
         k_eg_pass2<<<grid, 256, 0, st>>>(d, mv, count, per, table, size - 1, g_d);
@@ -245,12 +256,9 @@ extern "C" int hgp_exact_gains(hgp_handle *h, int32_t count, const int32_t *move
         e = cudaGetLastError();
     }
     if (e == cudaSuccess && rc == HGP_OK) e = cudaMemcpyAsync(host, out, sizeof(host), cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess && rc == HGP_OK) e = cudaMemcpyAsync(gains, g_d, sizeof(int64_t) * (size_t)count, cudaMemcpyDeviceToHost, st);
-    if (mv) pool_free(mv, st);
-    if (seen) pool_free(seen, st);
-    if (out) pool_free(out, st);
+    if (e == cudaSuccess && rc == HGP_OK) e = cudaMemcpyAsync(gains, g_d, g_bytes, cudaMemcpyDeviceToHost, st);
+    if (buf) pool_free(buf, st);
     if (table) pool_free(table, st);
-    if (g_d) pool_free(g_d, st);
     const cudaError_t e2 = stream_wait(st);
     if (e == cudaSuccess) e = e2;
     if (e != cudaSuccess) {
