@@ -205,10 +205,14 @@ __global__ void k_ct_narrow(const unsigned long long *w64, int64_t len, int32_t 
 
 // ---------------------------------------------------------------- per-net sort + dedupe
 // Fingerprint of a sorted, de-duplicated pin list: the sum of a 64-bit mix of every pin
-// (independent of how the pins are split over threads), mixed with the list's length.
+// (independent of how the pins are split over threads), mixed with the list's length.  Nets with equal
+// fingerprints are compared, so the mix of a pin is a short one: two odd multipliers, the upper half
+// folded into the lower after each.
 __device__ __forceinline__ unsigned long long pin_mix(int32_t v)
 {
-    return splitmix64_output(0x6a09e667f3bcc908ull ^ (uint64_t)(uint32_t)v);
+    uint64_t x = (uint64_t)((uint32_t)v + 1u) * 0x9e3779b97f4a7c15ull;
+    x = (x ^ (x >> 32)) * 0xd1342543de82ef95ull;
+    return x ^ (x >> 32);
 }
 
 __device__ __forceinline__ unsigned long long key_final(unsigned long long h, int32_t s)
@@ -235,11 +239,16 @@ constexpr int kClasses = 4;   // listed classes: 9..32, 33..kMid, kMid+1..kMediu
 
 // thread per net: nets of at most kTiny pins are sorted in registers (an unrolled sorting
 // network), de-duplicated and fingerprinted; larger nets go to the lists of the warp (9..32 pins,
-// ..kMid), CTA (..kMedium) and chunked (larger) kernels
-__global__ void k_ct_tiny(const int64_t *off, const int32_t *pins, int32_t m, const int32_t *map, int32_t *a,
-                          int32_t *size1, unsigned long long *key, int32_t *rep, int32_t *lists, int32_t *counts)
+// ..kMid), CTA (..kMedium) and chunked (larger) kernels.  A CTA reserves its places in a list with one
+// atomic (one per warp: 800k returning atomics on one sector for 10M nets, and this kernel 464 us
+// instead of 240).
+__global__ void __launch_bounds__(256) k_ct_tiny(const int64_t *off, const int32_t *pins, int32_t m,
+                                                 const int32_t *map, int32_t *a, int32_t *size1,
+                                                 unsigned long long *key, int32_t *rep, int32_t *lists,
+                                                 int32_t *counts)
 {
-    const int lane = threadIdx.x & 31;
+    __shared__ int32_t n_of[kClasses][8], at[kClasses];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     for (int64_t e0 = blockIdx.x * (int64_t)blockDim.x; e0 < m; e0 += (int64_t)gridDim.x * blockDim.x) {
         const int64_t e = e0 + threadIdx.x;
         int cls = -1;
@@ -274,24 +283,37 @@ __global__ void k_ct_tiny(const int64_t *off, const int32_t *pins, int32_t m, co
                 cls = s <= 32 ? 0 : (s <= kMid ? 1 : (s <= kMedium ? 2 : 3));
             }
         }
-        // warp-aggregated append of the larger nets to their class lists
+        // append of the larger nets to their class lists
+        unsigned mine = 0;
 #pragma unroll
         for (int c = 0; c < kClasses; ++c) {
             const unsigned mk = __ballot_sync(kFull, cls == c);
-            if (!mk) continue;
-            int32_t base = 0;
-            if (lane == __ffs(mk) - 1) base = atomicAdd(&counts[c], __popc(mk));
-            base = __shfl_sync(kFull, base, __ffs(mk) - 1);
-            if (cls == c) lists[(int64_t)c * m + base + __popc(mk & ((1u << lane) - 1))] = (int32_t)e;
+            if (cls == c) mine = mk;
+            if (lane == 0) n_of[c][wid] = __popc(mk);
         }
+        __syncthreads();
+        if (threadIdx.x < kClasses) {
+            int32_t total = 0;
+#pragma unroll
+            for (int w = 0; w < 8; ++w) {
+                const int32_t x = n_of[threadIdx.x][w];
+                n_of[threadIdx.x][w] = total;
+                total += x;
+            }
+            at[threadIdx.x] = total ? atomicAdd(&counts[threadIdx.x], total) : 0;
+        }
+        __syncthreads();
+        if (cls >= 0)
+            lists[(int64_t)cls * m + at[cls] + n_of[cls][wid] + __popc(mine & ((1u << lane) - 1))] = (int32_t)e;
+        __syncthreads();   // the counts are used again
     }
 }
 
 // Bitonic sort of 32 K values, K per lane in registers: ascending in the order lane * K + i.  Pairs
 // closer than K are in the lane, the others come by shuffle; no shared memory and no barriers
 // (sorting in shared memory, two accesses and a barrier per step, took 346 us for the nets of
-// 33..256 pins and 584 us for those of 257..2048 of a 10M-net power-law instance; 280 us for 33..512
-// and 138 for 513..2048 now).
+// 33..256 pins and 584 us for those of 257..2048 of a 10M-net power-law instance; 244 us for 33..512
+// and 135 for 513..2048 now).
 template <int K>
 __device__ __forceinline__ void warp_sort(int32_t (&v)[K])
 {
