@@ -14,10 +14,11 @@
 //                  ties to the smaller block; only blocks in the union of Lambda(e) over the
 //                  nets with Phi(e,a) = 1 can have positive gain (g_i <= omega of those nets
 //                  that contain i), so only those are evaluated.
-//   k_hist/k_select   per target block t whose candidates do not all fit (w(t) + sum c > L_max):
-//                  histogram of candidate weight by gain, scanned from the highest gain to
-//                  find the threshold gain G_t and the budget left for candidates with
-//                  gain == G_t (approval order (gain desc, id asc), inclusive prefix sums).
+//   k_select       per target block t whose candidates do not all fit (w(t) + sum c > L_max): the
+//                  histogram of candidate weight by gain, filled by k_gain, scanned from the
+//                  highest gain to find the threshold gain G_t and the budget left for
+//                  candidates with gain == G_t (approval order (gain desc, id asc), inclusive
+//                  prefix sums); k_hist refines gains beyond the histogram.
 //   k_tie_sum/k_tie_cut   per tile weight of the gain == G_t candidates, then the vertex id up to
 //                  which they fit the remaining budget (ties are approved in id order).
 //   k_apply        applies every approved move: Pi(u) = t, block weights, Phi(e,a)--,
@@ -26,10 +27,13 @@
 //                  the matching bit, so the final bits are right whatever the order).
 //   k_round_end    per-round objective and heaviest block; advances the device round state.
 //
+// A small instance runs all of this as one thread-block cluster in one launch (hgp_small.cuh).
+//
 // Every kernel takes the instance state as `const Dev *devs` in device memory and a list of
-// work items.  A single-handle launch passes items == nullptr: item i is the handle's own
-// tile / block i.  A batch launch passes (instance, local index) pairs covering many
-// handles at once, so one launch per phase refines a whole batch.
+// work items (k_gain and k_apply of one handle take the state as a parameter).  A single-handle
+// launch passes items == nullptr: item i is the handle's own tile / block i.  A batch launch passes
+// (instance, local index) pairs covering many handles at once, so one launch per phase refines a
+// whole batch.
 #include <cuda_runtime.h>
 #include <stddef.h>
 #include <stdint.h>
@@ -329,11 +333,12 @@ __device__ __forceinline__ Lam with_room(Lam T, const GainWarp &g, int32_t cu)
 // every block of Lambda(e) is a ripple-carry addition on whole bitsets, O(NP) word operations
 // whatever the number of blocks.  W(u) is known from creation, so NP is too (conn_t <= W(u) <
 // 2^NP).  kAhead records are in flight per lane, and the net ids of the next ones (32-byte records, 3
-// ahead on 3 CTAs per SM: 30.2 ms per power-law step, 2 on 4: 31.8, 4 on 3: 32.0, 1 on 4: 34.0).  Then the block of T with room with the largest
-// conn_t (smallest id among equals).  Against incidences spread over the lanes (a binary search
+// ahead on 3 CTAs per SM: 30.2 ms per power-law step, 2 on 4: 31.8, 4 on 3: 32.0, 1 on 4: 34.0).
+// Then the block of T with room with the largest conn_t (smallest id among equals).  Against incidences spread over the lanes (a binary search
 // and three shared-memory atomics each, (Lambda, omega) kept for a second pass over the nets):
-// row-net 2M, k = 8, records in L2: 93 -> 56 us per launch of 5 M gathers; power-law 50M, k = 64,
-// bound by random sectors from DRAM: 1.77 -> 1.65 ms per launch of 86 M.
+// row-net 2M, k = 8, records in L2: 93 -> 56 us per launch of 5 M gathers (47 with full segments and
+// overlapped launches); power-law 50M, k = 64, bound by random sectors from DRAM: 1.77 -> 1.65 ms per
+// launch of 86 M (1.53 with the net ids loaded ahead).
 template <typename Lam, typename Rec, int NP, bool UNIT, bool RB, bool COH>
 __device__ __forceinline__ void lane_best(const Rec *recs, const int32_t *inc, int32_t jb, int32_t je, int a, int32_t r,
                                           const GainWarp &g, int32_t cu, Lam kall, int32_t eq_value, Nets<Lam> &x,
@@ -1417,8 +1422,9 @@ __device__ __forceinline__ void apply_segs(const Dev &d, int32_t tile, int32_t s
 // it applies them over their incidences flattened across the lanes, so all atomics are in flight
 // at once.  (In a saturated sub-round a fifth of the candidates is approved: without the queue a
 // chunk had 6 moves and 40 of the 128 pins it can have in flight.  Row-net 2M 35 -> 32 us per
-// launch, power-law 50M 1.05 -> 0.98 ms; the queue with one candidate decided per lane at a time,
-// a chain of loads for every 32, was slower than no queue, 42 us and 1.19 ms.)
+// launch, power-law 50M 1.05 -> 0.98 ms, and 26 us and 0.73 ms since tiny nets, phi_move and stamps
+// by reductions; the queue with one candidate decided per lane at a time, a chain of loads for every
+// 32, was slower than no queue, 42 us and 1.19 ms.)
 // B as for k_gain.
 template <typename Rec, bool B, int KEY = KEY_T>
 __global__ void __launch_bounds__(kThreads, B ? 3 : 4) k_apply(const Dev d0, const Dev *devs, const int2 *items,
@@ -1562,8 +1568,9 @@ __global__ void __launch_bounds__(kThreads, B ? 3 : 4) k_apply(const Dev d0, con
 // move.  The apply step counts the movers of every net and the moved incidences of nets with
 // several movers; INSERT records max out, min in and |in| of those nets' (e, i) in an
 // open-addressing table sized to that count, EVAL sums the terms per move and marks the moves
-// whose sum is negative, and the revert step moves those back (Sec. 6).  Balance holds after it: each block's approval was
-// checked against its weight at the start of the sub-round, without credit for departures.
+// whose sum is negative, and the revert step moves those back (Sec. 6).  Balance holds after it: each
+// block's approval was checked against its weight at the start of the sub-round, without credit for
+// departures.
 struct alignas(16) RvSlot {
     unsigned long long key;   // e * 64 + i, kRvEmpty when free
     int32_t max_out;          // largest id of a mover that left block i (a pin of e), -1 if none
@@ -1584,13 +1591,14 @@ __device__ __forceinline__ uint64_t rv_slots(const Dev &d)
     return c;
 }
 
-// find (or insert) key by linear probing; at most `mask + 1` probes
-__device__ __forceinline__ RvSlot *rv_find(RvSlot *tab, uint64_t mask, unsigned long long key, bool insert)
+// find (or insert) key by linear probing from p, whose key is cur; at most `mask + 1` probes.  Keys are
+// read through L1: one that is there stays, and a free slot read too late is settled by the
+// compare-and-swap (the slots of a large net are read by all its movers).
+__device__ __forceinline__ RvSlot *rv_find(RvSlot *tab, uint64_t mask, uint64_t p, unsigned long long cur,
+                                           unsigned long long key, bool insert)
 {
-    uint64_t p = splitmix64_output(key) & mask;
     for (uint64_t probe = 0; probe <= mask; ++probe) {
         RvSlot *sl = tab + p;
-        unsigned long long cur = __ldcg(&sl->key);
         if (cur == key) return sl;
         if (cur == kRvEmpty) {
             if (!insert) return nullptr;
@@ -1598,25 +1606,33 @@ __device__ __forceinline__ RvSlot *rv_find(RvSlot *tab, uint64_t mask, unsigned 
             if (cur == kRvEmpty || cur == key) return sl;
         }
         p = (p + 1) & mask;
+        cur = tab[p].key;
     }
     return nullptr;
 }
 
+// the slots of (e, a) and (e, b); the first probes of both are in flight together
+__device__ __forceinline__ void rv_find_both(RvSlot *tab, uint64_t mask, int32_t e, int a, int b, bool insert,
+                                             RvSlot *&sa, RvSlot *&sb)
+{
+    const unsigned long long ka = (unsigned long long)e * 64 + a, kb = (unsigned long long)e * 64 + b;
+    const uint64_t pa = splitmix64_output(ka) & mask, pb = splitmix64_output(kb) & mask;
+    const unsigned long long ca = tab[pa].key, cb = tab[pb].key;
+    sa = rv_find(tab, mask, pa, ca, ka, insert);
+    sb = rv_find(tab, mask, pb, cb, kb, insert);
+}
+
+// half a slot per thread, so that a warp's store is one run and not every second 16 bytes of two.  With
+// this and the two changes above the revert launches of 5 rounds take 2.33 instead of 2.59 ms (power-law
+// 3M, k = 32), 27.8 instead of 30.5 (50M, k = 64).
 __global__ void k_rv_clear(const Dev d)
 {
     after_previous();
-    const uint64_t n = rv_slots(d);
-    RvSlot *tab = reinterpret_cast<RvSlot *>(d.rv_tab);
+    const uint64_t n = 2 * rv_slots(d);
+    int4 *tab = reinterpret_cast<int4 *>(d.rv_tab);
     for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < n;
-         i += (uint64_t)gridDim.x * blockDim.x) {
-        RvSlot sl;
-        sl.key = kRvEmpty;
-        sl.max_out = -1;
-        sl.min_in = 0x7fffffff;
-        sl.n_in = 0;
-        sl.pad[0] = sl.pad[1] = sl.pad[2] = 0;
-        tab[i] = sl;
-    }
+         i += (uint64_t)gridDim.x * blockDim.x)
+        tab[i] = i & 1 ? make_int4(0, 0, 0, 0) : make_int4(-1, -1, -1, 0x7fffffff);   // n_in; key, max_out, min_in
 }
 
 struct alignas(16) RvWarp {
@@ -1627,8 +1643,8 @@ struct alignas(16) RvWarp {
 
 enum { RV_INSERT = 0, RV_EVAL = 1 };
 
-// CTA per tile, a run of its segments per warp: the approved movers of each 32 candidates, their incidences flattened over
-// the lanes, one of the passes above per launch.
+// CTA per tile, a run of its segments per warp: the approved movers of each 32 candidates, their
+// incidences flattened over the lanes, one of the passes above per launch.
 template <typename Rec, int PASS>
 __global__ void __launch_bounds__(kThreads) k_rv_pass(const Dev d)
 {
@@ -1685,8 +1701,8 @@ __global__ void __launch_bounds__(kThreads) k_rv_pass(const Dev d)
             const int32_t av = rw.w.a[v], bv = rw.w.t[v], uv = rw.u[v];
             if (PASS == RV_INSERT) {
                 if (movers < 2) continue;
-                RvSlot *s_a = rv_find(tab, mask, (unsigned long long)ee * 64 + av, true);
-                RvSlot *s_b = rv_find(tab, mask, (unsigned long long)ee * 64 + bv, true);
+                RvSlot *s_a, *s_b;
+                rv_find_both(tab, mask, ee, av, bv, true, s_a, s_b);
                 if (!s_a || !s_b) {
                     lost = true;
                     continue;
@@ -1705,8 +1721,8 @@ __global__ void __launch_bounds__(kThreads) k_rv_pass(const Dev d)
                     if (pa == 0) g += w;
                     if (pb == 1) g -= w;
                 } else {
-                    const RvSlot *s_a = rv_find(tab, mask, (unsigned long long)ee * 64 + av, false);
-                    const RvSlot *s_b = rv_find(tab, mask, (unsigned long long)ee * 64 + bv, false);
+                    RvSlot *s_a, *s_b;
+                    rv_find_both(tab, mask, ee, av, bv, false, s_a, s_b);
                     if (!s_a || !s_b) {
                         lost = true;
                         continue;
@@ -1724,8 +1740,8 @@ __global__ void __launch_bounds__(kThreads) k_rv_pass(const Dev d)
     if (lost) atomicOr(d.err, ERR_TABLE);
 }
 
-// CTA per tile, a run of its segments per warp: the marked moves go back to their source blocks (Phi, Lambda, S1, block
-// weights, objective as in the apply step; the nets keep their round-r stamps).  Resets the
+// CTA per tile, a run of its segments per warp: the marked moves go back to their source blocks (Phi,
+// Lambda, S1, block weights, objective as in the apply step; the nets keep their round-r stamps).  Resets the
 // sub-round's moved-incidence count for the next sub-round.
 template <typename Rec>
 __global__ void __launch_bounds__(kThreads) k_rv_revert(const Dev d, int32_t rr)
@@ -2154,8 +2170,8 @@ Plan single_plan(hgp_handle *h)
 }
 
 // Whether a handle's rounds run as one cluster (hgp_small.cuh): instances of up to kSmallVertices
-// vertices and kSmallPins pins on a device that can hold the cluster.  Per-phase profiling and the revert variant take
-// the launches of the general path.
+// vertices and kSmallPins pins on a device that can hold the cluster.  Per-phase profiling and the
+// revert variant take the launches of the general path.
 bool small_plan(const Plan &p, int device, int32_t debug)
 {
     if (p.prof || p.revert || p.tiles || p.d0.n > kSmallVertices || (debug & 32)) return false;
