@@ -1216,14 +1216,14 @@ cudaError_t library_pool(cudaMemPool_t *out)
         // keep up to 1/64 of the device's memory (4.4 GB of 284) between handles: mapping it
         // afresh and unmapping it at the next synchronisation took as long as the work itself
         // (creating and closing a 5M-vertex level 6.4 -> 3.6 ms, a 500k-pin request 457 -> 261
-        // us, contraction of 10M vertices 10.4 -> 6.8 ms).  Memory freed on another stream is only
-        // reused once it is free there, never by making a stream wait for the other.
+        // us, contraction of 10M vertices 10.4 -> 6.8 ms).  The reuse policies stay at their defaults:
+        // when no more memory can be mapped, memory whose release is still queued on another stream
+        // is taken, and the allocating stream waits for that release (a handle created on a nearly
+        // full device while a destroyed one's rounds still run).
         size_t free_b = 0, total_b = 0;
         uint64_t keep = 0;
         if (cudaMemGetInfo(&free_b, &total_b) == cudaSuccess) keep = total_b / kPoolKeepShare;
-        int no = 0;
-        if (cudaMemPoolSetAttribute(g_pool[dev], cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess ||
-            cudaMemPoolSetAttribute(g_pool[dev], cudaMemPoolReuseAllowInternalDependencies, &no) != cudaSuccess)
+        if (cudaMemPoolSetAttribute(g_pool[dev], cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess)
             (void)cudaGetLastError();
         g_pool_ready[dev].store(g_pool[dev], std::memory_order_release);
     }

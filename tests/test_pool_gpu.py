@@ -1,0 +1,43 @@
+"""The library's memory pool: memory whose release is pending, and memory used before."""
+import gc
+
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+def _default_retention():
+    from paper_2010_10272_gb300.native import set_pool_retention
+    set_pool_retention(torch.cuda.mem_get_info()[1] // 64)
+
+
+def test_create_waits_for_a_pending_release_on_another_stream():
+    """On a nearly full device, a handle created while the rounds of a destroyed one still run takes
+    that one's memory once it is released, instead of failing."""
+    from paper_2010_10272_gb300 import HGP
+    from paper_2010_10272_gb300.native import set_pool_retention
+    n = m = 12_000_000                       # a handle of 1.1 GB, 0.6 more while it is created
+    dev = torch.device("cuda")
+    off = torch.arange(0, 4 * m + 1, 4, dtype=torch.int64, device=dev)
+    step = torch.tensor([0, 7, 11, 19], device=dev)
+    pins = ((torch.arange(m, device=dev)[:, None] + step) % n).sort(1)[0].to(torch.int32).reshape(-1).contiguous()
+    part = (torch.arange(n, device=dev) % 16).to(torch.int32)
+    try:
+        set_pool_retention(0)
+        a = HGP(n, m, off, pins, 16, 0.03, part, device=True, graph=1)
+        want = a.refine(2)
+        torch.cuda.synchronize()
+        gc.collect()
+        torch.cuda.empty_cache()
+        rest = torch.empty(torch.cuda.mem_get_info()[0] - (850 << 20), dtype=torch.uint8, device=dev)
+        a.refine(800, stats=False)           # one graph launch of about 0.4 s, still running below
+        a.close()
+        b = HGP(n, m, off, pins, 16, 0.03, part, device=True)
+        assert np.array_equal(b.refine(2), want)
+        b.close()
+    finally:
+        rest = None                          # noqa: F841
+        torch.cuda.empty_cache()
+        _default_retention()
