@@ -381,6 +381,9 @@ int hgp_coarse_copy_to_host(const hgp_coarse *c, int64_t *net_off, int32_t *pins
                             int32_t *net_w, int32_t *map);
 /* fine_part[u] = coarse_part[map[u]] (device int32 arrays of n' and n entries). */
 int hgp_coarse_project(const hgp_coarse *c, const int32_t *coarse_part, int32_t *fine_part);
+/* Waits for the device that holds the arrays and releases them to the library's pool (NULL is
+ * allowed), whichever device is current.  The two calls above run on the contraction's stream,
+ * which has to exist for them; it may be destroyed before this call. */
 void hgp_coarse_destroy(hgp_coarse *c);
 
 /*

@@ -20,6 +20,7 @@
 #include <stdint.h>
 
 #include <algorithm>
+#include <array>
 #include <new>
 #include <utility>
 
@@ -974,13 +975,7 @@ __global__ void k_ct_project(const int32_t *map, int32_t n, const int32_t *coars
         fine_part[u] = coarse_part[map[u]];
 }
 
-// the arrays go back to the library's pool (behind the work queued on the stream)
-void coarse_free(hgp_coarse *c)
-{
-    if (!c) return;
-    for (void *p : {(void *)c->net_off, (void *)c->pins, (void *)c->vw, (void *)c->nw, (void *)c->map}) dev_free(p, c->stream);
-    delete c;
-}
+std::array<void *, 5> coarse_arrays(const hgp_coarse *c) { return {c->net_off, c->pins, c->vw, c->nw, c->map}; }
 
 }  // namespace
 
@@ -1189,7 +1184,8 @@ done:
         rc = status_of(e);
     }
     if (rc != HGP_OK) {
-        coarse_free(c);
+        for (void *p : coarse_arrays(c)) dev_free(p, st);
+        delete c;
         return rc;
     }
     *out = c;
@@ -1255,7 +1251,15 @@ extern "C" int hgp_coarse_project(const hgp_coarse *c, const int32_t *coarse_par
 extern "C" void hgp_coarse_destroy(hgp_coarse *c)
 {
     if (!c) return;
-    // the arrays may be in use on any stream of the device (cudaFree would wait for them all, too)
-    if (cudaDeviceSynchronize() != cudaSuccess) (void)cudaGetLastError();
-    coarse_free(c);
+    // the arrays may be in use on any stream of their device: wait for that device, whichever is
+    // current, and release them without the contraction's stream, which may be gone by now
+    int now = 0;
+    const bool other = cudaGetDevice(&now) == cudaSuccess && now != c->device;
+    if (other) cudaSetDevice(c->device);
+    cudaDeviceSynchronize();
+    for (void *p : coarse_arrays(c))
+        if (p) cudaFree(p);
+    if (other) cudaSetDevice(now);
+    (void)cudaGetLastError();
+    delete c;
 }
