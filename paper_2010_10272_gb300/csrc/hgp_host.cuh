@@ -5,6 +5,7 @@
 #include <stdint.h>
 
 #include "hgp_internal.cuh"
+#include "hgp_rules.h"
 
 struct hgp_handle {
     hgp::Dev d{};
@@ -86,6 +87,11 @@ cudaError_t dev_alloc(void **p, size_t bytes, cudaStream_t st);
 void dev_free(void *p, cudaStream_t st);
 // the same for temporaries whose release status the caller checks
 inline cudaError_t pool_free(void *p, cudaStream_t st) { return p ? cudaFreeAsync(p, st) : cudaSuccess; }
+
+// Whether a kernel of `device` may read [p, p + bytes) where it is: one allocation of that device's
+// memory.  A caller's array that is anything else (host or managed memory, another device's, a part of
+// an allocation too short for it) is copied, which the runtime does or refuses.
+bool readable_in_place(const void *p, size_t bytes, int device);
 
 // Carves `bytes` (rounded up to 256) from the handle's arena; nullptr when it has no room left.
 inline void *arena_take(hgp_handle *h, size_t bytes)

@@ -5,6 +5,7 @@
 //     builds the same two adjacency arrays with prefix sums, Sec. 3.2);
 //   * Phi(e, i) from the partition (Sec. 2 / Sec. 5.1), Lambda(e), S1(e) and omega(e) in the
 //     per-net record, the block weights and the (lambda-1) objective (Sec. 2).
+#include <cuda.h>
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>
@@ -1283,6 +1284,29 @@ cudaError_t dev_alloc(void **p, size_t bytes, cudaStream_t st)
     return e;
 }
 
+bool readable_in_place(const void *p, size_t bytes, int device)
+{
+    typedef CUresult (*Range)(CUdeviceptr *, size_t *, CUdeviceptr);
+    static const Range range = [] {
+        void *f = nullptr;
+        cudaDriverEntryPointQueryResult found;
+        if (cudaGetDriverEntryPointByVersion("cuMemGetAddressRange", &f, 12000, cudaEnableDefault, &found) != cudaSuccess) {
+            (void)cudaGetLastError();
+            f = nullptr;
+        }
+        return reinterpret_cast<Range>(f);
+    }();
+    cudaPointerAttributes at;
+    if (!range || cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return false;
+    }
+    CUdeviceptr base = 0;
+    size_t size = 0;
+    return at.type == cudaMemoryTypeDevice && at.device == device &&
+           range(&base, &size, (CUdeviceptr)p) == CUDA_SUCCESS && range_inside((uintptr_t)p, bytes, (uintptr_t)base, size);
+}
+
 void dev_free(void *p, cudaStream_t st)
 {
     if (p && pool_free(p, st) != cudaSuccess) (void)cudaGetLastError();
@@ -1916,11 +1940,13 @@ int hgp_set_partition(hgp_handle *h, const int32_t *part, int32_t on_device)
     cudaStream_t st = h->stream;
     // two launches and one read-back: the check stages the 1-byte partition and its block weights, and
     // once it is known to be valid (else the handle keeps its state) k_init_nets does the rest.  A
-    // device partition is read where it is.  10k vertices: 110 -> 28 us a call.
+    // device partition is read where it is, if it is in this device's memory.  10k vertices: 110 ->
+    // 28 us a call.
     const int32_t *src = part;
     int32_t *tmp = nullptr;
     cudaError_t e = cudaSuccess;
-    if (!on_device || (reinterpret_cast<uintptr_t>(part) & 3)) {
+    if (!on_device || (reinterpret_cast<uintptr_t>(part) & 3) ||
+        !readable_in_place(part, sizeof(int32_t) * (size_t)d.n, h->device)) {
         tmp = h->scratch_n;
         if (!tmp) CK(dev_alloc(reinterpret_cast<void **>(&tmp), sizeof(int32_t) * (size_t)d.n, st));
         src = tmp;

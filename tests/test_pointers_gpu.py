@@ -1,0 +1,38 @@
+"""Device arrays of the caller, wherever they are."""
+import numpy as np
+import pytest
+
+import oracle
+import synth
+from parity_util import compare_state
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+def _allocated(kind, values):
+    """An int32 array in device memory at the end of its allocation, in managed or in page-locked host
+    memory: (address, owner)."""
+    import ctypes
+    rt = ctypes.CDLL("libcudart.so.%d" % int(torch.version.cuda.split(".")[0]))
+    p, nbytes = ctypes.c_void_p(), values.nbytes
+    room = -(-nbytes // (2 << 20)) * (2 << 20)
+    call = {"device": rt.cudaMalloc, "managed": rt.cudaMallocManaged, "pinned": rt.cudaMallocHost}[kind]
+    args = (ctypes.c_uint(1),) if kind == "managed" else ()
+    assert call(ctypes.byref(p), ctypes.c_size_t(room), *args) == 0
+    at = p.value + room - nbytes
+    assert rt.cudaMemcpy(ctypes.c_void_p(at), values.ctypes.data_as(ctypes.c_void_p), ctypes.c_size_t(nbytes), 4) == 0
+    return at, lambda: (rt.cudaFreeHost if kind == "pinned" else rt.cudaFree)(p)
+
+
+@pytest.mark.parametrize("kind", ["device", "managed", "pinned"])
+def test_device_partition_wherever_it_is(kind):
+    from paper_2010_10272_gb300 import HGP
+    hg = synth.random_small(4, 5003, 4000, 6, max_size=7)
+    second = np.random.default_rng(1).integers(0, 6, hg.n).astype(np.int32)
+    at, free = _allocated(kind, second)
+    h = HGP.from_hypergraph(hg)
+    h.set_partition(at, device=True)
+    compare_state(h, oracle.Oracle.from_hypergraph(hg, part=second))
+    h.close()
+    free()
