@@ -21,7 +21,7 @@
 
 #include <mutex>
 
-#include "hgp_internal.cuh"
+#include "hgp_host.cuh"
 
 using namespace hgp;
 
@@ -369,7 +369,11 @@ extern "C" int hgp_candidates_noalloc(int32_t n, int32_t m, const int32_t *net_o
     NaRec *recs = reinterpret_cast<NaRec *>(sc + kRecOffset);
 
     cudaError_t e = cudaSuccess;
-    if (!pins || !inc_nets) {   // allowed only without pins
+    int dev = 0;
+    cudaGetDevice(&dev);
+    // offsets that are not plainly this device's are read by a copy first, which refuses what is no
+    // device array; pins and lists may only be missing where there are no pins
+    if (!pins || !inc_nets || !readable_in_place(net_offsets, sizeof(int32_t) * ((size_t)m + 1), dev)) {
         int32_t P = 0;
         e = cudaMemcpyAsync(&P, net_offsets + m, sizeof(int32_t), cudaMemcpyDeviceToHost, st);
         if (e == cudaSuccess) e = cudaStreamSynchronize(st);
@@ -377,7 +381,7 @@ extern "C" int hgp_candidates_noalloc(int32_t n, int32_t m, const int32_t *net_o
             (void)cudaGetLastError();
             return HGP_ERR_CUDA;
         }
-        if (P != 0) return HGP_ERR_INVALID;
+        if (P < 0 || (P > 0 && (!pins || !inc_nets))) return HGP_ERR_INVALID;
     }
 
     // block weights start from zero and the error flag is cleared on every call

@@ -36,3 +36,24 @@ def test_device_partition_wherever_it_is(kind):
     compare_state(h, oracle.Oracle.from_hypergraph(hg, part=second))
     h.close()
     free()
+
+
+@pytest.mark.parametrize("kind", ["device", "managed", "pinned"])
+def test_allocation_free_offsets_wherever_they_are(kind):
+    from paper_2010_10272_gb300 import HGP
+    from paper_2010_10272_gb300.native import candidates_noalloc
+    hg = synth.random_small(4, 5003, 4000, 6, max_size=7)
+    net = np.repeat(np.arange(hg.m, dtype=np.int32), np.diff(hg.net_off))
+    voff = np.concatenate([[0], np.cumsum(np.bincount(hg.pins, minlength=hg.n))]).astype(np.int32)
+    pins, voff, inc, part = (torch.from_numpy(x).cuda() for x in
+                             (hg.pins, voff, net[np.argsort(hg.pins, kind="stable")], hg.part))
+    t = torch.empty(hg.n, dtype=torch.int32, device="cuda")
+    g = torch.empty(hg.n, dtype=torch.int64, device="cuda")
+    off, free = _allocated(kind, hg.net_off.astype(np.int32))
+    assert candidates_noalloc(hg.n, hg.m, off, pins, voff, inc, hg.k, hg.eps, part, t, g) == 0
+    assert candidates_noalloc(hg.n, hg.m, off, None, voff, None, hg.k, hg.eps, part, t, g) == 1
+    h = HGP.from_hypergraph(hg)
+    want_t, want_g = h.debug_candidates(0)
+    assert np.array_equal(t.cpu().numpy(), want_t) and np.array_equal(g.cpu().numpy(), want_g)
+    h.close()
+    free()
