@@ -240,6 +240,93 @@ __device__ __forceinline__ void na_planes(const NaRec *recs, const int32_t *inc,
     for (int p = 0; p < NP; ++p) conn_out |= (int32_t)((c[p] >> t_out) & 1) << p;
 }
 
+__device__ __forceinline__ void take_net(const NaRec &r, int a, int64_t &W, int64_t &b, uint64_t &T)
+{
+    W += r.w;
+    if ((r.s1 >> a) & 1) {
+        b += r.w;
+        T |= r.lam;
+    }
+}
+
+// blocks of T with room for weight cu
+__device__ __forceinline__ uint64_t na_room(uint64_t T, const long long *slack, int32_t cu)
+{
+    for (uint64_t x = T; x; x &= x - 1) {
+        const int t = __ffsll((long long)x) - 1;
+        if (slack[t] < cu) T &= ~(1ull << t);
+    }
+    return T;
+}
+
+// A vertex of many nets by the whole warp: the lanes stride over its nets, then each keeps the sums of
+// two blocks.  By one lane, which the 31 others of its warp wait for, 30k vertices with Zipf degrees up to
+// 1,378 took 2.02 ms a call; 0.89 so, of which 0.76 are the transpose check.
+constexpr int32_t kNaLaneDeg = 96;   // as kLaneDeg of the refinement rounds
+
+__device__ __forceinline__ int64_t warp_sum(int64_t v)
+{
+#pragma unroll
+    for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
+    return v;
+}
+
+__device__ __forceinline__ void na_hub(const NaRec *recs, const int32_t *inc, int32_t jb, int32_t je, int a, int32_t cu,
+                                       const long long *slack, int &t_best, int64_t &g_best)
+{
+    const int lane = threadIdx.x & 31;
+    const int32_t deg = je - jb;
+    int64_t W = 0, b = 0;
+    uint64_t T = 0;
+    for (int32_t i = lane; i < deg; i += 32) take_net(recs[inc[jb + i]], a, W, b, T);
+    W = warp_sum(W);
+    b = warp_sum(b);
+    T = (uint64_t)__reduce_or_sync(kFull, (uint32_t)T) | ((uint64_t)__reduce_or_sync(kFull, (uint32_t)(T >> 32)) << 32);
+    T = na_room(T & ~(1ull << a), slack, cu);
+    t_best = -1;
+    g_best = 0;
+    if (T == 0) return;
+    int64_t conn0 = 0, conn1 = 0;   // of blocks lane and lane + 32
+    for (int32_t i0 = 0; i0 < deg; i0 += 32) {
+        uint64_t lam = 0;
+        int32_t w = 0;
+        if (i0 + lane < deg) {
+            const NaRec &r = recs[inc[jb + i0 + lane]];
+            lam = r.lam & T;
+            w = r.w;
+        }
+        const int nn = min(32, deg - i0);
+        for (int q = 0; q < nn; ++q) {
+            const uint32_t lo = __shfl_sync(kFull, (uint32_t)lam, q), hi = __shfl_sync(kFull, (uint32_t)(lam >> 32), q);
+            const int32_t wq = __shfl_sync(kFull, w, q);
+            conn0 += ((lo >> lane) & 1) ? wq : 0;
+            conn1 += ((hi >> lane) & 1) ? wq : 0;
+        }
+    }
+    // the larger gain, then the smaller block
+    int64_t g = 0;
+    int t = -1;
+    if (((T >> lane) & 1) && b - W + conn0 > 0) {
+        g = b - W + conn0;
+        t = lane;
+    }
+    if (((T >> (lane + 32)) & 1) && b - W + conn1 > g) {
+        g = b - W + conn1;
+        t = lane + 32;
+    }
+#pragma unroll
+    for (int o = 16; o; o >>= 1) {
+        const int64_t g2 = __shfl_xor_sync(kFull, g, o);
+        const int t2 = __shfl_xor_sync(kFull, t, o);
+        if (g2 > g || (g2 == g && t2 >= 0 && t2 < t)) {
+            g = g2;
+            t = t2;
+        }
+    }
+    t_best = t;
+    g_best = g;
+}
+
 // The gain step of round 0 (every vertex eligible) for sub-round s, as in the refinement rounds:
 // T = blocks of Lambda(e) over nets with Phi(e,a) = 1, minus a and the blocks without room; best t in
 // T by g_t = b(u) - W + omega({e : t in Lambda(e)}), smallest block on ties; no candidate unless the
@@ -282,33 +369,33 @@ __global__ void __launch_bounds__(256) k_na_candidates(int32_t n, int32_t k, dou
             }
         }
         __syncwarp();
-        for (int i = lane; i < cnt; i += 32) {
-            const int64_t u = base + list[i];
-            int32_t t_best = -1;
+        for (int i0 = 0; i0 < cnt; i0 += 32) {
+            const bool on = i0 + lane < cnt;
+            int64_t u = 0;
+            int t_best = -1, a = 0;
             int64_t g_best = 0;
-            const int a = part[u];
-            const int32_t cu = vw ? vw[u] : 1;
-            const int32_t jb = vtx_off[u], je = vtx_off[u + 1];
+            int32_t cu = 1, jb = 0, je = 0;
+            if (on) {
+                u = base + list[i0 + lane];
+                a = part[u];
+                cu = vw ? vw[u] : 1;
+                jb = vtx_off[u];
+                je = vtx_off[u + 1];
+            }
+            const bool hub = je - jb > kNaLaneDeg;
             int64_t W = 0, b = 0;
             uint64_t T = 0;
-            for (int32_t j = jb; j < je; ++j) {
-                const NaRec &r = recs[inc[j]];
-                W += r.w;
-                if ((r.s1 >> a) & 1) {
-                    b += r.w;
-                    T |= r.lam;
-                }
+            if (!hub) {
+                for (int32_t j = jb; j < je; ++j) take_net(recs[inc[j]], a, W, b, T);
+                T = na_room(T & ~(1ull << a), slack, cu);
             }
-            T &= ~(1ull << a);
-            for (uint64_t x = T; x; x &= x - 1) {
-                const int t = __ffsll((long long)x) - 1;
-                if (slack[t] < cu) T &= ~(1ull << t);
-            }
-            if (T != 0 && W < 2048) {
+            const bool planes = T != 0 && W < 2048;
+            const bool wide = __any_sync(kFull, planes && W >= 64);   // the warp takes one path
+            if (planes) {
                 int t;
                 int32_t conn;
-                if (W < 64) na_planes<6>(recs, inc, jb, je, T, t, conn);
-                else na_planes<11>(recs, inc, jb, je, T, t, conn);
+                if (wide) na_planes<11>(recs, inc, jb, je, T, t, conn);
+                else na_planes<6>(recs, inc, jb, je, T, t, conn);
                 const int64_t g = b - W + conn;
                 if (g > 0) {
                     g_best = g;
@@ -330,8 +417,21 @@ __global__ void __launch_bounds__(256) k_na_candidates(int32_t n, int32_t k, dou
                     }
                 }
             }
-            target[u] = t_best;
-            gain[u] = g_best;
+            for (unsigned hm = __ballot_sync(kFull, hub); hm; hm &= hm - 1) {
+                const int src = __ffs(hm) - 1;
+                int t;
+                int64_t g;
+                na_hub(recs, inc, __shfl_sync(kFull, jb, src), __shfl_sync(kFull, je, src), __shfl_sync(kFull, a, src),
+                       __shfl_sync(kFull, cu, src), slack, t, g);
+                if (lane == src) {
+                    t_best = t;
+                    g_best = g;
+                }
+            }
+            if (on) {
+                target[u] = t_best;
+                gain[u] = g_best;
+            }
         }
         __syncwarp();
     }

@@ -1,0 +1,57 @@
+"""Vertices of many nets beside vertices of few, numbered at random or by falling degree."""
+import numpy as np
+import pytest
+
+import oracle
+import synth
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+def hubs(seed, n, m, k, order="random", vertex_w=4, net_w=9, eps=0.1):
+    """Nets of 2 to 7 pins, each pin the vertex of rank n x^5 for a uniform x (a few vertices are in a large
+    part of all nets), ids by rank or at random."""
+    rng = np.random.default_rng(seed)
+    ids = np.arange(n) if order == "falling" else rng.permutation(n)
+    nets = [np.unique(ids[np.minimum((n * rng.random(s) ** 5).astype(np.int64), n - 1)]) for s in rng.integers(2, 8, m)]
+    hg = synth.random_small(seed, n, m, k, max_size=2, weighted=True, eps=eps)
+    hg.net_off = np.concatenate([[0], np.cumsum([len(x) for x in nets])]).astype(hg.net_off.dtype)
+    hg.pins = np.concatenate(nets).astype(np.int32)
+    hg.vertex_w = rng.integers(1, vertex_w + 1, n).astype(np.int32) if vertex_w else None
+    hg.net_w = rng.integers(1, net_w + 1, m).astype(np.int32) if net_w else None
+    part = rng.integers(0, k, n).astype(np.int32)
+    part[ids] = np.where(rng.random(n) < 0.7, np.arange(n) * k // n, part[ids])     # neighbours by rank together
+    hg.part = part
+    return hg
+
+
+def degrees(hg):
+    return np.bincount(hg.pins, minlength=hg.n)
+
+
+@pytest.mark.parametrize("k", [2, 33, 64])
+@pytest.mark.parametrize("order", ["random", "falling"])
+@pytest.mark.parametrize("net_w", [0, 9, 3000])
+def test_allocation_free_candidates(k, order, net_w):
+    from paper_2010_10272_gb300.native import candidates_noalloc
+    hg = hubs(k, 700, 6000, k, order, net_w=net_w)
+    deg = degrees(hg)
+    assert (deg > 96).sum() > 20 and (deg < 96).sum() > 300
+    net = np.repeat(np.arange(hg.m, dtype=np.int32), np.diff(hg.net_off))
+    dev = torch.device("cuda")
+    args = [torch.from_numpy(np.ascontiguousarray(x)).to(dev) for x in
+            (hg.net_off.astype(np.int32), hg.pins, np.concatenate([[0], np.cumsum(deg)]).astype(np.int32),
+             net[np.argsort(hg.pins, kind="stable")])]
+    part, vw = torch.from_numpy(hg.part).to(dev), torch.from_numpy(hg.vertex_w).to(dev)
+    nw = torch.from_numpy(hg.net_w).to(dev) if net_w else None
+    t = torch.empty(hg.n, dtype=torch.int32, device=dev)
+    g = torch.empty(hg.n, dtype=torch.int64, device=dev)
+    o = oracle.Oracle.from_hypergraph(hg, subrounds=2, seed=5)
+    found = 0
+    for s in range(2):
+        assert candidates_noalloc(hg.n, hg.m, *args, k, hg.eps, part, t, g, vw, nw, subrounds=2, seed=5, s=s) == 0
+        want_t, want_g = o.candidates(s)
+        assert np.array_equal(t.cpu().numpy(), want_t) and np.array_equal(g.cpu().numpy(), want_g)
+        found += (want_t[deg > 96] >= 0).sum()
+    assert found > 0
