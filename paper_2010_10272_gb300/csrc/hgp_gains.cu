@@ -70,29 +70,38 @@ __device__ __forceinline__ void find_both(Slot *table, uint64_t mask, unsigned l
 }
 
 // validation: vertex in range, moved once, from = Pi(u), to in range and different; and the sum of
-// the degrees of the moved vertices (each contributes 2 keys per incident net).  out: error, sum
+// the degrees of the moved vertices (each contributes 2 keys per incident net).  out: error, sum, largest
+// degree
 __global__ void k_eg_check(Dev d, const int32_t *moves, int32_t count, int32_t *seen, unsigned long long *out)
 {
     unsigned long long s = 0;
+    int32_t most = 0;
     for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < count;
          j += (int64_t)gridDim.x * blockDim.x) {
         const int32_t u = moves[3 * j], a = moves[3 * j + 1], b = moves[3 * j + 2];
         bool bad = u < 0 || u >= d.n || b < 0 || b >= d.k || a == b;
         if (!bad) {
             bad = d.part[u] != a || atomicExch(&seen[u], 1) != 0;
-            s += (unsigned long long)(d.vtx_off[u + 1] - d.vtx_off[u]);
+            const int32_t deg = d.vtx_off[u + 1] - d.vtx_off[u];
+            s += (unsigned long long)deg;
+            most = max(most, deg);
         }
         if (bad) atomicOr(&out[0], 1ull);
     }
     for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(kFull, s, o);
-    if ((threadIdx.x & 31) == 0 && s) atomicAdd(&out[1], s);
+    most = (int32_t)__reduce_max_sync(kFull, (unsigned)most);
+    if ((threadIdx.x & 31) == 0 && s) {
+        atomicAdd(&out[1], s);
+        atomicMax(&out[2], (unsigned long long)most);
+    }
 }
 
 // Up to this many moves (all of whose warps run at once) a warp takes one each: the chain of dependent
 // accesses per 32 incidences is what a short sequence waits for (5k moves of 4 nets, 8 per warp: 144
 // us, one: 119 us).
 constexpr int kEgWarps = 152 * 32;
-constexpr uint64_t kEgDense = 1 << 20;   // slots (32 MB) from which a table may be two thirds full
+constexpr uint64_t kEgDense = 1 << 20;   // slots (32 MB) from which a table may be two thirds full,
+constexpr uint64_t kEgHub = 128;         // unless a move has more nets than this
 
 // `per` (at most 32) moves of a warp, about 32 incidences in all, one run that the lanes walk
 // flattened (a warp per move left most lanes idle, 6 nets of 32; 32 moves per warp were as slow, too
@@ -180,8 +189,17 @@ __global__ void __launch_bounds__(256) k_eg_pass2(Dev d, const int32_t *moves, i
     const Rec32 *r32 = reinterpret_cast<const Rec32 *>(d.rec);
     for (int64_t j0 = ((int64_t)blockIdx.x * 8 + (threadIdx.x >> 5)) * per; j0 < count; j0 += warps * per) {
         const int32_t total = w.load(d, moves, j0, count, per);
+        // a lane's sum over the incidences of one move, added to the move's when the lane leaves it (32
+        // lanes adding to one hub's sum at every step: 15.3 instead of 14.5 ms in the case below)
+        long long g = 0;
+        int at = 0;
         for (int32_t i = lane; i < total; i += 32) {
             const int v = w.slot(i);
+            if (v != at) {
+                if (g) atomicAdd(&w.g[at], (unsigned long long)g);
+                g = 0;
+                at = v;
+            }
             const int32_t j = (int32_t)j0 + v, a = w.a[v], b = w.b[v];
             const int32_t eraw = d.inc[w.jb[v] + (i - w.off[v])];
             const int32_t e = eraw & kNetMask;
@@ -190,11 +208,10 @@ __global__ void __launch_bounds__(256) k_eg_pass2(Dev d, const int32_t *moves, i
             const int32_t we = (d.k <= 32 ? r16[e].w : r32[e].w) & 0x7fffffff;
             Slot *sa, *sb;
             find_both(table, mask, (unsigned long long)e, a, b, false, sa, sb);
-            long long g = 0;
             if (sa && sa->max_out == j && sa->min_in > (uint32_t)j && sa->n_out + 1 == phi_get(d, e, a, wide, wrow)) g += we;
             if (sb && sb->min_in == (uint32_t)j && sb->max_out < j && sb->n_out + 1 == phi_get(d, e, b, wide, wrow)) g -= we;
-            if (g) atomicAdd(&w.g[v], (unsigned long long)g);
         }
+        if (g) atomicAdd(&w.g[at], (unsigned long long)g);
         __syncwarp();
         if (lane < per && j0 + lane < count) gains[j0 + lane] = (int64_t)w.g[lane];
         __syncwarp();
@@ -220,9 +237,9 @@ extern "C" int hgp_exact_gains(hgp_handle *h, int32_t count, const int32_t *move
     cudaStream_t st = h->stream;
     Slot *table = nullptr;
     char *buf = nullptr;
-    unsigned long long host[2] = {0, 0};
+    unsigned long long host[3] = {0, 0, 0};
     int rc = HGP_OK;
-    // one buffer (five took 10 us more): error and degree sum, seen flags (both zeroed), gains, moves
+    // one buffer (five took 10 us more): error, degree sum and maximum, seen flags (both zeroed), gains, moves
     const size_t zero_bytes = (sizeof(host) + sizeof(int32_t) * (size_t)d.n + 15) / 16 * 16;
     const size_t g_bytes = sizeof(int64_t) * (size_t)count;
     cudaError_t e = dev_alloc(reinterpret_cast<void **>(&buf), zero_bytes + g_bytes + sizeof(int32_t) * 3 * (size_t)count, st);
@@ -240,10 +257,12 @@ extern "C" int hgp_exact_gains(hgp_handle *h, int32_t count, const int32_t *move
     if (e == cudaSuccess) e = cudaMemcpyAsync(host, out, sizeof(host), cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = stream_wait(st);
     if (e == cudaSuccess && host[0]) rc = HGP_ERR_INVALID;
-    // at most 2 keys per incident net of a moved vertex; the table is at most half full while it is small
-    // (long runs of probes are what few moves wait for: 5.4k moves 114 -> 96 us), two thirds above
+    // at most 2 keys per incident net of a moved vertex.  The table is at most half full while it is small
+    // or a move has many nets, two thirds above: a chain of accesses waits for the longest run of probes of
+    // every 32, and few moves (5.4k: 114 -> 96 us) or one of a hub wait for a chain (50k moves of 1M
+    // vertices with Zipf degrees, one of 21,185 nets: 14.5 ms two thirds full, 8.1 half full)
     uint64_t size = 64;
-    while (size < (size < kEgDense ? 4 : 3) * (uint64_t)host[1]) size <<= 1;
+    while (size < (size < kEgDense || host[2] > kEgHub ? 4 : 3) * (uint64_t)host[1]) size <<= 1;
     if (e == cudaSuccess && rc == HGP_OK) e = dev_alloc(reinterpret_cast<void **>(&table), sizeof(Slot) * size, st);
     if (e == cudaSuccess && rc == HGP_OK) e = cudaMemsetAsync(table, 0xFF, sizeof(Slot) * size, st);
     if (e == cudaSuccess && rc == HGP_OK) {

@@ -55,3 +55,21 @@ def test_allocation_free_candidates(k, order, net_w):
         assert np.array_equal(t.cpu().numpy(), want_t) and np.array_equal(g.cpu().numpy(), want_g)
         found += (want_t[deg > 96] >= 0).sum()
     assert found > 0
+
+
+@pytest.mark.parametrize("order", ["random", "falling"])
+@pytest.mark.parametrize("n,m,k,count", [(60_000, 70_000, 5, 60_000), (60_000, 70_000, 40, 30_000), (900, 9000, 3, 800)])
+def test_exact_gains(n, m, k, count, order):
+    """Hubs among the few moves and among the many of a warp, in tables of half and of more than a
+    million slots."""
+    from paper_2010_10272_gb300 import HGP
+    rng = np.random.default_rng(count)
+    hg = hubs(n + k, n, m, k, order)
+    u = rng.permutation(hg.n)[:count]
+    hub = np.argsort(degrees(hg))[-40:]
+    u = rng.permutation(np.unique(np.concatenate([u, hub])))
+    a = hg.part[u]
+    moves = np.stack([u, a, (a + rng.integers(1, k, u.size)) % k], 1).astype(np.int32)
+    h = HGP.from_hypergraph(hg)
+    assert np.array_equal(h.exact_gains(moves), oracle.Oracle.from_hypergraph(hg).exact_gains(moves))
+    h.close()
