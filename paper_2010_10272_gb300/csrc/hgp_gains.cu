@@ -263,7 +263,14 @@ extern "C" int hgp_exact_gains(hgp_handle *h, int32_t count, const int32_t *move
     // vertices with Zipf degrees, one of 21,185 nets: 14.5 ms two thirds full, 8.1 half full)
     uint64_t size = 64;
     while (size < (size < kEgDense || host[2] > kEgHub ? 4 : 3) * (uint64_t)host[1]) size <<= 1;
-    if (e == cudaSuccess && rc == HGP_OK) e = dev_alloc(reinterpret_cast<void **>(&table), sizeof(Slot) * size, st);
+    if (e == cudaSuccess && rc == HGP_OK) {
+        e = dev_alloc(reinterpret_cast<void **>(&table), sizeof(Slot) * size, st);
+        // on a nearly full device, half the slots if those still hold every key
+        if (e == cudaErrorMemoryAllocation && size / 2 >= 2 * (uint64_t)host[1]) {
+            size /= 2;
+            e = dev_alloc(reinterpret_cast<void **>(&table), sizeof(Slot) * size, st);
+        }
+    }
     if (e == cudaSuccess && rc == HGP_OK) e = cudaMemsetAsync(table, 0xFF, sizeof(Slot) * size, st);
     if (e == cudaSuccess && rc == HGP_OK) {
         const uint64_t fit = 32 * (uint64_t)count / std::max<uint64_t>(1, host[1]);   // moves of 32 incidences

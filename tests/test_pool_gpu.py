@@ -41,3 +41,31 @@ def test_create_waits_for_a_pending_release_on_another_stream():
         rest = None                          # noqa: F841
         torch.cuda.empty_cache()
         _default_retention()
+
+
+def test_exact_gains_on_a_nearly_full_device():
+    """16M incidences moved: with less free memory than the usual table takes, a smaller one is used."""
+    from paper_2010_10272_gb300 import HGP
+    from paper_2010_10272_gb300.native import set_pool_retention
+    n = m = 4_000_000
+    dev = torch.device("cuda")
+    off = torch.arange(0, 4 * m + 1, 4, dtype=torch.int64, device=dev)
+    step = torch.tensor([0, 7, 11, 19], device=dev)
+    pins = ((torch.arange(m, device=dev)[:, None] + step) % n).sort(1)[0].to(torch.int32).reshape(-1).contiguous()
+    part = (torch.arange(n, device=dev) % 16).to(torch.int32)
+    u = np.random.default_rng(0).permutation(n)
+    moves = np.stack([u, u % 16, (u + 5) % 16], 1).astype(np.int32)
+    h = HGP(n, m, off, pins, 16, 0.03, part, device=True)
+    try:
+        set_pool_retention(0)
+        want = h.exact_gains(moves)
+        torch.cuda.synchronize()
+        gc.collect()
+        torch.cuda.empty_cache()
+        rest = torch.empty(torch.cuda.mem_get_info()[0] - (1850 << 20), dtype=torch.uint8, device=dev)
+        assert np.array_equal(h.exact_gains(moves), want)
+    finally:
+        rest = None                          # noqa: F841
+        torch.cuda.empty_cache()
+        _default_retention()
+        h.close()
