@@ -270,7 +270,12 @@ constexpr int32_t kPlaneMaxW = 2047;   // W(u) up to this uses bit planes (NP <=
 // degrees above this are walked by the whole warp: its two passes cost about as many issue slots
 // as a lane's walk of this length with the other lanes idle
 constexpr int32_t kLaneDeg = 96;
-constexpr int kRbSegs = 6;             // segments of a rebalancing item
+// Segments of a rebalancing item (gain and apply step) with S sub-rounds: about the active vertices of 256
+// consecutive ones.  Its candidates lie together, so a larger item also gives more of a run of hubs to
+// one warp.  Vertices numbered by falling Zipf degree, S = 4, 2 / 3 / 6 segments: 5M 8.2 / 9.3 / 15.5 ms
+// (exponent 0.5), 55 / 61 / 84 (0.75); power-law 5M with few hubs 2.44 / 2.25 / 2.43; S = 16, 1 / 2 / 6:
+// 12.0 / 15.2 / 20.3 (0.5).
+inline int32_t rb_segments(int32_t S) { return std::min(6, std::max(1, 8 / S)); }
 constexpr int kFeasW = 8;              // vertex weights up to this have a mask of blocks with room
 
 // Per-warp state of the gain step that depends on the instance.
@@ -291,6 +296,7 @@ struct RbArgs {
     int32_t r;       // round number of the sub-round hash for this pass
     int32_t phase;   // 1: gain >= 0 only; 2: any gain
     int32_t off;     // added to the gain to make the approval priority non-negative
+    int32_t segs;    // segments of an item
 };
 
 // What one pass over a vertex's nets gives.
@@ -689,7 +695,7 @@ __device__ __forceinline__ void load_dev(Dev &dst, const Dev *src)
 }
 
 // Persistent: each warp walks work items, a segment of one tile's sub-round list each (a
-// rebalancing item is kRbSegs segments, few of whose vertices take part), one vertex per lane
+// rebalancing item is RbArgs::segs segments, few of whose vertices take part), one vertex per lane
 // (lane_best).  Only blocks in T can have a positive gain, since g_t <= omega({e : Phi(e,a) = 1,
 // t in Lambda(e)}); the best of them has the largest g_t = b(u) - W + conn_t.  Vertices with more
 // than kLaneDeg nets or W > kPlaneMaxW are walked by the whole warp.
@@ -701,7 +707,7 @@ __device__ __forceinline__ void load_dev(Dev &dst, const Dev *src)
 template <typename Rec, bool B, bool RB = false>
 __global__ void __launch_bounds__(kThreads, sizeof(Rec) == 16 || RB ? 4 : 3) k_gain(const Dev d0, const Dev *devs, const int2 *items,
                                                       int32_t n_items, int32_t per_tile, int32_t take, int32_t s,
-                                                      int32_t rr, RbArgs rb = RbArgs{0, 0, 0})
+                                                      int32_t rr, RbArgs rb = RbArgs{0, 0, 0, 1})
 {
     after_previous();
     typedef typename RecIO<Rec>::Lam Lam;
@@ -727,7 +733,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(Rec) == 16 || RB ? 4 : 3) k_g
         const int32_t it1 = min(n_it, (group + 1) * take);
         for (int32_t it = group * take; it < it1; ++it) {
             int32_t tile = it / per_tile;
-            const int32_t seg = (it - tile * per_tile) * (RB ? kRbSegs : 1);
+            const int32_t seg = (it - tile * per_tile) * (RB ? rb.segs : 1);
             int32_t nel = 0;
             if (B) {
                 const int2 im = items[tile];
@@ -754,7 +760,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(Rec) == 16 || RB ? 4 : 3) k_g
                     if (RB) gi.r = rb.r;
                     inst_prev = 0;
                 }
-                const int32_t seg_end = RB ? min(d0.nseg, seg + kRbSegs) : seg + 1;
+                const int32_t seg_end = RB ? min(d0.nseg, seg + rb.segs) : seg + 1;
                 const int32_t nout = gain_seg<Rec, RB>(d0, tile, seg, seg_end, s, ws[wid], picked[RB ? wid : 0], gi, nel,
                                                        rb);
                 int32_t *cnt = d0.cand_cnt + (int64_t)tile * d0.nseg + seg;
@@ -2036,10 +2042,10 @@ void launch(void (*kernel)(KA...), int64_t grid, unsigned block, cudaStream_t st
 cudaError_t launch_gain(const Plan &p, int32_t s, int32_t rr)
 {
     const bool b = p.tiles != nullptr;
-    if (p.rec32 && b) launch(k_gain<Rec32, true>, p.grid_gain, kThreads, p.st, p.d0, p.devs, p.tiles, p.n_tiles, p.nseg, p.take, s, rr, RbArgs{0, 0, 0});
-    else if (p.rec32) launch(k_gain<Rec32, false>, p.grid_gain, kThreads, p.st, p.d0, p.devs, p.tiles, p.n_tiles, p.nseg, p.take, s, rr, RbArgs{0, 0, 0});
-    else if (b) launch(k_gain<Rec16, true>, p.grid_gain, kThreads, p.st, p.d0, p.devs, p.tiles, p.n_tiles, p.nseg, p.take, s, rr, RbArgs{0, 0, 0});
-    else launch(k_gain<Rec16, false>, p.grid_gain, kThreads, p.st, p.d0, p.devs, p.tiles, p.n_tiles, p.nseg, p.take, s, rr, RbArgs{0, 0, 0});
+    if (p.rec32 && b) launch(k_gain<Rec32, true>, p.grid_gain, kThreads, p.st, p.d0, p.devs, p.tiles, p.n_tiles, p.nseg, p.take, s, rr, RbArgs{0, 0, 0, 1});
+    else if (p.rec32) launch(k_gain<Rec32, false>, p.grid_gain, kThreads, p.st, p.d0, p.devs, p.tiles, p.n_tiles, p.nseg, p.take, s, rr, RbArgs{0, 0, 0, 1});
+    else if (b) launch(k_gain<Rec16, true>, p.grid_gain, kThreads, p.st, p.d0, p.devs, p.tiles, p.n_tiles, p.nseg, p.take, s, rr, RbArgs{0, 0, 0, 1});
+    else launch(k_gain<Rec16, false>, p.grid_gain, kThreads, p.st, p.d0, p.devs, p.tiles, p.n_tiles, p.nseg, p.take, s, rr, RbArgs{0, 0, 0, 1});
     *p.launches += 1;
     return cudaGetLastError();
 }
@@ -2465,14 +2471,14 @@ cudaError_t launch_rebalance_pass(const Plan &p, int32_t pass, RbArgs rb, bool l
     launch(k_round_prep, p.n_tiles, kThreads, p.st, p.devs, p.tiles, p.n_tiles, rb.r);
     *p.launches += 1;
     for (int32_t s = 0; s < p.S_max; ++s) {
-        launch(k_gain<Rec, false, true>, p.grid_gain, kThreads, p.st, p.d0, p.devs, p.tiles, p.n_tiles, (p.nseg + kRbSegs - 1) / kRbSegs, 1, s,
+        launch(k_gain<Rec, false, true>, p.grid_gain, kThreads, p.st, p.d0, p.devs, p.tiles, p.n_tiles, (p.nseg + rb.segs - 1) / rb.segs, 1, s,
                                                                     pass, rb);
         *p.launches += 1;
         *p.launches += launch_stage<KEY_A>(p, levels, bins);
         launch(k_rb_mark, p.grid_apply, kThreads, p.st, p.d0);
         *p.launches += 1;
         *p.launches += launch_stage<KEY_TS>(p, levels, bins);
-        launch(k_apply<Rec, false, KEY_TS>, p.grid_apply, kThreads, p.st, p.d0, p.devs, p.tiles, p.n_tiles, p.nseg, p.per, pass);
+        launch(k_apply<Rec, false, KEY_TS>, p.grid_apply, kThreads, p.st, p.d0, p.devs, p.tiles, p.n_tiles, p.nseg, std::min(p.per, rb.segs), pass);
         *p.launches += 1;
     }
     launch(k_round_end, 1, 128, p.st, p.devs, 1, pass, 0);
@@ -2518,6 +2524,7 @@ extern "C" int hgp_rebalance(hgp_handle *h, int32_t max_passes, hgp_round_stats 
         rb.r = (1 << 30) + pass;
         rb.phase = phase;
         rb.off = phase == 2 ? (int32_t)off : 0;
+        rb.segs = rb_segments(h->d.S);
         const int64_t top = phase == 2 ? 2 * off : off;   // largest priority
         const bool levels = top >= kBins - 1;
         const int32_t bins = (int32_t)std::min<int64_t>(kBins, (top + kThreads) / kThreads * kThreads);

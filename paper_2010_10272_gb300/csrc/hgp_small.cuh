@@ -265,7 +265,7 @@ __global__ void __launch_bounds__(kSmThreads, 1) k_small(const Dev d, int32_t ro
                 }
                 int t_best;
                 int32_t g_best;
-                const bool elig = gain_vertex<Rec, false, true>(d, inc, sh.g[wid], gi, RbArgs{0, 0, 0}, valid, a, cu, jb, je, W,
+                const bool elig = gain_vertex<Rec, false, true>(d, inc, sh.g[wid], gi, RbArgs{0, 0, 0, 1}, valid, a, cu, jb, je, W,
                                                                 t_best, g_best);
                 nelig += elig;
                 const unsigned cm = __ballot_sync(kFull, t_best >= 0);

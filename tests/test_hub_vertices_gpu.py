@@ -4,6 +4,7 @@ import pytest
 
 import oracle
 import synth
+from parity_util import compare_state
 
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
@@ -72,4 +73,21 @@ def test_exact_gains(n, m, k, count, order):
     moves = np.stack([u, a, (a + rng.integers(1, k, u.size)) % k], 1).astype(np.int32)
     h = HGP.from_hypergraph(hg)
     assert np.array_equal(h.exact_gains(moves), oracle.Oracle.from_hypergraph(hg).exact_gains(moves))
+    h.close()
+
+
+@pytest.mark.parametrize("S", [1, 2, 3, 4, 16, 64])
+@pytest.mark.parametrize("k,order", [(4, "falling"), (40, "falling"), (40, "random")])
+def test_rebalancing(S, k, order):
+    """Items of one to six segments, ending inside a tile's list, hubs side by side in the first."""
+    from paper_2010_10272_gb300 import HGP
+    hg = hubs(S + k, 9001, 14_000, k, order, eps=0.05)
+    part = hg.part.copy()
+    part[::3] = 0
+    h = HGP.from_hypergraph(hg, part=part, subrounds=S, seed=2)
+    o = oracle.Oracle.from_hypergraph(hg, part=part, subrounds=S, seed=2)
+    st, ph = h.rebalance(8)
+    want, wph = o.rebalance(8)[:2]
+    assert np.array_equal(st[:, :5], want[:, :5]) and np.array_equal(ph, wph) and len(ph) > 0
+    compare_state(h, o)
     h.close()
