@@ -270,6 +270,8 @@ constexpr int32_t kPlaneMaxW = 2047;   // W(u) up to this uses bit planes (NP <=
 // degrees above this are walked by the whole warp: its two passes cost about as many issue slots
 // as a lane's walk of this length with the other lanes idle
 constexpr int32_t kLaneDeg = 96;
+constexpr int kHubPlanes = 13;         // bit planes of such a walk (with 16, kernels that keep within their
+constexpr int32_t kHubMaxW = (1 << kHubPlanes) - 1;   // registers spill: row-net 2M 3.57 -> 3.66 ms)
 // Segments of a rebalancing item (gain and apply step) with S sub-rounds: about the active vertices of 256
 // consecutive ones.  Its candidates lie together, so a larger item also gives more of a run of hubs to
 // one warp.  Vertices numbered by falling Zipf degree, S = 4, 2 / 3 / 6 segments: 5M 8.2 / 9.3 / 15.5 ms
@@ -440,6 +442,54 @@ __device__ __forceinline__ void count_gain(const Dev &d, bool ok, int key, int32
     if ((int)(threadIdx.x & 31) == __ffs(peers) - 1) atomicAdd(&d.hist[(int64_t)key * kBins + bin], sum);
 }
 
+// The sums conn_t of a vertex of many nets, those of blocks lane and lane + 32 in each lane: every lane
+// adds its nets' weights into bit planes over the blocks of T (as lane_best; with 64 blocks a net has two
+// lanes, one for either half, so that the planes are 32-bit words), and the lanes' planes are added
+// pairwise.  Every net's bits passed around the warp instead (32 steps per 32 nets): 2M vertices, k = 8,
+// numbered by falling degree (3,030 nets at most), gain step of 5 rounds 15.7 -> 9.7 ms with 4 sub-rounds,
+// 57.9 -> 41.1 with 64; 5M power-law, k = 64, 64 sub-rounds 124 -> 107.
+template <typename Lam, typename Rec, bool COH>
+__device__ __forceinline__ void hub_planes(const Rec *recs, const int32_t *inc, int32_t jb, int32_t je, Lam T, int32_t &acc0,
+                                           int32_t &acc1)
+{
+    constexpr bool kWide = sizeof(Lam) == 8;
+    constexpr int NP = kHubPlanes, kNets = kWide ? 16 : 32;   // nets of a step
+    const int lane = threadIdx.x & 31;
+    const uint32_t mine = kWide && lane >= 16 ? hi32(T) : lo32(T);
+    uint32_t c[NP];
+#pragma unroll
+    for (int p = 0; p < NP; ++p) c[p] = 0;
+    for (int32_t j = jb + lane % kNets; j < je; j += kNets) {
+        Lam lam;
+        int32_t w;
+        RecIO<Rec>::template load_b<COH>(recs + (load_inc<COH>(inc, j) & kNetMask), lam, w);
+        const uint32_t x = (kWide && lane >= 16 ? hi32(lam) : lo32(lam)) & mine;
+        uint32_t carry = 0;
+#pragma unroll
+        for (int p = 0; p < NP; ++p) {
+            const uint32_t ad = ((w >> p) & 1) ? x : 0u, cp = c[p];
+            c[p] = cp ^ ad ^ carry;
+            carry = (cp & ad) | (carry & (cp ^ ad));
+        }
+    }
+    __syncwarp();
+#pragma unroll 1
+    for (int o = kNets / 2; o; o >>= 1) {
+        uint32_t carry = 0;
+#pragma unroll
+        for (int p = 0; p < NP; ++p) {
+            const uint32_t ad = __shfl_xor_sync(kFull, c[p], o), cp = c[p];
+            c[p] = cp ^ ad ^ carry;
+            carry = (cp & ad) | (carry & (cp ^ ad));
+        }
+    }
+#pragma unroll
+    for (int p = 0; p < NP; ++p) {
+        acc0 |= (int32_t)((__shfl_sync(kFull, c[p], 0) >> lane) & 1) << p;
+        if (kWide) acc1 |= (int32_t)((__shfl_sync(kFull, c[p], 16) >> lane) & 1) << p;
+    }
+}
+
 // The best target of the vertex in this lane (a = its block, cu its weight, [jb, je) its nets, W their
 // weight, inc the incidence lists): block t_best (-1: none) and its gain; returns eligibility.  The
 // warp calls it together.
@@ -520,7 +570,8 @@ __device__ __forceinline__ bool gain_vertex(const Dev &d, const int32_t *inc, co
         const uint32_t Tlo = lo32(hT), Thi = hi32(hT);
         const int32_t hbw = y.b - hW;
         int32_t acc0 = 0, acc1 = 0;
-        for (int32_t j0 = hjb; j0 < hje; j0 += 32) {
+        if (hW <= kHubMaxW) hub_planes<Lam, Rec, COH>(recs, inc, hjb, hje, hT, acc0, acc1);
+        else for (int32_t j0 = hjb; j0 < hje; j0 += 32) {
             const int32_t j = j0 + lane;
             Lam lam = 0;
             int32_t w = 0;

@@ -91,3 +91,46 @@ def test_rebalancing(S, k, order):
     assert np.array_equal(st[:, :5], want[:, :5]) and np.array_equal(ph, wph) and len(ph) > 0
     compare_state(h, o)
     h.close()
+
+
+@pytest.mark.parametrize("k", [3, 32, 33, 64])
+@pytest.mark.parametrize("net_w", [0, 2, 60, 800_000])
+@pytest.mark.parametrize("variant", [{}, {"balance_moves": True}])
+def test_rounds(k, net_w, variant):
+    """Hubs whose nets weigh up to and more than 8191 (13 bit planes), by the cluster and by the launches."""
+    from paper_2010_10272_gb300 import HGP
+    hg = hubs(k, 700, 6000, k, "falling", net_w=net_w)
+    net = np.repeat(np.arange(hg.m), np.diff(hg.net_off))
+    W = np.bincount(hg.pins, weights=(hg.net_w if net_w else np.ones(hg.m))[net], minlength=hg.n)
+    hub = degrees(hg) > 96
+    assert (W[hub] <= 8191).any() or net_w > 60
+    assert (W[hub] > 8191).any() == (net_w >= 60)
+    o = oracle.Oracle.from_hypergraph(hg, subrounds=2, seed=9, **variant)
+    want, _ = o.refine(3)
+    for debug in (0, 32):
+        h = HGP.from_hypergraph(hg, subrounds=2, seed=9, debug=debug, **variant)
+        assert np.array_equal(h.refine(3)[:, :5], want[:, :5])
+        compare_state(h, o)
+        h.close()
+
+
+@pytest.mark.parametrize("W", [8190, 8191, 8192])
+@pytest.mark.parametrize("k", [2, 40])
+def test_largest_sum_of_the_bit_planes(W, k):
+    """One vertex whose W nets all reach one other block, at the last value the planes hold and beyond."""
+    from paper_2010_10272_gb300 import HGP
+    n = W + 200
+    off = np.arange(0, 2 * W + 1, 2, dtype=np.int64)
+    pins = np.stack([np.zeros(W, np.int32), np.arange(1, W + 1, dtype=np.int32)], 1).reshape(-1)
+    part = np.zeros(n, np.int32)
+    part[1:W + 1] = 1                          # every net of vertex 0 has its other pin there
+    part[W + 1:] = 2 + np.arange(n - W - 1) % (k - 2) if k > 2 else 0
+    vw = np.ones(n, np.int32)
+    vw[W + 1:] = 2000                          # so that the block has room
+    h = HGP(n, W, off, pins, k, 0.99, part, vw, subrounds=1, debug=32)
+    o = oracle.Oracle(n, W, off, pins, k, 0.99, part, vw, subrounds=1)
+    t, g = h.debug_candidates(0)
+    want_t, want_g = o.candidates(0)
+    assert np.array_equal(t, want_t) and np.array_equal(g, want_g)
+    assert (t[0], g[0]) == (1, W)
+    h.close()
