@@ -431,6 +431,12 @@ void hgp_destroy(hgp_handle *h);
  */
 int hgp_set_pool_retention(int64_t bytes);
 
+/* The pool of the current device: bytes in use (by handles, batches, coarse hypergraphs and calls), and
+ * bytes it keeps of what was freed, which the system counts as used but the library's next allocations
+ * take first, and which the driver gives to other allocations that find no free memory.  Either may be
+ * NULL. */
+int hgp_get_pool_usage(int64_t *used, int64_t *kept);
+
 /* Host waits inside the library (read-backs, the end of hgp_create, statistics): on = 0
  * (default) spins in cudaStreamSynchronize; on = 1 sleeps on a blocking-sync event recorded on
  * the stream, which frees the CPU core while the device works (for callers where many threads

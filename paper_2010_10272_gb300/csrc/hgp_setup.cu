@@ -1882,6 +1882,22 @@ int hgp_set_pool_retention(int64_t bytes)
     return HGP_OK;
 }
 
+int hgp_get_pool_usage(int64_t *used, int64_t *kept)
+{
+    cudaMemPool_t pool = nullptr;
+    uint64_t in_use = 0, reserved = 0;
+    cudaError_t e = hgp::library_pool(&pool);
+    if (e == cudaSuccess) e = cudaMemPoolGetAttribute(pool, cudaMemPoolAttrUsedMemCurrent, &in_use);
+    if (e == cudaSuccess) e = cudaMemPoolGetAttribute(pool, cudaMemPoolAttrReservedMemCurrent, &reserved);
+    if (e != cudaSuccess) {
+        (void)cudaGetLastError();
+        return status_of(e);
+    }
+    if (used) *used = (int64_t)in_use;
+    if (kept) *kept = (int64_t)(reserved > in_use ? reserved - in_use : 0);
+    return HGP_OK;
+}
+
 const char *hgp_strerror(int code)
 {
     switch (code) {

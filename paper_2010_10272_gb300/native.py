@@ -130,6 +130,8 @@ def load_library():
             getattr(lib, name).restype = ctypes.c_int
         lib.hgp_set_pool_retention.argtypes = [i64]
         lib.hgp_set_pool_retention.restype = ctypes.c_int
+        lib.hgp_get_pool_usage.argtypes = [P, P]
+        lib.hgp_get_pool_usage.restype = ctypes.c_int
         lib.hgp_batch_destroy.argtypes = [P]
         lib.hgp_batch_destroy.restype = None
         lib.hgp_probe_gather.argtypes = [i64, i64, P, P]
@@ -465,6 +467,14 @@ def set_pool_retention(nbytes: int):
     keeps for reuse (default: 1/64 of the device's memory; 0 = give it back at the next
     synchronisation)."""
     _check(load_library().hgp_set_pool_retention(int(nbytes)), "hgp_set_pool_retention")
+
+
+def pool_usage():
+    """hgp_get_pool_usage: (bytes in use, bytes kept of what was freed) of the library's pool on the
+    current device."""
+    used, kept = ctypes.c_int64(), ctypes.c_int64()
+    _check(load_library().hgp_get_pool_usage(ctypes.byref(used), ctypes.byref(kept)), "hgp_get_pool_usage")
+    return used.value, kept.value
 
 
 def set_blocking_waits(on: bool):

@@ -34,7 +34,7 @@ from typing import Deque, Dict, List, Optional
 
 import numpy as np
 
-from .native import HGP, Batch, set_blocking_waits
+from .native import HGP, Batch, pool_usage, set_blocking_waits
 
 _RANGE = 256
 _TILE = 2048
@@ -123,7 +123,7 @@ class Server:
     """Continuous-batching refinement server for one GPU (see the module docstring).
 
     memory_budget: device bytes the server may hold for requests (default: the free device
-    memory when the server starts, minus reserve_bytes).  max_active: requests refined at once;
+    memory when the server starts, with what the library's pool keeps, minus reserve_bytes).  max_active: requests refined at once;
     max_staged: requests created (or being created) ahead of the batch they will join;
     creators: threads that create and retire request state (0: the serving thread itself);
     ctas_per_sm: persistent grid of the batch's gain and apply kernels (0: by occupancy; fewer
@@ -149,7 +149,8 @@ class Server:
         self.reserve = int(reserve_bytes)
         if memory_budget is None:
             free, _ = torch.cuda.mem_get_info()
-            memory_budget = max(0, int(free) - self.reserve)
+            kept = pool_usage()[1] if torch.cuda.is_available() else 0
+            memory_budget = max(0, int(free) + kept - self.reserve)
         self.memory_budget = int(memory_budget)
         self.max_active = int(max_active)
         self.max_staged = int(max_staged)
