@@ -533,6 +533,10 @@ constexpr int32_t kHostSizesMaxNets = 1 << 20;
 // device inputs with fewer nets than this carve their buffers from one allocation, too (about 30 pool
 // calls at creation otherwise: 256 handles of 1k to 200k vertices 900 -> 55-154 ms)
 constexpr int32_t kDeviceArenaMaxNets = 1 << 18;
+// what such a handle may keep of its creation's scratch and as unused room in Phi.  Given back by all of
+// 256 handles, the holes between them made every later call that waits 5 us longer (set_partition 29 ->
+// 35 us); kept by handles of many vertices it was 8 bytes a vertex.
+constexpr int64_t kKeptSpare = 8 << 20;
 // in internal order, nets of at least kBigNet pins (a prefix) get their own CTAs at creation and
 // initialisation (a power of two: size classes are powers of two)
 
@@ -1317,11 +1321,11 @@ void dev_free(void *p, cudaStream_t st)
 namespace {
 
 template <typename T>
-cudaError_t dalloc(hgp_handle *h, T **p, int64_t count)
+cudaError_t dalloc(hgp_handle *h, T **p, int64_t count, bool in_arena = true)
 {
     *p = nullptr;
     if (count < 1) count = 1;
-    if (void *a = arena_take(h, (size_t)count * sizeof(T))) {
+    if (void *a = in_arena ? arena_take(h, (size_t)count * sizeof(T)) : nullptr) {
         *p = reinterpret_cast<T *>(a);
         return cudaSuccess;
     }
@@ -1385,27 +1389,46 @@ int init_state(hgp_handle *h, const uint8_t *part, const int32_t *guard)
 
 constexpr int kSmallN = 72 + kAccN;   // int64 entries of a handle's small state (see create_impl)
 
-// Device bytes of every buffer create_impl (and the first refine) allocates for a handle of few
-// nets (see kHostSizesMaxNets, kDeviceArenaMaxNets), each rounded up to 256 bytes: the arena
-// those buffers are carved from.  It covers the direct transpose in input net order without
-// wide nets; buffers of any other path (or beyond a miscount) come from the pool instead.
+size_t aligned_bytes(int64_t bytes) { return (size_t)((bytes < 1 ? 1 : bytes) + 255) / 256 * 256; }
+
+// What a creation uses and the handle does not keep: the int64 offsets, the int32 partition, and the scan
+// scratch (block sums, counts).
+struct CreateScratch {
+    int64_t off64, part_in, block_sums, tmp;   // entries
+    CreateScratch(int32_t n, int32_t m)
+    {
+        const int64_t nm = n > m ? n : m;
+        const int64_t nr_ctas = m > 0 ? std::min<int64_t>(((int64_t)m + 2047) / 2048, 1216) : 0;
+        const int64_t scan_count = std::max<int64_t>(nm + 1, kNrRanks * nr_ctas + 1);
+        off64 = (int64_t)m + 1;
+        part_in = n;
+        block_sums = (scan_count + kScanChunk - 1) / kScanChunk + 1;
+        tmp = nm + 1;
+    }
+    size_t bytes() const
+    {
+        return aligned_bytes(8 * off64) + aligned_bytes(4 * part_in) + aligned_bytes(4 * block_sums) + aligned_bytes(4 * tmp);
+    }
+};
+
+// Device bytes of every buffer a handle of few nets (see kHostSizesMaxNets, kDeviceArenaMaxNets) keeps,
+// each rounded up to 256 bytes: the arena those buffers are carved from.  It covers the direct transpose
+// in input net order without wide nets; buffers of any other path (or beyond a miscount) come from the
+// pool instead.  max_size < 0: the largest net is not known yet, and Phi not part of the arena.
 size_t small_handle_bytes(int32_t n, int32_t m, int64_t P, int32_t k, const hgp_options &o, int32_t max_size,
                           bool has_vw, bool has_nw)
 {
-    auto A = [](int64_t bytes) -> size_t { return (size_t)((bytes < 1 ? 1 : bytes) + 255) / 256 * 256; };
+    auto A = [](int64_t bytes) { return aligned_bytes(bytes); };
     const int64_t n_tiles = ((int64_t)n + kTile - 1) / kTile, nseg = segments_of(o.subrounds);
-    const int64_t S = o.subrounds, nm = n > m ? n : m;
+    const int64_t S = o.subrounds;
     const int w = o.phi_width ? o.phi_width : (max_size <= 255 ? 1 : 2);
-    const int64_t nr_ctas = m > 0 ? std::min<int64_t>((m + 2047) / 2048, 1216) : 0;
-    const int64_t scan_count = std::max<int64_t>(nm + 1, kNrRanks * nr_ctas + 1);
-    const int64_t nb = (scan_count + kScanChunk - 1) / kScanChunk;
     size_t b = 0;
-    b += A(8 * (m + 1)) + A(4 * (m + 1)) + A(4 * P) + A(4 * (int64_t)n);   // inputs
+    b += A(4 * ((int64_t)m + 1)) + A(4 * P);                                         // inputs
     if (has_vw) b += A(4 * (int64_t)n);
     if (has_nw) b += A(4 * (int64_t)m) + A(4 * (int64_t)n);                           // and W(u)
-    b += A(4 * (nb + 1)) + A(4 * (nm + 1));                                          // scan scratch
     b += A(4 * ((int64_t)n + 1)) + A(4 * P);                                         // vtx_off, inc
-    b += 2 * A(n) + A(4 * (((int64_t)m * k * w + 7) / 8 * 2)) + A((int64_t)m * (k <= 32 ? 16 : 32)) + A(8 * kSmallN);
+    if (max_size >= 0) b += A(4 * (((int64_t)m * k * w + 7) / 8 * 2));
+    b += 2 * A(n) + A((int64_t)m * (k <= 32 ? 16 : 32)) + A(8 * kSmallN);
     b += A(2 * n_tiles * kTile) + A(2 * n_tiles * (S + 1)) + A(8 * n_tiles * kTile) + A(4 * n_tiles * nseg);
     b += A(8 * (int64_t)k * kBins) + A((int64_t)sizeof(Sel) * 64) + A(8 * (int64_t)k * n_tiles);
     if (o.revert_negative) {
@@ -1518,26 +1541,43 @@ int create_impl(int32_t n, int32_t m, const int64_t *net_offsets, const int32_t 
         if (lo < 0) return fail(HGP_ERR_INVALID);   // then every size is at most P < 2^31
         max_size = (int32_t)hi;
     }
+    const CreateScratch cs(n, m);
+    int64_t *off64 = nullptr;
+    int32_t *part_in = nullptr, *tmp = nullptr, *block_sums = nullptr;
+    // device inputs: the largest net is not known yet, so Phi gets room for 2-byte entries.  That and the
+    // scratch stay with the handle where they are little; else the scratch is an allocation of its own,
+    // given back at the end, and Phi another one.
+    const bool whole = host_sizes || (int64_t)cs.bytes() + (int64_t)m * k <= kKeptSpare;
     if (host_sizes || m < kDeviceArenaMaxNets) {
-        // device inputs: the largest net is not known yet, so Phi gets room for 2-byte entries
-        const size_t bytes = small_handle_bytes(n, m, P, k, o, host_sizes ? max_size : 65535, vertex_w != nullptr,
-                                                net_w != nullptr);
+        const size_t keep = small_handle_bytes(n, m, P, k, o, host_sizes ? max_size : (whole ? 65535 : -1), vertex_w != nullptr,
+                                               net_w != nullptr);
+        const size_t bytes = keep + (whole ? cs.bytes() : 0);
         void *a = nullptr;
         if (dev_alloc(&a, bytes, st) == cudaSuccess) {   // else every buffer comes from the pool
             h->allocs[h->n_allocs++] = a;
             h->arena = static_cast<char *>(a);
             h->arena_size = bytes;
         }
+        if (!whole && dev_alloc(&a, cs.bytes(), st) == cudaSuccess) {
+            h->allocs[h->n_allocs++] = a;                // released as off64's
+            char *at = static_cast<char *>(a);
+            off64 = reinterpret_cast<int64_t *>(at);
+            part_in = reinterpret_cast<int32_t *>(at += aligned_bytes(8 * cs.off64));
+            block_sums = reinterpret_cast<int32_t *>(at += aligned_bytes(4 * cs.part_in));
+            tmp = reinterpret_cast<int32_t *>(at += aligned_bytes(4 * cs.block_sums));
+        }
+    }
+    if (!off64) {
+        CKF(dalloc(h, &off64, cs.off64));
+        CKF(dalloc(h, &part_in, cs.part_in));
+        CKF(dalloc(h, &block_sums, cs.block_sums));
+        CKF(dalloc(h, &tmp, cs.tmp));
     }
 
     // ---- inputs
-    int64_t *off64 = nullptr;
-    int32_t *part_in = nullptr, *tmp = nullptr;
     int32_t *net_off = nullptr, *pins_d = nullptr, *vw_d = nullptr, *nw_d = nullptr;
-    CKF(dalloc(h, &off64, (int64_t)m + 1));
     CKF(dalloc(h, &net_off, (int64_t)m + 1));
     CKF(dalloc(h, &pins_d, P));
-    CKF(dalloc(h, &part_in, n));
     // small state: block weights [64], objective, largest W(u), error flag and largest net (int32
     // each), round state (2 int32), then the sums of a state initialisation; zeroed once
     int64_t *small = nullptr;
@@ -1590,12 +1630,8 @@ int create_impl(int32_t n, int32_t m, const int64_t *net_offsets, const int32_t 
         max_size = host_err[1];
     }
 
-    // ---- scan scratch (shared by the scans below)
-    const int64_t nr_ctas = m > 0 ? (m + 2047) / 2048 < 1216 ? (m + 2047) / 2048 : 1216 : 0;
-    const int64_t scan_count = std::max((int64_t)(n > m ? n : m) + 1, kNrRanks * nr_ctas + 1);
-    const int64_t nb = (scan_count + kScanChunk - 1) / kScanChunk;
-    int32_t *block_sums = nullptr;
-    CKF(dalloc(h, &block_sums, nb + 1));
+    // ---- scans (in block_sums, shared by all of them)
+    const int64_t nr_ctas = m > 0 ? std::min<int64_t>(((int64_t)m + 2047) / 2048, 1216) : 0;
     auto scan = [&](const int32_t *in, int32_t *outp, int64_t count) -> cudaError_t {
         const int64_t blocks = (count + kScanChunk - 1) / kScanChunk;
         const int64_t bl = blocks < 1 ? 1 : blocks;
@@ -1606,7 +1642,6 @@ int create_impl(int32_t n, int32_t m, const int64_t *net_offsets, const int32_t 
     };
 
     // ---- internal net order (largest size class first); the input-order arrays are released
-    CKF(dalloc(h, &tmp, (int64_t)(n > m ? n : m) + 1));
     const int64_t avg_size = m > 0 ? (P + m - 1) / m : 0;
     const bool reorder = m > 0 && !(o.debug & 8) &&
                          ((o.debug & 4) || (m >= kReorderMinNets && max_size >= kReorderSkew * avg_size));
@@ -1762,7 +1797,7 @@ int create_impl(int32_t n, int32_t m, const int64_t *net_offsets, const int32_t 
     const int64_t entries = (int64_t)phi_rows * k;
     const int64_t words = (entries * w + 7) / 8 * 2;
     uint32_t *phi = nullptr;
-    CKF(dalloc(h, &phi, words));
+    CKF(dalloc(h, &phi, words, whole));
     d.phi = phi;   // written whole by init_state
     const size_t rec_bytes = k <= 32 ? sizeof(Rec16) : sizeof(Rec32);
     uint4 *rec = nullptr;

@@ -69,3 +69,24 @@ def test_exact_gains_on_a_nearly_full_device():
         torch.cuda.empty_cache()
         _default_retention()
         h.close()
+
+
+def test_a_handle_keeps_no_creation_scratch():
+    """A handle made from device arrays of few nets and many vertices holds what its rounds use, not the
+    buffers of its creation (8 bytes a vertex more)."""
+    from paper_2010_10272_gb300 import HGP
+    from paper_2010_10272_gb300.native import pool_usage
+    n, m, k = 30_000_000, 1000, 8
+    dev = torch.device("cuda")
+    off = torch.arange(0, 64 * m + 1, 64, dtype=torch.int64, device=dev)
+    pins = (torch.arange(m, device=dev)[:, None] * 29_000 + torch.arange(64, device=dev) * 400).to(torch.int32).reshape(-1)
+    part = (torch.arange(n, device=dev) % k).to(torch.int32)
+    before = pool_usage()[0]
+    h = HGP(n, m, off, pins, k, 0.03, part, device=True)
+    h.refine(1)
+    torch.cuda.synchronize()
+    kept = pool_usage()[0] - before
+    tiles = -(-n // 2048)
+    need = 4 * n + 2 * n + tiles * 2048 * (2 + 8) + 8 * k * tiles + 8 * k * 4096    # offsets, Pi twice, lists, candidates, ties
+    assert need <= kept <= need + (64 << 20)
+    h.close()
