@@ -362,7 +362,7 @@ __global__ void __launch_bounds__(1024) k_nr_pins_big(const int32_t *off_int, co
     __shared__ int32_t win[kBigWin], src[kBigWin];
     __shared__ int32_t first;
     const int32_t p0 = blockIdx.x * kBigChunk;
-    const int32_t p1 = min(off_int[m_big], p0 + kBigChunk);
+    const int32_t len = chunk_length(p0, off_int[m_big], kBigChunk);
     if (threadIdx.x == 0) first = net_of_pin(off_int, m_big, p0);
     __syncthreads();
     if (threadIdx.x < kBigWin) {
@@ -371,7 +371,8 @@ __global__ void __launch_bounds__(1024) k_nr_pins_big(const int32_t *off_int, co
     }
     __syncthreads();
 #pragma unroll 4
-    for (int32_t j = p0 + threadIdx.x; j < p1; j += blockDim.x) {
+    for (int32_t i = threadIdx.x; i < len; i += blockDim.x) {
+        const int32_t j = p0 + i;
         const int sl = win_slot(win, j);
         pins_int[j] = pins[src[sl] + (j - win[sl])];
     }
@@ -557,7 +558,7 @@ __global__ void k_scatter(const int32_t *off, const int32_t *pins, int32_t m, in
     for (int64_t e = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; e < m; e += warps) {
         const int32_t b = off[e], end = off[e + 1];
         const int32_t ef = (int32_t)((uint32_t)e | (end - b > narrow_max ? kWideFlag : 0u));
-        for (int32_t j = b + lane; j < end; j += 32) {
+        for (int64_t j = (int64_t)b + lane; j < end; j += 32) {
             const int32_t pos = atomicAdd(&fill[pins[j]], 1);
             inc[pos] = ef;
         }
@@ -673,9 +674,8 @@ __global__ void __launch_bounds__(kTpThreads) k_tp_scatter_big(const int32_t *of
     __shared__ int32_t cur[kTpMaxBuckets];
     __shared__ int32_t win[kBigWin];
     __shared__ int32_t first;
-    const int32_t p_end = off[m_big];
     const int32_t p0 = blockIdx.x * kBigChunk;
-    const int32_t p1 = min(p_end, p0 + kBigChunk);
+    const int32_t len = chunk_length(p0, off[m_big], kBigChunk);
     if (threadIdx.x == 0) first = net_of_pin(off, m_big, p0);
     for (int i = threadIdx.x; i < nb; i += blockDim.x) cur[i] = 0;
     __syncthreads();
@@ -683,7 +683,8 @@ __global__ void __launch_bounds__(kTpThreads) k_tp_scatter_big(const int32_t *of
     if (threadIdx.x < kBigWin) win[threadIdx.x] = off[min(m_big, e_f + (int32_t)threadIdx.x)];
     __syncthreads();
     for (int pass = 0; pass < 2; ++pass) {
-        for (int32_t j = p0 + threadIdx.x; j < p1; j += blockDim.x) {
+        for (int32_t i = threadIdx.x; i < len; i += blockDim.x) {
+            const int32_t j = p0 + i;
             const int32_t v = pins[j];
             const int32_t pos = atomicAdd(&cur[v >> bshift], 1);
             if (pass == 1) {
@@ -728,11 +729,11 @@ __global__ void __launch_bounds__(1024) k_tp_place(const unsigned long long *pai
     __syncthreads();
     // kTpPlaceBatch pairs per thread are loaded before any is used (the loads' latencies overlap)
     const int32_t step = (int32_t)blockDim.x * kTpPlaceBatch;
-    for (int32_t i0 = p0 + threadIdx.x; i0 < p1; i0 += step) {
+    for (int64_t i0 = (int64_t)p0 + threadIdx.x; i0 < p1; i0 += step) {
         unsigned long long pr[kTpPlaceBatch];
 #pragma unroll
         for (int q = 0; q < kTpPlaceBatch; ++q) {
-            const int32_t i = i0 + q * (int32_t)blockDim.x;
+            const int64_t i = i0 + q * (int32_t)blockDim.x;
             pr[q] = i < p1 ? pairs[i] : ~0ull;            // read again below: keep in L2
         }
 #pragma unroll
@@ -753,11 +754,11 @@ __global__ void __launch_bounds__(1024) k_tp_place(const unsigned long long *pai
     }
     if (bkt == nb - 1 && threadIdx.x == 0) vtx_off[n] = p1;
     __syncthreads();
-    for (int32_t i0 = p0 + threadIdx.x; i0 < p1; i0 += step) {
+    for (int64_t i0 = (int64_t)p0 + threadIdx.x; i0 < p1; i0 += step) {
         unsigned long long pr[kTpPlaceBatch];
 #pragma unroll
         for (int q = 0; q < kTpPlaceBatch; ++q) {
-            const int32_t i = i0 + q * (int32_t)blockDim.x;
+            const int64_t i = i0 + q * (int32_t)blockDim.x;
             pr[q] = i < p1 ? __ldcs(&pairs[i]) : ~0ull;
         }
 #pragma unroll

@@ -21,3 +21,13 @@ def test_range_inside(tmp_path):
     got = run_cpp(tmp_path, "".join(f'printf("%d ", hgp::range_inside({p}ull, {b}ull, {base}ull, {size}ull));'
                                     for p, b, base, size, _ in cases))
     assert [int(x) for x in got] == [c[-1] for c in cases]
+
+
+def test_chunks_of_a_list_that_ends_at_the_largest_index(tmp_path):
+    """The chunks of a pin array of up to 2^31 - 1 entries cover it once, the last one included."""
+    chunk = 8192
+    for end in (1, 8191, 8192, 8193, 2**31 - 1, 2**31 - 8192, 2**31 - 8193, 2**31 - 8191):
+        first = max(0, (end - 1) // chunk - 2)
+        got = run_cpp(tmp_path, "".join(f'printf("%d ", hgp::chunk_length({c * chunk}, {end}, {chunk}));'
+                                        for c in range(first, (end + chunk - 1) // chunk)))
+        assert [int(x) for x in got] == [min(chunk, end - c * chunk) for c in range(first, (end + chunk - 1) // chunk)]
