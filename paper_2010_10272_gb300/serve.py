@@ -28,6 +28,7 @@ from __future__ import annotations
 import collections
 import concurrent.futures
 import dataclasses
+import math
 import threading
 import time
 from typing import Deque, Dict, List, Optional
@@ -36,7 +37,6 @@ import numpy as np
 
 from .native import HGP, Batch, pool_usage, set_blocking_waits
 
-_RANGE = 256
 _TILE = 2048
 _BINS = 4096
 _ALLOC_SLACK = 64 << 20
@@ -49,17 +49,18 @@ def estimate_device_bytes(n: int, m: int, pins: int, k: int, max_net_size: int,
                           phi_width: int = 0) -> int:
     """Peak device bytes hgp_create needs for one hypergraph (mirrors its allocations)."""
     w = phi_width or (1 if max_net_size <= 255 else 2)
-    n_ranges = (n + _RANGE - 1) // _RANGE
-    n_tiles = (n_ranges + 7) // 8
+    tiles = (n + _TILE - 1) // _TILE
+    mean = _TILE / subrounds                                   # segments of a tile's sub-round list
+    seg = int(min(_TILE // 32, max(1, math.ceil((mean + 2 * math.sqrt(mean * (1 - 1 / subrounds))) / 32))))
     rec = 16 if k <= 32 else 32
     b = 0
-    b += (m + 1) * 12 + pins * 8 + (n + 1) * 4 + n * 4 + n     # offsets, pins, inc, vtx_off, part
+    b += (m + 1) * 4 + pins * 8 + (n + 1) * 4 + 2 * n          # offsets, pins, inc, vtx_off, part twice
     b += n * 4 if weighted_vertices else 0
-    b += m * 4 if weighted_nets else 0
-    b += (m * k * w + 3) // 4 * 4 + m * rec                    # Phi, net records
-    b += n_ranges * _RANGE * 9 + n_ranges * (subrounds + 1) * 2 + n_ranges * 4   # sub-round lists, candidates
-    b += k * _BINS * 8 + k * n_tiles * 8 + 64 * 40             # approval scratch
-    b += (max(n, m) + 1) * 4 + n * 4 + (m + 1) * 8            # creation temporaries
+    b += (m + n) * 4 if weighted_nets else 0                   # weights, and W(u)
+    b += (m * k * w + 7) // 8 * 8 + m * rec                    # Phi, net records
+    b += tiles * (_TILE * (2 + 8) + (subrounds + 1) * 2 + seg * 4)    # sub-round lists, candidates
+    b += k * _BINS * 8 + k * tiles * 8 + 64 * 40               # approval scratch
+    b += (max(n, m) + 1) * 4 + n * 4 + (m + 1) * 8             # creation temporaries
     if m >= _REORDER_MIN_NETS and max_net_size >= 8 * -(-pins // max(m, 1)):
         b += m * 4                                            # internal net order: input -> internal ids
     if n > _DIRECT_TRANSPOSE_MAX_N:

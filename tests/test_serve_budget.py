@@ -29,3 +29,18 @@ def test_pool_usage():
     used, kept = pool_usage()
     assert used == before and kept >= live
     set_pool_retention(torch.cuda.mem_get_info()[1] // 64)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("n,m,k,weighted", [(3000, 2000, 2, False), (200_000, 150_000, 40, True), (1_500_000, 1_100_000, 16, True)])
+def test_estimate_covers_a_handle(n, m, k, weighted):
+    import synth
+    from paper_2010_10272_gb300 import HGP
+    from paper_2010_10272_gb300.native import pool_usage
+    from paper_2010_10272_gb300.serve import estimate_device_bytes
+    hg = synth.random_small(n, n, m, k, max_size=6, weighted=weighted)
+    before = pool_usage()[0]
+    h = HGP.from_hypergraph(hg)
+    h.refine(1)
+    assert pool_usage()[0] - before <= estimate_device_bytes(n, m, int(hg.net_off[-1]), k, 6, weighted, weighted)
+    h.close()
