@@ -421,12 +421,12 @@ void hgp_destroy(hgp_handle *h);
  * Memory pool (no counterpart in the paper).  Handles and batches take their device memory
  * from a stream-ordered pool the library keeps per device (allocations and releases are
  * queued on the owner's stream and never synchronise the device, so handles can be created
- * and destroyed while other handles' kernels run).  By default the pool keeps up to 1/64 of the
- * device's memory of what was freed, for the next handles; more than that goes back to the system
- * at the next synchronisation.  When no more memory can be mapped, an allocation takes memory whose
- * release is still queued on another stream and makes its own stream wait for that release; one
- * that fails even so gives back what the pool keeps unused and is tried once more.  This call sets
- * how many bytes the pool of the current device may keep (0: give everything back at the next
+ * and destroyed while other handles' kernels run).  What was freed stays in the pool for the next
+ * handles while the pool holds, in use and kept, at most 1/64 of the device's memory; above that it goes
+ * back to the system at the next synchronisation.  When no more memory can be mapped, an allocation
+ * takes memory whose release is still queued on another stream and makes its own stream wait for that
+ * release; one that fails even so gives back what the pool keeps unused and is tried once more.  This
+ * call sets that size for the pool of the current device, in bytes (0: everything goes back at the next
  * synchronisation).  HGP_ERR_INVALID for bytes < 0.
  */
 int hgp_set_pool_retention(int64_t bytes);

@@ -1040,7 +1040,7 @@ extern "C" int hgp_contract(int32_t n, int32_t m, const int64_t *net_off, const 
     // (2) map and cluster weights
     CT(dev_alloc(reinterpret_cast<void **>(&c->map), sizeof(int32_t) * (size_t)n, st));
     CT(dev_alloc(reinterpret_cast<void **>(&c->vw), sizeof(int32_t) * (size_t)n2, st));
-    CT(dev_alloc(reinterpret_cast<void **>(&w64), sizeof(unsigned long long) * (size_t)(n > mm ? n : mm), st));
+    CT(dev_alloc(reinterpret_cast<void **>(&w64), sizeof(unsigned long long) * (size_t)n2, st));
     CT(cudaMemsetAsync(w64, 0, sizeof(unsigned long long) * (size_t)n2, st));
     k_ct_map<<<grid_of(n, 256), 256, 0, st>>>(cluster, n, cid, vertex_w, c->map, w64);
     k_ct_narrow<<<grid_of(n2, 256), 256, 0, st>>>(w64, n2, c->vw, err);

@@ -26,7 +26,7 @@ namespace hgp {
 constexpr int kSeg = 32;                 // list entries of a segment: one per lane
 constexpr int kWarps = 8;                // warps per tile CTA
 constexpr int kRvSlotBytes = 32;         // one slot of the revert variant's hash table
-constexpr int kWqPerRow = 128;           // work counters per stats row: 64 sub-rounds x 2 kernels
+constexpr int kWqPerRow = 64;            // work counters per stats row: the gain step's, one per sub-round
 constexpr int kThreads = 32 * kWarps;
 // consecutive vertices whose sub-round lists are built together.  A warp takes a list 32 entries
 // (a segment) at a time: the longer the list, the fewer of its segments are partly empty (with
@@ -127,8 +127,8 @@ struct Dev {
     Sel *sel;               // [k]
     int64_t *tie;           // [k * n_tiles] weight of the candidates at the threshold gain
     int64_t *stats;         // [rounds * ST_N]
-    int32_t *wq;            // [rounds * kWqPerRow] work counters of the single-instance persistent
-                            // kernels (nullptr in batches: static assignment)
+    int32_t *wq;            // [rounds * kWqPerRow] work counters of the gain step (a batch's launches
+                            // share one set, passed beside the members' states)
     int32_t *err;
     unsigned long long *acc;  // [kAccN] sums of a state initialisation, zero between them
     uint64_t seed;          // sub-round hash seed

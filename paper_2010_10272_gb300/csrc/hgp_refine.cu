@@ -281,7 +281,6 @@ inline int32_t rb_segments(int32_t S) { return std::min(6, std::max(1, 8 / S)); 
 constexpr int kFeasW = 8;              // vertex weights up to this have a mask of blocks with room
 
 // Per-warp state of the gain step that depends on the instance.
-template <typename Lam>
 struct GainInst {
     int32_t r;           // round number
     int32_t all_elig;    // first round: every vertex eligible
@@ -495,7 +494,7 @@ __device__ __forceinline__ void hub_planes(const Rec *recs, const int32_t *inc, 
 // warp calls it together.
 template <typename Rec, bool RB, bool COH>
 __device__ __forceinline__ bool gain_vertex(const Dev &d, const int32_t *inc, const GainWarp &g,
-                                            const GainInst<typename RecIO<Rec>::Lam> &gi, const RbArgs &rb, bool valid, int32_t a, int32_t cu, int32_t jb, int32_t je,
+                                            const GainInst &gi, const RbArgs &rb, bool valid, int32_t a, int32_t cu, int32_t jb, int32_t je,
                                             int32_t W, int &t_best, int32_t &g_best)
 {
     typedef typename RecIO<Rec>::Lam Lam;
@@ -651,7 +650,7 @@ __device__ __forceinline__ bool gain_vertex(const Dev &d, const int32_t *inc, co
 template <typename Rec, bool RB>
 __device__ __forceinline__ int32_t gain_seg(const Dev &d, int32_t tile, int32_t seg, int32_t seg_end, int32_t s,
                                             const GainWarp &g, uint16_t *picked,
-                                            const GainInst<typename RecIO<Rec>::Lam> &gi, int32_t &nel, const RbArgs &rb)
+                                            const GainInst &gi, int32_t &nel, const RbArgs &rb)
 {
     const int lane = threadIdx.x & 31;
     const bool unit = d.nw == nullptr;
@@ -728,7 +727,7 @@ __device__ __forceinline__ void room_tables(const Dev &d, const int64_t *bw, Gai
 }
 
 template <typename Rec>
-__device__ __forceinline__ void gain_refresh(const Dev &d, GainWarp &g, GainInst<typename RecIO<Rec>::Lam> &gi)
+__device__ __forceinline__ void gain_refresh(const Dev &d, GainWarp &g, GainInst &gi)
 {
     room_tables(d, d.bw, g);
     gi.r = d.rs[0];
@@ -770,12 +769,12 @@ __global__ void __launch_bounds__(kThreads, sizeof(Rec) == 16 || RB ? 4 : 3) k_g
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     if (tid == 0) { cnt_s[0] = 0; cnt_s[1] = 0; warps_done = 0; }
     __syncthreads();   // before any warp adds into them
-    GainInst<Lam> gi;
+    GainInst gi;
     int32_t nelig = 0, ncand = 0;
     int inst_prev = -1;
     const int32_t n_it = (B ? n_items : d0.n_tiles) * per_tile;
     const int32_t warps = gridDim.x * kWarps;
-    int32_t *wq = d0.wq + ((int64_t)rr * 64 + s) * 2;
+    int32_t *wq = d0.wq + (int64_t)rr * kWqPerRow + s;
     int32_t group = blockIdx.x * kWarps + wid;
     while ((int64_t)group * take < n_it) {
         // issued by lane 0 now, read (broadcast) when the items are done
@@ -2288,8 +2287,7 @@ int ensure_stats(hgp_handle *h, int32_t rounds)
     int32_t cap = h->stats_cap ? h->stats_cap : 16;
     while (cap < rounds) cap *= 2;
     int64_t *dev = nullptr, *host = nullptr;
-    // stats rows, then the work counters of the persistent kernels: 64 sub-rounds x (gain, apply)
-    // per row
+    // stats rows, then the gain step's work counters
     const size_t bytes = sizeof(int64_t) * ST_N * (size_t)cap + sizeof(int32_t) * kWqPerRow * (size_t)cap;
     cudaError_t e = cudaSuccess;
     dev = static_cast<int64_t *>(arena_take(h, bytes));

@@ -109,7 +109,6 @@ __global__ void k_scan_final(const int32_t *in, int32_t *out, int64_t count, con
 }
 
 // ------------------------------------------------------------------ validation
-// warp per net: pins in range and strictly increasing; largest net size
 // Warp-wide: the pins of nets e0 .. e0 + 31 (clipped to e_hi) are contiguous; off33 receives
 // their exclusive offsets inside that run (off33[32] = its length) and the run's first pin index
 // is returned.  Lanes then walk the run flattened, one pin each, with pin_net to find the net.
@@ -1219,8 +1218,9 @@ cudaError_t library_pool(cudaMemPool_t *out)
             g_pool[dev] = nullptr;
             return e;
         }
-        // keep up to 1/64 of the device's memory (4.4 GB of 284) between handles: mapping it
-        // afresh and unmapping it at the next synchronisation took as long as the work itself
+        // keep freed memory between handles while the pool holds at most 1/64 of the device's (4.4 GB of
+        // 284), in use and kept: mapping it afresh and unmapping it at the next
+        // synchronisation took as long as the work itself
         // (creating and closing a 5M-vertex level 6.4 -> 3.6 ms, a 500k-pin request 457 -> 261
         // us, contraction of 10M vertices 10.4 -> 6.8 ms).  The reuse policies stay at their defaults:
         // when no more memory can be mapped, memory whose release is still queued on another stream

@@ -18,7 +18,7 @@
 // The records and pin counts live in global memory as in the general path; another SM's updates
 // are read from L2 (RecIO<..>::load_full<true>, atomics), ordered by the cluster barriers.
 //
-// 10k vertices (k = 2, 60k pins, 5 rounds): 740 -> 200 us a call.
+// 10k vertices (k = 2, 60k pins, 5 rounds), new partition and read-back included: 777 -> 239 us a call.
 
 constexpr int kSmWarps = 16;
 constexpr int kSmThreads = 32 * kSmWarps;
@@ -75,8 +75,8 @@ struct SmallCand {
     uint32_t uat;   // offset << 12 | source << 6 | target
 };
 
-// digit of a candidate's key at pass p (the gain's nd digits from the top, inverted so that larger
-// gains come first, then the id's two)
+// A candidate's key: the gain's nd digits, inverted so that larger gains come first, then the id's two.  Pass
+// p of the approval takes its p-th digit from the top.
 __device__ __forceinline__ unsigned long long small_key(int32_t g, int32_t u, int nd)
 {
     const unsigned long long inv = ((1ull << (kSmDigit * nd)) - 1) - (unsigned long long)(uint32_t)g;
@@ -202,7 +202,7 @@ __global__ void __launch_bounds__(kSmThreads, 1) k_small(const Dev d, int32_t ro
     const bool unit = d.nw == nullptr;
     const int32_t S = d.S;
     const bool pow2 = (S & (S - 1)) == 0;
-    GainInst<typename RecIO<Rec>::Lam> gi;
+    GainInst gi;
     const int32_t r0 = d.rs[0], started = d.rs[1];
     for (int i = tid; i < kSmPerHome * kSmRow; i += kSmThreads) (&sh.row[0][0])[i] = 0;
     if (tid < 64) {

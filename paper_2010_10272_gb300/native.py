@@ -463,9 +463,9 @@ def _stats_array(buf, count: int) -> np.ndarray:
 
 
 def set_pool_retention(nbytes: int):
-    """hgp_set_pool_retention: freed device memory the library's pool of the current device
-    keeps for reuse (default: 1/64 of the device's memory; 0 = give it back at the next
-    synchronisation)."""
+    """hgp_set_pool_retention: the size, in use and kept, up to which the library's pool of the current
+    device keeps freed memory for reuse (default: 1/64 of the device's memory; 0 = give it back at
+    the next synchronisation)."""
     _check(load_library().hgp_set_pool_retention(int(nbytes)), "hgp_set_pool_retention")
 
 

@@ -15,7 +15,7 @@ def kept():
     """The pool keeps what was freed, among it arrays of other values."""
     from paper_2010_10272_gb300 import HGP
     from paper_2010_10272_gb300.native import pool_usage, set_pool_retention
-    set_pool_retention(4 << 30)
+    set_pool_retention(1 << 40)               # whatever else is alive
     hg = synth.random_small(1, 400_000, 300_000, 64, max_size=9, weighted=True)
     hs = [HGP.from_hypergraph(hg, revert_negative=True) for _ in range(2)]
     for h in hs:

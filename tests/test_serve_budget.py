@@ -18,7 +18,7 @@ def test_pool_usage():
     import synth
     from paper_2010_10272_gb300 import HGP
     from paper_2010_10272_gb300.native import pool_usage, set_pool_retention
-    set_pool_retention(1 << 30)
+    set_pool_retention(1 << 40)
     hg = synth.random_small(3, 300_000, 200_000, 8, max_size=6)
     before = pool_usage()[0]
     h = HGP.from_hypergraph(hg)
