@@ -1481,13 +1481,16 @@ int create_impl(int32_t n, int32_t m, const int64_t *net_offsets, const int32_t 
     Dev &d = h->d;
     cudaGetDevice(&h->device);
     auto release = [&](void *ptr) {   // frees one of the handle's allocations before the end
-        if (in_arena(h, ptr)) return;
+        if (!ptr || in_arena(h, ptr)) return;
         for (int i = 0; i < h->n_allocs; ++i)
             if (h->allocs[i] == ptr) {
                 dev_free(h->allocs[i], h->stream);
-                h->allocs[i] = nullptr;
+                h->allocs[i] = h->allocs[--h->n_allocs];
+                return;
             }
     };
+    // a temporary from the pool: the handle's until release(), so that a creation that fails frees it
+    auto temporary = [&](auto **ptr, int64_t count) { return dalloc(h, ptr, count, false); };
     if (o.cuda_stream) {
         h->stream = (cudaStream_t)o.cuda_stream;
     } else {
@@ -1651,7 +1654,7 @@ int create_impl(int32_t n, int32_t m, const int64_t *net_offsets, const int32_t 
         const int32_t per_cta = (int32_t)((m + nr_ctas - 1) / nr_ctas);
         const int32_t nslots = (int32_t)(kNrRanks * nr_ctas);
         int32_t *cnt = nullptr, *perm = nullptr, *off_int = nullptr, *pins_int = nullptr, *nw_int = nullptr;
-        CKF(dev_alloc(reinterpret_cast<void **>(&cnt), sizeof(int32_t) * (2 * (size_t)nslots + 1), st));
+        CKF(temporary(&cnt, 2 * (int64_t)nslots + 1));
         int32_t *base = cnt + nslots;
         CKF(dalloc(h, &perm, m));
         CKF(dalloc(h, &off_int, (int64_t)m + 1));
@@ -1673,7 +1676,7 @@ int create_impl(int32_t n, int32_t m, const int64_t *net_offsets, const int32_t 
         h->m_huge = below(kHugeNet);
         for (int i = 0; i < 4; ++i) d.tiny[i] = first[kNrTiny + i];
         int32_t *src_big = nullptr;   // where the pins of the large-net prefix come from
-        if (mb > 0) CKF(dev_alloc(reinterpret_cast<void **>(&src_big), sizeof(int32_t) * (size_t)mb, st));
+        if (mb > 0) CKF(temporary(&src_big, mb));
         k_nr_place<<<(unsigned)nr_ctas, kNrThreads, 0, st>>>(net_off, m, per_cta, base, perm, tmp, mb, src_big);
         h->launches++;
         CKF(scan(tmp, off_int, m));   // sizes in internal order -> offsets (off_int[m] = P)
@@ -1688,8 +1691,8 @@ int create_impl(int32_t n, int32_t m, const int64_t *net_offsets, const int32_t 
             h->launches++;
             CKF(cudaGetLastError());
         }
-        CKF(pool_free(cnt, st));
-        if (src_big) CKF(pool_free(src_big, st));
+        release(cnt);
+        release(src_big);
         h->m_big = mb;
         h->m_big32 = (int32_t)std::min((int64_t)m, ((int64_t)mb + 31) / 32 * 32);
         release(net_off);
@@ -1751,8 +1754,8 @@ int create_impl(int32_t n, int32_t m, const int64_t *net_offsets, const int32_t 
         const int64_t per_cta = std::min<int64_t>(kTpMaxPins, std::max<int64_t>(kTpMinPins, p_rest / kTpMinCtas));
         int32_t *bk = nullptr;           // counts [nbk + 1], offsets [nbk + 1], cursors [nbk]
         unsigned long long *pairs = nullptr;
-        CKF(dev_alloc(reinterpret_cast<void **>(&bk), sizeof(int32_t) * (3 * (size_t)nbk + 2), st));
-        CKF(dev_alloc(reinterpret_cast<void **>(&pairs), sizeof(unsigned long long) * (size_t)P, st));
+        CKF(temporary(&bk, 3 * (int64_t)nbk + 2));
+        CKF(temporary(&pairs, P));
         int32_t *bk_cnt = bk, *bk_off = bk + nbk + 1, *bk_cur = bk + 2 * nbk + 2;
         CKF(cudaMemsetAsync(bk_cnt, 0, sizeof(int32_t) * ((size_t)nbk + 1), st));
         k_tp_hist<<<grid_for(P, 256, 152 * 8), 256, 0, st>>>(pins_d, P, bshift, nbk, bk_cnt, guard); h->launches++;
@@ -1777,8 +1780,8 @@ int create_impl(int32_t n, int32_t m, const int64_t *net_offsets, const int32_t 
         }
         h->launches++;
         CKF(cudaGetLastError());
-        CKF(pool_free(pairs, st));
-        CKF(pool_free(bk, st));
+        release(pairs);
+        release(bk);
     } else {
         CKF(cudaMemsetAsync(vtx_off, 0, sizeof(int32_t) * ((size_t)n + 1), st));
     }

@@ -90,3 +90,43 @@ def test_a_handle_keeps_no_creation_scratch():
     need = 4 * n + 2 * n + tiles * 2048 * (2 + 8) + 8 * k * tiles + 8 * k * 4096    # offsets, Pi twice, lists, candidates, ties
     assert need <= kept <= need + (64 << 20)
     h.close()
+
+
+@pytest.mark.parametrize("skewed", [False, True])
+def test_a_failed_creation_leaves_nothing(skewed):
+    """Creations that run out of memory at one allocation or another free what they had."""
+    from paper_2010_10272_gb300 import HGP, HGPError
+    from paper_2010_10272_gb300.native import pool_usage, set_pool_retention
+    n = m = 4_000_000
+    dev = torch.device("cuda")
+    size = torch.full((m,), 4, dtype=torch.int64, device=dev)
+    first = torch.arange(m, device=dev)
+    if skewed:                                # large nets: internal order
+        size[:40] = 100_000
+    off = torch.zeros(m + 1, dtype=torch.int64, device=dev)
+    off[1:] = torch.cumsum(size, 0)
+    net = torch.repeat_interleave(first, size)
+    pins = (torch.clamp(net, max=n - 100_000) + torch.arange(net.numel(), device=dev) - off[net]).to(torch.int32)
+    part = (torch.arange(n, device=dev) % 16).to(torch.int32)
+    del net, size, first
+    failed = 0
+    try:
+        set_pool_retention(0)
+        for free_mb in list(range(60, 700, 40)) + [1500]:
+            torch.cuda.synchronize()
+            torch.cuda.empty_cache()
+            before = pool_usage()[0]
+            rest = torch.empty(torch.cuda.mem_get_info()[0] - (free_mb << 20), dtype=torch.uint8, device=dev)
+            try:
+                HGP(n, m, off, pins, 16, 0.03, part, device=True).close()
+            except HGPError as e:
+                assert e.code == 2
+                failed += 1
+            torch.cuda.synchronize()
+            assert pool_usage()[0] == before, free_mb
+            del rest
+        assert 3 <= failed <= 16
+    finally:
+        rest = None                          # noqa: F841
+        torch.cuda.empty_cache()
+        _default_retention()
