@@ -326,6 +326,7 @@ int hgp_candidates_noalloc(int32_t n, int32_t m, const int32_t *net_offsets, con
 /*
  * Sets the persistent grids of the handle's gain and apply kernels (CTAs per SM; 0 = derived
  * from occupancy), as the options of the same names do at creation.  Results never depend on
+ * them, and a small instance that runs as one cluster (see hgp_options.debug, bit 5) does not use
  * them.  Waits for the handle's stream; drops a captured CUDA graph.
  */
 int hgp_set_launch_shape(hgp_handle *h, int32_t gain_ctas_per_sm, int32_t apply_ctas_per_sm);

@@ -272,12 +272,18 @@ constexpr int32_t kPlaneMaxW = 2047;   // W(u) up to this uses bit planes (NP <=
 constexpr int32_t kLaneDeg = 96;
 constexpr int kHubPlanes = 13;         // bit planes of such a walk (with 16, kernels that keep within their
 constexpr int32_t kHubMaxW = (1 << kHubPlanes) - 1;   // registers spill: row-net 2M 3.57 -> 3.66 ms)
-// Segments of a rebalancing item (gain and apply step) with S sub-rounds: about the active vertices of 256
-// consecutive ones.  Its candidates lie together, so a larger item also gives more of a run of hubs to
-// one warp.  Vertices numbered by falling Zipf degree, S = 4, 2 / 3 / 6 segments: 5M 8.2 / 9.3 / 15.5 ms
-// (exponent 0.5), 55 / 61 / 84 (0.75); power-law 5M with few hubs 2.44 / 2.25 / 2.43; S = 16, 1 / 2 / 6:
-// 12.0 / 15.2 / 20.3 (0.5).
-inline int32_t rb_segments(int32_t S) { return std::min(6, std::max(1, 8 / S)); }
+// Segments of a rebalancing item, of the gain and of the apply step alike, with S sub-rounds: the active
+// vertices of 256, 384 or 512 consecutive ids, as `share`, the vertices per warp of the apply step, grows.
+// Its candidates lie together, so a larger item fills more lanes but also gives more of a run of hubs to
+// one warp.  S = 4, ms a call with 2 / 3 / 4 segments (and with 6 in the gain and up to 9 in the apply step):
+// planted 2M (share 411) 0.40 / 0.44 / 0.45 (0.48); power-law 5M (1,028) 1.79 / 1.67 / 1.71 (1.88) and
+// numbered by falling Zipf degree 7.9 / 9.0 / 10.2 (15.2); 10M 2.93 / 2.68 / 2.60 (2.84); 50M (10,280)
+// 13.3 / 12.0 / 11.2 (11.3), falling 32 / 35 / 37 (51).  S = 16, 5M falling, 1 / 2 / 6: 12.0 / 15.2 / 20.3.
+inline int32_t rb_segments(int32_t S, int64_t share)
+{
+    const int32_t ids = share < 640 ? 256 : (share < 3200 ? 384 : 512);
+    return std::min(6, std::max(1, ids / (kSeg * S)));
+}
 constexpr int kFeasW = 8;              // vertex weights up to this have a mask of blocks with room
 
 // Per-warp state of the gain step that depends on the instance.
@@ -2573,7 +2579,7 @@ extern "C" int hgp_rebalance(hgp_handle *h, int32_t max_passes, hgp_round_stats 
         rb.r = (1 << 30) + pass;
         rb.phase = phase;
         rb.off = phase == 2 ? (int32_t)off : 0;
-        rb.segs = rb_segments(h->d.S);
+        rb.segs = rb_segments(h->d.S, h->d.n / ((int64_t)p.grid_apply * kWarps));
         const int64_t top = phase == 2 ? 2 * off : off;   // largest priority
         const bool levels = top >= kBins - 1;
         const int32_t bins = (int32_t)std::min<int64_t>(kBins, (top + kThreads) / kThreads * kThreads);

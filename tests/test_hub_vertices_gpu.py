@@ -134,3 +134,25 @@ def test_largest_sum_of_the_bit_planes(W, k):
     assert np.array_equal(t, want_t) and np.array_equal(g, want_g)
     assert (t[0], g[0]) == (1, W)
     h.close()
+
+
+@pytest.mark.parametrize("n,S", [(800_001, 1), (800_001, 3), (800_001, 4), (4_000_001, 4)])
+def test_rebalancing_with_larger_items(n, S):
+    """Items of up to 384 and 512 ids' active vertices: many vertices per warp (one CTA per SM)."""
+    from paper_2010_10272_gb300 import HGP
+    rng = np.random.default_rng(S)
+    m, k = n // 4, 5
+    pins = np.sort(rng.integers(0, n, (m, 3), dtype=np.int32), 1)
+    pins = pins[(np.diff(pins, axis=1) > 0).all(1)]
+    m = len(pins)
+    off = np.arange(0, 3 * m + 1, 3, dtype=np.int64)
+    part = rng.integers(0, k, n).astype(np.int32)
+    part[rng.random(n) < 0.3] = 2
+    args = (n, m, off, np.ascontiguousarray(pins.reshape(-1)), k, 0.03, part)
+    h = HGP(*args, subrounds=S, apply_ctas_per_sm=1)
+    o = oracle.Oracle(*args, subrounds=S)
+    st, ph = h.rebalance(6)
+    want, wph = o.rebalance(6)[:2]
+    assert np.array_equal(st[:, :5], want[:, :5]) and np.array_equal(ph, wph)
+    assert np.array_equal(h.partition(), o.partition())
+    h.close()
