@@ -1291,25 +1291,26 @@ cudaError_t dev_alloc(void **p, size_t bytes, cudaStream_t st)
 
 bool readable_in_place(const void *p, size_t bytes, int device)
 {
-    typedef CUresult (*Range)(CUdeviceptr *, size_t *, CUdeviceptr);
-    static const Range range = [] {
+    typedef CUresult (*Query)(unsigned, CUpointer_attribute *, void **, CUdeviceptr);
+    static const Query query = [] {
         void *f = nullptr;
         cudaDriverEntryPointQueryResult found;
-        if (cudaGetDriverEntryPointByVersion("cuMemGetAddressRange", &f, 12000, cudaEnableDefault, &found) != cudaSuccess) {
+        if (cudaGetDriverEntryPointByVersion("cuPointerGetAttributes", &f, 12000, cudaEnableDefault, &found) != cudaSuccess) {
             (void)cudaGetLastError();
             f = nullptr;
         }
-        return reinterpret_cast<Range>(f);
+        return reinterpret_cast<Query>(f);
     }();
-    cudaPointerAttributes at;
-    if (!range || cudaPointerGetAttributes(&at, p) != cudaSuccess) {
-        (void)cudaGetLastError();
-        return false;
-    }
+    // one call for all of them; what an address does not have stays zero
+    unsigned type = 0, managed = 0;
+    int owner = -1;
     CUdeviceptr base = 0;
     size_t size = 0;
-    return at.type == cudaMemoryTypeDevice && at.device == device &&
-           range(&base, &size, (CUdeviceptr)p) == CUDA_SUCCESS && range_inside((uintptr_t)p, bytes, (uintptr_t)base, size);
+    CUpointer_attribute what[] = {CU_POINTER_ATTRIBUTE_MEMORY_TYPE, CU_POINTER_ATTRIBUTE_IS_MANAGED, CU_POINTER_ATTRIBUTE_DEVICE_ORDINAL,
+                                  CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, CU_POINTER_ATTRIBUTE_RANGE_SIZE};
+    void *to[] = {&type, &managed, &owner, &base, &size};
+    return query && query(5, what, to, (CUdeviceptr)p) == CUDA_SUCCESS && type == CU_MEMORYTYPE_DEVICE && !managed &&
+           owner == device && range_inside((uintptr_t)p, bytes, (uintptr_t)base, size);
 }
 
 void dev_free(void *p, cudaStream_t st)
