@@ -1257,8 +1257,8 @@ extern "C" void hgp_coarse_destroy(hgp_coarse *c)
     const bool other = cudaGetDevice(&now) == cudaSuccess && now != c->device;
     if (other) cudaSetDevice(c->device);
     cudaDeviceSynchronize();
-    for (void *p : coarse_arrays(c))
-        if (p) cudaFree(p);
+    for (void *p : coarse_arrays(c))   // on the default stream (cudaFree would leave the pool's count of used bytes as it was)
+        if (p && cudaFreeAsync(p, nullptr) != cudaSuccess) cudaFree(p);
     if (other) cudaSetDevice(now);
     (void)cudaGetLastError();
     delete c;

@@ -44,3 +44,18 @@ def test_released_after_its_stream_was_destroyed():
         assert min(free[1:]) >= free[0] - (64 << 20)
     finally:
         set_pool_retention(torch.cuda.mem_get_info()[1] // 64)
+
+
+def test_released_arrays_are_the_pools_again():
+    from paper_2010_10272_gb300.native import pool_usage, set_pool_retention
+    set_pool_retention(1 << 40)
+    hg = synth.random_small(12, 200_000, 120_000, 2, max_size=6)
+    cluster = (np.arange(hg.n) // 2).astype(np.int32)
+    before = pool_usage()[0]
+    c = _contract(hg, cluster, None)
+    live = pool_usage()[0] - before
+    assert live > 4 * c.num_pins
+    c.close()
+    used, kept = pool_usage()
+    assert used == before and kept >= live
+    set_pool_retention(torch.cuda.mem_get_info()[1] // 64)
