@@ -1256,9 +1256,10 @@ extern "C" void hgp_coarse_destroy(hgp_coarse *c)
     int now = 0;
     const bool other = cudaGetDevice(&now) == cudaSuccess && now != c->device;
     if (other) cudaSetDevice(c->device);
-    cudaDeviceSynchronize();
-    for (void *p : coarse_arrays(c))   // on the default stream (cudaFree would leave the pool's count of used bytes as it was)
-        if (p && cudaFreeAsync(p, nullptr) != cudaSuccess) cudaFree(p);
+    // (a device that cannot be waited for, as during a stream capture, keeps them, as cudaFree would)
+    if (cudaDeviceSynchronize() == cudaSuccess)
+        for (void *p : coarse_arrays(c))   // on the default stream; cudaFree would not count them as given back
+            if (p && cudaFreeAsync(p, nullptr) != cudaSuccess) cudaFree(p);
     if (other) cudaSetDevice(now);
     (void)cudaGetLastError();
     delete c;
